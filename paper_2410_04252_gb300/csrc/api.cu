@@ -95,6 +95,7 @@ GatePassArgs gate_args(int n, const GatePass &gp) {
     a.area = gp.area;
     a.mem_begin = gp.mem_begin;
     a.mem_end = gp.mem_end;
+    a.dense = gp.dense;
     return a;
 }
 
@@ -124,13 +125,17 @@ struct QsuEntry {
     uint64_t key = 0;
     QsuPlan plan;
     std::vector<GatePassArgs> args;
-    DevBuf ops, gparam, csr_off, csr_idx, phases, steps, dblocks, dmembers;
+    DevBuf ops, gparam, csr_off, csr_idx, phases, steps, dblocks, dmembers, prep, pargs, imoffs;
+    std::vector<uint64_t> image;    // register-blocked passes: offset of the pass's tables, else unused
+    size_t image_bytes = 0;         // of one direction
+    int nimages = 0;
     int m = 0, np = 0;
     double plan_ms = 0;
     uint64_t last_use = 0;
     void release() {
         ops.release(); gparam.release(); csr_off.release(); csr_idx.release(); phases.release(); steps.release();
-        dblocks.release(); dmembers.release();
+        dblocks.release(); dmembers.release(); prep.release();
+        pargs.release(); imoffs.release();
     }
 };
 
@@ -164,7 +169,7 @@ struct sv_handle {
     uint64_t tick = 0;
     std::vector<std::unique_ptr<QsuEntry>> qsu;
     std::vector<std::unique_ptr<EvcEntry>> evc, hps;
-    DevBuf params, coef, mats, part, slotval, opval, grad, scal, per_term, status;
+    DevBuf params, coef, mats, pmats, images, part, slotval, opval, grad, scal, per_term, status;
     // forward bookkeeping for SV_FORWARD_DONE
     uint64_t last_qsu_key = 0;
     bool forward_valid = false;
@@ -396,12 +401,25 @@ sv_status get_qsu(sv_handle *h, const sv_gate *gates, size_t m, size_t np, sv_sc
     ent->key = key;
     ent->m = (int)m;
     ent->np = (int)np;
-    for (auto &gp : ent->plan.passes) ent->args.push_back(gate_args(h->n, gp));
+    std::vector<GatePassArgs> rargs;
+    std::vector<uint64_t> roffs;
+    for (auto &gp : ent->plan.passes) {
+        ent->args.push_back(gate_args(h->n, gp));
+        ent->image.push_back(ent->image_bytes);
+        if (gp.ph_begin < 0) continue;
+        rargs.push_back(ent->args.back());
+        roffs.push_back(ent->image_bytes);
+        ent->image_bytes += reg_image_bytes(h->dt, ent->args.back());
+    }
+    ent->nimages = (int)rargs.size();
+    SV_CK(upload(ent->pargs, rargs, h->stream));
+    SV_CK(upload(ent->imoffs, roffs, h->stream));
     SV_CK(upload(ent->ops, ent->plan.ops, h->stream));
     SV_CK(upload(ent->phases, ent->plan.phases, h->stream));
     SV_CK(upload(ent->steps, ent->plan.steps, h->stream));
     SV_CK(upload(ent->dblocks, ent->plan.dblocks, h->stream));
     SV_CK(upload(ent->dmembers, ent->plan.dmembers, h->stream));
+    SV_CK(upload(ent->prep, ent->plan.prep, h->stream));
     std::vector<int32_t> gparam(m);
     for (size_t i = 0; i < m; ++i) gparam[i] = gates[i].param;
     bool parametric_kind[8] = {true, true, false, true, true, false, false, false};
@@ -454,7 +472,10 @@ sv_status evc_entry_upload(sv_handle *h, EvcEntry *ent, const double *coeffs, si
         ss[i].coef = ent->plan.strings[i].coef;
         ss[i].nY = ent->plan.strings[i].nY;
         ss[i].bz = ent->plan.strings[i].bz;
+        ss[i].pad = 0;
     }
+    for (auto &g : ent->plan.groups)
+        for (int32_t q = g.s_begin; q < g.s_end; ++q) ss[q].X = g.X;
     SV_CK(upload(ent->groups, gs, h->stream));
     SV_CK(upload(ent->strings, ss, h->stream));
     SV_CK(upload(ent->term_slot, ent->plan.term_slot, h->stream));
@@ -523,8 +544,9 @@ sv_status get_evc(sv_handle *h, const sv_pauli *p, const double *c, size_t nterm
     return SV_OK;
 }
 
+// dir0, ndirs: the directions whose pass tables are made (0 forward, 1 reverse)
 sv_status upload_params(sv_handle *h, QsuEntry *q, const double *params, size_t np, const double *mats,
-                        size_t nmats, sv_stats *st) {
+                        size_t nmats, int dir0, int ndirs, sv_stats *st) {
     for (size_t i = 0; i < np; ++i)
         if (!std::isfinite(params[i])) return fail(SV_EINVAL, "non-finite parameter");
     std::vector<double> pv(params, params + np);
@@ -545,6 +567,20 @@ sv_status upload_params(sv_handle *h, QsuEntry *q, const double *params, size_t 
         }
     } else {
         SV_CK(h->mats.ensure(16));
+    }
+    SV_CK(h->images.ensure(std::max<size_t>(2 * q->image_bytes, 16)));
+    if (q->nimages) {
+        Rec r(h, st, SV_K_AUX, 0.0);
+        SV_CK(launch_reg_image(h->dt, h->stream, q->pargs.as<GatePassArgs>(), q->imoffs.as<uint64_t>(), q->nimages,
+                               q->ops.as<DevOp>(), q->phases.as<Phase>(), q->steps.as<RegStep>(), h->coef.p,
+                               q->dblocks.as<DiagBlock>(), q->dmembers.as<DiagMember>(), h->images.p, q->image_bytes,
+                               dir0, ndirs));
+    }
+    SV_CK(h->pmats.ensure(std::max<size_t>((size_t)q->plan.prep_elems * h->es, 16)));
+    if (!q->plan.prep.empty()) {
+        Rec r(h, st, SV_K_AUX, 0.0);
+        SV_CK(launch_prep_mats(h->dt, h->stream, q->prep.as<PrepMat>(), (int)q->plan.prep.size(), h->mats.p,
+                               h->pmats.p));
     }
     return SV_OK;
 }
@@ -587,16 +623,14 @@ sv_status run_forward(sv_handle *h, QsuEntry *q, sv_stats *st) {
         }
         for (; pi < P.passes.size() && P.passes[pi].tile == (int)t; ++pi) {
             const GatePassArgs &a = q->args[pi];
-            int grid = gate_pass_grid(h->dt, a.k, a.nlow, a.op_end - a.op_begin, threads, h->opt.blocks_per_sm);
-            uint64_t ntiles = 1ull << a.nout;
-            if ((uint64_t)grid > ntiles) grid = (int)ntiles;
             if (a.ph_begin >= 0) {
                 Rec r(h, st, SV_K_GATE, 2.0 * (double)h->state_bytes());
-                const int rg = (int)std::min<uint64_t>(ntiles, (uint64_t)device_sms());
-                SV_CK(launch_gate_reg(h->dt, h->stream, rg, h->psi, a, q->ops.as<DevOp>(), q->phases.as<Phase>(),
-                                      q->steps.as<RegStep>(), h->coef.p, h->mats.p, q->dblocks.as<DiagBlock>(),
-                                      q->dmembers.as<DiagMember>()));
+                const int rg = reg_pass_grid(h->dt, a, false, h->opt.blocks_per_sm);
+                SV_CK(launch_gate_reg(h->dt, h->stream, rg, h->psi, a, h->images.as<char>() + q->image[pi], h->pmats.p));
             } else {
+                int grid = gate_pass_grid(h->dt, a.k, a.nlow, a.op_end - a.op_begin, threads, h->opt.blocks_per_sm);
+                const uint64_t ntiles = 1ull << a.nout;
+                if ((uint64_t)grid > ntiles) grid = (int)ntiles;
                 Rec r(h, st, SV_K_GATE, 2.0 * (double)h->state_bytes());
                 SV_CK(launch_gate_pass(h->dt, h->stream, grid, threads, h->psi, a, q->ops.as<DevOp>(), h->coef.p,
                                        h->mats.p));
@@ -620,7 +654,10 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
     const int nslots = (int)P.strings.size();
     int E = 1;
     for (auto &cp : P.passes) E = std::max(E, 1 << (cp.kl + cp.m));
-    const int grid = coset_grid(h->dt, E, h->opt.blocks_per_sm, false);
+    // a small state's cosets are shared by several CTAs; every pass then writes a row per coset
+    bool slices = !e->args.empty();
+    for (auto &a : e->args) slices = slices && coset_slices_pay(h->dt, a) && a.nfree == e->args[0].nfree;
+    const int grid = slices ? 1 << e->args[0].nfree : coset_grid(h->dt, E, h->opt.blocks_per_sm, false);
     SV_CK(h->part.ensure((size_t)grid * std::max(nslots, 1) * sizeof(double)));
     SV_CK(h->slotval.ensure(std::max(nslots, 1) * sizeof(double)));
     SV_CK(h->scal.ensure(4 * sizeof(double)));
@@ -634,6 +671,11 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
         }
         for (int pi = P.tile_pass_begin[t]; pi < P.tile_pass_end[t]; ++pi) {
             Rec r(h, st, SV_K_EVC, (double)h->state_bytes());
+            if (slices) {
+                SV_CK(launch_evc_slice(h->dt, h->stream, h->psi, e->args[pi], e->strings.as<DevString>(),
+                                       h->part.as<double>(), nslots));
+                continue;
+            }
             SV_CK(launch_evc_pass(h->dt, h->stream, grid, h->psi, e->args[pi], e->groups.as<DevGroup>(),
                                   e->strings.as<DevString>(), h->part.as<double>(), nslots, h->status.as<int>(),
                                   (long long)h->opt.wait_limit));
@@ -668,7 +710,8 @@ sv_status run_hpsi(sv_handle *h, EvcEntry *e, sv_stats *st) {
     int E = 1;
     for (auto &cp : P.passes) E = std::max(E, 1 << (cp.kl + cp.m));
     const int grid = coset_grid(h->dt, E, h->opt.blocks_per_sm, true);
-    SV_CK(h->part.ensure((size_t)grid * sizeof(double) + 64));
+    SV_CK(h->part.ensure((size_t)std::max(grid, 2 * device_sms()) * sizeof(double) + 64));
+    int rows = grid;         // energy partials of the last pass
     SV_CK(h->scal.ensure(4 * sizeof(double)));
     const int np = (int)P.passes.size();
     if (np == 0) {
@@ -678,13 +721,18 @@ sv_status run_hpsi(sv_handle *h, EvcEntry *e, sv_stats *st) {
     }
     for (int pi = 0; pi < np; ++pi) {
         Rec r(h, st, SV_K_HPSI, (pi == 0 ? 2.0 : 3.0) * (double)h->state_bytes());
+        if (coset_slices_pay(h->dt, e->args[pi])) {
+            SV_CK(launch_hpsi_slice(h->dt, h->stream, h->psi, h->lam, e->args[pi], e->strings.as<DevString>(), pi == 0,
+                                    pi == np - 1, h->part.as<double>(), &rows));
+            continue;
+        }
         SV_CK(launch_hpsi_pass(h->dt, h->stream, grid, h->psi, h->lam, e->args[pi], e->groups.as<DevGroup>(),
                                e->strings.as<DevString>(), pi == 0, pi == np - 1, h->part.as<double>(),
                                h->status.as<int>(), (long long)h->opt.wait_limit));
     }
     {
         Rec r(h, st, SV_K_AUX, 0.0);
-        SV_CK(launch_reduce_rows(h->stream, h->part.as<double>(), grid, 1, 0, 1, h->scal.as<double>() + 1));
+        SV_CK(launch_reduce_rows(h->stream, h->part.as<double>(), rows, 1, 0, 1, h->scal.as<double>() + 1));
     }
     if (st) st->hpsi_passes = np;
     return SV_OK;
@@ -695,8 +743,17 @@ sv_status run_reverse(sv_handle *h, QsuEntry *q, sv_stats *st) {
     const int threads = adj_threads(h);
     const int nops = (int)P.ops.size();
     int grid = 1;
-    for (auto &a : q->args)
-        grid = std::max(grid, adj_pass_grid(h->dt, a.k, a.nlow, a.op_end - a.op_begin, threads, h->opt.blocks_per_sm));
+    // one grid for all passes, so that every pass writes the same partial rows
+    for (auto &a : q->args) {
+        int ga;
+        if (a.ph_begin >= 0 && !a.dense) {
+            ga = reg_pass_grid(h->dt, a, true, h->opt.blocks_per_sm);
+        } else {
+            ga = adj_pass_grid(h->dt, a.k, a.nlow, a.op_end - a.op_begin, threads, h->opt.blocks_per_sm);
+            ga = (int)std::min<uint64_t>((uint64_t)ga, 1ull << a.nout);
+        }
+        grid = std::max(grid, ga);
+    }
     SV_CK(h->part.ensure((size_t)grid * std::max(nops, 1) * sizeof(double)));
     SV_CK(h->opval.ensure(std::max(nops, 1) * sizeof(double)));
     SV_CK(h->grad.ensure(std::max(q->np, 1) * sizeof(double)));
@@ -712,11 +769,10 @@ sv_status run_reverse(sv_handle *h, QsuEntry *q, sv_stats *st) {
                                               c.host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, h->stream));
                     }
             Rec r(h, st, SV_K_ADJ, 4.0 * (double)h->state_bytes());
-            if (a.ph_begin >= 0)
-                SV_CK(launch_adj_reg(h->dt, h->stream, grid, h->psi, h->lam, a, q->ops.as<DevOp>(),
-                                     q->phases.as<Phase>(), q->steps.as<RegStep>(), h->coef.p, h->mats.p,
-                                     h->part.as<double>(), nops, q->dblocks.as<DiagBlock>(),
-                                     q->dmembers.as<DiagMember>()));
+            if (a.ph_begin >= 0 && !a.dense)
+                SV_CK(launch_adj_reg(h->dt, h->stream, grid, h->psi, h->lam, a,
+                                     h->images.as<char>() + q->image_bytes + q->image[pi], h->pmats.p,
+                                     h->part.as<double>(), nops));
             else
                 SV_CK(launch_adj_pass(h->dt, h->stream, grid, threads, h->psi, h->lam, a, q->ops.as<DevOp>(),
                                       h->coef.p, h->mats.p, h->part.as<double>(), nops));
@@ -819,7 +875,7 @@ void sv_destroy(sv_handle *h) {
     for (auto &e : h->qsu) e->release();
     for (auto &e : h->evc) e->release();
     for (auto &e : h->hps) e->release();
-    for (DevBuf *b : {&h->params, &h->coef, &h->mats, &h->part, &h->slotval, &h->opval, &h->grad, &h->scal,
+    for (DevBuf *b : {&h->params, &h->coef, &h->mats, &h->pmats, &h->images, &h->part, &h->slotval, &h->opval, &h->grad, &h->scal,
                       &h->per_term, &h->status})
         b->release();
     h->drop_ckpts();
@@ -951,7 +1007,7 @@ sv_status sv_apply_circuit(sv_handle *h, const sv_gate *gates, size_t m, const d
     SV_TRY(ensure_psi(h));
     QsuEntry *q = nullptr;
     SV_TRY(get_qsu(h, gates, m, np, sched, &q, st));
-    SV_TRY(upload_params(h, q, params, np, mats, nmats, st));
+    SV_TRY(upload_params(h, q, params, np, mats, nmats, 0, 1, st));
     SV_TRY(run_forward(h, q, st));
     h->last_qsu_key = q->key;
     h->forward_valid = true;
@@ -1025,11 +1081,11 @@ sv_status sv_grad(sv_handle *h, const sv_gate *gates, size_t m, const double *pa
         uint64_t gk = qsu_key(h, gates, m, np, sched);
         (void)gk;
         if (q->m != (int)m || q->np != (int)np) return fail(SV_ESTATE, "SV_FORWARD_DONE with a different circuit");
-        SV_TRY(upload_params(h, q, params, np, mats, nmats, st));
+        SV_TRY(upload_params(h, q, params, np, mats, nmats, 1, 1, st));
         SV_TRY(relayout(h, q->plan.final_l2p, false, st));
     } else {
         SV_TRY(get_qsu(h, gates, m, np, sched, &q, st));
-        SV_TRY(upload_params(h, q, params, np, mats, nmats, st));
+        SV_TRY(upload_params(h, q, params, np, mats, nmats, 0, 2, st));
         SV_TRY(run_forward(h, q, st));
     }
     EvcEntry *e = nullptr;
@@ -1233,6 +1289,7 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
     const int hio = std::max(8, kmax - o.low_bits);
     PlanOptions po = plan_options(o);
     po.max_diag = 0;                     // the batched kernel applies RZ / CZ one by one
+    po.reg_threads = 512;
     po.reg_pairs = false;                // and runs register phases of RY / RZ / CZ / 1-qubit matrices only
     std::vector<int32_t> l2p(n);
     for (int q = 0; q < n; ++q) l2p[q] = q;
@@ -1314,7 +1371,10 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
         ss[i].coef = H.strings[i].coef;
         ss[i].nY = H.strings[i].nY;
         ss[i].bz = H.strings[i].bz;
+        ss[i].pad = 0;
     }
+    for (auto &g : H.groups)
+        for (int32_t q = g.s_begin; q < g.s_end; ++q) ss[q].X = g.X;
     std::vector<int32_t> order(batch);
     for (int b = 0; b < batch; ++b) order[b] = b;
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return gsize[x] > gsize[y]; });

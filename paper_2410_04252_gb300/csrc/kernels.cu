@@ -233,10 +233,6 @@ __device__ __forceinline__ DevOp resolve_out(DevOp op, uint64_t gbase) {
     return op;
 }
 
-__device__ __forceinline__ bool has_out_target(const DevOp &op) {
-    return op.t[0] >= kOutTarget || (op.kind == SV_CZ && op.t[1] >= kOutTarget);
-}
-
 template <typename R>
 __device__ void apply_op(Cx<R> *t, int k, const DevOp &op, const R *coef, const Cx<R> *mats, bool adj) {
     const uint32_t T = 1u << k;
@@ -836,9 +832,9 @@ __device__ __forceinline__ void phase_index(uint32_t rmask, int k, uint32_t &bas
 // The thread's tile bits outside rmask when the lane bits of the thread
 // index hold the tile bits in `lanes` (ascending) and the other thread index
 // bits hold the remaining non-register bits (ascending).
-__device__ __forceinline__ uint32_t phase_base(uint32_t rmask, uint32_t lanes, int k) {
+__device__ __forceinline__ uint32_t phase_base(uint32_t rmask, uint32_t lanes, int k, uint32_t t) {
     const uint32_t all = (k >= 32) ? 0xFFFFFFFFu : ((1u << k) - 1u);
-    uint32_t base = 0, t = threadIdx.x;
+    uint32_t base = 0;
     for (uint32_t m = lanes; m; m &= m - 1, t >>= 1)
         if (t & 1u) base |= m & (0u - m);
     for (uint32_t m = all & ~rmask & ~lanes; m; m &= m - 1, t >>= 1)
@@ -1064,31 +1060,6 @@ __device__ __forceinline__ R ra_pair_grad(const RA<R> *p, const RA<R> *l) {
     return g;
 }
 
-// Givens rotation on register bits (A, B), A holding the "1" of u; and the
-// double excitation on the four register bits with u's pair MU.
-#define SV_GIVENS_SWITCH(ra, rb, CALL)                                                       \
-    switch ((ra) * 4 + (rb)) {                                                               \
-    case 1: CALL(1, 2); break;   case 2: if constexpr (RB > 2) { CALL(1, 4); } break;        \
-    case 3: if constexpr (RB > 3) { CALL(1, 8); } break;                                     \
-    case 4: CALL(2, 1); break;   case 6: if constexpr (RB > 2) { CALL(2, 4); } break;        \
-    case 7: if constexpr (RB > 3) { CALL(2, 8); } break;                                     \
-    case 8: if constexpr (RB > 2) { CALL(4, 1); } break;                                     \
-    case 9: if constexpr (RB > 2) { CALL(4, 2); } break;                                     \
-    case 11: if constexpr (RB > 3) { CALL(4, 8); } break;                                    \
-    case 12: if constexpr (RB > 3) { CALL(8, 1); } break;                                    \
-    case 13: if constexpr (RB > 3) { CALL(8, 2); } break;                                    \
-    case 14: if constexpr (RB > 3) { CALL(8, 4); } break;                                    \
-    default: break;                                                                          \
-    }
-#define SV_DEXC_SWITCH(mu, CALL)                                                             \
-    if constexpr (RB == 4) {                                                                 \
-        switch (mu) {                                                                        \
-        case 3: CALL(3, 12); break;  case 5: CALL(5, 10); break;  case 6: CALL(6, 9); break; \
-        case 9: CALL(9, 6); break;   case 10: CALL(10, 5); break; case 12: CALL(12, 3); break; \
-        default: break;                                                                      \
-        }                                                                                    \
-    }
-
 // Four values reduced over a warp at once: lane L ends with the warp total
 // of value L >> 3 (6 shuffles instead of 20).
 template <typename R>
@@ -1106,129 +1077,169 @@ __device__ __forceinline__ R warp_sum4(R v0, R v1, R v2, R v3) {
     return k;
 }
 
-template <typename R, int V, int B>
-__device__ __forceinline__ void ra_mat1(RA<R> *x, const Cx<R> *M, bool adj) {
-    const Cx<R> m00 = mel<R>(M, 2, 0, 0, adj), m01 = mel<R>(M, 2, 0, 1, adj);
-    const Cx<R> m10 = mel<R>(M, 2, 1, 0, adj), m11 = mel<R>(M, 2, 1, 1, adj);
+// Register bits (A, B) of a Givens rotation, A holding the "1" of u, and the
+// pairs (MU, MV) of a double excitation, as one operation code each; the
+// codes of a step's operation in the register-blocked passes (RegOp).
+enum : uint32_t {
+    RO_GIVENS = 0,     // + 3 ra + (rb - (rb > ra)): 12 ordered pairs
+    RO_DEXC = 12,      // + index of mu in {3, 5, 6, 9, 10, 12}
+    RO_MAT1 = 18,      // + register bit
+    RO_MAT2 = 22,      // + index of the bit pair 01 02 03 12 13 23
+    RO_MAT4 = 28,
+    RO_RZ = 29,        // + register bit
+    RO_RZ_THREAD = 33, // t0: tile bit
+    RO_CZ = 34,        // t0, t1: tile bits
+    RO_RZ_OUT = 35,    // t0 - kOutTarget: physical bit outside the tile
+    RO_CZ_OUT = 36,    // t0 or t1 (or both) outside the tile
+    RO_NOP = 37
+};
+#define SV_RO_GIVENS(CALL)                                                                       \
+    case 0: CALL(1, 2); break;  case 1: CALL(1, 4); break;  case 2: CALL(1, 8); break;           \
+    case 3: CALL(2, 1); break;  case 4: CALL(2, 4); break;  case 5: CALL(2, 8); break;           \
+    case 6: CALL(4, 1); break;  case 7: CALL(4, 2); break;  case 8: CALL(4, 8); break;           \
+    case 9: CALL(8, 1); break;  case 10: CALL(8, 2); break; case 11: CALL(8, 4); break;          \
+    case 12: CALL(3, 12); break; case 13: CALL(5, 10); break; case 14: CALL(6, 9); break;        \
+    case 15: CALL(9, 6); break;  case 16: CALL(10, 5); break; case 17: CALL(12, 3); break;
+
+// Prepared 1-, 2- and 4-qubit matrices (k_prep_mats: indexed by register
+// bits, conjugate transpose already taken for the adjoint) on the register
+// amplitudes.  Every thread reads the same element, 16 bytes at a time.
+template <typename R, int DIM> struct MatRow { Cx<R> m[DIM]; };
+template <typename R, int DIM>
+__device__ __forceinline__ MatRow<R, DIM> mat_row(const Cx<R> *M, int u) {
+    MatRow<R, DIM> r;
+    constexpr int PER = 16 / sizeof(Cx<R>);
+    const float4 *p = reinterpret_cast<const float4 *>(M + u * DIM);
+    float4 t[DIM / PER];
+#pragma unroll
+    for (int i = 0; i < DIM / PER; ++i) {
+        // complex128: volatile, so that the rows of a 4-qubit matrix are not all
+        // loaded ahead (they would not fit the registers beside the amplitudes)
+        if constexpr (sizeof(R) == 8)
+            asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(t[i].x), "=f"(t[i].y), "=f"(t[i].z), "=f"(t[i].w) : "l"(p + i));
+        else
+            t[i] = __ldg(p + i);
+    }
+    memcpy(&r, t, sizeof(r));
+    return r;
+}
+template <typename R, int DIM>
+__device__ __forceinline__ Cx<R> row_dot(const MatRow<R, DIM> &m, const Cx<R> *x) {
+    R re = 0, im = 0;
+#pragma unroll
+    for (int w = 0; w < DIM; ++w) {
+        re += m.m[w].x * x[w].x - m.m[w].y * x[w].y;
+        im += m.m[w].x * x[w].y + m.m[w].y * x[w].x;
+    }
+    return mk<R>(re, im);
+}
+// the dim x dim matrix on register bits B0 (and B1 > B0)
+template <typename R, int B0, int B1>
+__device__ __forceinline__ void reg_mat(RA<R> *x, const Cx<R> *M) {
+    constexpr int NB = B1 > B0 ? 2 : 1, DIM = 1 << NB, V = 1 << kRegBits;
+    constexpr int MASK = (1 << B0) | (NB == 2 ? 1 << B1 : 0);
+    MatRow<R, DIM> row[DIM];
+#pragma unroll
+    for (int u = 0; u < DIM; ++u) row[u] = mat_row<R, DIM>(M, u);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        if (v & (1 << B)) continue;
-        const int w = v | (1 << B);
-        const Cx<R> a = ra_cx<R>(x[v]), b = ra_cx<R>(x[w]);
-        x[v] = cx_ra<R>(mk<R>(m00.x * a.x - m00.y * a.y + m01.x * b.x - m01.y * b.y,
-                              m00.x * a.y + m00.y * a.x + m01.x * b.y + m01.y * b.x));
-        x[w] = cx_ra<R>(mk<R>(m10.x * a.x - m10.y * a.y + m11.x * b.x - m11.y * b.y,
-                              m10.x * a.y + m10.y * a.x + m11.x * b.y + m11.y * b.x));
+        if (v & MASK) continue;
+        Cx<R> in[DIM];
+#pragma unroll
+        for (int u = 0; u < DIM; ++u) in[u] = ra_cx<R>(x[v | ((u & 1) << B0) | (NB == 2 ? (u >> 1) << B1 : 0)]);
+#pragma unroll
+        for (int u = 0; u < DIM; ++u)
+            x[v | ((u & 1) << B0) | (NB == 2 ? (u >> 1) << B1 : 0)] = cx_ra<R>(row_dot<R, DIM>(row[u], in));
     }
 }
+template <typename R>
+__device__ __forceinline__ void reg_mat4(RA<R> *x, const Cx<R> *M) {
+    Cx<R> in[16];
+#pragma unroll
+    for (int v = 0; v < 16; ++v) in[v] = ra_cx<R>(x[v]);
+#pragma unroll
+    for (int v = 0; v < 16; ++v) x[v] = cx_ra<R>(row_dot<R, 16>(mat_row<R, 16>(M, v), in));
+}
 
-#define SV_RB_SWITCH(b, CALL)                                    \
-    switch (b) {                                                 \
-    case 0: CALL(0); break;                                      \
-    case 1: if constexpr (RB > 1) { CALL(1); } break;            \
-    case 2: if constexpr (RB > 2) { CALL(2); } break;            \
-    case 3: if constexpr (RB > 3) { CALL(3); } break;            \
-    default: break;                                              \
+// the register amplitudes v whose bit b is set
+__device__ __forceinline__ uint32_t reg_bit_mask(uint32_t b) {
+    return b == 0 ? 0xAAAAu : b == 1 ? 0xCCCCu : b == 2 ? 0xF0F0u : 0xFF00u;
+}
+// the register amplitudes on which a CZ of in-tile bits t0, t1 is -1
+__device__ __forceinline__ uint32_t cz_negmask(uint32_t t0, uint32_t t1, uint32_t rmask, uint32_t base) {
+    uint32_t m = 0xFFFFu;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t t = i ? t1 : t0;
+        if ((rmask >> t) & 1u) m &= reg_bit_mask(__popc(rmask & ((1u << t) - 1u)));
+        else if (!((base >> t) & 1u)) m = 0;
     }
+    return m;
+}
+template <typename R>
+__device__ __forceinline__ void reg_neg_mask(RA<R> *x, uint32_t m) {
+#pragma unroll
+    for (int v = 0; v < (1 << kRegBits); ++v)
+        if ((m >> v) & 1u) x[v] = ra_neg<R>(x[v]);
+}
+template <typename R, int B>
+__device__ __forceinline__ void reg_rz_bit(RA<R> *x, Cx<R> k) {
+    const Cx<R> w0 = mk<R>(k.x, -k.y), w1 = mk<R>(k.x, k.y);
+#pragma unroll
+    for (int v = 0; v < (1 << kRegBits); ++v) x[v] = ra_cmul<R>(x[v], ((v >> B) & 1) ? w1 : w0);
+}
+template <typename R>
+__device__ __forceinline__ void reg_phase_all(RA<R> *x, Cx<R> k, bool one) {
+    const Cx<R> w = mk<R>(k.x, one ? k.y : -k.y);
+#pragma unroll
+    for (int v = 0; v < (1 << kRegBits); ++v) x[v] = ra_cmul<R>(x[v], w);
+}
+// sign mask of a CZ with a target outside the tile (constant over the tile)
+__device__ __forceinline__ uint32_t cz_out_negmask(uint32_t t0, uint32_t t1, uint32_t rmask, uint32_t base,
+                                                   uint64_t gbase) {
+    const bool o0 = t0 >= (uint32_t)kOutTarget, o1 = t1 >= (uint32_t)kOutTarget;
+    if (o0 && !((gbase >> (t0 - kOutTarget)) & 1ull)) return 0;
+    if (o1 && !((gbase >> (t1 - kOutTarget)) & 1ull)) return 0;
+    if (o0 && o1) return 0xFFFFu;
+    const uint32_t t = o0 ? t1 : t0;
+    return cz_negmask(t, t, rmask, base);
+}
 
-// One operation applied by the generic path (OP steps) on register
-// amplitudes: base = the thread's tile bits outside rmask; cs = (cos, sin)
-// of the half angle (sin already negated for an inverse).
-template <typename R, int RB>
-__device__ void ra_apply_op(RA<R> *x, DevOp op, uint32_t rmask, uint32_t base, Cx<R> cs, const Cx<R> *mats,
-                            bool adj) {
-    constexpr int V = 1 << RB;
-    const int t0 = op.t[0];
-    const int b0 = __popc(rmask & ((1u << (t0 & 31)) - 1u));
-    switch (op.kind) {
-    case SV_RY: {
-        const RotK<R> k = rotk<R>(cs.x, cs.y);
-#define SV_C(B) ra_rot<R, V, B>(x, k)
-        SV_RB_SWITCH(b0, SV_C)
+// One operation of a step (code and targets packed in `a`: code | t0 << 8 |
+// t1 << 16) on the register amplitudes; k = (cos, sin), sin negated for an
+// inverse; M = the prepared matrix.  DENSE: 2- and 4-qubit matrices too
+// (their reverse passes run in k_adj_pass).
+template <typename R, bool DENSE>
+__device__ __forceinline__ void reg_op(RA<R> *x, uint32_t a, uint32_t rmask, uint32_t base, uint64_t gbase,
+                                       Cx<R> k, const Cx<R> *M) {
+    constexpr int V = 1 << kRegBits;
+    const uint32_t t0 = (a >> 8) & 255u, t1 = (a >> 16) & 255u;
+    const RotK<R> rk = rotk<R>(k.x, k.y);
+    switch (a & 255u) {
+#define SV_C(MU, MV) ra_pair_rot<R, V, MU, MV>(x, rk)
+        SV_RO_GIVENS(SV_C)
 #undef SV_C
-        break;
-    }
-    case SV_MAT1: {
-        const Cx<R> *M = mats + op.mat;
-#define SV_C(B) ra_mat1<R, V, B>(x, M, adj)
-        SV_RB_SWITCH(b0, SV_C)
-#undef SV_C
-        break;
-    }
-    case SV_GIVENS: {
-        const RotK<R> k = rotk<R>(cs.x, cs.y);
-        const int b1 = __popc(rmask & ((1u << op.t[1]) - 1u));
-#define SV_C(MU, MV) ra_pair_rot<R, V, MU, MV>(x, k)
-        SV_GIVENS_SWITCH(b0, b1, SV_C)
-#undef SV_C
-        break;
-    }
-    case SV_DEXC: {
-        const RotK<R> k = rotk<R>(cs.x, cs.y);
-        const int mu = (1 << b0) | (1 << __popc(rmask & ((1u << op.t[1]) - 1u)));
-#define SV_C(MU, MV) ra_pair_rot<R, V, MU, MV>(x, k)
-        SV_DEXC_SWITCH(mu, SV_C)
-#undef SV_C
-        break;
-    }
-    case SV_RZ: {
-        if ((rmask >> t0) & 1u) {
-            const Cx<R> w0 = mk<R>(cs.x, -cs.y), w1 = mk<R>(cs.x, cs.y);
-#pragma unroll
-            for (int v = 0; v < V; ++v) x[v] = ra_cmul<R>(x[v], ((v >> b0) & 1) ? w1 : w0);
-        } else {
-            const Cx<R> w = mk<R>(cs.x, ((base >> t0) & 1u) ? cs.y : -cs.y);
-#pragma unroll
-            for (int v = 0; v < V; ++v) x[v] = ra_cmul<R>(x[v], w);
-        }
-        break;
-    }
-    case SV_CZ: {
-        const int t1 = op.t[1];
-        const bool r0 = (rmask >> t0) & 1u, r1 = (rmask >> t1) & 1u;
-        uint32_t negmask = 0;   // register amplitudes that change sign
-        if (r0 && r1) {
-            const int b1 = __popc(rmask & ((1u << t1) - 1u));
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                if ((v >> b0) & (v >> b1) & 1) negmask |= 1u << v;
-        } else if (r0 || r1) {
-            const int tr = r0 ? t0 : t1, tt = r0 ? t1 : t0;
-            if ((base >> tt) & 1u) {
-                const int br = __popc(rmask & ((1u << tr) - 1u));
-#pragma unroll
-                for (int v = 0; v < V; ++v)
-                    if ((v >> br) & 1) negmask |= 1u << v;
-            }
-        } else if (((base >> t0) & (base >> t1)) & 1u) {
-            negmask = 0xFFFFFFFFu;
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-            if ((negmask >> v) & 1u) x[v] = ra_neg<R>(x[v]);
-        break;
-    }
-    case SV_OP_PHASE: {
-        const Cx<R> w = mk<R>(cs.x, op.t[0] ? cs.y : -cs.y);
-#pragma unroll
-        for (int v = 0; v < V; ++v) x[v] = ra_cmul<R>(x[v], w);
-        break;
-    }
-    case SV_OP_ZSIGN: {
-        const bool reg = (rmask >> t0) & 1u;
-        const bool thr = !reg && ((base >> t0) & 1u);
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-            if (reg ? ((v >> b0) & 1) : thr) x[v] = ra_neg<R>(x[v]);
-        break;
-    }
-    case SV_OP_NEG: {
-#pragma unroll
-        for (int v = 0; v < V; ++v) x[v] = ra_neg<R>(x[v]);
-        break;
-    }
-    default:
-        break;
+    case RO_MAT1: reg_mat<R, 0, 0>(x, M); break;
+    case RO_MAT1 + 1: reg_mat<R, 1, 1>(x, M); break;
+    case RO_MAT1 + 2: reg_mat<R, 2, 2>(x, M); break;
+    case RO_MAT1 + 3: reg_mat<R, 3, 3>(x, M); break;
+    case RO_MAT2: if constexpr (DENSE) reg_mat<R, 0, 1>(x, M); break;
+    case RO_MAT2 + 1: if constexpr (DENSE) reg_mat<R, 0, 2>(x, M); break;
+    case RO_MAT2 + 2: if constexpr (DENSE) reg_mat<R, 0, 3>(x, M); break;
+    case RO_MAT2 + 3: if constexpr (DENSE) reg_mat<R, 1, 2>(x, M); break;
+    case RO_MAT2 + 4: if constexpr (DENSE) reg_mat<R, 1, 3>(x, M); break;
+    case RO_MAT2 + 5: if constexpr (DENSE) reg_mat<R, 2, 3>(x, M); break;
+    case RO_MAT4: if constexpr (DENSE) reg_mat4<R>(x, M); break;
+    case RO_RZ: reg_rz_bit<R, 0>(x, k); break;
+    case RO_RZ + 1: reg_rz_bit<R, 1>(x, k); break;
+    case RO_RZ + 2: reg_rz_bit<R, 2>(x, k); break;
+    case RO_RZ + 3: reg_rz_bit<R, 3>(x, k); break;
+    case RO_RZ_THREAD: reg_phase_all<R>(x, k, (base >> t0) & 1u); break;
+    case RO_RZ_OUT: reg_phase_all<R>(x, k, (gbase >> (t0 - kOutTarget)) & 1ull); break;
+    case RO_CZ: reg_neg_mask<R>(x, cz_negmask(t0, t1, rmask, base)); break;
+    case RO_CZ_OUT: reg_neg_mask<R>(x, cz_out_negmask(t0, t1, rmask, base, gbase)); break;
+    default: break;
     }
 }
 
@@ -1239,40 +1250,39 @@ __device__ __forceinline__ R ra_imdot(RA<R> l, RA<R> p) {
     return a.x * b.y - a.y * b.x;
 }
 
-// Adjoint of one OP step: gradient part Im<lambda|G|psi> (RY: Y, RZ: Z), then
-// U^dagger on both register sets.  cs holds (cos, -sin).
-template <typename R, int RB>
-__device__ R ra_adjoint_op(RA<R> *p, RA<R> *l, DevOp op, uint32_t rmask, uint32_t base, Cx<R> cs,
-                           const Cx<R> *mats) {
-    constexpr int V = 1 << RB;
-    const int t0 = op.t[0];
-    const int b0 = __popc(rmask & ((1u << (t0 & 31)) - 1u));
+// Adjoint of one operation: gradient part Im<lambda|G|psi> (the subspace Y of
+// a rotation, Z of an RZ), then U^dagger on both register sets.
+__device__ __forceinline__ bool reg_op_param(uint32_t a) {
+    const uint32_t c = a & 255u;
+    return c < RO_MAT1 || (c >= RO_RZ && c <= RO_RZ_THREAD) || c == RO_RZ_OUT;
+}
+template <typename R>
+__device__ __forceinline__ R reg_op_adj(RA<R> *p, RA<R> *l, uint32_t a, uint32_t rmask, uint32_t base, uint64_t gbase,
+                                        Cx<R> k, const Cx<R> *M) {
+    constexpr int V = 1 << kRegBits;
+    const uint32_t t0 = (a >> 8) & 255u;
+    const uint32_t c = a & 255u;
     R g = 0;
-    if (op.kind == SV_RY) {
-#define SV_C(B) g = ra_ry_grad<R, V, B>(p, l)
-        SV_RB_SWITCH(b0, SV_C)
-#undef SV_C
-    } else if (op.kind == SV_GIVENS) {
-        const int b1 = __popc(rmask & ((1u << op.t[1]) - 1u));
+    if (c < RO_MAT1) {
+        switch (c) {
 #define SV_C(MU, MV) g = ra_pair_grad<R, V, MU, MV>(p, l)
-        SV_GIVENS_SWITCH(b0, b1, SV_C)
+            SV_RO_GIVENS(SV_C)
 #undef SV_C
-    } else if (op.kind == SV_DEXC) {
-        const int mu = (1 << b0) | (1 << __popc(rmask & ((1u << op.t[1]) - 1u)));
-#define SV_C(MU, MV) g = ra_pair_grad<R, V, MU, MV>(p, l)
-        SV_DEXC_SWITCH(mu, SV_C)
-#undef SV_C
-    } else if (op.kind == SV_RZ || op.kind == SV_OP_PHASE) {
-        const bool reg = op.kind == SV_RZ && ((rmask >> t0) & 1u);
-        const bool one = op.kind == SV_OP_PHASE ? op.t[0] != 0 : ((base >> t0) & 1u) != 0;
+        default: break;
+        }
+    } else if (reg_op_param(a)) {
+        // amplitudes on which Z is -1
+        const uint32_t neg = c == RO_RZ_THREAD ? (((base >> t0) & 1u) ? 0xFFFFu : 0u)
+                             : c == RO_RZ_OUT  ? (((gbase >> (t0 - kOutTarget)) & 1ull) ? 0xFFFFu : 0u)
+                                               : reg_bit_mask((c - RO_RZ) & 3u);
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             const R im = ra_imdot<R>(l[v], p[v]);
-            g += (reg ? ((v >> b0) & 1) : one) ? -im : im;
+            g += ((neg >> v) & 1u) ? -im : im;
         }
     }
-    ra_apply_op<R, RB>(p, op, rmask, base, cs, mats, true);
-    ra_apply_op<R, RB>(l, op, rmask, base, cs, mats, true);
+    reg_op<R, false>(p, a, rmask, base, gbase, k, M);
+    reg_op<R, false>(l, a, rmask, base, gbase, k, M);
     return g;
 }
 
@@ -1302,7 +1312,7 @@ __device__ __forceinline__ void load_tile_async(E *tile, const Cx<R> *psi, uint6
 // Shared-memory layout of a register-blocked pass (both kernels): the tiles,
 // then these tables (offsets in bytes from the end of the tiles).
 struct RegLayout {
-    uint32_t hioff, cs, steps, blocks, mem, pbase, prb, acc, tot, sc, area, total;
+    uint32_t hioff, chunk, cs, steps, blocks, mem, phases, pbase, prb, sc, area, image, acc, tot, total;
 };
 // FP64 is 1/64 of the FP32 rate on this part: per-tile gradient partials stay
 // in FP32 slots and reach FP64 once every kAdjFlush tiles
@@ -1312,146 +1322,234 @@ __host__ __device__ inline RegLayout reg_layout(const GatePassArgs &a, int amp, 
     RegLayout L;
     const uint32_t nops = (uint32_t)(a.op_end - a.op_begin), nst = (uint32_t)(a.st_end - a.st_begin);
     const uint32_t nph = (uint32_t)(a.ph_end - a.ph_begin), nb = (uint32_t)(a.db_end - a.db_begin);
+    const uint32_t nt = 1u << (a.k - kRegBits);
     uint32_t o = 0;
     L.hioff = o; o = align16u(o + 8u * (1u << (a.k - a.nlow)));
+    L.chunk = o; o = align16u(o + 16u * 16u);
     L.cs = o;    o = align16u(o + (uint32_t)amp * nops);
     L.steps = o; o = align16u(o + 16u * nst);
     L.blocks = o; o = align16u(o + (uint32_t)sizeof(DiagBlock) * nb);
     L.mem = o;   o = align16u(o + (uint32_t)sizeof(DiagMember) * (uint32_t)(a.mem_end - a.mem_begin));
-    L.pbase = o; o = align16u(o + 2u * kRegThreads * nph);
+    L.phases = o; o = align16u(o + 16u * nph);
+    L.pbase = o; o = align16u(o + 2u * nt * nph);
     L.prb = o;   o = align16u(o + 8u * nph);
-    // adjoint gradient slots: per op and warp a partial of the state's real
-    // type, and for complex64 an FP64 total per op (flushed every kAdjFlush tiles)
-    L.acc = o;   o = align16u(o + (adj ? ((uint32_t)amp / 2u) * kAdjSlotStride * nops : 0u));
-    L.tot = o;   o = align16u(o + (adj && amp == 8 ? 8u * nops : 0u));
     // factored RYs: per step the product of the factors applied before it
     // (adjoint), and the pass's total factor (entry nst)
     L.sc = o;    o = align16u(o + ((uint32_t)amp / 2u) * (nst + 1u));
     L.area = o;  o = align16u(o + (uint32_t)a.area);
+    L.image = o;                                   // the tables up to here come from k_reg_image
+    // adjoint gradient slots: per op and warp a partial of the state's real
+    // type, and for complex64 an FP64 total per op (flushed every kAdjFlush tiles)
+    L.acc = o;   o = align16u(o + (adj ? ((uint32_t)amp / 2u) * kAdjSlotStride * nops : 0u));
+    L.tot = o;   o = align16u(o + (adj && amp == 8 ? 8u * nops : 0u));
     L.total = o;
     return L;
 }
 
-// Per-launch set-up shared by both kernels: high offsets, (cos, sin) per op
-// (sin negated for the adjoint), steps, blocks, each phase's thread base and
-// swizzled register-bit offsets, and the diagonal blocks' data (of D, or of
-// D^dagger for the adjoint): a register block's table T[v][zm] and every
-// thread's zm, a thread block's factor per thread.
-template <typename R, int RB>
-__device__ void reg_setup(unsigned char *sm, const RegLayout &L, const GatePassArgs &a, const DevOp *ops,
-                          const Phase *phases, const RegStep *steps, const R *coef, const DiagBlock *dblocks,
-                          const DiagMember *dmem, bool adj) {
-    constexpr int V = 1 << RB;
-    const int NT = blockDim.x, tid = threadIdx.x;
-    uint64_t *hioff = reinterpret_cast<uint64_t *>(sm + L.hioff);
-    Cx<R> *cs = reinterpret_cast<Cx<R> *>(sm + L.cs);
-    RegStep *st = reinterpret_cast<RegStep *>(sm + L.steps);
-    DiagBlock *bl = reinterpret_cast<DiagBlock *>(sm + L.blocks);
-    uint16_t *pbase = reinterpret_cast<uint16_t *>(sm + L.pbase);
-    uint16_t *prb = reinterpret_cast<uint16_t *>(sm + L.prb);
-    const uint32_t nh = 1u << (a.k - a.nlow);
-    for (uint32_t j = tid; j < nh; j += NT) hioff[j] = deposit(j, a.hi, a.nhi);
-    for (int o = a.op_begin + tid; o < a.op_end; o += NT) {
+// A chunk of a tile: the 16-byte pieces a thread moves are element j = P tid
+// + i P NT (P amplitudes per piece), i < 16 / P; their places are the
+// thread's XOR / OR these per-chunk constants.
+struct ChunkOff {
+    uint64_t g;    // global element offset of tile bits i P NT
+    uint32_t s;    // shared slot of the same
+    uint32_t pad;
+};
+struct PhaseS {
+    uint32_t rmask;
+    int32_t st_begin, st_end;   // relative to the pass
+    uint32_t pad;
+};
+
+// The tables of a register-blocked pass, made once per call by k_reg_image in
+// global memory and copied into shared memory by every CTA of the pass: high
+// and chunk offsets, (cos, sin) per op (sin negated for the adjoint) with the
+// RYs of ROT steps factored, decoded steps, blocks, phases with their thread
+// bases and swizzled register-bit offsets, the factors' prefix products, and
+// the diagonal blocks' data (of D, or of D^dagger for the adjoint): a register
+// block's table T[v][zm] and every thread's zm, a thread block's factor per
+// thread.  Made inside the pass kernels they were most of a launch on a small
+// state (n = 14: 49 of 52 us a gate pass, serial in one CTA's 64 threads), and
+// every CTA of every pass repeated them.  Block (pass, slice, direction): the
+// slices share a pass's phases and blocks, slice 0 writes the rest.
+constexpr int kImageSlices = 8;
+template <typename R>
+__global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restrict__ pargs,
+                                                   const uint64_t *__restrict__ offs, const DevOp *__restrict__ ops,
+                                                   const Phase *__restrict__ phases,
+                                                   const RegStep *__restrict__ steps, const R *__restrict__ coef,
+                                                   const DiagBlock *__restrict__ dblocks,
+                                                   const DiagMember *__restrict__ dmem, unsigned char *out0,
+                                                   uint64_t dir_stride, int dir0) {
+    constexpr int RB = kRegBits, V = 1 << RB;
+    constexpr uint32_t P = 16 / sizeof(Cx<R>);
+    __shared__ GatePassArgs a;
+    __shared__ Cx<R> cs[kMaxPassOps];
+    __shared__ RegStep st[kMaxPassOps];
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const bool adj = (int)blockIdx.z + dir0 != 0, first = blockIdx.y == 0;
+    for (int i = tid; i < (int)(sizeof(GatePassArgs) / 4); i += nthr)
+        reinterpret_cast<uint32_t *>(&a)[i] = reinterpret_cast<const uint32_t *>(pargs + blockIdx.x)[i];
+    __syncthreads();
+    unsigned char *out = out0 + (adj ? dir_stride : 0) + offs[blockIdx.x];
+    const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), adj);
+    const int NT = 1 << (a.k - RB), nph = a.ph_end - a.ph_begin, nst = a.st_end - a.st_begin;
+    for (int o = a.op_begin + tid; o < a.op_end; o += nthr) {
         const int gi = ops[o].gate;
         cs[o - a.op_begin] = mk<R>(coef[2 * gi], adj ? -coef[2 * gi + 1] : coef[2 * gi + 1]);
+    }
+    // the steps: operation records decoded to (code and targets, op, prepared matrix)
+    for (int s = tid; s < nst; s += nthr) {
+        RegStep S = steps[a.st_begin + s];
+        if (S.type == SV_STEP_OP && first) {
+            int ph = a.ph_begin;
+            while (phases[ph].st_end <= a.st_begin + s) ++ph;
+            const uint32_t rmask = phases[ph].rmask;
+            const DevOp op = ops[S.a];
+            const uint32_t t0 = (uint8_t)op.t[0], t1 = (uint8_t)op.t[1];
+            auto reg = [&](uint32_t t) { return (uint32_t)__popc(rmask & ((1u << (t & 31u)) - 1u)); };
+            uint32_t code = RO_NOP;
+            if (op.kind == SV_GIVENS) {
+                const uint32_t ra = reg(t0), rb = reg(t1);
+                code = RO_GIVENS + 3u * ra + rb - (rb > ra ? 1u : 0u);
+            } else if (op.kind == SV_DEXC) {
+                const uint32_t mu = (1u << reg(t0)) | (1u << reg(t1));
+                code = RO_DEXC + (mu == 3u ? 0u : mu == 5u ? 1u : mu == 6u ? 2u : mu == 9u ? 3u : mu == 10u ? 4u : 5u);
+            } else if (op.kind == SV_MAT1) {
+                code = RO_MAT1 + reg(t0);
+            } else if (op.kind == SV_MAT2) {
+                const uint32_t lo = min(reg(t0), reg(t1)), hi = max(reg(t0), reg(t1));
+                code = RO_MAT2 + (lo == 0u ? hi - 1u : lo == 1u ? hi + 1u : 5u);
+            } else if (op.kind == SV_MAT4) {
+                code = RO_MAT4;
+            } else if (op.kind == SV_RZ) {
+                code = t0 >= (uint32_t)kOutTarget ? (uint32_t)RO_RZ_OUT
+                       : ((rmask >> t0) & 1u)     ? RO_RZ + reg(t0)
+                                                  : (uint32_t)RO_RZ_THREAD;
+            } else if (op.kind == SV_CZ) {
+                code = (t0 >= (uint32_t)kOutTarget || t1 >= (uint32_t)kOutTarget) ? RO_CZ_OUT : RO_CZ;
+            }
+            S.op_begin = S.a - a.op_begin;
+            S.a = (int32_t)(code | (t0 << 8) | (t1 << 16));
+            S.op_end = op.pm;
+        }
+        st[s] = S;
     }
     __syncthreads();
     // the RYs of ROT steps as (t, factor), each step carrying their forms
     // (bit 8 + register bit set: form B)
-    for (int s = a.st_begin + tid; s < a.st_end; s += NT) {
-        RegStep S = steps[s];
-        if (S.type == SV_STEP_ROT) {
-            int o = S.op_begin;
-            for (int b = 0; b < RB; ++b) {
-                if (!((S.a >> b) & 1)) continue;
-                const Cx<R> k = cs[o - a.op_begin];
-                int fb;
-                cs[o - a.op_begin] = ry_factored<R>(k.x, k.y, fb);
-                if (fb) S.a |= 1 << (8 + b);
-                ++o;
-            }
+    for (int s = tid; s < nst; s += nthr) {
+        if (st[s].type != SV_STEP_ROT) continue;
+        int o = st[s].op_begin - a.op_begin, forms = st[s].a;
+        for (int b = 0; b < RB; ++b) {
+            if (!((st[s].a >> b) & 1)) continue;
+            const Cx<R> k = cs[o];
+            int fb;
+            cs[o] = ry_factored<R>(k.x, k.y, fb);
+            if (fb) forms |= 1 << (8 + b);
+            ++o;
         }
-        st[s - a.st_begin] = S;
+        st[s].a = forms;
     }
-    // prefix products of the factors in execution order (forward: ascending
-    // steps; adjoint: descending), entry nst = the pass's total factor
-    if (tid == 0) {
-        R *sc = reinterpret_cast<R *>(sm + L.sc);
-        const int nst = a.st_end - a.st_begin;
-        R f = 1;
-        for (int i = 0; i < nst; ++i) {
-            const int s = adj ? a.st_end - 1 - i : a.st_begin + i;
-            sc[s - a.st_begin] = f;
-            const RegStep S = steps[s];
-            if (S.type != SV_STEP_ROT) continue;
-            for (int o = S.op_begin; o < S.op_end; ++o) {
-                const int gi = ops[o].gate;
-                const R c = coef[2 * gi], sn = adj ? -coef[2 * gi + 1] : coef[2 * gi + 1];
-                int fb;
-                f *= ry_factored<R>(c, sn, fb).y;
-            }
+    __syncthreads();
+    if (first) {
+        const uint32_t nh = 1u << (a.k - a.nlow), lowmask = (1u << a.nlow) - 1u;
+        uint64_t *hioff = reinterpret_cast<uint64_t *>(out + L.hioff);
+        for (uint32_t j = tid; j < nh; j += nthr) hioff[j] = deposit(j, a.hi, a.nhi);
+        ChunkOff *chunk = reinterpret_cast<ChunkOff *>(out + L.chunk);
+        for (uint32_t i = tid; i < 16u / P; i += nthr) {
+            const uint32_t j = i * P * (uint32_t)NT;
+            chunk[i] = {(j & lowmask) | deposit(j >> a.nlow, a.hi, a.nhi), swz_tile(j), 0u};
         }
-        sc[nst] = f;
-    }
-    for (int b = a.db_begin + tid; b < a.db_end; b += NT) bl[b - a.db_begin] = dblocks[b];
-    DiagMember *mem = reinterpret_cast<DiagMember *>(sm + L.mem);
-    for (int m = a.mem_begin + tid; m < a.mem_end; m += NT) mem[m - a.mem_begin] = dmem[m];
-    for (int ph = a.ph_begin; ph < a.ph_end; ++ph) {
-        const uint32_t rmask = phases[ph].rmask;
-        const uint32_t base = phase_base(rmask, phases[ph].lanes, a.k);
-        pbase[(ph - a.ph_begin) * NT + tid] = (uint16_t)base;
-        if (tid < 4) {
-            uint32_t rm = rmask, bitv = 0;
-            for (int i = 0; i <= tid && rm; ++i) {
-                bitv = rm & (0u - rm);
-                rm ^= bitv;
+        for (int o = tid; o < a.op_end - a.op_begin; o += nthr) reinterpret_cast<Cx<R> *>(out + L.cs)[o] = cs[o];
+        for (int s = tid; s < nst; s += nthr) reinterpret_cast<RegStep *>(out + L.steps)[s] = st[s];
+        for (int b = a.db_begin + tid; b < a.db_end; b += nthr)
+            reinterpret_cast<DiagBlock *>(out + L.blocks)[b - a.db_begin] = dblocks[b];
+        for (int m = a.mem_begin + tid; m < a.mem_end; m += nthr)
+            reinterpret_cast<DiagMember *>(out + L.mem)[m - a.mem_begin] = dmem[m];
+        for (int q = tid; q < nph; q += nthr) {
+            const Phase F = phases[a.ph_begin + q];
+            reinterpret_cast<PhaseS *>(out + L.phases)[q] = {F.rmask, F.st_begin - a.st_begin, F.st_end - a.st_begin, 0u};
+            uint32_t rm = F.rmask;
+            for (int i = 0; i < RB; ++i, rm &= rm - 1u)
+                reinterpret_cast<uint16_t *>(out + L.prb)[q * 4 + i] = (uint16_t)swz_tile(rm & (0u - rm));
+        }
+        // prefix products of the factors in execution order (forward: ascending
+        // steps; adjoint: descending), entry nst = the pass's total factor
+        R *sc = reinterpret_cast<R *>(out + L.sc);
+        for (int i = tid; i <= nst; i += nthr) {
+            R f = 1;
+            for (int q = 0; q < i; ++q) {
+                const RegStep S = st[adj ? nst - 1 - q : q];
+                if (S.type != SV_STEP_ROT) continue;
+                for (int o = S.op_begin - a.op_begin; o < S.op_end - a.op_begin; ++o) f *= cs[o].y;
             }
-            prb[(ph - a.ph_begin) * 4 + tid] = (uint16_t)(tid < RB ? swz_tile(bitv) : 0u);
+            sc[i == nst ? nst : (adj ? nst - 1 - i : i)] = f;
         }
     }
-    unsigned char *area = sm + L.area;
-    for (int b = a.db_begin; b < a.db_end; ++b) {
-        const DiagBlock B = dblocks[b];
-        const uint32_t base = phase_base(B.rmask, B.lanes, a.k);
+    // this slice's phases: the tile bits of every thread
+    for (int e = tid; e < nph * NT; e += nthr) {
+        const int q = e / NT, t = e % NT;
+        if (q % kImageSlices != (int)blockIdx.y) continue;
+        const Phase F = phases[a.ph_begin + q];
+        reinterpret_cast<uint16_t *>(out + L.pbase)[e] = (uint16_t)phase_base(F.rmask, F.lanes, a.k, (uint32_t)t);
+    }
+    // this slice's diagonal blocks: tables and per-thread data
+    unsigned char *area = out + L.area;
+    for (int b = (int)blockIdx.y; b < a.db_end - a.db_begin; b += kImageSlices) {
+        const DiagBlock B = dblocks[a.db_begin + b];
+        const DiagMember *mb = dmem + B.m_begin;
+        const int nm = B.m_end - B.m_begin;
         if (B.kind == 0) {
             Cx<R> *tab = reinterpret_cast<Cx<R> *>(area + B.smem);
             uint8_t *zmv = area + B.smem + V * V * (int)sizeof(Cx<R>);
-            if (tid < V * V) {
-                const int v = tid / V, zm = tid % V;
+            for (int q = tid; q < V * V; q += nthr) {
+                const int v = q / V, zm = q % V;
                 Cx<R> r = mk<R>(((__popc((uint32_t)(v & zm)) & 1) ? -1 : 1), 0);
-                for (int mi = B.m_begin; mi < B.m_end; ++mi) {
-                    const DiagMember m = dmem[mi];
+                for (int mi = 0; mi < nm; ++mi) {
+                    const DiagMember m = mb[mi];
                     if (m.type == SV_DM_REG_RZ) {
-                        const int gi = ops[m.op].gate;
-                        const R c = coef[2 * gi], s = adj ? -coef[2 * gi + 1] : coef[2 * gi + 1];
-                        r = cmul<R>(r, mk<R>(c, ((v >> m.a) & 1) ? s : -s));
+                        const Cx<R> k = cs[m.op - a.op_begin];
+                        r = cmul<R>(r, mk<R>(k.x, ((v >> m.a) & 1) ? k.y : -k.y));
                     } else if (m.type == SV_DM_REG_CZ) {
                         if ((v >> m.a) & (v >> m.b) & 1) r = mk<R>(-r.x, -r.y);
                     }
                 }
-                tab[v * V + zm] = r;
+                tab[q] = r;
             }
-            uint32_t zm = 0;
-            for (int mi = B.m_begin; mi < B.m_end; ++mi) {
-                const DiagMember m = dmem[mi];
-                if (m.type == SV_DM_MIX_CZ && ((base >> m.b) & 1u)) zm ^= 1u << m.a;
-            }
-            zmv[tid] = (uint8_t)zm;
-        } else {
-            Cx<R> w = mk<R>(1, 0);
-            for (int mi = B.m_begin; mi < B.m_end; ++mi) {
-                const DiagMember m = dmem[mi];
-                if (m.type == SV_DM_THR_RZ) {
-                    const int gi = ops[m.op].gate;
-                    const R c = coef[2 * gi], s = adj ? -coef[2 * gi + 1] : coef[2 * gi + 1];
-                    w = cmul<R>(w, mk<R>(c, ((base >> m.a) & 1u) ? s : -s));
-                } else if (m.type == SV_DM_THR_CZ) {
-                    if ((base >> m.a) & (base >> m.b) & 1u) w = mk<R>(-w.x, -w.y);
+            for (int t = tid; t < NT; t += nthr) {
+                const uint32_t base = phase_base(B.rmask, B.lanes, a.k, (uint32_t)t);
+                uint32_t zm = 0;
+                for (int mi = 0; mi < nm; ++mi) {
+                    const DiagMember m = mb[mi];
+                    if (m.type == SV_DM_MIX_CZ && ((base >> m.b) & 1u)) zm ^= 1u << m.a;
                 }
+                zmv[t] = (uint8_t)zm;
             }
-            reinterpret_cast<Cx<R> *>(area + B.smem)[tid] = w;
+        } else {
+            for (int t = tid; t < NT; t += nthr) {
+                const uint32_t base = phase_base(B.rmask, B.lanes, a.k, (uint32_t)t);
+                Cx<R> w = mk<R>(1, 0);
+                for (int mi = 0; mi < nm; ++mi) {
+                    const DiagMember m = mb[mi];
+                    if (m.type == SV_DM_THR_RZ) {
+                        const Cx<R> k = cs[m.op - a.op_begin];
+                        w = cmul<R>(w, mk<R>(k.x, ((base >> m.a) & 1u) ? k.y : -k.y));
+                    } else if (m.type == SV_DM_THR_CZ) {
+                        if ((base >> m.a) & (base >> m.b) & 1u) w = mk<R>(-w.x, -w.y);
+                    }
+                }
+                reinterpret_cast<Cx<R> *>(area + B.smem)[t] = w;
+            }
         }
     }
+}
+
+// A pass's tables from global into shared memory (16 bytes at a time)
+__device__ __forceinline__ void reg_image_load(unsigned char *sm, const unsigned char *image, uint32_t bytes) {
+    for (uint32_t i = 16u * threadIdx.x; i < bytes; i += 16u * blockDim.x) cp_async16(sm + i, image + i);
+    cp_async_commit();
+    cp_async_wait0();
+    __syncthreads();
 }
 
 // x[v] *= the block's factor (register block: table entry [v][zm]; thread block: one factor)
@@ -1496,47 +1594,110 @@ __device__ __forceinline__ void reg_diag2(RA<R> *x, RA<R> *y, const DiagBlock &B
     }
 }
 
-// The thread's 2^RB shared-memory indices of a phase (swizzled; the swizzle
-// is linear, so index(base | sp[v]) = swz(base) ^ XOR of swz(register bits)).
-template <int RB>
-__device__ __forceinline__ void phase_slots(uint32_t *idx, uint32_t base, const uint16_t *prb) {
+// The thread's 16 shared-memory slots of a phase (the swizzle is linear, so
+// slot(base | v) = slot(base) ^ XOR of the register bits' slots), and the
+// gather and scatter of its amplitudes.  A phase that holds tile bit 0 moves
+// complex64 pairs (v, v | 1) by one 16-byte access: with 8-byte accesses its
+// lanes could only reach half of the banks.
+__device__ __forceinline__ void phase_slots16(uint32_t *idx, uint32_t base, const uint16_t *prb) {
+    const ushort4 r = *reinterpret_cast<const ushort4 *>(prb);
+    const uint32_t rb[4] = {r.x, r.y, r.z, r.w};
     idx[0] = swz_tile(base);
 #pragma unroll
-    for (int v = 1; v < (1 << RB); ++v) idx[v] = idx[v & (v - 1)] ^ prb[__ffs(v) - 1];
+    for (int v = 1; v < 16; ++v) idx[v] = idx[v & (v - 1)] ^ rb[(v & 1) ? 0 : (v & 2) ? 1 : (v & 4) ? 2 : 3];
+}
+template <typename R>
+__device__ __forceinline__ void phase_gather(RA<R> *x, const RA<R> *tile, const uint32_t *idx, bool pairs) {
+    if (sizeof(R) == 4 && pairs) {
+#pragma unroll
+        for (int v = 0; v < 16; v += 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(&tile[idx[v]]);
+            memcpy(&x[v], &w.x, 8);
+            memcpy(&x[v + 1], &w.y, 8);
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < 16; ++v) x[v] = tile[idx[v]];
+    }
+}
+template <typename R>
+__device__ __forceinline__ void phase_scatter(const RA<R> *x, RA<R> *tile, const uint32_t *idx, bool pairs) {
+    if (sizeof(R) == 4 && pairs) {
+#pragma unroll
+        for (int v = 0; v < 16; v += 2) {
+            ulonglong2 w;
+            memcpy(&w.x, &x[v], 8);
+            memcpy(&w.y, &x[v + 1], 8);
+            *reinterpret_cast<ulonglong2 *>(&tile[idx[v]]) = w;
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < 16; ++v) tile[idx[v]] = x[v];
+    }
 }
 
-template <typename R, int RB>
-__global__ void __launch_bounds__(512, 1) k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a,
-                                                     const DevOp *__restrict__ ops, const Phase *__restrict__ phases,
-                                                     const RegStep *__restrict__ steps, const R *__restrict__ coef,
-                                                     const Cx<R> *__restrict__ mats,
-                                                     const DiagBlock *__restrict__ dblocks,
-                                                     const DiagMember *__restrict__ dmem) {
-    constexpr int V = 1 << RB;
+// 16-byte copies of a tile between global memory and its swizzled place
+template <typename R>
+__device__ __forceinline__ void reg_tile_load(RA<R> *tile, const Cx<R> *src, const ChunkOff *chunk, uint32_t slot) {
+    constexpr int C = (int)sizeof(Cx<R>);   // 16 / P chunks
+#pragma unroll
+    for (int i = 0; i < C; ++i) cp_async16(&tile[slot ^ chunk[i].s], src + chunk[i].g);
+}
+template <typename R>
+__device__ __forceinline__ void reg_tile_store(Cx<R> *dst, const RA<R> *tile, const ChunkOff *chunk, uint32_t slot,
+                                               R f) {
+    constexpr int C = (int)sizeof(Cx<R>);
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        const ChunkOff c = chunk[i];
+        if constexpr (sizeof(R) == 4) {
+            float4 v = *reinterpret_cast<const float4 *>(&tile[slot ^ c.s]);
+            v.x *= f; v.y *= f; v.z *= f; v.w *= f;
+            *reinterpret_cast<float4 *>(dst + c.g) = v;
+        } else {
+            const double2 v = tile[slot ^ c.s];
+            dst[c.g] = make_double2(v.x * f, v.y * f);
+        }
+    }
+}
+
+// What bounds the register-blocked passes is the issue of their own
+// instructions, not memory: a pass applies tens of gates per round trip to
+// HBM.  So everything that does not depend on the amplitudes is done once per
+// call (k_reg_image) or kept as per-chunk constants, tiles move by 16-byte
+// accesses, and a step's operation is one switch on a decoded code.
+template <typename R>
+__global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256, 1)
+k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *__restrict__ image,
+           const Cx<R> *__restrict__ pmats) {
+    constexpr int RB = kRegBits, V = 1 << RB;
+    constexpr uint32_t P = 16 / sizeof(Cx<R>);
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t T = 1u << a.k;
     RA<R> *tiles = reinterpret_cast<RA<R> *>(smem);          // two tiles: the next one streams in
     unsigned char *sm = smem + 2 * T * sizeof(RA<R>);
     const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), false);
-    reg_setup<R, RB>(sm, L, a, ops, phases, steps, coef, dblocks, dmem, false);
-    __syncthreads();
+    reg_image_load(sm, image, L.image);
     const R ftot = reinterpret_cast<const R *>(sm + L.sc)[a.st_end - a.st_begin];   // product of the RY factors
     const uint64_t *hioff = reinterpret_cast<const uint64_t *>(sm + L.hioff);
+    const ChunkOff *chunk = reinterpret_cast<const ChunkOff *>(sm + L.chunk);
     const Cx<R> *cs = reinterpret_cast<const Cx<R> *>(sm + L.cs);
     const RegStep *st = reinterpret_cast<const RegStep *>(sm + L.steps);
     const DiagBlock *bl = reinterpret_cast<const DiagBlock *>(sm + L.blocks);
+    const PhaseS *phs = reinterpret_cast<const PhaseS *>(sm + L.phases);
     const uint16_t *pbase = reinterpret_cast<const uint16_t *>(sm + L.pbase);
     const uint16_t *prb = reinterpret_cast<const uint16_t *>(sm + L.prb);
     const unsigned char *area = sm + L.area;
-    const int NT = blockDim.x;
+    const int NT = blockDim.x, nph = a.ph_end - a.ph_begin;
     const uint64_t ntiles = 1ull << a.nout;
-    const uint32_t lowmask = (1u << a.nlow) - 1u;
     const uint64_t mine = blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    const uint32_t j0 = P * threadIdx.x, slot = swz_tile(j0);
+    Cx<R> *mypsi = psi + (hioff[j0 >> a.nlow] | (j0 & ((1u << a.nlow) - 1u)));
     // tile bases walked with masked additions (current, and two ahead)
     const BitWalk bw = bit_walk(a.out, a.nout, gridDim.x);
     uint64_t base_pf = deposit(blockIdx.x, a.out, a.nout), base_cur = base_pf;
     for (uint64_t k = 0; k < 2; ++k) {
-        if (k < mine) load_tile_async<R>(tiles + k * T, psi, base_pf, hioff, a.nlow, T);
+        if (k < mine) reg_tile_load<R>(tiles + k * T, mypsi + base_pf, chunk, slot);
         cp_async_commit();
         base_pf = walk_next(base_pf, bw);
     }
@@ -1546,16 +1707,15 @@ __global__ void __launch_bounds__(512, 1) k_gate_reg(Cx<R> *__restrict__ psi, co
         RA<R> *tile = tiles + (it & 1) * T;
         cp_async_wait1();
         __syncthreads();
-        for (int ph = a.ph_begin; ph < a.ph_end; ++ph) {
-            const Phase P = phases[ph];
-            const uint32_t base = pbase[(ph - a.ph_begin) * NT + threadIdx.x];
+        for (int ph = 0; ph < nph; ++ph) {
+            const PhaseS F = phs[ph];
+            const uint32_t base = pbase[ph * NT + threadIdx.x];
             uint32_t idx[V];
-            phase_slots<RB>(idx, base, prb + (ph - a.ph_begin) * 4);
+            phase_slots16(idx, base, prb + ph * 4);
             RA<R> x[V];
-#pragma unroll
-            for (int v = 0; v < V; ++v) x[v] = tile[idx[v]];
-            for (int s = P.st_begin; s < P.st_end; ++s) {
-                const RegStep S = st[s - a.st_begin];
+            phase_gather<R>(x, tile, idx, F.rmask & 1u);
+            for (int s = F.st_begin; s < F.st_end; ++s) {
+                const RegStep S = st[s];
                 if (S.type == SV_STEP_ROT) {
                     // factored RYs (t, factor): the factors are applied at the store
                     const Cx<R> *c = cs + (S.op_begin - a.op_begin);
@@ -1568,41 +1728,32 @@ __global__ void __launch_bounds__(512, 1) k_gate_reg(Cx<R> *__restrict__ psi, co
                 } else if (S.type == SV_STEP_DIAG) {
                     reg_diag<R, RB>(x, bl[S.a - a.db_begin], area);
                 } else {
-                    DevOp op = ops[S.a];
-                    if (has_out_target(op)) op = resolve_out(op, gbase);
-                    ra_apply_op<R, RB>(x, op, P.rmask, base, cs[S.a - a.op_begin], mats, false);
+                    reg_op<R, true>(x, (uint32_t)S.a, F.rmask, base, gbase, cs[S.op_begin], pmats + S.op_end);
                 }
             }
-#pragma unroll
-            for (int v = 0; v < V; ++v) tile[idx[v]] = x[v];
+            phase_scatter<R>(x, tile, idx, F.rmask & 1u);
             __syncthreads();
         }
-        const Cx<R> *tc = reinterpret_cast<const Cx<R> *>(tile);
-        for (uint32_t j = threadIdx.x; j < T; j += NT) {
-            const Cx<R> v = tc[swz_tile(j)];
-            psi[gbase | hioff[j >> a.nlow] | (j & lowmask)] = mk<R>(v.x * ftot, v.y * ftot);
-        }
-        __syncthreads();
-        if (it + 2 < mine) load_tile_async<R>(tile, psi, base_pf, hioff, a.nlow, T);
+        reg_tile_store<R>(mypsi + gbase, tile, chunk, slot, ftot);
+        // a thread reloads exactly the slots it has just stored from
+        if (it + 2 < mine) reg_tile_load<R>(tile, mypsi + base_pf, chunk, slot);
         cp_async_commit();
         base_pf = walk_next(base_pf, bw);
     }
 }
 
-template <typename R, int RB>
-__global__ void __launch_bounds__(512, 1) k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam,
-                                                    const GatePassArgs a, const DevOp *__restrict__ ops,
-                                                    const Phase *__restrict__ phases, const RegStep *__restrict__ steps,
-                                                    const R *__restrict__ coef, const Cx<R> *__restrict__ mats,
-                                                    double *__restrict__ part, int part_stride,
-                                                    const DiagBlock *__restrict__ dblocks,
-                                                    const DiagMember *__restrict__ dmem) {
-    constexpr int V = 1 << RB;
+template <typename R>
+__global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256, 1)
+k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam, const GatePassArgs a,
+          const unsigned char *__restrict__ image, const Cx<R> *__restrict__ pmats, double *__restrict__ part,
+          int part_stride) {
+    constexpr int RB = kRegBits, V = 1 << RB;
+    constexpr uint32_t P = 16 / sizeof(Cx<R>);
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t T = 1u << a.k;
-    const int nops = a.op_end - a.op_begin;
+    const int nops = a.op_end - a.op_begin, nph = a.ph_end - a.ph_begin;
     const int NT = blockDim.x, nwarps = NT >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // slot row stride nwarps + 1: the lanes 0, 8, 16, 24 that add the four
+    // slot row stride 17: the lanes 0, 8, 16, 24 that add the four
     // gradients of a step (ops o .. o+3) hit four different banks
     const int AS = kAdjSlotStride;
     RA<R> *tl = reinterpret_cast<RA<R> *>(smem);           // lambda tile, then the psi tile
@@ -1614,29 +1765,35 @@ __global__ void __launch_bounds__(512, 1) k_adj_reg(Cx<R> *__restrict__ psi, Cx<
     for (int j = threadIdx.x; j < nops * AS; j += NT) acc[j] = 0;
     if constexpr (sizeof(R) == 4)
         for (int j = threadIdx.x; j < nops; j += NT) tot64[j] = 0.0;
-    reg_setup<R, RB>(sm, L, a, ops, phases, steps, coef, dblocks, dmem, true);
-    __syncthreads();
+    reg_image_load(sm, image, L.image);
     // factored RYs: before step s both registers sets hold the true vectors
     // divided by scf[s], so a gradient part computed there is scaled by
     // scf[s]^2; the stores multiply by the total factor
     const R *scf = reinterpret_cast<const R *>(sm + L.sc);
     const R ftot = scf[a.st_end - a.st_begin];
     const uint64_t *hioff = reinterpret_cast<const uint64_t *>(sm + L.hioff);
+    const ChunkOff *chunk = reinterpret_cast<const ChunkOff *>(sm + L.chunk);
     const Cx<R> *cs = reinterpret_cast<const Cx<R> *>(sm + L.cs);
     const RegStep *st = reinterpret_cast<const RegStep *>(sm + L.steps);
     const DiagBlock *bl = reinterpret_cast<const DiagBlock *>(sm + L.blocks);
+    const PhaseS *phs = reinterpret_cast<const PhaseS *>(sm + L.phases);
     const uint16_t *pbase = reinterpret_cast<const uint16_t *>(sm + L.pbase);
     const uint16_t *prb = reinterpret_cast<const uint16_t *>(sm + L.prb);
     const unsigned char *area = sm + L.area;
     const DiagMember *mem = reinterpret_cast<const DiagMember *>(sm + L.mem);
     const uint64_t ntiles = 1ull << a.nout;
-    const uint32_t lowmask = (1u << a.nlow) - 1u;
     const uint64_t mine = blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    const uint32_t j0 = P * threadIdx.x, slot = swz_tile(j0);
+    const uint64_t toff = hioff[j0 >> a.nlow] | (j0 & ((1u << a.nlow) - 1u));
     const BitWalk bw = bit_walk(a.out, a.nout, gridDim.x);
     uint64_t gnext = deposit(blockIdx.x, a.out, a.nout);
     for (uint64_t it = 0; it < mine; ++it) {
         const uint64_t gbase = gnext;
         gnext = walk_next(gnext, bw);
+        // a thread's pieces go to the slots that it stored from last
+        reg_tile_load<R>(tp, psi + (gbase | toff), chunk, slot);
+        reg_tile_load<R>(tl, lam + (gbase | toff), chunk, slot);
+        cp_async_commit();
         if (it + 1 < mine) {
             // the next tile's psi and lambda runs head for L2 while this one is processed
             const uint64_t gn = gnext;
@@ -1646,47 +1803,19 @@ __global__ void __launch_bounds__(512, 1) k_adj_reg(Cx<R> *__restrict__ psi, Cx<
                 prefetch_l2(lam + (gn | hioff[j]), runbytes);
             }
         }
-        {
-            Cx<R> *tpc = reinterpret_cast<Cx<R> *>(tp), *tlc = reinterpret_cast<Cx<R> *>(tl);
-            if (T == (uint32_t)(V * NT)) {
-                // every load of the thread in flight before the first store
-                Cx<R> vp[V], vl[V];
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const uint32_t j = threadIdx.x + (uint32_t)v * NT;
-                    const uint64_t gi = gbase | hioff[j >> a.nlow] | (j & lowmask);
-                    vp[v] = psi[gi];
-                    vl[v] = lam[gi];
-                }
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const uint32_t j = threadIdx.x + (uint32_t)v * NT;
-                    tpc[swz_tile(j)] = vp[v];
-                    tlc[swz_tile(j)] = vl[v];
-                }
-            } else {
-                for (uint32_t j = threadIdx.x; j < T; j += NT) {
-                    const uint64_t gi = gbase | hioff[j >> a.nlow] | (j & lowmask);
-                    tpc[swz_tile(j)] = psi[gi];
-                    tlc[swz_tile(j)] = lam[gi];
-                }
-            }
-        }
+        cp_async_wait0();
         __syncthreads();
-        for (int ph = a.ph_end - 1; ph >= a.ph_begin; --ph) {
-            const Phase P = phases[ph];
-            const uint32_t base = pbase[(ph - a.ph_begin) * NT + threadIdx.x];
+        for (int ph = nph - 1; ph >= 0; --ph) {
+            const PhaseS F = phs[ph];
+            const uint32_t base = pbase[ph * NT + threadIdx.x];
             uint32_t idx[V];
-            phase_slots<RB>(idx, base, prb + (ph - a.ph_begin) * 4);
+            phase_slots16(idx, base, prb + ph * 4);
             RA<R> xp[V], xl[V];
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                xp[v] = tp[idx[v]];
-                xl[v] = tl[idx[v]];
-            }
-            for (int s = P.st_end - 1; s >= P.st_begin; --s) {
-                const RegStep S = st[s - a.st_begin];
-                const R fs = scf[s - a.st_begin], fs2 = fs * fs;
+            phase_gather<R>(xp, tp, idx, F.rmask & 1u);
+            phase_gather<R>(xl, tl, idx, F.rmask & 1u);
+            for (int s = F.st_end - 1; s >= F.st_begin; --s) {
+                const RegStep S = st[s];
+                const R fs = scf[s], fs2 = fs * fs;
                 if (S.type == SV_STEP_ROT) {
                     // every RY of the step: gradient part at the step's end (they commute), then RY^dagger
                     R g[4] = {0, 0, 0, 0};
@@ -1695,10 +1824,9 @@ __global__ void __launch_bounds__(512, 1) k_adj_reg(Cx<R> *__restrict__ psi, Cx<
                         if (!((S.a >> b) & 1)) continue;
                         switch (b) {
                         case 0: g[0] = ra_ry_grad<R, V, 0>(xp, xl); break;
-                        case 1: if constexpr (RB > 1) g[1] = ra_ry_grad<R, V, 1>(xp, xl); break;
-                        case 2: if constexpr (RB > 2) g[2] = ra_ry_grad<R, V, 2>(xp, xl); break;
-                        case 3: if constexpr (RB > 3) g[3] = ra_ry_grad<R, V, 3>(xp, xl); break;
-                        default: break;
+                        case 1: g[1] = ra_ry_grad<R, V, 1>(xp, xl); break;
+                        case 2: g[2] = ra_ry_grad<R, V, 2>(xp, xl); break;
+                        default: g[3] = ra_ry_grad<R, V, 3>(xp, xl); break;
                         }
                     }
                     const R tot = warp_sum4<R>(g[0], g[1], g[2], g[3]) * fs2;
@@ -1757,34 +1885,23 @@ __global__ void __launch_bounds__(512, 1) k_adj_reg(Cx<R> *__restrict__ psi, Cx<
                     }
                     reg_diag2<R, RB>(xp, xl, B, area);
                 } else {
-                    DevOp op = ops[S.a];
-                    if (has_out_target(op)) op = resolve_out(op, gbase);
-                    R g = ra_adjoint_op<R, RB>(xp, xl, op, P.rmask, base, cs[S.a - a.op_begin], mats);
-                    if (has_param(op.kind)) {
+                    // the prepared matrix is followed by its conjugate transpose (1-qubit matrices: 4 elements)
+                    R g = reg_op_adj<R>(xp, xl, (uint32_t)S.a, F.rmask, base, gbase, cs[S.op_begin],
+                                        pmats + S.op_end + 4);
+                    if (reg_op_param((uint32_t)S.a)) {
                         g = warp_sum<R>(g) * fs2;
-                        if (lane == 0) acc[(S.a - a.op_begin) * AS + warp] += g;
+                        if (lane == 0) acc[S.op_begin * AS + warp] += g;
                     }
                 }
             }
             // the slots again (fewer registers live across the steps)
-            phase_slots<RB>(idx, pbase[(ph - a.ph_begin) * NT + threadIdx.x], prb + (ph - a.ph_begin) * 4);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                tp[idx[v]] = xp[v];
-                tl[idx[v]] = xl[v];
-            }
+            phase_slots16(idx, pbase[ph * NT + threadIdx.x], prb + ph * 4);
+            phase_scatter<R>(xp, tp, idx, F.rmask & 1u);
+            phase_scatter<R>(xl, tl, idx, F.rmask & 1u);
             __syncthreads();
         }
-        {
-            const Cx<R> *tpc = reinterpret_cast<const Cx<R> *>(tp), *tlc = reinterpret_cast<const Cx<R> *>(tl);
-            for (uint32_t j = threadIdx.x; j < T; j += NT) {
-                const uint64_t gi = gbase | hioff[j >> a.nlow] | (j & lowmask);
-                const Cx<R> p = tpc[swz_tile(j)], l = tlc[swz_tile(j)];
-                psi[gi] = mk<R>(p.x * ftot, p.y * ftot);
-                lam[gi] = mk<R>(l.x * ftot, l.y * ftot);
-            }
-        }
-        __syncthreads();
+        reg_tile_store<R>(psi + (gbase | toff), tp, chunk, slot, ftot);
+        reg_tile_store<R>(lam + (gbase | toff), tl, chunk, slot, ftot);
         if constexpr (sizeof(R) == 4) {
             // the next writes to the slots follow the next tile's barrier
             if (((it + 1) % kAdjFlush) == 0 || it + 1 == mine) {
@@ -1808,7 +1925,24 @@ __global__ void __launch_bounds__(512, 1) k_adj_reg(Cx<R> *__restrict__ psi, Cx<
         part[(size_t)blockIdx.x * part_stride + a.op_begin + o] = tsum;
     }
 }
-#undef SV_RB_SWITCH
+
+// Prepared matrices (PrepMat), one block each.
+template <typename R>
+__global__ void k_prep_mats(const PrepMat *__restrict__ prep, const Cx<R> *__restrict__ mats, Cx<R> *__restrict__ out) {
+    const PrepMat p = prep[blockIdx.x];
+    const int dim = 1 << p.nq;
+    auto caller = [&](int u) {
+        int j = 0;
+        for (int t = 0; t < p.nq; ++t) j |= ((u >> p.perm[t]) & 1) << t;
+        return j;
+    };
+    for (int q = threadIdx.x; q < dim * dim; q += blockDim.x) {
+        const int ju = caller(q >> p.nq), jw = caller(q & (dim - 1));
+        out[p.dst + q] = mats[p.src + ju * dim + jw];
+        const Cx<R> c = mats[p.src + jw * dim + ju];
+        out[p.dst + dim * dim + q] = mk<R>(c.x, -c.y);
+    }
+}
 
 // -------------------------------------------------------------------- K-QR --
 struct SwapArgs {
@@ -3091,15 +3225,19 @@ __device__ __forceinline__ void hpsi_row16(float2 *acc, uint32_t Bl, uint32_t g0
 // sign bits parity(l & z) ^ parity(a0 & bz) ^ nY of every string.  Per coset
 // one ballot gives parity(rep & z) of every string.
 constexpr int kHpsiTab = 32;
+// The same for passes with more strings (several per X/Y mask), in dynamic
+// shared memory; tz gives the coset-independent sign, parity(tid & tz).
+struct HpsiStr {
+    uint64_t z;
+    uint32_t X, g, w, tz;
+};
+static_assert(sizeof(HpsiStr) == 24, "HpsiStr layout");
 struct HpsiTab {
     uint64_t z[kHpsiTab];
     uint32_t X[kHpsiTab], g[kHpsiTab], w[kHpsiTab];
 };
 
-__device__ __forceinline__ void hpsi_tab_string(float2 *acc, const HpsiTab &T, int k, uint32_t sb, uint32_t bmask) {
-    const uint32_t Xo = T.X[k];
-    const uint32_t g0 = T.g[k] ^ (((bmask >> k) & 1u) << 31);
-    const uint32_t w = T.w[k];
+__device__ __forceinline__ void hpsi_string(float2 *acc, uint32_t Xo, uint32_t g0, uint32_t w, uint32_t sb) {
     const uint32_t Bl = sb + ((threadIdx.x ^ (Xo & 511u)) << 3);
     switch (((Xo >> 9) & 15u) | ((Xo >> 31) << 4)) {
 #define SV_HC(C) case C: hpsi_row16<((C) >> 4) != 0, (C) & 15>(acc, Bl, g0, w); break;
@@ -3110,6 +3248,9 @@ __device__ __forceinline__ void hpsi_tab_string(float2 *acc, const HpsiTab &T, i
 #undef SV_HC
     default: break;
     }
+}
+__device__ __forceinline__ void hpsi_tab_string(float2 *acc, const HpsiTab &T, int k, uint32_t sb, uint32_t bmask) {
+    hpsi_string(acc, T.X[k], T.g[k] ^ (((bmask >> k) & 1u) << 31), T.w[k], sb);
 }
 
 template <typename R, int EPT>
@@ -3122,6 +3263,7 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
     const uint32_t E = 1u << (a.kl + a.m);
     Cx<R> *buf = reinterpret_cast<Cx<R> *>(smem);
     uint64_t *spanv = reinterpret_cast<uint64_t *>(buf + 2 * E);
+    HpsiStr *many = reinterpret_cast<HpsiStr *>(spanv + (1u << a.m));   // passes of more than kHpsiTab strings
     __shared__ double wsum[32];
     coset_span(a, spanv);
     const ThreadCoset tc = thread_coset(a.kl);
@@ -3144,21 +3286,28 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
     uint32_t tmask = 0;
     if constexpr (sizeof(R) == 4 && EPT == 16) {
         if (fast) {
-            for (int gi = a.g_begin; gi < a.g_end; ++gi) {
-                const DevGroup G = groups[gi];
-                for (int sidx = G.s_begin; sidx < G.s_end; ++sidx, ++ns) {
-                    if (ns >= kHpsiTab) continue;
-                    const DevString S = strs[sidx];
-                    tmask |= (uint32_t)((__popcll(tc.l & S.z) ^ __popc(tc.a0 & S.bz) ^ S.nY) & 1) << ns;
-                    if (threadIdx.x == 0) {
-                        const float g = (S.nY & 2) ? -(float)S.coef : (float)S.coef;
-                        tabs.z[ns] = S.z;
-                        tabs.X[ns] = G.X | ((uint32_t)(S.nY & 1) << 31);
-                        tabs.g[ns] = __float_as_uint(g);
-                        tabs.w[ns] = S.bz >> tc.ash;
-                    }
+            ns = a.s_end - a.s_begin;
+            for (int q = (int)threadIdx.x; q < ns; q += 512) {
+                const DevString S = strs[a.s_begin + q];
+                const float g = (S.nY & 2) ? -(float)S.coef : (float)S.coef;
+                if (ns <= kHpsiTab) {
+                    tabs.z[q] = S.z;
+                    tabs.X[q] = S.X | ((uint32_t)(S.nY & 1) << 31);
+                    tabs.g[q] = __float_as_uint(g);
+                    tabs.w[q] = S.bz >> tc.ash;
+                } else {
+                    many[q].z = S.z;
+                    many[q].X = S.X | ((uint32_t)(S.nY & 1) << 31);
+                    many[q].g = __float_as_uint((S.nY & 1) ? -g : g);
+                    many[q].w = S.bz >> tc.ash;
+                    many[q].tz = (uint32_t)(S.z & ((1ull << a.kl) - 1ull)) | ((S.bz & ((1u << tc.ash) - 1u)) << a.kl);
                 }
             }
+            if (ns <= kHpsiTab)
+                for (int q = 0; q < ns; ++q) {
+                    const DevString S = strs[a.s_begin + q];
+                    tmask |= (uint32_t)((__popcll(tc.l & S.z) ^ __popc(tc.a0 & S.bz) ^ S.nY) & 1) << q;
+                }
             __syncthreads();
         }
     }
@@ -3189,21 +3338,23 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
                     hpsi_tab_string(reinterpret_cast<float2 *>(acc), tabs, k, sb, bmask);
             }
         }
-        for (int gi = tabbed ? a.g_end : a.g_begin; gi < a.g_end; ++gi) {
+        if constexpr (sizeof(R) == 4 && EPT == 16) {
+            if (fast && !tabbed) {
+                const uint32_t sb = smem_u32(t);
+                for (int k = 0; k < ns; ++k) {
+                    const HpsiStr h = many[k];
+                    const uint32_t neg = (uint32_t)(__popcll(rep & h.z) ^ __popc(threadIdx.x & h.tz)) & 1u;
+                    hpsi_string(reinterpret_cast<float2 *>(acc), h.X, h.g ^ (neg << 31), h.w, sb);
+                }
+            }
+        }
+        const bool staged = sizeof(R) == 4 && EPT == 16 && fast;
+        for (int gi = staged ? a.g_end : a.g_begin; gi < a.g_end; ++gi) {
             const DevGroup G = groups[gi];
             for (int s = G.s_begin; s < G.s_end; ++s) {
                 const DevString S = strs[s];
                 const int base = (__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz) ^ S.nY) & 1;
                 const R g = (S.nY & 2) ? -(R)S.coef : (R)S.coef;
-                if constexpr (sizeof(R) == 4 && EPT == 16) {
-                    if (fast) {
-                        const uint32_t g0 = __float_as_uint((float)g) ^ ((uint32_t)base << 31);
-                        const uint32_t B = (threadIdx.x ^ G.X) * 8u;
-                        if (S.nY & 1) hpsi_gray16<true>(reinterpret_cast<float2 *>(acc), smem_u32(t), B, g0, S.bz >> tc.ash);
-                        else hpsi_gray16<false>(reinterpret_cast<float2 *>(acc), smem_u32(t), B, g0, S.bz >> tc.ash);
-                        continue;
-                    }
-                }
                 const uint32_t jm = walsh_mask(S.bz >> tc.ash);
                 if (fast) {
                     const uint32_t sm = base ? ~jm : jm;
@@ -3255,6 +3406,202 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
     }
 }
 
+// ------------------------------------------------ slices of small states --
+// Few cosets (a small state) leave most SMs idle when a CTA takes whole
+// cosets with all of a pass's strings: n = 14 has 2 cosets of 2^13, so 2 of
+// 152 CTAs worked through 256 strings each (230 us a pass).  Here S CTAs
+// share a coset: each stages all of it (64 KB, from L2) and evaluates its
+// slice of the strings (expectation) or of the outputs (H|psi>), so nothing
+// is combined across CTAs and the result does not depend on S.
+
+// Element-index mask of string S in a coset: parity(b & z) for b = rep ^
+// span(e >> kl) ^ (e mod 2^kl) is parity(rep & z) ^ parity(e & tau).
+__device__ __forceinline__ uint32_t coset_tau(const DevString &S, int kl) {
+    return (uint32_t)(S.z & ((1ull << kl) - 1ull)) | (S.bz << kl);
+}
+
+// <psi|P|psi> over one coset, a warp per string: lane L takes the elements
+// e = L + 32 i.  With a flipped bit h >= 5 only the elements with bit h clear
+// are taken (one of each pair, times 2); else every element (each pair from
+// both sides).  Eight elements at a time, signed by the Walsh function of
+// the low three bits of i, the rest of i's parity once per eight.
+template <typename R>
+__global__ void __launch_bounds__(512) k_evc_slice(const Cx<R> *__restrict__ psi, const CosetArgs a,
+                                                   const DevString *__restrict__ strs, double *__restrict__ part,
+                                                   int part_stride, int slices) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const uint32_t E = 1u << (a.kl + a.m);
+    Cx<R> *t = reinterpret_cast<Cx<R> *>(smem);
+    uint64_t *spanv = reinterpret_cast<uint64_t *>(t + E);
+    const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t c = blockIdx.x / (uint32_t)slices, sl = blockIdx.x % (uint32_t)slices;
+    coset_span(a, spanv);
+    const uint64_t rep = deposit(c, a.freeb, a.nfree);
+    load_coset<R>(t, psi, rep, spanv, a.kl, E);
+    cp_async_commit();
+    cp_async_wait0();
+    __syncthreads();
+    for (int q = a.s_begin + (int)sl * nwarps + warp; q < a.s_end; q += nwarps * slices) {
+        const DevString S = strs[q];
+        const uint32_t X = S.X, tau = coset_tau(S, a.kl);
+        const bool odd = S.nY & 1;
+        const int hb = X ? 31 - __clz(X) : 0;
+        const bool half = hb >= 5;
+        const uint32_t n8 = (half ? E >> 1 : E) >> 8;      // groups of 8 x 32 elements
+        // i runs over the selected rows; bit hb - 5 is inserted as 0
+        const int ib = half ? hb - 5 : 31;
+        R acc = 0;
+        if (n8 == 0) {                                      // tiny cosets
+            for (uint32_t i = 0; i < ((half ? E >> 1 : E) + 31) / 32; ++i) {
+                const uint32_t row = half ? ins0(i, ib) : i, e = (row << 5) | lane;
+                if (e >= E) continue;
+                const Cx<R> u = t[e], v = t[e ^ X];
+                const R val = odd ? (v.x * u.y - v.y * u.x) : (v.x * u.x + v.y * u.y);
+                acc += (__popc(e & tau) & 1) ? -val : val;
+            }
+        }
+        R sg[8];
+        uint32_t r8[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t row = half ? ins0((uint32_t)k, ib) : (uint32_t)k;
+            r8[k] = row << 5;
+            sg[k] = (__popc((row << 5) & tau) & 1) ? (R)-1 : (R)1;
+        }
+        for (uint32_t g = 0; g < n8; ++g) {
+            const uint32_t e0 = ((half ? ins0(g << 3, ib) : g << 3) << 5) | lane;
+            R sub = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const uint32_t e = e0 | r8[k];
+                const Cx<R> u = t[e], v = t[e ^ X];
+                const R val = odd ? (v.x * u.y - v.y * u.x) : (v.x * u.x + v.y * u.y);
+                sub = fma(sg[k], val, sub);
+            }
+            acc += (__popc(e0 & tau) & 1) ? -sub : sub;
+        }
+        if (half) acc *= 2;
+        if (__popcll(rep & S.z) & 1) acc = -acc;
+        if (X && ((S.nY == 1) | (S.nY == 2))) acc = -acc;
+        double v = (double)acc;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) part[(size_t)c * part_stride + q] = v;
+    }
+}
+
+// lambda over one coset, the outputs split into S slices of O: with O >= 512
+// a thread holds EPT = O / 512 outputs and takes every string; with fewer,
+// 512 / O groups of warps share the strings and are summed in a fixed order.
+template <typename R> struct HSliceStr { R g; uint32_t X, tau; };   // X bit 31: nY odd
+constexpr int kHSliceTab = 256;                                     // strings staged at a time
+template <typename R, int EPT>
+__global__ void __launch_bounds__(512) k_hpsi_slice(const Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam,
+                                                    const CosetArgs a, const DevString *__restrict__ strs, int first,
+                                                    int last, double *__restrict__ epart, int slices) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const uint32_t E = 1u << (a.kl + a.m), O = E / (uint32_t)slices;
+    Cx<R> *t = reinterpret_cast<Cx<R> *>(smem);
+    uint64_t *spanv = reinterpret_cast<uint64_t *>(t + E);
+    HSliceStr<R> *tab = reinterpret_cast<HSliceStr<R> *>(spanv + (1u << a.m));
+    Cx<R> *red = reinterpret_cast<Cx<R> *>(tab + kHSliceTab);        // [512] when strings are shared
+    __shared__ double wsum[16];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t c = blockIdx.x / (uint32_t)slices, sl = blockIdx.x % (uint32_t)slices;
+    coset_span(a, spanv);
+    const uint64_t rep = deposit(c, a.freeb, a.nfree);
+    load_coset<R>(t, psi, rep, spanv, a.kl, E);
+    cp_async_commit();
+    const uint32_t lm = (1u << a.kl) - 1u;
+    const uint32_t OT = O < 512u ? O : 512u;                         // output threads
+    const uint32_t e0 = sl * O + (threadIdx.x & (OT - 1u)), sgrp = threadIdx.x / OT, nsg = 512u / OT;
+    const bool owner = sgrp == 0;
+    Cx<R> old[EPT], acc[EPT];
+#pragma unroll
+    for (int j = 0; j < EPT; ++j) {
+        const uint32_t e = e0 + j * 512u;
+        old[j] = mk<R>(0, 0);
+        if (!first && owner) old[j] = lam[rep ^ spanv[e >> a.kl] ^ (e & lm)];
+        acc[j] = mk<R>(0, 0);
+    }
+    for (int q0 = a.s_begin; q0 < a.s_end; q0 += kHSliceTab) {
+        const int nq = min(kHSliceTab, a.s_end - q0);
+        __syncthreads();                                             // the previous part of the table is used up
+        for (int q = threadIdx.x; q < nq; q += 512) {
+            const DevString S = strs[q0 + q];
+            HSliceStr<R> h;
+            const bool neg = ((S.nY >> 1) ^ S.nY ^ __popcll(rep & S.z)) & 1;
+            h.g = neg ? -(R)S.coef : (R)S.coef;
+            h.X = S.X | ((uint32_t)(S.nY & 1) << 31);
+            h.tau = coset_tau(S, a.kl);
+            tab[q] = h;
+        }
+        cp_async_wait0();
+        __syncthreads();
+#pragma unroll 4
+        for (int q = (int)sgrp; q < nq; q += (int)nsg) {
+            const HSliceStr<R> h = tab[q];
+            const uint32_t X = h.X & 0x7FFFFFFFu;
+            const R g = (__popc(e0 & h.tau) & 1) ? -h.g : h.g;
+            // parity of j's bits (element bits 9 and up) against tau
+            const uint32_t jm = EPT > 1 ? walsh_mask((h.tau >> 9) & (EPT - 1)) : 0u;
+            if (h.X >> 31) {          // i * f * v
+#pragma unroll
+                for (int j = 0; j < EPT; ++j) {
+                    const Cx<R> v = t[(e0 + j * 512u) ^ X];
+                    const R f = ((jm >> j) & 1u) ? -g : g;
+                    acc[j].x -= f * v.y;
+                    acc[j].y += f * v.x;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < EPT; ++j) {
+                    const Cx<R> v = t[(e0 + j * 512u) ^ X];
+                    const R f = ((jm >> j) & 1u) ? -g : g;
+                    acc[j].x += f * v.x;
+                    acc[j].y += f * v.y;
+                }
+            }
+        }
+    }
+    cp_async_wait0();
+    __syncthreads();
+    if (nsg > 1) {
+        red[threadIdx.x] = acc[0];
+        __syncthreads();
+        if (owner) {
+            for (uint32_t k = 1; k < nsg; ++k) {
+                const Cx<R> v = red[k * OT + threadIdx.x];
+                acc[0].x += v.x;
+                acc[0].y += v.y;
+            }
+        }
+    }
+    double ev = 0;
+    if (owner) {
+        R el = 0;
+#pragma unroll
+        for (int j = 0; j < EPT; ++j) {
+            const uint32_t e = e0 + j * 512u;
+            acc[j].x += old[j].x;
+            acc[j].y += old[j].y;
+            lam[rep ^ spanv[e >> a.kl] ^ (e & lm)] = acc[j];
+            const Cx<R> p = t[e];
+            el += p.x * acc[j].x + p.y * acc[j].y;
+        }
+        ev = (double)el;
+    }
+    if (last) {
+        for (int o = 16; o > 0; o >>= 1) ev += __shfl_xor_sync(0xffffffffu, ev, o);
+        if (lane == 0) wsum[warp] = ev;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < 16; ++w) s += wsum[w];
+            epart[blockIdx.x] = s;
+        }
+    }
+}
+
 // ----------------------------------------------------------------- K-BATCH --
 // Many independent small states in ONE persistent launch.  A CTA takes a whole
 // state at a time from an atomic work counter (states pre-sorted longest
@@ -3272,6 +3619,36 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     return t;
 }
 
+// A thread's amplitudes of a phase (tile indices base | sp[v]); a phase that
+// holds tile bit 0 moves complex64 pairs by one 16-byte access, as
+// phase_gather does.
+template <typename R, int V>
+__device__ __forceinline__ void batch_gather(Cx<R> *x, const Cx<R> *tile, uint32_t base, const uint32_t *sp, bool pairs) {
+    if (sizeof(R) == 4 && pairs) {
+#pragma unroll
+        for (int v = 0; v < V; v += 2) {
+            const float4 w = *reinterpret_cast<const float4 *>(&tile[swz_tile(base | sp[v])]);
+            x[v] = mk<R>((R)w.x, (R)w.y);
+            x[v + 1] = mk<R>((R)w.z, (R)w.w);
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) x[v] = tile[swz_tile(base | sp[v])];
+    }
+}
+template <typename R, int V>
+__device__ __forceinline__ void batch_scatter(const Cx<R> *x, Cx<R> *tile, uint32_t base, const uint32_t *sp, bool pairs) {
+    if (sizeof(R) == 4 && pairs) {
+#pragma unroll
+        for (int v = 0; v < V; v += 2)
+            *reinterpret_cast<float4 *>(&tile[swz_tile(base | sp[v])]) =
+                make_float4((float)x[v].x, (float)x[v].y, (float)x[v + 1].x, (float)x[v + 1].y);
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) tile[swz_tile(base | sp[v])] = x[v];
+    }
+}
+
 // Register-phased tile of a gate pass inside the batched kernel (512
 // threads): the tile is staged swizzled, each phase gathers the thread's
 // 2^RB amplitudes, applies its gates in registers, scatters them back.
@@ -3283,13 +3660,11 @@ __device__ __noinline__ void batch_reg_forward(Cx<R> *tile, const GatePassArgs &
         const Phase F = phases[ph];
         uint32_t base, sp[V];
         phase_index<RB>(F.rmask, P.k, base, sp);
-        base = phase_base(F.rmask, F.lanes, P.k);   // the phase's lane bits (conflict-free half-warps)
+        base = phase_base(F.rmask, F.lanes, P.k, threadIdx.x);   // the phase's lane bits (conflict-free half-warps)
         Cx<R> x[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) x[v] = tile[swz_tile(base | sp[v])];
+        batch_gather<R, V>(x, tile, base, sp, F.rmask & 1u);
         for (int o = F.op_begin; o < F.op_end; ++o) reg_apply<R, RB>(x, ops[o], F.rmask, base, coef, nullptr, false);
-#pragma unroll
-        for (int v = 0; v < V; ++v) tile[swz_tile(base | sp[v])] = x[v];
+        batch_scatter<R, V>(x, tile, base, sp, F.rmask & 1u);
         __syncthreads();
     }
 }
@@ -3325,14 +3700,10 @@ __device__ __noinline__ void batch_reg_adjoint(Cx<R> *tp, Cx<R> *tl, const GateP
         const Phase F = phases[ph];
         uint32_t base, sp[V];
         phase_index<RB>(F.rmask, P.k, base, sp);
-        base = phase_base(F.rmask, F.lanes, P.k);   // the phase's lane bits (conflict-free half-warps)
+        base = phase_base(F.rmask, F.lanes, P.k, threadIdx.x);   // the phase's lane bits (conflict-free half-warps)
         Cx<R> xp[V], xl[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const uint32_t si = swz_tile(base | sp[v]);
-            xp[v] = tp[si];
-            xl[v] = tl[si];
-        }
+        batch_gather<R, V>(xp, tp, base, sp, F.rmask & 1u);
+        batch_gather<R, V>(xl, tl, base, sp, F.rmask & 1u);
         for (int o = F.op_end - 1; o >= F.op_begin; --o) {
             const DevOp op = ops[o];
             R g = reg_adjoint<R, RB>(xp, xl, op, F.rmask, base, coef, nullptr);
@@ -3341,12 +3712,8 @@ __device__ __noinline__ void batch_reg_adjoint(Cx<R> *tp, Cx<R> *tl, const GateP
                 if (lane == 0) opacc[(o - o0) * nwarps + warp] += g;
             }
         }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const uint32_t si = swz_tile(base | sp[v]);
-            tp[si] = xp[v];
-            tl[si] = xl[v];
-        }
+        batch_scatter<R, V>(xp, tp, base, sp, F.rmask & 1u);
+        batch_scatter<R, V>(xl, tl, base, sp, F.rmask & 1u);
         __syncthreads();
     }
 }
@@ -3837,65 +4204,6 @@ cudaError_t launch_gate_pass(sv_dtype dt, cudaStream_t st, int grid, int threads
     return cudaGetLastError();
 }
 
-template <typename R>
-cudaError_t gate_reg_dispatch(cudaStream_t st, int grid, void *psi, const GatePassArgs &a, const DevOp *ops,
-                              const Phase *phases, const RegStep *steps, const void *coef, const void *mats,
-                              const DiagBlock *dblocks, const DiagMember *dmem) {
-    const size_t sm = gate_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
-    switch (a.k - 9) {
-#define SV_GR(RB)                                                                                            \
-    case RB:                                                                                                 \
-        allow_smem(k_gate_reg<R, RB>, sm);                                                                   \
-        k_gate_reg<R, RB><<<grid, kRegThreads, sm, st>>>((Cx<R> *)psi, a, ops, phases, steps, (const R *)coef, \
-                                                         (const Cx<R> *)mats, dblocks, dmem);                \
-        break;
-        SV_GR(2) SV_GR(3)
-    case 4:   // complex128 tiles hold at most 2^12 amplitudes
-        if constexpr (sizeof(R) == 4) {
-            allow_smem(k_gate_reg<R, 4>, sm);
-            k_gate_reg<R, 4><<<grid, kRegThreads, sm, st>>>((Cx<R> *)psi, a, ops, phases, steps, (const R *)coef,
-                                                            (const Cx<R> *)mats, dblocks, dmem);
-            break;
-        }
-        return cudaErrorInvalidValue;
-#undef SV_GR
-    default:
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-template <typename R>
-cudaError_t adj_reg_dispatch(cudaStream_t st, int grid, void *psi, void *lam, const GatePassArgs &a,
-                             const DevOp *ops, const Phase *phases, const RegStep *steps, const void *coef,
-                             const void *mats, double *part, int part_stride, const DiagBlock *dblocks,
-                             const DiagMember *dmem) {
-    const size_t sm = adj_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
-    switch (a.k - 9) {
-#define SV_AR(RB)                                                                                            \
-    case RB:                                                                                                 \
-        allow_smem(k_adj_reg<R, RB>, sm);                                                                    \
-        k_adj_reg<R, RB><<<grid, kRegThreads, sm, st>>>((Cx<R> *)psi, (Cx<R> *)lam, a, ops, phases, steps,   \
-                                                        (const R *)coef, (const Cx<R> *)mats, part, part_stride, \
-                                                        dblocks, dmem);                                      \
-        break;
-        SV_AR(2) SV_AR(3)
-    case 4:
-        if constexpr (sizeof(R) == 4) {
-            allow_smem(k_adj_reg<R, 4>, sm);
-            k_adj_reg<R, 4><<<grid, kRegThreads, sm, st>>>((Cx<R> *)psi, (Cx<R> *)lam, a, ops, phases, steps,
-                                                           (const R *)coef, (const Cx<R> *)mats, part, part_stride,
-                                                           dblocks, dmem);
-            break;
-        }
-        return cudaErrorInvalidValue;
-#undef SV_AR
-    default:
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
 size_t gate_reg_smem(sv_dtype dt, const GatePassArgs &a) {
     const int amp = dt == SV_C64 ? 8 : 16;
     return 2 * ((size_t)1 << a.k) * amp + reg_layout(a, amp, false).total;
@@ -3906,22 +4214,76 @@ size_t adj_reg_smem(sv_dtype dt, const GatePassArgs &a) {
     return 2 * ((size_t)1 << a.k) * amp + reg_layout(a, amp, true).total;
 }
 
+int reg_pass_grid(sv_dtype dt, const GatePassArgs &a, bool adj, int blocks_per_sm) {
+    const size_t sm = (adj ? adj_reg_smem(dt, a) : gate_reg_smem(dt, a)) + 1024;
+    const int nt = 1 << (a.k - kRegBits);
+    // resident CTAs by shared memory, by the launch bound's register share and by the block limit
+    int per = (int)std::min<size_t>((size_t)228 * 1024 / sm, (size_t)((dt == SV_C64 ? 512 : 256) / nt));
+    per = std::max(1, std::min(per, 16));
+    if (blocks_per_sm > 0) per = std::min(per, blocks_per_sm);
+    const uint64_t ntiles = 1ull << a.nout;
+    return (int)std::min<uint64_t>(ntiles, (uint64_t)per * device_sms());
+}
+
+template <typename R>
+cudaError_t gate_reg_dispatch(cudaStream_t st, int grid, void *psi, const GatePassArgs &a, const void *image,
+                              const void *pmats) {
+    const size_t sm = gate_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
+    const int nt = 1 << (a.k - kRegBits);
+    if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
+    allow_smem(k_gate_reg<R>, sm);
+    k_gate_reg<R><<<grid, nt, sm, st>>>((Cx<R> *)psi, a, (const unsigned char *)image, (const Cx<R> *)pmats);
+    return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t adj_reg_dispatch(cudaStream_t st, int grid, void *psi, void *lam, const GatePassArgs &a,
+                             const void *image, const void *pmats, double *part, int part_stride) {
+    const size_t sm = adj_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
+    const int nt = 1 << (a.k - kRegBits);
+    if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
+    allow_smem(k_adj_reg<R>, sm);
+    k_adj_reg<R><<<grid, nt, sm, st>>>((Cx<R> *)psi, (Cx<R> *)lam, a, (const unsigned char *)image,
+                                       (const Cx<R> *)pmats, part, part_stride);
+    return cudaGetLastError();
+}
+
+size_t reg_image_bytes(sv_dtype dt, const GatePassArgs &a) {
+    return (reg_layout(a, dt == SV_C64 ? 8 : 16, false).image + 255) & ~(size_t)255;
+}
+
+cudaError_t launch_reg_image(sv_dtype dt, cudaStream_t st, const GatePassArgs *pargs, const uint64_t *offs, int npasses,
+                             const DevOp *ops, const Phase *phases, const RegStep *steps, const void *coef,
+                             const DiagBlock *dblocks, const DiagMember *dmem, void *out, uint64_t dir_stride, int dir0,
+                             int ndirs) {
+    if (npasses <= 0) return cudaSuccess;
+    const dim3 grid(npasses, kImageSlices, ndirs);
+    if (dt == SV_C64)
+        k_reg_image<float><<<grid, 256, 0, st>>>(pargs, offs, ops, phases, steps, (const float *)coef, dblocks, dmem,
+                                                 (unsigned char *)out, dir_stride, dir0);
+    else
+        k_reg_image<double><<<grid, 256, 0, st>>>(pargs, offs, ops, phases, steps, (const double *)coef, dblocks, dmem,
+                                                  (unsigned char *)out, dir_stride, dir0);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_prep_mats(sv_dtype dt, cudaStream_t st, const PrepMat *prep, int count, const void *mats, void *out) {
+    if (count <= 0) return cudaSuccess;
+    if (dt == SV_C64) k_prep_mats<float><<<count, 256, 0, st>>>(prep, (const float2 *)mats, (float2 *)out);
+    else k_prep_mats<double><<<count, 256, 0, st>>>(prep, (const double2 *)mats, (double2 *)out);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_gate_reg(sv_dtype dt, cudaStream_t st, int grid, void *psi, const GatePassArgs &a,
-                            const DevOp *ops, const Phase *phases, const RegStep *steps, const void *coef,
-                            const void *mats, const DiagBlock *dblocks, const DiagMember *dmem) {
-    if (dt == SV_C64) return gate_reg_dispatch<float>(st, grid, psi, a, ops, phases, steps, coef, mats, dblocks, dmem);
-    return gate_reg_dispatch<double>(st, grid, psi, a, ops, phases, steps, coef, mats, dblocks, dmem);
+                            const void *image, const void *pmats) {
+    if (dt == SV_C64) return gate_reg_dispatch<float>(st, grid, psi, a, image, pmats);
+    return gate_reg_dispatch<double>(st, grid, psi, a, image, pmats);
 }
 
 cudaError_t launch_adj_reg(sv_dtype dt, cudaStream_t st, int grid, void *psi, void *lam, const GatePassArgs &a,
-                           const DevOp *ops, const Phase *phases, const RegStep *steps, const void *coef,
-                           const void *mats, double *part, int part_stride, const DiagBlock *dblocks,
-                           const DiagMember *dmem) {
-    if (dt == SV_C64)
-        return adj_reg_dispatch<float>(st, grid, psi, lam, a, ops, phases, steps, coef, mats, part, part_stride,
-                                       dblocks, dmem);
-    return adj_reg_dispatch<double>(st, grid, psi, lam, a, ops, phases, steps, coef, mats, part, part_stride,
-                                    dblocks, dmem);
+                           const void *image, const void *pmats, double *part, int part_stride) {
+    if (dt == SV_C64) return adj_reg_dispatch<float>(st, grid, psi, lam, a, image, pmats, part, part_stride);
+    return adj_reg_dispatch<double>(st, grid, psi, lam, a, image, pmats, part, part_stride);
 }
 
 cudaError_t launch_adj_pass(sv_dtype dt, cudaStream_t st, int grid, int threads, void *psi, void *lam,
@@ -4089,7 +4451,8 @@ cudaError_t hpsi_dispatch(cudaStream_t st, int grid, const void *psi, void *lam,
                           const DevGroup *groups, const DevString *strs, int first, int last, double *epart,
                           int *status, long long limit) {
     const int E = 1 << (a.kl + a.m);
-    const size_t sm = 2 * (size_t)E * sizeof(Cx<R>) + ((size_t)1 << a.m) * 8;
+    const size_t sm = 2 * (size_t)E * sizeof(Cx<R>) + ((size_t)1 << a.m) * 8 +
+                      (a.s_end - a.s_begin > kHpsiTab ? (size_t)(a.s_end - a.s_begin) * sizeof(HpsiStr) : 0);
     // a multiple of the run length, at least one warp, at most 512
     const int threads = std::max(std::max(32, 1 << a.kl), std::min(E, 512));
     const int ept = std::max(1, E / threads);
@@ -4117,6 +4480,61 @@ cudaError_t launch_hpsi_pass(sv_dtype dt, cudaStream_t st, int grid, const void 
                              int last, double *epart, int *status, long long limit) {
     if (dt == SV_C64) return hpsi_dispatch<float>(st, grid, psi, lam, a, groups, strs, first, last, epart, status, limit);
     return hpsi_dispatch<double>(st, grid, psi, lam, a, groups, strs, first, last, epart, status, limit);
+}
+
+// Slices of a coset for the kernels above: about two CTAs for each SM in all,
+// as far as the strings (a warp each) or the outputs (at least 32) go.  The
+// line between whole cosets and slices is two cosets per SM: with fewer, the
+// double-buffered kernels have nothing to overlap (measured on random strings,
+// complex64, per H|psi> pass: see the kernel's comment).
+bool coset_slices_pay(sv_dtype dt, const CosetArgs &a) {
+    return a.kl + a.m >= 6 && a.nfree < 16 && (1 << a.nfree) < (dt == SV_C64 ? 2 : 1) * device_sms();
+}
+
+cudaError_t launch_evc_slice(sv_dtype dt, cudaStream_t st, const void *psi, const CosetArgs &a, const DevString *strs,
+                             double *part, int part_stride) {
+    const int E = 1 << (a.kl + a.m), ncos = 1 << a.nfree;
+    const int want = (2 * device_sms() + ncos - 1) / ncos, most = (a.s_end - a.s_begin + 15) / 16;
+    const int S = std::max(1, std::min(want, most));
+    const size_t es = dt == SV_C64 ? 8 : 16, sm = (size_t)E * es + ((size_t)8 << a.m);
+    if (dt == SV_C64) {
+        allow_smem(k_evc_slice<float>, sm);
+        k_evc_slice<float><<<ncos * S, 512, sm, st>>>((const float2 *)psi, a, strs, part, part_stride, S);
+    } else {
+        allow_smem(k_evc_slice<double>, sm);
+        k_evc_slice<double><<<ncos * S, 512, sm, st>>>((const double2 *)psi, a, strs, part, part_stride, S);
+    }
+    return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t hpsi_slice_dispatch(cudaStream_t st, const void *psi, void *lam, const CosetArgs &a, const DevString *strs,
+                                int first, int last, double *epart, int *rows) {
+    const int E = 1 << (a.kl + a.m), ncos = 1 << a.nfree;
+    int S = 1;
+    while (ncos * S < device_sms() && E / (2 * S) >= 32) S *= 2;
+    const int ept = std::max(1, E / S / 512);
+    const size_t sm = (size_t)E * sizeof(Cx<R>) + ((size_t)8 << a.m) + kHSliceTab * sizeof(HSliceStr<R>) +
+                      512 * sizeof(Cx<R>);
+    *rows = ncos * S;
+#define SV_HS_CASE(N)                                                                                                case N:                                                                                                              allow_smem(k_hpsi_slice<R, N>, sm);                                                                              k_hpsi_slice<R, N><<<ncos * S, 512, sm, st>>>((const Cx<R> *)psi, (Cx<R> *)lam, a, strs, first, last, epart, S);         break;
+    switch (ept) {
+        SV_HS_CASE(1)
+        SV_HS_CASE(2)
+        SV_HS_CASE(4)
+        SV_HS_CASE(8)
+        SV_HS_CASE(16)
+    default:
+        return cudaErrorInvalidValue;
+    }
+#undef SV_HS_CASE
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hpsi_slice(sv_dtype dt, cudaStream_t st, const void *psi, void *lam, const CosetArgs &a,
+                              const DevString *strs, int first, int last, double *epart, int *rows) {
+    if (dt == SV_C64) return hpsi_slice_dispatch<float>(st, psi, lam, a, strs, first, last, epart, rows);
+    return hpsi_slice_dispatch<double>(st, psi, lam, a, strs, first, last, epart, rows);
 }
 
 cudaError_t launch_reduce_rows(cudaStream_t st, const double *part, int nblocks, int stride, int s_begin,

@@ -18,6 +18,7 @@ struct GatePassArgs {
     int st_begin, st_end;    // steps of the pass's register phases
     int area;                // bytes of the diagonal-block data
     int mem_begin, mem_end;  // diagonal-block members of the pass
+    int dense;               // the phases hold 2- or 4-qubit matrices (the reverse pass runs in k_adj_pass)
     int8_t hi[40];
     int8_t out[64];
 };
@@ -43,6 +44,8 @@ struct DevString {
     double coef;
     int32_t nY;
     uint32_t bz;      // parities of the pass's span basis against z
+    uint32_t X;       // the group's partner offset
+    uint32_t pad;
 };
 
 // Few-string expectation passes (every group one string): at most this many groups.
@@ -88,16 +91,25 @@ cudaError_t launch_gate_pass(sv_dtype dt, cudaStream_t st, int grid, int threads
 cudaError_t launch_adj_pass(sv_dtype dt, cudaStream_t st, int grid, int threads, void *psi, void *lam,
                             const GatePassArgs &a, const DevOp *ops, const void *coef, const void *mats,
                             double *part, int part_stride);
-// Register-blocked passes (512 threads; a.ph_begin >= 0, 11 <= k <= 13): the
+// Register-blocked passes (2^(k - kRegBits) threads; a.ph_begin >= 0): the
 // phases' steps (RegStep) are executed in order (forward) or in reverse
 // (adjoint); part receives the FP64 gradient partials of every operation.
+// pmats: the prepared matrices of launch_prep_mats.
+int reg_pass_grid(sv_dtype dt, const GatePassArgs &a, bool adj, int blocks_per_sm);
+cudaError_t launch_prep_mats(sv_dtype dt, cudaStream_t st, const PrepMat *prep, int count, const void *mats, void *out);
+// The tables of the register-blocked passes, made on the device once per call
+// (they hold the parameters): pass p's tables are reg_image_bytes(args[p])
+// bytes at out + offs[p], those of the reverse pass dir_stride further;
+// directions dir0 .. dir0 + ndirs - 1 (0 forward, 1 reverse) are made.
+size_t reg_image_bytes(sv_dtype dt, const GatePassArgs &a);
+cudaError_t launch_reg_image(sv_dtype dt, cudaStream_t st, const GatePassArgs *pargs, const uint64_t *offs, int npasses,
+                             const DevOp *ops, const Phase *phases, const RegStep *steps, const void *coef,
+                             const DiagBlock *dblocks, const DiagMember *dmem, void *out, uint64_t dir_stride, int dir0,
+                             int ndirs);
 cudaError_t launch_gate_reg(sv_dtype dt, cudaStream_t st, int grid, void *psi, const GatePassArgs &a,
-                            const DevOp *ops, const Phase *phases, const RegStep *steps, const void *coef,
-                            const void *mats, const DiagBlock *dblocks, const DiagMember *dmem);
+                            const void *image, const void *pmats);
 cudaError_t launch_adj_reg(sv_dtype dt, cudaStream_t st, int grid, void *psi, void *lam, const GatePassArgs &a,
-                           const DevOp *ops, const Phase *phases, const RegStep *steps, const void *coef,
-                           const void *mats, double *part, int part_stride, const DiagBlock *dblocks,
-                           const DiagMember *dmem);
+                           const void *image, const void *pmats, double *part, int part_stride);
 // Shared memory of a register-blocked pass (forward / adjoint).
 size_t gate_reg_smem(sv_dtype dt, const GatePassArgs &a);
 size_t adj_reg_smem(sv_dtype dt, const GatePassArgs &a);
@@ -113,6 +125,13 @@ cudaError_t launch_evc_pass(sv_dtype dt, cudaStream_t st, int grid, const void *
 cudaError_t launch_hpsi_pass(sv_dtype dt, cudaStream_t st, int grid, const void *psi, void *lam,
                              const CosetArgs &a, const DevGroup *groups, const DevString *strs,
                              int first, int last, double *epart, int *status, long long limit);
+// Few cosets (coset_slices_pay): several CTAs share a coset.  Expectation:
+// part rows are the 2^nfree cosets; H|psi>: *rows energy partials.
+bool coset_slices_pay(sv_dtype dt, const CosetArgs &a);
+cudaError_t launch_evc_slice(sv_dtype dt, cudaStream_t st, const void *psi, const CosetArgs &a, const DevString *strs,
+                             double *part, int part_stride);
+cudaError_t launch_hpsi_slice(sv_dtype dt, cudaStream_t st, const void *psi, void *lam, const CosetArgs &a,
+                              const DevString *strs, int first, int last, double *epart, int *rows);
 // out[s] = sum over b < nblocks of part[b * stride + s], s in [s_begin, s_end); fixed order.
 cudaError_t launch_reduce_rows(cudaStream_t st, const double *part, int nblocks, int stride,
                                int s_begin, int s_end, double *out);

@@ -425,6 +425,7 @@ void plan_gate_passes(QsuPlan &P, const std::vector<Op> &ops, int k, int low, in
                 }
                 d.gate = u;
                 d.mat = ops[u].mat;
+                d.pm = -1;
                 P.ops.push_back(d);
             }
             gp.op_end = (int32_t)P.ops.size();
@@ -440,9 +441,9 @@ void plan_gate_passes(QsuPlan &P, const std::vector<Op> &ops, int k, int low, in
 }
 
 // ------------------------------------------------------- register phases --
-// A pass made only of RY, RZ, CZ and 1-qubit matrices is run register
-// blocked: every thread holds 2^r amplitudes spanned by r tile bits (the
-// register set).  Non-diagonal gates need their target in the register set;
+// A pass is run register blocked: every thread holds 2^r amplitudes spanned
+// by r tile bits (the register set; r = 4, or k less the thread bits of a
+// given CTA size).  Non-diagonal gates need their targets in the register set;
 // diagonal gates (RZ, CZ) apply in any layout.  Phases are built like the
 // tiles: the register set takes the targets of the earliest remaining
 // non-diagonal gates (padded with the lowest free tile bits), then the phase
@@ -491,19 +492,25 @@ uint32_t phase_lanes(uint32_t rmask, int k) {
     return lanes;
 }
 
-void plan_phases(QsuPlan &P, bool pairs) {
+void plan_phases(QsuPlan &P, bool pairs, int threads) {
     for (auto &gp : P.passes) {
-        const int r = gp.k - 9;                       // 512 threads
-        if (r < 2) continue;
-        bool ok = true;
+        int r = kRegBits;
+        if (threads) {
+            r = gp.k;
+            for (int t = threads; t > 1; t >>= 1) --r;
+        }
+        if (r < 2 || (!threads && gp.k < kRegMinTile)) continue;
+        bool ok = true, dense = false;
         for (int o = gp.op_begin; o < gp.op_end; ++o) {
             const int kd = P.ops[o].kind;
-            // a double excitation needs four register bits
-            if (kd != SV_RY && kd != SV_RZ && kd != SV_CZ && kd != SV_MAT1 && !(pairs && kd == SV_GIVENS) &&
-                !(pairs && kd == SV_DEXC && r == 4))
-                ok = false;
+            // Givens rotations, double excitations and dense 2- and 4-qubit
+            // matrices need their targets among four register bits
+            const bool pair = kd == SV_GIVENS || kd == SV_DEXC || kd == SV_MAT2 || kd == SV_MAT4;
+            if (kd != SV_RY && kd != SV_RZ && kd != SV_CZ && kd != SV_MAT1 && !(pairs && pair)) ok = false;
+            if (kd == SV_MAT2 || kd == SV_MAT4) dense = true;
         }
         if (!ok) continue;
+        gp.dense = dense;
         const uint32_t all = (gp.k >= 32) ? 0xFFFFFFFFu : ((1u << gp.k) - 1u);
         auto tmask = [&](const DevOp &d) {
             uint32_t m = 0;
@@ -544,6 +551,21 @@ void plan_phases(QsuPlan &P, bool pairs) {
                 }
             }
             ph.op_end = gp.op_begin + (int32_t)out.size();
+            for (int o = ph.op_begin - gp.op_begin; o < (int)out.size(); ++o) {
+                DevOp &d = out[o];
+                if (threads || (d.kind != SV_MAT1 && d.kind != SV_MAT2 && d.kind != SV_MAT4)) continue;
+                // the targets' places among the gate's register bits, ascending
+                PrepMat pm;
+                pm.nq = op_qubits(d.kind);
+                pm.src = d.mat;
+                pm.dst = P.prep_elems;
+                const uint32_t tm = tmask(d);
+                for (int t = 0; t < 4; ++t)
+                    pm.perm[t] = (int8_t)(t < pm.nq ? __builtin_popcount(tm & ((1u << d.t[t]) - 1u)) : 0);
+                d.pm = pm.dst;
+                P.prep_elems += 2 << (2 * pm.nq);
+                P.prep.push_back(pm);
+            }
             P.phases.push_back(ph);
             remain.swap(next);
         }
@@ -1156,7 +1178,7 @@ std::string plan_qsu(int n, int g, const sv_gate *gates, size_t m, bool lazy, co
     if (P.tiles.empty()) P.final_l2p = l2p_init;
     int k = std::max(o.tile_bits, std::min(o.low_bits, P.nL) + 4);
     plan_gate_passes(P, ops, k, o.low_bits, o.fuse_max, o.diag_exempt);
-    plan_phases(P, o.reg_pairs);
+    plan_phases(P, o.reg_pairs, o.reg_threads);
     plan_steps(P, std::min(o.max_diag, kMaxPassDiag), o.amp_bytes);
     return "";
 }

@@ -46,6 +46,16 @@ struct DevOp {
     int8_t t[4];
     int32_t gate;     // index in the caller's gate list (coefficient / gradient slot)
     int32_t mat;      // complex offset into the matrix array, or -1
+    int32_t pm;       // register-blocked passes: complex offset of the prepared matrix (PrepMat), else -1
+};
+
+// A caller matrix of a register-blocked pass, prepared once per call: M'[u][w]
+// = M[j(u)][j(w)] with u, w over the gate's register bits in ascending order
+// and j the caller's index (bit t of j = bit perm[t] of u), followed by its
+// conjugate transpose (dim * dim elements each).
+struct PrepMat {
+    int32_t nq, src, dst;    // targets; complex offsets into the caller's and the prepared array
+    int8_t perm[4];
 };
 
 // One shared-memory pass of K-GATE / K-ADJ.
@@ -55,6 +65,7 @@ struct GatePass {
     uint64_t bits = 0;                // physical staged bits
     int32_t op_begin = 0, op_end = 0; // into QsuPlan::ops
     int32_t ph_begin = -1, ph_end = -1;  // register phases (register-blocked passes), else -1
+    int32_t dense = 0;                   // 1: the phases hold 2- or 4-qubit matrices (forward only)
     int32_t db_begin = 0, db_end = 0;    // diagonal blocks of the pass (register-blocked passes)
     int32_t st_begin = 0, st_end = 0;    // steps of the pass's phases
     int32_t area = 0;                    // bytes of the pass's diagonal-block data (shared memory)
@@ -87,7 +98,10 @@ struct DiagMember {
     int32_t op;       // index into QsuPlan::ops (coefficient and gradient slot)
 };
 constexpr int kMaxPassDiag = 24;       // diagonal blocks per register-blocked pass
-constexpr int kRegThreads = 512;       // CTA size of register-blocked passes (r = k - 9)
+// Register-blocked passes: each thread holds 2^kRegBits amplitudes of a tile,
+// so a tile of 2^k amplitudes takes 2^(k - kRegBits) threads, at least a warp.
+constexpr int kRegBits = 4;
+constexpr int kRegMinTile = kRegBits + 5;
 
 // A register phase of a register-blocked pass: each thread holds the
 // amplitudes spanned by the tile bits in rmask; ops [op_begin, op_end) are
@@ -107,30 +121,39 @@ struct Phase {
 // members.  OP: one operation (a = op_begin), applied by the generic code.
 enum { SV_STEP_ROT = 0, SV_STEP_DIAG = 1, SV_STEP_OP = 2 };
 // The shared-memory slot of tile index i in the register-blocked passes: a
-// linear (XOR) swizzle of the low 4 bits by bits 4..11, so that slot(a | b)
-// = slot(a) ^ slot(b) for disjoint a, b.
+// linear (XOR) swizzle, so that slot(a | b) = slot(a) ^ slot(b) for disjoint
+// a, b.  It keeps bit 0 (an even index and its successor stay one 16-byte
+// pair of complex64, so tiles move by 16-byte accesses and a phase that holds
+// tile bit 0 gathers pairs) and XORs bits 1..3 with the bit triples 4..6 and
+// 7..9 and with independent mixtures of bits 10..12: whatever 4 of 13 bits a
+// phase holds in registers, the others still reach every value of the low
+// bits (at most 7 of the 12 bits fall into any one plane of the three).
 #ifdef __CUDACC__
 #define SV_HD __host__ __device__
 #else
 #define SV_HD
 #endif
-SV_HD inline uint32_t swz_slot(uint32_t i) { return i ^ (((i >> 4) ^ (i >> 8)) & 15u); }
-// Shared memory of a register-blocked pass of k staged bits (512 threads,
-// amplitudes of amp bytes): the block area needs at most this much beyond
-// the tiles, tables and accumulators, and each block takes
-// diag_block_bytes() of it.
+SV_HD inline uint32_t swz_slot(uint32_t i) {
+    const uint32_t y = (i >> 10) & 7u;
+    return i ^ ((((i >> 4) ^ (i >> 7) ^ y ^ (y << 1) ^ (y >> 2)) & 7u) << 1);
+}
+// Shared memory of a register-blocked pass of k staged bits (amplitudes of
+// amp bytes): the block area needs at most this much beyond the tiles, tables
+// and accumulators, and each block takes diag_block_bytes() of it.
 constexpr int kRegSmemLimit = 226 * 1024;
-constexpr int kAdjSlotStride = kRegThreads / 32 + 1;   // adjoint gradient slots per op (one per warp, padded)
+constexpr int kAdjSlotStride = 17;   // adjoint gradient slots per op (one per warp, padded)
 inline int diag_block_bytes(int kind, int k, int amp) {
-    const int V = 1 << (k - 9);
-    return kind == 0 ? V * V * amp + 512 : 512 * amp;
+    const int V = 1 << kRegBits, NT = 1 << (k - kRegBits);
+    return kind == 0 ? V * V * amp + NT : NT * amp;
 }
 inline int reg_pass_fixed_bytes(int k, int nlow, int nops, int nsteps, int nphases, int amp) {
-    // adjoint (the larger): psi and lambda tiles, high offsets, (c, s) per op,
-    // steps, block headers, per-phase thread bases and register offsets,
-    // per-warp gradient slots, the RY factor per step, alignment
-    return 2 * (1 << k) * amp + 8 * (1 << (k - nlow)) + nops * amp + 16 * nsteps + 32 * kMaxPassDiag +
-           16 * nops + nphases * (2 * kRegThreads + 8) + nops * kAdjSlotStride * 8 + 8 * (nsteps + 1) + 272;
+    // adjoint (the larger): psi and lambda tiles, high offsets, chunk offsets,
+    // (c, s) per op, steps, block headers and members, phases with their
+    // thread bases and register offsets, per-warp gradient slots, the RY
+    // factor per step, alignment
+    return 2 * (1 << k) * amp + 8 * (1 << (k - nlow)) + 256 + nops * amp + 16 * nsteps + 32 * kMaxPassDiag +
+           16 * nops + nphases * (2 * (1 << (k - kRegBits)) + 8 + 32) + nops * kAdjSlotStride * 8 +
+           8 * (nsteps + 1) + 320;
 }
 struct RegStep {
     int32_t type, a;
@@ -147,6 +170,8 @@ struct QsuPlan {
     std::vector<RegStep> steps;       // steps of the register phases
     std::vector<DiagBlock> dblocks;   // diagonal blocks of register phases
     std::vector<DiagMember> dmembers;
+    std::vector<PrepMat> prep;        // caller matrices of register phases
+    int32_t prep_elems = 0;           // complex elements of the prepared array
     std::vector<int32_t> init_l2p, final_l2p;
     int32_t nqr() const {
         int32_t c = 0;
@@ -202,7 +227,8 @@ struct PlanOptions {
     int hier_intra = -1;         // >= 0: hierarchical tiling (Alg. 4/5) with this many intra qubits
     int max_diag = kMaxPassDiag; // diagonal blocks per register-blocked pass (shared-memory budget)
     int amp_bytes = 8;           // 8 complex64, 16 complex128 (shared-memory budget of the blocks)
-    bool reg_pairs = true;       // Givens / double excitations may run in register phases
+    bool reg_pairs = true;       // Givens, double excitations and dense matrices may run in register phases
+    int reg_threads = 0;         // register phases on CTAs of this size (the batched kernel), 0 = 2^(k - kRegBits)
     bool diag_exempt = false;    // QSU: diagonal gates (RZ, CZ) never ask for a QR (per-chunk phases)
     // One greedy step of Alg. 6 done elsewhere (on the device): given the
     // distinct X/Y supports xs with remaining weights w, return the rank of
