@@ -614,19 +614,22 @@ sv_status run_forward(sv_handle *h, QsuEntry *q, sv_stats *st) {
     const int threads = gate_threads(h);
     h->drop_ckpts();
     size_t pi = 0;
+    int launched = 0;    // kernels since the passes' tables were made
     for (size_t t = 0; t < P.tiles.size(); ++t) {
         const Tile &T = P.tiles[t];
         if (!T.pairs.empty()) {
             const int s = (int)T.pairs.size() / 2;
             Rec r(h, st, SV_K_QR, 2.0 * (1.0 - std::ldexp(1.0, -s)) * (double)h->state_bytes());
             SV_CK(launch_bitswap(h->dt, h->stream, h->psi, h->n, T.pairs.data(), s, h->opt.blocks_per_sm));
+            ++launched;
         }
-        for (; pi < P.passes.size() && P.passes[pi].tile == (int)t; ++pi) {
+        for (; pi < P.passes.size() && P.passes[pi].tile == (int)t; ++pi, ++launched) {
             const GatePassArgs &a = q->args[pi];
             if (a.ph_begin >= 0) {
                 Rec r(h, st, SV_K_GATE, 2.0 * (double)h->state_bytes());
                 const int rg = reg_pass_grid(h->dt, a, false, h->opt.blocks_per_sm);
-                SV_CK(launch_gate_reg(h->dt, h->stream, rg, h->psi, a, h->images.as<char>() + q->image[pi], h->pmats.p));
+                SV_CK(launch_gate_reg(h->dt, h->stream, rg, h->psi, a, h->images.as<char>() + q->image[pi], h->pmats.p,
+                                      launched > 0));
             } else {
                 int grid = gate_pass_grid(h->dt, a.k, a.nlow, a.op_end - a.op_begin, threads, h->opt.blocks_per_sm);
                 const uint64_t ntiles = 1ull << a.nout;
@@ -758,6 +761,7 @@ sv_status run_reverse(sv_handle *h, QsuEntry *q, sv_stats *st) {
     SV_CK(h->opval.ensure(std::max(nops, 1) * sizeof(double)));
     SV_CK(h->grad.ensure(std::max(q->np, 1) * sizeof(double)));
     int pi = (int)P.passes.size() - 1;
+    int launched = 0;    // reverse passes so far (the tables may have been made right before the first)
     for (int t = (int)P.tiles.size() - 1; t >= 0; --t) {
         for (; pi >= 0 && P.passes[pi].tile == t; --pi) {
             const GatePassArgs &a = q->args[pi];
@@ -772,7 +776,7 @@ sv_status run_reverse(sv_handle *h, QsuEntry *q, sv_stats *st) {
             if (a.ph_begin >= 0 && !a.dense)
                 SV_CK(launch_adj_reg(h->dt, h->stream, grid, h->psi, h->lam, a,
                                      h->images.as<char>() + q->image_bytes + q->image[pi], h->pmats.p,
-                                     h->part.as<double>(), nops));
+                                     h->part.as<double>(), nops, launched++ > 0));
             else
                 SV_CK(launch_adj_pass(h->dt, h->stream, grid, threads, h->psi, h->lam, a, q->ops.as<DevOp>(),
                                       h->coef.p, h->mats.p, h->part.as<double>(), nops));

@@ -21,6 +21,9 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <map>
+#include <mutex>
+#include <tuple>
 
 #include "kernels.h"
 
@@ -31,6 +34,15 @@ template <typename R> struct CxT;
 template <> struct CxT<float> { using T = float2; };
 template <> struct CxT<double> { using T = double2; };
 template <typename R> using Cx = typename CxT<R>::T;
+
+// Programmatic dependent launch: pdl_wait() returns when every earlier kernel
+// of the stream is complete and its writes are visible; pdl_next() lets the
+// next kernel's blocks start (their own pdl_wait() holds them back).  Called
+// in this order, so what runs before a kernel's pdl_wait() may read anything
+// that was written before its predecessor began -- plan tables, never the
+// predecessor's output -- and writes nothing but shared memory.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename R>
 __device__ __forceinline__ Cx<R> mk(R a, R b) {
@@ -461,6 +473,8 @@ __global__ void __launch_bounds__(512) k_gate_pass(Cx<R> *__restrict__ psi, cons
     uint64_t *hioff = reinterpret_cast<uint64_t *>(tile + T);
     for (uint32_t j = threadIdx.x; j < nh; j += blockDim.x) hioff[j] = deposit(j, a.hi, a.nhi);
     __syncthreads();
+    pdl_wait();
+    pdl_next();
     const uint64_t ntiles = 1ull << a.nout;
     const uint32_t lowmask = (1u << a.nlow) - 1u;
     for (uint64_t ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
@@ -497,6 +511,8 @@ __global__ void __launch_bounds__(512) k_adj_pass(Cx<R> *__restrict__ psi, Cx<R>
     for (uint32_t j = threadIdx.x; j < nh; j += blockDim.x) hioff[j] = deposit(j, a.hi, a.nhi);
     for (int j = threadIdx.x; j < nops * nwarps; j += blockDim.x) acc[j] = 0.0;
     __syncthreads();
+    pdl_wait();
+    pdl_next();
     const uint64_t ntiles = 1ull << a.nout;
     const uint32_t lowmask = (1u << a.nlow) - 1u;
     for (uint64_t ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
@@ -1393,6 +1409,8 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
     unsigned char *out = out0 + (adj ? dir_stride : 0) + offs[blockIdx.x];
     const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), adj);
     const int NT = 1 << (a.k - RB), nph = a.ph_end - a.ph_begin, nst = a.st_end - a.st_begin;
+    pdl_wait();
+    pdl_next();
     for (int o = a.op_begin + tid; o < a.op_end; o += nthr) {
         const int gi = ops[o].gate;
         cs[o - a.op_begin] = mk<R>(coef[2 * gi], adj ? -coef[2 * gi + 1] : coef[2 * gi + 1]);
@@ -1669,7 +1687,7 @@ __device__ __forceinline__ void reg_tile_store(Cx<R> *dst, const RA<R> *tile, co
 template <typename R>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256, 1)
 k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *__restrict__ image,
-           const Cx<R> *__restrict__ pmats) {
+           const Cx<R> *__restrict__ pmats, int early) {
     constexpr int RB = kRegBits, V = 1 << RB;
     constexpr uint32_t P = 16 / sizeof(Cx<R>);
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1677,7 +1695,11 @@ k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *_
     RA<R> *tiles = reinterpret_cast<RA<R> *>(smem);          // two tiles: the next one streams in
     unsigned char *sm = smem + 2 * T * sizeof(RA<R>);
     const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), false);
+    // early: the tables were complete before the kernel before this one began
+    if (!early) pdl_wait();
     reg_image_load(sm, image, L.image);
+    pdl_wait();
+    pdl_next();
     const R ftot = reinterpret_cast<const R *>(sm + L.sc)[a.st_end - a.st_begin];   // product of the RY factors
     const uint64_t *hioff = reinterpret_cast<const uint64_t *>(sm + L.hioff);
     const ChunkOff *chunk = reinterpret_cast<const ChunkOff *>(sm + L.chunk);
@@ -1746,7 +1768,7 @@ template <typename R>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256, 1)
 k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam, const GatePassArgs a,
           const unsigned char *__restrict__ image, const Cx<R> *__restrict__ pmats, double *__restrict__ part,
-          int part_stride) {
+          int part_stride, int early) {
     constexpr int RB = kRegBits, V = 1 << RB;
     constexpr uint32_t P = 16 / sizeof(Cx<R>);
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1765,7 +1787,11 @@ k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam, const GatePassArgs a
     for (int j = threadIdx.x; j < nops * AS; j += NT) acc[j] = 0;
     if constexpr (sizeof(R) == 4)
         for (int j = threadIdx.x; j < nops; j += NT) tot64[j] = 0.0;
+    // early: the tables were complete before the kernel before this one began
+    if (!early) pdl_wait();
     reg_image_load(sm, image, L.image);
+    pdl_wait();
+    pdl_next();
     // factored RYs: before step s both registers sets hold the true vectors
     // divided by scf[s], so a gradient part computed there is scaled by
     // scf[s]^2; the stores multiply by the total factor
@@ -1930,6 +1956,8 @@ k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam, const GatePassArgs a
 template <typename R>
 __global__ void k_prep_mats(const PrepMat *__restrict__ prep, const Cx<R> *__restrict__ mats, Cx<R> *__restrict__ out) {
     const PrepMat p = prep[blockIdx.x];
+    pdl_wait();
+    pdl_next();
     const int dim = 1 << p.nq;
     auto caller = [&](int u) {
         int j = 0;
@@ -1997,7 +2025,7 @@ __global__ void __launch_bounds__(256) k_bitswap(Cx<R> *__restrict__ psi, const 
     __syncthreads();
     const uint32_t runmask = (1u << a.L) - 1u;
     const uint64_t ntiles = 1ull << a.nout;
-    const bool vec = (VEC == 2) && a.L >= 1;
+    const bool vec = VEC == 1 || a.L >= 1;
     // no in-tile exchange moves bit 0: the source slots of a 16-byte pair are
     // adjacent (the swizzle keeps bit 0), so the pair is one 16-byte load
     bool bit0_fixed = true;
@@ -2005,6 +2033,8 @@ __global__ void __launch_bounds__(256) k_bitswap(Cx<R> *__restrict__ psi, const 
         if (a.la[i] == 0 || a.lb[i] == 0) bit0_fixed = false;
     const BitWalk bw = bit_walk(a.out, a.nout, gridDim.x);
     uint64_t bnext = deposit(blockIdx.x, a.out, a.nout);
+    pdl_wait();
+    pdl_next();
     for (uint64_t ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
         const uint64_t b0 = bnext;
         bnext = walk_next(bnext, bw);
@@ -2014,7 +2044,7 @@ __global__ void __launch_bounds__(256) k_bitswap(Cx<R> *__restrict__ psi, const 
         if (self && a.nlo == 0) continue;
         if (vec) {
             // 16-byte copies straight into shared memory (j even and bit 0 of b0, b1 clear: both ends aligned)
-            for (uint32_t j = 2 * threadIdx.x; j < T; j += 2 * blockDim.x) {
+            for (uint32_t j = VEC * threadIdx.x; j < T; j += VEC * blockDim.x) {
                 const uint64_t off = hioff[j >> a.L] | (j & runmask);
                 const uint32_t s = swz<R>(j);
                 cp_async16(&A[s], &psi[b0 | off]);
@@ -2031,7 +2061,7 @@ __global__ void __launch_bounds__(256) k_bitswap(Cx<R> *__restrict__ psi, const 
             }
         }
         __syncthreads();
-        if (vec && bit0_fixed) {
+        if (vec && VEC == 2 && bit0_fixed) {
             for (uint32_t j = 2 * threadIdx.x; j < T; j += 2 * blockDim.x) {
                 const uint64_t off = hioff[j >> a.L] | (j & runmask);
                 const uint32_t s0 = pt[j >> 1] & 0xFFFFu;
@@ -2040,7 +2070,7 @@ __global__ void __launch_bounds__(256) k_bitswap(Cx<R> *__restrict__ psi, const 
                 if (!self)
                     *reinterpret_cast<float4 *>(&psi[b1 | off]) = *reinterpret_cast<const float4 *>(&A[s0]);
             }
-        } else if (vec) {
+        } else if (vec && VEC == 2) {
             for (uint32_t j = 2 * threadIdx.x; j < T; j += 2 * blockDim.x) {
                 const uint64_t off = hioff[j >> a.L] | (j & runmask);
                 const uint32_t pp = pt[j >> 1], s0 = pp & 0xFFFFu, s1 = pp >> 16;
@@ -2474,6 +2504,8 @@ __global__ void __launch_bounds__(512, 1) k_evc_pass(const Cx<R> *__restrict__ p
     // current iteration, rep_pf of the one two ahead (the next copy issued)
     const BitWalk bw = bit_walk(a.freeb, a.nfree, gridDim.x);
     uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
+    pdl_wait();
+    pdl_next();
     for (uint64_t k = 0; k < 2; ++k) {
         if (k < mine) load_coset<R>(buf + k * E, psi, rep_pf, spanv, a.kl, E);
         cp_async_commit();
@@ -2719,6 +2751,8 @@ __global__ void __launch_bounds__(1 << LOGNT, 1) k_evc_few(const Cx<R> *__restri
     // current iteration, rep_pf of the one two ahead (the next copy issued)
     const BitWalk bw = bit_walk(a.freeb, a.nfree, gridDim.x);
     uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
+    pdl_wait();
+    pdl_next();
     for (uint64_t k = 0; k < 2; ++k) {
         if (k < mine) load_coset<R>(buf + k * E, psi, rep_pf, spanv, a.kl, E);
         cp_async_commit();
@@ -3003,6 +3037,8 @@ __global__ void __launch_bounds__(1 << LOGNT, 1) k_evc_ring(const Cx<R> *__restr
     const bool rl = a.kl <= LOGNT + (sizeof(R) == 4 ? 1 : 0) && (16u >> a.kl) <= (uint32_t)sizeof(Cx<R>) &&
                     (EPT * sizeof(Cx<R>)) % 16 == 0;
     const RingLoad RL = ring_load_setup<R, NT>(rl ? a.kl : 0);
+    pdl_wait();
+    pdl_next();
     for (uint64_t k = 0; k < 2; ++k) {
         if (k < mine) {
             if (rl) ring_load<R, EPT, NT>(buf + k * E, psi, rep_pf, spanv, RL);
@@ -3253,7 +3289,10 @@ __device__ __forceinline__ void hpsi_tab_string(float2 *acc, const HpsiTab &T, i
     hpsi_string(acc, T.X[k], T.g[k] ^ (((bmask >> k) & 1u) << 31), T.w[k], sb);
 }
 
-template <typename R, int EPT>
+// MANY: complex64 passes of 8192 staged with more than kHpsiTab strings (a
+// variant of its own: the two string loops in one kernel cost the passes of
+// few strings 4 %).
+template <typename R, int EPT, bool MANY>
 __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam,
                                                       const CosetArgs a, const DevGroup *__restrict__ groups,
                                                       const DevString *__restrict__ strs, int first, int last,
@@ -3275,6 +3314,8 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
     // current iteration, rep_pf of the one two ahead (the next copy issued)
     const BitWalk bw = bit_walk(a.freeb, a.nfree, gridDim.x);
     uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
+    pdl_wait();
+    pdl_next();
     for (uint64_t k = 0; k < 2; ++k) {
         if (k < mine) load_coset<R>(buf + k * E, psi, rep_pf, spanv, a.kl, E);
         cp_async_commit();
@@ -3290,20 +3331,20 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
             for (int q = (int)threadIdx.x; q < ns; q += 512) {
                 const DevString S = strs[a.s_begin + q];
                 const float g = (S.nY & 2) ? -(float)S.coef : (float)S.coef;
-                if (ns <= kHpsiTab) {
-                    tabs.z[q] = S.z;
-                    tabs.X[q] = S.X | ((uint32_t)(S.nY & 1) << 31);
-                    tabs.g[q] = __float_as_uint(g);
-                    tabs.w[q] = S.bz >> tc.ash;
-                } else {
+                if constexpr (MANY) {
                     many[q].z = S.z;
                     many[q].X = S.X | ((uint32_t)(S.nY & 1) << 31);
                     many[q].g = __float_as_uint((S.nY & 1) ? -g : g);
                     many[q].w = S.bz >> tc.ash;
                     many[q].tz = (uint32_t)(S.z & ((1ull << a.kl) - 1ull)) | ((S.bz & ((1u << tc.ash) - 1u)) << a.kl);
+                } else {
+                    tabs.z[q] = S.z;
+                    tabs.X[q] = S.X | ((uint32_t)(S.nY & 1) << 31);
+                    tabs.g[q] = __float_as_uint(g);
+                    tabs.w[q] = S.bz >> tc.ash;
                 }
             }
-            if (ns <= kHpsiTab)
+            if constexpr (!MANY)
                 for (int q = 0; q < ns; ++q) {
                     const DevString S = strs[a.s_begin + q];
                     tmask |= (uint32_t)((__popcll(tc.l & S.z) ^ __popc(tc.a0 & S.bz) ^ S.nY) & 1) << q;
@@ -3311,7 +3352,7 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
             __syncthreads();
         }
     }
-    const bool tabbed = ns > 0 && ns <= kHpsiTab;
+    const bool tabbed = ns > 0;
     const int lane = threadIdx.x & 31;
     double eacc = 0.0;
     R eblk = 0;
@@ -3329,7 +3370,14 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
         }
         cp_async_wait1();
         __syncthreads();
-        if constexpr (sizeof(R) == 4 && EPT == 16) {
+        if constexpr (sizeof(R) == 4 && EPT == 16 && MANY) {
+            const uint32_t sb = smem_u32(t);
+            for (int k = 0; k < ns; ++k) {
+                const HpsiStr h = many[k];
+                const uint32_t neg = (uint32_t)(__popcll(rep & h.z) ^ __popc(threadIdx.x & h.tz)) & 1u;
+                hpsi_string(reinterpret_cast<float2 *>(acc), h.X, h.g ^ (neg << 31), h.w, sb);
+            }
+        } else if constexpr (sizeof(R) == 4 && EPT == 16) {
             if (tabbed) {
                 const bool pb = lane < ns && ((__popcll(rep & tabs.z[lane < ns ? lane : 0]) & 1) != 0);
                 const uint32_t bmask = tmask ^ __ballot_sync(0xffffffffu, pb);
@@ -3338,18 +3386,7 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
                     hpsi_tab_string(reinterpret_cast<float2 *>(acc), tabs, k, sb, bmask);
             }
         }
-        if constexpr (sizeof(R) == 4 && EPT == 16) {
-            if (fast && !tabbed) {
-                const uint32_t sb = smem_u32(t);
-                for (int k = 0; k < ns; ++k) {
-                    const HpsiStr h = many[k];
-                    const uint32_t neg = (uint32_t)(__popcll(rep & h.z) ^ __popc(threadIdx.x & h.tz)) & 1u;
-                    hpsi_string(reinterpret_cast<float2 *>(acc), h.X, h.g ^ (neg << 31), h.w, sb);
-                }
-            }
-        }
-        const bool staged = sizeof(R) == 4 && EPT == 16 && fast;
-        for (int gi = staged ? a.g_end : a.g_begin; gi < a.g_end; ++gi) {
+        for (int gi = tabbed ? a.g_end : a.g_begin; gi < a.g_end; ++gi) {
             const DevGroup G = groups[gi];
             for (int s = G.s_begin; s < G.s_end; ++s) {
                 const DevString S = strs[s];
@@ -3437,6 +3474,8 @@ __global__ void __launch_bounds__(512) k_evc_slice(const Cx<R> *__restrict__ psi
     const uint32_t c = blockIdx.x / (uint32_t)slices, sl = blockIdx.x % (uint32_t)slices;
     coset_span(a, spanv);
     const uint64_t rep = deposit(c, a.freeb, a.nfree);
+    pdl_wait();
+    pdl_next();
     load_coset<R>(t, psi, rep, spanv, a.kl, E);
     cp_async_commit();
     cp_async_wait0();
@@ -3509,6 +3548,8 @@ __global__ void __launch_bounds__(512) k_hpsi_slice(const Cx<R> *__restrict__ ps
     const uint32_t c = blockIdx.x / (uint32_t)slices, sl = blockIdx.x % (uint32_t)slices;
     coset_span(a, spanv);
     const uint64_t rep = deposit(c, a.freeb, a.nfree);
+    pdl_wait();
+    pdl_next();
     load_coset<R>(t, psi, rep, spanv, a.kl, E);
     cp_async_commit();
     const uint32_t lm = (1u << a.kl) - 1u;
@@ -4041,6 +4082,8 @@ __global__ void k_alg6_step(const uint64_t *__restrict__ xs, const int32_t *__re
 template <typename R>
 __global__ void k_prep(const int32_t *__restrict__ gparam, const double *__restrict__ params, int m,
                        R *__restrict__ coef) {
+    pdl_wait();
+    pdl_next();
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= m) return;
     const int p = gparam[g];
@@ -4052,11 +4095,15 @@ __global__ void k_prep(const int32_t *__restrict__ gparam, const double *__restr
 
 template <typename R>
 __global__ void k_set_one(Cx<R> *psi, uint64_t index) {
+    pdl_wait();
+    pdl_next();
     psi[index] = mk<R>(1, 0);
 }
 
 __global__ void k_reduce_rows(const double *__restrict__ part, int nblocks, int stride, int s_begin, int s_end,
                               double *__restrict__ out) {
+    pdl_wait();
+    pdl_next();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int s = s_begin + w;
     if (s >= s_end) return;
@@ -4068,6 +4115,8 @@ __global__ void k_reduce_rows(const double *__restrict__ part, int nblocks, int 
 
 __global__ void k_scatter(const double *__restrict__ opval, const int32_t *__restrict__ off,
                           const int32_t *__restrict__ idx, int np, double *__restrict__ grad) {
+    pdl_wait();
+    pdl_next();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np) return;
     double s = 0.0;
@@ -4079,6 +4128,8 @@ __global__ void k_energy(const double *__restrict__ slotval, const int32_t *__re
                          const double *__restrict__ coeffs, int nterms, double *__restrict__ per_term,
                          double *__restrict__ energy) {
     __shared__ double red[256];
+    pdl_wait();
+    pdl_next();
     double s = 0.0;
     for (int t = threadIdx.x; t < nterms; t += blockDim.x) {
         const double v = slotval[term_slot[t]];
@@ -4100,26 +4151,81 @@ __global__ void k_copy(Cx<R> *__restrict__ dst, const Cx<R> *__restrict__ src, s
         dst[i] = src[i];
 }
 
-template <typename K>
-int occupancy(K kernel, int threads, size_t smem) {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem) != cudaSuccess) nb = 1;
-    return nb < 1 ? 1 : nb;
+// Per-device answers of the runtime that every launch asks for (a launch of a
+// small state's pass takes a few microseconds, a query one of them).
+constexpr int kMaxDevices = 64;
+std::mutex g_query_mu;
+int current_device() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return dev;
 }
 
-// Largest dynamic shared memory a block may opt in to on the current device.
-int smem_optin() {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || v <= 0)
-        v = 48 * 1024;
+int occupancy(const void *kernel, int threads, size_t smem) {
+    static std::map<std::tuple<int, const void *, int, size_t>, int> known;
+    const auto key = std::make_tuple(current_device(), kernel, threads, smem);
+    std::lock_guard<std::mutex> lock(g_query_mu);
+    auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem) != cudaSuccess) return 1;
+    nb = nb < 1 ? 1 : nb;
+    if (known.size() < 4096) known[key] = nb;
+    return nb;
+}
+template <typename... A>
+int occupancy(void (*kernel)(A...), int threads, size_t smem) {
+    return occupancy((const void *)kernel, threads, smem);
+}
+
+int device_attribute(cudaDeviceAttr what, int fallback) {
+    static int known[2][kMaxDevices];
+    const int dev = current_device(), row = what == cudaDevAttrMultiProcessorCount ? 0 : 1;
+    std::lock_guard<std::mutex> lock(g_query_mu);
+    if (dev >= 0 && dev < kMaxDevices && known[row][dev]) return known[row][dev];
+    int v = 0;
+    if (cudaDeviceGetAttribute(&v, what, dev) != cudaSuccess || v <= 0) return fallback;
+    if (dev >= 0 && dev < kMaxDevices) known[row][dev] = v;
     return v;
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t smem) {
+// Largest dynamic shared memory a block may opt in to on the current device.
+int smem_optin() { return device_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin, 48 * 1024); }
+
+// Raise a kernel's dynamic shared memory limit to the largest size asked for.
+cudaError_t allow_smem_of(const void *kernel, size_t smem) {
+    static std::map<std::pair<int, const void *>, size_t> allowed;
+    const auto key = std::make_pair(current_device(), kernel);
+    std::lock_guard<std::mutex> lock(g_query_mu);
+    size_t &have = allowed[key];
+    if (smem <= have) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) have = smem;
+    return e;
+}
+template <typename... A>
+cudaError_t allow_smem(void (*kernel)(A...), size_t smem) {
     if (smem <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return allow_smem_of((const void *)kernel, smem);
+}
+
+// A launch whose set-up may overlap the kernel before it on the stream
+// (programmatic dependent launch): every kernel launched so runs pdl_wait()
+// in all threads before it touches anything that earlier work on the stream
+// reads or writes.
+template <typename... A, typename... V>
+cudaError_t launch(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st, V... v) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, A(v)...);
 }
 
 size_t gate_smem(sv_dtype dt, int k, int nlow) {
@@ -4137,12 +4243,7 @@ size_t coset_smem(sv_dtype dt, int E, int m, int nslots, int nwarps) {
 
 }  // namespace
 
-int device_sms() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
-}
+int device_sms() { return device_attribute(cudaDevAttrMultiProcessorCount, 1); }
 
 int gate_pass_grid(sv_dtype dt, int k, int nlow, int nops, int threads, int blocks_per_sm) {
     (void)nops;
@@ -4176,17 +4277,15 @@ cudaError_t launch_prep(sv_dtype dt, cudaStream_t st, const int32_t *gparam, con
                         void *coef) {
     if (m <= 0) return cudaSuccess;
     const int th = 128, bl = (m + th - 1) / th;
-    if (dt == SV_C64) k_prep<float><<<bl, th, 0, st>>>(gparam, params, m, (float *)coef);
-    else k_prep<double><<<bl, th, 0, st>>>(gparam, params, m, (double *)coef);
-    return cudaGetLastError();
+    if (dt == SV_C64) return launch(k_prep<float>, bl, th, 0, st, gparam, params, m, (float *)coef);
+    return launch(k_prep<double>, bl, th, 0, st, gparam, params, m, (double *)coef);
 }
 
 cudaError_t launch_set_basis(sv_dtype dt, cudaStream_t st, void *psi, size_t bytes, uint64_t index) {
     cudaError_t e = cudaMemsetAsync(psi, 0, bytes, st);
     if (e != cudaSuccess) return e;
-    if (dt == SV_C64) k_set_one<float><<<1, 1, 0, st>>>((float2 *)psi, index);
-    else k_set_one<double><<<1, 1, 0, st>>>((double2 *)psi, index);
-    return cudaGetLastError();
+    if (dt == SV_C64) return launch(k_set_one<float>, 1, 1, 0, st, (float2 *)psi, index);
+    return launch(k_set_one<double>, 1, 1, 0, st, (double2 *)psi, index);
 }
 
 cudaError_t launch_gate_pass(sv_dtype dt, cudaStream_t st, int grid, int threads, void *psi,
@@ -4194,14 +4293,12 @@ cudaError_t launch_gate_pass(sv_dtype dt, cudaStream_t st, int grid, int threads
     size_t sm = gate_smem(dt, a.k, a.nlow);
     if (dt == SV_C64) {
         allow_smem(k_gate_pass<float>, sm);
-        k_gate_pass<float><<<grid, threads, sm, st>>>((float2 *)psi, a, ops, (const float *)coef,
-                                                      (const float2 *)mats);
-    } else {
-        allow_smem(k_gate_pass<double>, sm);
-        k_gate_pass<double><<<grid, threads, sm, st>>>((double2 *)psi, a, ops, (const double *)coef,
-                                                       (const double2 *)mats);
+        return launch(k_gate_pass<float>, grid, threads, sm, st, (float2 *)psi, a, ops, (const float *)coef,
+                      (const float2 *)mats);
     }
-    return cudaGetLastError();
+    allow_smem(k_gate_pass<double>, sm);
+    return launch(k_gate_pass<double>, grid, threads, sm, st, (double2 *)psi, a, ops, (const double *)coef,
+                  (const double2 *)mats);
 }
 
 size_t gate_reg_smem(sv_dtype dt, const GatePassArgs &a) {
@@ -4227,25 +4324,24 @@ int reg_pass_grid(sv_dtype dt, const GatePassArgs &a, bool adj, int blocks_per_s
 
 template <typename R>
 cudaError_t gate_reg_dispatch(cudaStream_t st, int grid, void *psi, const GatePassArgs &a, const void *image,
-                              const void *pmats) {
+                              const void *pmats, bool early) {
     const size_t sm = gate_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
     const int nt = 1 << (a.k - kRegBits);
     if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
     allow_smem(k_gate_reg<R>, sm);
-    k_gate_reg<R><<<grid, nt, sm, st>>>((Cx<R> *)psi, a, (const unsigned char *)image, (const Cx<R> *)pmats);
-    return cudaGetLastError();
+    return launch(k_gate_reg<R>, grid, nt, sm, st, (Cx<R> *)psi, a, (const unsigned char *)image,
+                  (const Cx<R> *)pmats, early ? 1 : 0);
 }
 
 template <typename R>
 cudaError_t adj_reg_dispatch(cudaStream_t st, int grid, void *psi, void *lam, const GatePassArgs &a,
-                             const void *image, const void *pmats, double *part, int part_stride) {
+                             const void *image, const void *pmats, double *part, int part_stride, bool early) {
     const size_t sm = adj_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
     const int nt = 1 << (a.k - kRegBits);
     if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
     allow_smem(k_adj_reg<R>, sm);
-    k_adj_reg<R><<<grid, nt, sm, st>>>((Cx<R> *)psi, (Cx<R> *)lam, a, (const unsigned char *)image,
-                                       (const Cx<R> *)pmats, part, part_stride);
-    return cudaGetLastError();
+    return launch(k_adj_reg<R>, grid, nt, sm, st, (Cx<R> *)psi, (Cx<R> *)lam, a, (const unsigned char *)image,
+                  (const Cx<R> *)pmats, part, part_stride, early ? 1 : 0);
 }
 
 size_t reg_image_bytes(sv_dtype dt, const GatePassArgs &a) {
@@ -4259,31 +4355,28 @@ cudaError_t launch_reg_image(sv_dtype dt, cudaStream_t st, const GatePassArgs *p
     if (npasses <= 0) return cudaSuccess;
     const dim3 grid(npasses, kImageSlices, ndirs);
     if (dt == SV_C64)
-        k_reg_image<float><<<grid, 256, 0, st>>>(pargs, offs, ops, phases, steps, (const float *)coef, dblocks, dmem,
-                                                 (unsigned char *)out, dir_stride, dir0);
-    else
-        k_reg_image<double><<<grid, 256, 0, st>>>(pargs, offs, ops, phases, steps, (const double *)coef, dblocks, dmem,
-                                                  (unsigned char *)out, dir_stride, dir0);
-    return cudaGetLastError();
+        return launch(k_reg_image<float>, grid, 256, 0, st, pargs, offs, ops, phases, steps, (const float *)coef, dblocks,
+                      dmem, (unsigned char *)out, dir_stride, dir0);
+    return launch(k_reg_image<double>, grid, 256, 0, st, pargs, offs, ops, phases, steps, (const double *)coef, dblocks,
+                  dmem, (unsigned char *)out, dir_stride, dir0);
 }
 
 cudaError_t launch_prep_mats(sv_dtype dt, cudaStream_t st, const PrepMat *prep, int count, const void *mats, void *out) {
     if (count <= 0) return cudaSuccess;
-    if (dt == SV_C64) k_prep_mats<float><<<count, 256, 0, st>>>(prep, (const float2 *)mats, (float2 *)out);
-    else k_prep_mats<double><<<count, 256, 0, st>>>(prep, (const double2 *)mats, (double2 *)out);
-    return cudaGetLastError();
+    if (dt == SV_C64) return launch(k_prep_mats<float>, count, 256, 0, st, prep, (const float2 *)mats, (float2 *)out);
+    return launch(k_prep_mats<double>, count, 256, 0, st, prep, (const double2 *)mats, (double2 *)out);
 }
 
 cudaError_t launch_gate_reg(sv_dtype dt, cudaStream_t st, int grid, void *psi, const GatePassArgs &a,
-                            const void *image, const void *pmats) {
-    if (dt == SV_C64) return gate_reg_dispatch<float>(st, grid, psi, a, image, pmats);
-    return gate_reg_dispatch<double>(st, grid, psi, a, image, pmats);
+                            const void *image, const void *pmats, bool early) {
+    if (dt == SV_C64) return gate_reg_dispatch<float>(st, grid, psi, a, image, pmats, early);
+    return gate_reg_dispatch<double>(st, grid, psi, a, image, pmats, early);
 }
 
 cudaError_t launch_adj_reg(sv_dtype dt, cudaStream_t st, int grid, void *psi, void *lam, const GatePassArgs &a,
-                           const void *image, const void *pmats, double *part, int part_stride) {
-    if (dt == SV_C64) return adj_reg_dispatch<float>(st, grid, psi, lam, a, image, pmats, part, part_stride);
-    return adj_reg_dispatch<double>(st, grid, psi, lam, a, image, pmats, part, part_stride);
+                           const void *image, const void *pmats, double *part, int part_stride, bool early) {
+    if (dt == SV_C64) return adj_reg_dispatch<float>(st, grid, psi, lam, a, image, pmats, part, part_stride, early);
+    return adj_reg_dispatch<double>(st, grid, psi, lam, a, image, pmats, part, part_stride, early);
 }
 
 cudaError_t launch_adj_pass(sv_dtype dt, cudaStream_t st, int grid, int threads, void *psi, void *lam,
@@ -4292,15 +4385,12 @@ cudaError_t launch_adj_pass(sv_dtype dt, cudaStream_t st, int grid, int threads,
     size_t sm = adj_smem(dt, a.k, a.nlow, a.op_end - a.op_begin, threads);
     if (dt == SV_C64) {
         allow_smem(k_adj_pass<float>, sm);
-        k_adj_pass<float><<<grid, threads, sm, st>>>((float2 *)psi, (float2 *)lam, a, ops, (const float *)coef,
-                                                     (const float2 *)mats, part, part_stride);
-    } else {
-        allow_smem(k_adj_pass<double>, sm);
-        k_adj_pass<double><<<grid, threads, sm, st>>>((double2 *)psi, (double2 *)lam, a, ops,
-                                                      (const double *)coef, (const double2 *)mats, part,
-                                                      part_stride);
+        return launch(k_adj_pass<float>, grid, threads, sm, st, (float2 *)psi, (float2 *)lam, a, ops,
+                      (const float *)coef, (const float2 *)mats, part, part_stride);
     }
-    return cudaGetLastError();
+    allow_smem(k_adj_pass<double>, sm);
+    return launch(k_adj_pass<double>, grid, threads, sm, st, (double2 *)psi, (double2 *)lam, a, ops,
+                  (const double *)coef, (const double2 *)mats, part, part_stride);
 }
 
 cudaError_t launch_bitswap(sv_dtype dt, cudaStream_t st, void *psi, int n, const int32_t *pairs, int npairs,
@@ -4309,8 +4399,10 @@ cudaError_t launch_bitswap(sv_dtype dt, cudaStream_t st, void *psi, int n, const
     SwapArgs a;
     memset(&a, 0, sizeof(a));
     a.n = n;
-    // tile = the longest low run L with L + (partners of paired run bits) <= TB
-    const int TB = dt == SV_C64 ? 12 : 11;
+    // tile = the longest low run L with L + (partners of paired run bits) <= TB;
+    // a small state takes smaller tiles, so that they are more than the SMs
+    // (n = 12 complex128: 2 CTAs of 2^11 amplitudes took 9 us a QR)
+    const int TB = std::max(7, std::min(dt == SV_C64 ? 12 : 11, n - 9));
     int L = std::min(n, TB);
     for (; L > 1; --L) {
         int partners = 0;
@@ -4349,7 +4441,7 @@ cudaError_t launch_bitswap(sv_dtype dt, cudaStream_t st, void *psi, int n, const
         if (!(inside >> b & 1)) a.out[a.nout++] = (int8_t)b;
     const size_t es = dt == SV_C64 ? 8 : 16;
     const size_t sm = 2 * ((size_t)1 << a.ntb) * es + ((size_t)1 << (a.ntb - a.L)) * 8 + ((size_t)1 << a.ntb) * 2;
-    const int threads = 256;
+    const int threads = std::max(32, std::min(256, (1 << a.ntb) / (dt == SV_C64 ? 4 : 2)));
     int grid;
     if (dt == SV_C64) {
         allow_smem(k_bitswap<float>, sm);
@@ -4362,9 +4454,8 @@ cudaError_t launch_bitswap(sv_dtype dt, cudaStream_t st, void *psi, int n, const
     grid *= device_sms();
     const uint64_t ntiles = 1ull << a.nout;
     if ((uint64_t)grid > ntiles) grid = (int)ntiles;
-    if (dt == SV_C64) k_bitswap<float><<<grid, threads, sm, st>>>((float2 *)psi, a);
-    else k_bitswap<double><<<grid, threads, sm, st>>>((double2 *)psi, a);
-    return cudaGetLastError();
+    if (dt == SV_C64) return launch(k_bitswap<float>, grid, threads, sm, st, (float2 *)psi, a);
+    return launch(k_bitswap<double>, grid, threads, sm, st, (double2 *)psi, a);
 }
 
 template <typename R>
@@ -4380,8 +4471,8 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
 #define SV_EVCR_CASE(N)                                                                                      \
     case N:                                                                                                  \
         allow_smem(k_evc_ring<R, N, 9>, smr);                                                                \
-        k_evc_ring<R, N, 9><<<grid, 512, smr, st>>>((const Cx<R> *)psi, a, groups, strs, part, part_stride); \
-        return cudaGetLastError();
+        return launch(k_evc_ring<R, N, 9>, grid, 512, smr, st, (const Cx<R> *)psi, a, groups, strs, part,    \
+                      part_stride);
         switch (ept) {
             SV_EVCR_CASE(2)
             SV_EVCR_CASE(4)
@@ -4398,9 +4489,8 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
 #define SV_EVCF_CASE(N)                                                                                      \
     case N:                                                                                                  \
         allow_smem(k_evc_few<R, N, 9>, smf);                                                                 \
-        k_evc_few<R, N, 9><<<grid, threads, smf, st>>>((const Cx<R> *)psi, a, groups, strs, part,            \
-                                                      part_stride);                                          \
-        return cudaGetLastError();
+        return launch(k_evc_few<R, N, 9>, grid, threads, smf, st, (const Cx<R> *)psi, a, groups, strs, part, \
+                      part_stride);
         switch (ept) {
             SV_EVCF_CASE(1)
             SV_EVCF_CASE(2)
@@ -4423,9 +4513,8 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
 #define SV_EVC_CASE(N)                                                                                       \
     case N:                                                                                                  \
         allow_smem(k_evc_pass<R, N>, sm);                                                                    \
-        k_evc_pass<R, N><<<grid, threads, sm, st>>>((const Cx<R> *)psi, a, groups, strs, part, part_stride, \
-                                                    xform);                                                  \
-        break;
+        return launch(k_evc_pass<R, N>, grid, threads, sm, st, (const Cx<R> *)psi, a, groups, strs, part,    \
+                      part_stride, xform);
     switch (ept) {
         SV_EVC_CASE(1)
         SV_EVC_CASE(2)
@@ -4456,12 +4545,19 @@ cudaError_t hpsi_dispatch(cudaStream_t st, int grid, const void *psi, void *lam,
     // a multiple of the run length, at least one warp, at most 512
     const int threads = std::max(std::max(32, 1 << a.kl), std::min(E, 512));
     const int ept = std::max(1, E / threads);
+    // eight strings or so per pass are random masks, hundreds Jordan-Wigner ones
+    if constexpr (sizeof(R) == 4) {
+        if (ept == 16 && threads == 512 && a.s_end - a.s_begin > kHpsiTab) {
+            allow_smem(k_hpsi_pass<R, 16, true>, sm);
+            return launch(k_hpsi_pass<R, 16, true>, grid, threads, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, groups,
+                          strs, first, last, epart, status, limit);
+        }
+    }
 #define SV_HPSI_CASE(N)                                                                                      \
     case N:                                                                                                  \
-        allow_smem(k_hpsi_pass<R, N>, sm);                                                                   \
-        k_hpsi_pass<R, N><<<grid, threads, sm, st>>>((const Cx<R> *)psi, (Cx<R> *)lam, a, groups, strs,     \
-                                                     first, last, epart, status, limit);                     \
-        break;
+        allow_smem(k_hpsi_pass<R, N, false>, sm);                                                            \
+        return launch(k_hpsi_pass<R, N, false>, grid, threads, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a,  \
+                      groups, strs, first, last, epart, status, limit);
     switch (ept) {
         SV_HPSI_CASE(1)
         SV_HPSI_CASE(2)
@@ -4499,12 +4595,10 @@ cudaError_t launch_evc_slice(sv_dtype dt, cudaStream_t st, const void *psi, cons
     const size_t es = dt == SV_C64 ? 8 : 16, sm = (size_t)E * es + ((size_t)8 << a.m);
     if (dt == SV_C64) {
         allow_smem(k_evc_slice<float>, sm);
-        k_evc_slice<float><<<ncos * S, 512, sm, st>>>((const float2 *)psi, a, strs, part, part_stride, S);
-    } else {
-        allow_smem(k_evc_slice<double>, sm);
-        k_evc_slice<double><<<ncos * S, 512, sm, st>>>((const double2 *)psi, a, strs, part, part_stride, S);
+        return launch(k_evc_slice<float>, ncos * S, 512, sm, st, (const float2 *)psi, a, strs, part, part_stride, S);
     }
-    return cudaGetLastError();
+    allow_smem(k_evc_slice<double>, sm);
+    return launch(k_evc_slice<double>, ncos * S, 512, sm, st, (const double2 *)psi, a, strs, part, part_stride, S);
 }
 
 template <typename R>
@@ -4517,7 +4611,11 @@ cudaError_t hpsi_slice_dispatch(cudaStream_t st, const void *psi, void *lam, con
     const size_t sm = (size_t)E * sizeof(Cx<R>) + ((size_t)8 << a.m) + kHSliceTab * sizeof(HSliceStr<R>) +
                       512 * sizeof(Cx<R>);
     *rows = ncos * S;
-#define SV_HS_CASE(N)                                                                                                case N:                                                                                                              allow_smem(k_hpsi_slice<R, N>, sm);                                                                              k_hpsi_slice<R, N><<<ncos * S, 512, sm, st>>>((const Cx<R> *)psi, (Cx<R> *)lam, a, strs, first, last, epart, S);         break;
+#define SV_HS_CASE(N)                                                                                        \
+    case N:                                                                                                  \
+        allow_smem(k_hpsi_slice<R, N>, sm);                                                                  \
+        return launch(k_hpsi_slice<R, N>, ncos * S, 512, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, strs,  \
+                      first, last, epart, S);
     switch (ept) {
         SV_HS_CASE(1)
         SV_HS_CASE(2)
@@ -4543,21 +4641,18 @@ cudaError_t launch_reduce_rows(cudaStream_t st, const double *part, int nblocks,
     if (ns <= 0) return cudaSuccess;
     const int th = 256, warps_per = th / 32;
     const int bl = (ns + warps_per - 1) / warps_per;
-    k_reduce_rows<<<bl, th, 0, st>>>(part, nblocks, stride, s_begin, s_end, out);
-    return cudaGetLastError();
+    return launch(k_reduce_rows, bl, th, 0, st, part, nblocks, stride, s_begin, s_end, out);
 }
 
 cudaError_t launch_scatter(cudaStream_t st, const double *opval, const int32_t *off, const int32_t *idx, int np,
                            double *grad) {
     if (np <= 0) return cudaSuccess;
-    k_scatter<<<(np + 127) / 128, 128, 0, st>>>(opval, off, idx, np, grad);
-    return cudaGetLastError();
+    return launch(k_scatter, (np + 127) / 128, 128, 0, st, opval, off, idx, np, grad);
 }
 
 cudaError_t launch_energy(cudaStream_t st, const double *slotval, const int32_t *term_slot, const double *coeffs,
                           int nterms, double *per_term, double *energy) {
-    k_energy<<<1, 256, 0, st>>>(slotval, term_slot, coeffs, nterms, per_term, energy);
-    return cudaGetLastError();
+    return launch(k_energy, 1, 256, 0, st, slotval, term_slot, coeffs, nterms, per_term, energy);
 }
 
 cudaError_t launch_copy(sv_dtype dt, cudaStream_t st, void *dst, const void *src, size_t n) {

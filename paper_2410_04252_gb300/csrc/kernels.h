@@ -1,5 +1,7 @@
 // Launchers of the device kernels (kernels.cu).  All take a stream and return
-// the CUDA error of the launch.
+// the CUDA error of the launch.  The kernels' set-up may overlap the kernel
+// before them on the stream (programmatic dependent launch); their own reads
+// and writes of global memory follow it as usual.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -101,15 +103,17 @@ cudaError_t launch_prep_mats(sv_dtype dt, cudaStream_t st, const PrepMat *prep, 
 // (they hold the parameters): pass p's tables are reg_image_bytes(args[p])
 // bytes at out + offs[p], those of the reverse pass dir_stride further;
 // directions dir0 .. dir0 + ndirs - 1 (0 forward, 1 reverse) are made.
+// early: at least one kernel ran on the stream between the tables' kernels and
+// this pass, so it may read them while its predecessor still runs.
 size_t reg_image_bytes(sv_dtype dt, const GatePassArgs &a);
 cudaError_t launch_reg_image(sv_dtype dt, cudaStream_t st, const GatePassArgs *pargs, const uint64_t *offs, int npasses,
                              const DevOp *ops, const Phase *phases, const RegStep *steps, const void *coef,
                              const DiagBlock *dblocks, const DiagMember *dmem, void *out, uint64_t dir_stride, int dir0,
                              int ndirs);
 cudaError_t launch_gate_reg(sv_dtype dt, cudaStream_t st, int grid, void *psi, const GatePassArgs &a,
-                            const void *image, const void *pmats);
+                            const void *image, const void *pmats, bool early);
 cudaError_t launch_adj_reg(sv_dtype dt, cudaStream_t st, int grid, void *psi, void *lam, const GatePassArgs &a,
-                           const void *image, const void *pmats, double *part, int part_stride);
+                           const void *image, const void *pmats, double *part, int part_stride, bool early);
 // Shared memory of a register-blocked pass (forward / adjoint).
 size_t gate_reg_smem(sv_dtype dt, const GatePassArgs &a);
 size_t adj_reg_smem(sv_dtype dt, const GatePassArgs &a);
