@@ -143,11 +143,15 @@ struct EvcEntry {
     uint64_t key = 0;
     EvcPlan plan;
     std::vector<CosetArgs> args;
-    DevBuf groups, strings, term_slot, coeffs;
+    std::vector<CosetArgs> rest;    // what register phases leave of a pass (g_begin == g_end: nothing)
+    DevBuf groups, strings, term_slot, coeffs, rphases, rgroups, ritems;
     int nterms = 0;
     double plan_ms = 0;
     uint64_t last_use = 0;
-    void release() { groups.release(); strings.release(); term_slot.release(); coeffs.release(); }
+    void release() {
+        groups.release(); strings.release(); term_slot.release(); coeffs.release();
+        rphases.release(); rgroups.release(); ritems.release();
+    }
 };
 
 constexpr size_t kCacheSize = 6;
@@ -455,6 +459,13 @@ sv_status get_qsu(sv_handle *h, const sv_gate *gates, size_t m, size_t np, sv_sc
     return SV_OK;
 }
 
+int reg_groups(const EvcPlan &P, const CosetPass &cp) {
+    return P.rphases[cp.rp_end - 1].g_end - P.rphases[cp.rp_begin].g_begin;
+}
+int reg_items(const EvcPlan &P, const CosetPass &cp) {
+    return P.rphases[cp.rp_end - 1].i_end - P.rphases[cp.rp_begin].i_begin;
+}
+
 sv_status evc_entry_upload(sv_handle *h, EvcEntry *ent, const double *coeffs, size_t nterms) {
     std::vector<DevGroup> gs(ent->plan.groups.size());
     for (size_t i = 0; i < gs.size(); ++i) {
@@ -481,7 +492,24 @@ sv_status evc_entry_upload(sv_handle *h, EvcEntry *ent, const double *coeffs, si
     SV_CK(upload(ent->term_slot, ent->plan.term_slot, h->stream));
     std::vector<double> c(coeffs, coeffs + nterms);
     SV_CK(upload(ent->coeffs, c, h->stream));
-    for (auto &cp : ent->plan.passes) ent->args.push_back(coset_args(h->n, cp));
+    SV_CK(upload(ent->rphases, ent->plan.rphases, h->stream));
+    SV_CK(upload(ent->rgroups, ent->plan.rgroups, h->stream));
+    SV_CK(upload(ent->ritems, ent->plan.ritems, h->stream));
+    for (auto &cp : ent->plan.passes) {
+        ent->args.push_back(coset_args(h->n, cp));
+        CosetArgs &a = ent->args.back();
+        if (cp.rp_end > cp.rp_begin &&
+            !evc_reg_fits(h->dt, a, cp.s_reg - cp.s_begin, cp.rp_end - cp.rp_begin, reg_groups(ent->plan, cp),
+                          reg_items(ent->plan, cp))) {
+            cp.rp_end = cp.rp_begin;
+            cp.g_reg = cp.g_begin;
+            cp.s_reg = cp.s_begin;
+        }
+        CosetPass left = cp;
+        left.g_begin = cp.g_reg;
+        left.s_begin = cp.s_reg;
+        ent->rest.push_back(coset_args(h->n, left));
+    }
     return SV_OK;
 }
 
@@ -533,6 +561,10 @@ sv_status get_evc(sv_handle *h, const sv_pauli *p, const double *c, size_t nterm
                           ? plan_hpsi(h->n, p, c, nterms, po, h->l2p, ent->plan)
                           : plan_evc(h->n, h->g, p, c, nterms, sched != SV_SCHED_EAGER, po, h->l2p, ent->plan);
     if (!err.empty()) return fail(SV_EINVAL, std::string(hpsi ? "H|psi> plan: " : "EVC plan: ") + err);
+    if (!hpsi) {
+        const int r = h->dt == SV_C64 ? 5 : 4;
+        plan_evc_phases(ent->plan, r + 8, r);
+    }
     ent->plan_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     ent->key = key;
     ent->nterms = (int)nterms;
@@ -679,7 +711,16 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
                                        h->part.as<double>(), nslots));
                 continue;
             }
-            SV_CK(launch_evc_pass(h->dt, h->stream, grid, h->psi, e->args[pi], e->groups.as<DevGroup>(),
+            // masks of one or two staged bits in register phases, the rest of the pass (if any) by the general kernels
+            const CosetPass &cp = P.passes[pi];
+            if (cp.rp_end > cp.rp_begin) {
+                SV_CK(launch_evc_reg(h->dt, h->stream, grid, h->psi, e->args[pi], e->rphases.as<EvcRegPhase>() + cp.rp_begin,
+                                     cp.rp_end - cp.rp_begin, e->rgroups.as<EvcRegGroup>(), reg_groups(P, cp),
+                                     e->ritems.as<EvcRegItem>(), reg_items(P, cp), cp.s_reg - cp.s_begin,
+                                     h->part.as<double>(), nslots));
+                if (e->rest[pi].g_begin == e->rest[pi].g_end) continue;
+            }
+            SV_CK(launch_evc_pass(h->dt, h->stream, grid, h->psi, e->rest[pi], e->groups.as<DevGroup>(),
                                   e->strings.as<DevString>(), h->part.as<double>(), nslots, h->status.as<int>(),
                                   (long long)h->opt.wait_limit));
         }

@@ -2399,7 +2399,6 @@ __device__ __forceinline__ void pair_terms_sel(const float2 *t, const float2 *ow
     }
 }
 
-constexpr int kXformMinStrings = 16;  // groups with at least this many strings take the transform path
 // shared-memory layout of k_evc_pass: two staged cosets, the span table, per
 // string and warp a partial of the state's real type (FP64 is 1/64 of the
 // FP32 rate here: complex64 partials reach an FP64 total per string every
@@ -3142,6 +3141,294 @@ __global__ void __launch_bounds__(1 << LOGNT, 1) k_evc_ring(const Cx<R> *__restr
         double tsum = 0.0;
         for (int w = 0; w < NT / 32; ++w) tsum += wsum[threadIdx.x][w];
         part[(size_t)blockIdx.x * part_stride + a.s_begin + threadIdx.x] = tsum;
+    }
+}
+
+// ---- K-EVC in register phases (many masks of one or two staged bits) ----
+// A Jordan-Wigner pass has tens of X/Y masks of two qubits, a few strings
+// each.  The general kernel read every partner from shared memory and paid
+// each group's and string's fixed cost on 16 elements a thread (compute
+// bound: 64k clocks per 64 KB coset, 3k of which HBM would need).  Here a
+// phase's threads hold the amplitudes of r staged bits in registers (32 for
+// complex64), so one gather serves the pairs of up to ten masks; the strings
+// that differ only at the pair's other end (XX and YY, XY and YX) share one
+// signed sum up to its last level.  The coset is only read, so the warps run
+// their (phase, eighth of the coset) units without barriers; what remains per
+// string is its sign bit and its share of a four-value warp reduction.
+// n = 28, 4096 strings (16 passes): 106 -> see DESIGN.
+template <typename R> struct EvcVal;
+template <> struct EvcVal<float> { using T = unsigned long long; };   // packed halves of the products
+template <> struct EvcVal<double> { using T = double; };
+template <typename R> using EV = typename EvcVal<R>::T;
+
+template <bool IM> __device__ __forceinline__ unsigned long long ev_prod(unsigned long long v, unsigned long long u) {
+    if (!IM) return f2_mul(v, u);
+    const float2 h = f2_unpack(v);
+    return f2_mul(f2_pack(h.y, h.x), u);
+}
+template <bool IM> __device__ __forceinline__ double ev_prod(double2 v, double2 u) {
+    return IM ? v.x * u.y - v.y * u.x : v.x * u.x + v.y * u.y;
+}
+__device__ __forceinline__ unsigned long long ev_fold(unsigned long long s, unsigned long long b, unsigned long long a) {
+    return f2_fma(s, b, a);
+}
+__device__ __forceinline__ double ev_fold(double s, double b, double a) { return fma(s, b, a); }
+template <bool IM> __device__ __forceinline__ float ev_end(unsigned long long r) { return f2_combine<IM>(r); }
+template <bool IM> __device__ __forceinline__ double ev_end(double r) { return r; }
+__device__ __forceinline__ float ev_sign(float v, uint32_t neg) {
+    return __uint_as_float(__float_as_uint(v) ^ (neg << 31));
+}
+__device__ __forceinline__ double ev_sign(double v, uint32_t neg) { return neg ? -v : v; }
+
+// the element of pair p: bit H clear, the top bit of p at bit L, the others ascending
+template <int RB, int H, int L>
+__host__ __device__ constexpr int ev_elem(int p) {
+    int v = 0, c = 0;
+    for (int b = 0; b < RB; ++b) {
+        if (b == H || b == L) continue;
+        v |= ((p >> c) & 1) << b;
+        ++c;
+    }
+    return v | (((p >> (RB - 2)) & 1) << L);
+}
+template <typename R, int RB, int H, int L, bool ONE, bool IM>
+__device__ __forceinline__ void ev_products(EV<R> *P, const RA<R> *x) {
+    constexpr int XR = (1 << H) | (ONE ? 0 : 1 << L);
+#pragma unroll
+    for (int p = 0; p < (1 << (RB - 1)); ++p) {
+        const int v = ev_elem<RB, H, L>(p);
+        P[p] = ev_prod<IM>(x[v ^ XR], x[v]);
+    }
+}
+template <typename R, int RB, bool IM>
+__device__ __forceinline__ void ev_group_products(EV<R> *P, const RA<R> *x, int code) {
+#define SV_EP(H, L)                                                                              \
+    case H * 8 + L: if constexpr (H < RB) ev_products<R, RB, H, L, false, IM>(P, x); break;
+#define SV_EO(H, L)                                                                              \
+    case 64 + H * 8 + L: if constexpr (H < RB) ev_products<R, RB, H, L, true, IM>(P, x); break;
+    switch (code) {
+        SV_EP(1, 0) SV_EP(2, 0) SV_EP(2, 1) SV_EP(3, 0) SV_EP(3, 1) SV_EP(3, 2)
+        SV_EP(4, 0) SV_EP(4, 1) SV_EP(4, 2) SV_EP(4, 3)
+        SV_EO(0, 1) SV_EO(1, 0) SV_EO(2, 0) SV_EO(3, 0) SV_EO(4, 0)
+    default: break;
+    }
+#undef SV_EP
+#undef SV_EO
+}
+
+template <typename R> struct EvcItemS {
+    EV<R> lev[3];           // signs of the fold's levels
+    uint32_t slots, neg;    // sum slot | difference slot << 16 (0xFFFF: none)
+};
+template <typename R> __host__ __device__ constexpr int evc_reg_bits() { return sizeof(R) == 4 ? 5 : 4; }
+
+// Shared memory beyond the two staged cosets: span table, per string and
+// eighth a partial, FP64 totals (complex64), phases, groups, items.
+struct EvcRegLayout {
+    uint32_t span, acc, tot, phases, prb, pbase, tmask, groups, items, zs, total;
+};
+__host__ __device__ inline EvcRegLayout evc_reg_layout(int m, int nslots, int nph, int ngr, int nit, int rbytes) {
+    EvcRegLayout L;
+    uint32_t o = 0;
+    L.span = o;   o = align16u(o + (8u << m));
+    L.acc = o;    o = align16u(o + (uint32_t)nslots * 8u * (uint32_t)rbytes);
+    L.tot = o;    o = align16u(o + (rbytes == 4 ? 8u * (uint32_t)nslots : 0u));
+    L.phases = o; o = align16u(o + (uint32_t)sizeof(EvcRegPhase) * (uint32_t)nph);
+    L.prb = o;    o = align16u(o + 16u * (uint32_t)nph);
+    L.pbase = o;  o = align16u(o + 512u * (uint32_t)nph);
+    L.tmask = o;  o = align16u(o + 1024u * (uint32_t)nph);
+    L.groups = o; o = align16u(o + 16u * (uint32_t)ngr);
+    L.items = o;  o = align16u(o + 32u * (uint32_t)nit);
+    L.zs = o;     o = align16u(o + 8u * (uint32_t)nit);
+    L.total = o;
+    return L;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ psi, const CosetArgs a,
+                                                    const EvcRegPhase *__restrict__ phases, int nph,
+                                                    const EvcRegGroup *__restrict__ rgroups,
+                                                    const EvcRegItem *__restrict__ ritems, int nslots,
+                                                    double *__restrict__ part, int part_stride) {
+    constexpr int RB = evc_reg_bits<R>(), V = 1 << RB, NP = V / 2, LOGE = RB + 8;
+    constexpr uint32_t E = 1u << LOGE;
+    extern __shared__ __align__(16) unsigned char smem[];
+    RA<R> *buf = reinterpret_cast<RA<R> *>(smem);
+    unsigned char *sm = smem + 2 * (size_t)E * sizeof(Cx<R>);
+    const int g0 = phases[0].g_begin, i0 = phases[0].i_begin;
+    const int ngr = phases[nph - 1].g_end - g0, nit = phases[nph - 1].i_end - i0;
+    const EvcRegLayout L = evc_reg_layout(a.m, nslots, nph, ngr, nit, (int)sizeof(R));
+    uint64_t *spanv = reinterpret_cast<uint64_t *>(sm + L.span);
+    R *acc = reinterpret_cast<R *>(sm + L.acc);
+    double *tot64 = reinterpret_cast<double *>(sm + L.tot);
+    EvcRegPhase *phs = reinterpret_cast<EvcRegPhase *>(sm + L.phases);
+    uint16_t *prb = reinterpret_cast<uint16_t *>(sm + L.prb);
+    uint16_t *pbase = reinterpret_cast<uint16_t *>(sm + L.pbase);
+    uint32_t *tmask = reinterpret_cast<uint32_t *>(sm + L.tmask);
+    EvcRegGroup *grs = reinterpret_cast<EvcRegGroup *>(sm + L.groups);
+    EvcItemS<R> *its = reinterpret_cast<EvcItemS<R> *>(sm + L.items);
+    uint64_t *zs = reinterpret_cast<uint64_t *>(sm + L.zs);
+    const int tid = threadIdx.x, NT = blockDim.x, warp = tid >> 5, lane = tid & 31, nwarps = NT >> 5;
+    for (int j = tid; j < nslots * 8; j += NT) acc[j] = 0;
+    if constexpr (sizeof(R) == 4)
+        for (int j = tid; j < nslots; j += NT) tot64[j] = 0.0;
+    for (int p = tid; p < nph; p += NT) {
+        EvcRegPhase F = phases[p];
+        uint32_t rm = F.rmask;
+        for (int i = 0; i < RB; ++i, rm &= rm - 1u) prb[p * 8 + i] = (uint16_t)swz_tile(rm & (0u - rm));
+        F.g_begin -= g0; F.g_end -= g0; F.i_begin -= i0; F.i_end -= i0;
+        phs[p] = F;
+    }
+    for (int g = tid; g < ngr; g += NT) {
+        EvcRegGroup G = rgroups[g0 + g];
+        G.i_begin -= i0;
+        grs[g] = G;
+    }
+    for (int i = tid; i < nit; i += NT) {
+        const EvcRegItem t = ritems[i0 + i];
+        EvcItemS<R> s;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const float sg = ((t.w >> l) & 1u) ? -1.f : 1.f;
+            if constexpr (sizeof(R) == 4) s.lev[l] = f2_pack(sg, sg);
+            else s.lev[l] = (double)sg;
+        }
+        s.slots = (uint32_t)(t.slot_sum & 0xFFFF) | ((uint32_t)t.slot_dif << 16);
+        s.neg = t.neg;
+        its[i] = s;
+        zs[i] = t.z;
+    }
+    coset_span(a, spanv);
+    for (int e = tid; e < nph * 256; e += NT) {
+        const EvcRegPhase F = phs[e >> 8];
+        const uint32_t base = phase_base(F.rmask, F.lanes, LOGE, (uint32_t)e & 255u);
+        uint32_t m = 0;
+        for (int i = F.i_begin; i < F.i_end; ++i)
+            m |= (uint32_t)(__popc(base & ritems[i0 + i].tau) & 1) << (i - F.i_begin);
+        pbase[e] = (uint16_t)base;
+        tmask[e] = m;
+    }
+    const uint64_t ncos = 1ull << a.nfree;
+    const uint64_t mine = blockIdx.x < ncos ? (ncos - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    const BitWalk bw = bit_walk(a.freeb, a.nfree, gridDim.x);
+    uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
+    const uint32_t lowmask = (1u << a.kl) - 1u;
+    constexpr uint32_t PER = 16 / sizeof(Cx<R>);
+    auto load = [&](RA<R> *dst, uint64_t rep) {
+        for (uint32_t q = tid; q < E / PER; q += (uint32_t)NT) {
+            const uint32_t e = q * PER;
+            cp_async16(dst + swz_tile(e), psi + (rep ^ spanv[e >> a.kl] ^ (e & lowmask)));
+        }
+    };
+    pdl_wait();
+    pdl_next();
+    for (uint64_t k = 0; k < 2; ++k) {
+        if (k < mine) load(buf + k * E, rep_pf);
+        cp_async_commit();
+        rep_pf = walk_next(rep_pf, bw);
+    }
+    for (uint64_t it = 0; it < mine; ++it) {
+        const uint64_t rep = rep_cur;
+        rep_cur = walk_next(rep_cur, bw);
+        const RA<R> *t = buf + (it & 1) * E;
+        cp_async_wait1();
+        __syncthreads();
+        for (int u = warp; u < nph * 8; u += nwarps) {
+            const int p = u >> 3, wt = u & 7, th = (p << 8) | (wt << 5) | lane;
+            const EvcRegPhase F = phs[p];
+            const bool zb = lane < F.i_end - F.i_begin && (__popcll(rep & zs[min(F.i_begin + lane, nit - 1)]) & 1);
+            const uint32_t mask = tmask[th] ^ __ballot_sync(0xffffffffu, zb);
+            RA<R> x[V];
+            {
+                const uint4 r = *reinterpret_cast<const uint4 *>(prb + p * 8);
+                const uint32_t rb[5] = {r.x & 0xFFFFu, r.x >> 16, r.y & 0xFFFFu, r.y >> 16, r.z & 0xFFFFu};
+                uint32_t idx[V];
+                idx[0] = swz_tile(pbase[th]);
+#pragma unroll
+                for (int v = 1; v < V; ++v)
+                    idx[v] = idx[v & (v - 1)] ^ rb[(v & 1) ? 0 : (v & 2) ? 1 : (v & 4) ? 2 : (v & 8) ? 3 : 4];
+                if (sizeof(R) == 4 && (F.rmask & 1u)) {
+#pragma unroll
+                    for (int v = 0; v < V; v += 2) {
+                        const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(&t[idx[v]]);
+                        memcpy(&x[v], &w.x, 8);
+                        memcpy(&x[v + 1], &w.y, 8);
+                    }
+                } else {
+#pragma unroll
+                    for (int v = 0; v < V; ++v) x[v] = t[idx[v]];
+                }
+            }
+            // results of two items are reduced together
+            R v0 = 0, v1 = 0;
+            uint32_t pend = 0xFFFFFFFFu;
+            auto flush = [&](R w0, R w1, uint32_t slots) {
+                const R red = warp_sum4<R>(v0, v1, w0, w1);
+                const uint32_t two = (lane & 16) ? slots : pend, sl = (lane & 8) ? two >> 16 : two & 0xFFFFu;
+                if ((lane & 7) == 0 && sl != 0xFFFFu) acc[sl * 8 + wt] += red;
+                pend = 0xFFFFFFFFu;
+            };
+            for (int g = F.g_begin; g < F.g_end; ++g) {
+                const EvcRegGroup G = grs[g];
+#pragma unroll
+                for (int im = 0; im < 2; ++im) {
+                    const int n = im ? G.nim : G.nre, ib = G.i_begin + (im ? G.nre : 0);
+                    if (n == 0) continue;
+                    EV<R> P[NP];
+                    if (im) ev_group_products<R, RB, true>(P, x, G.code);
+                    else ev_group_products<R, RB, false>(P, x, G.code);
+                    for (int i = ib; i < ib + n; ++i) {
+                        const EvcItemS<R> S = its[i];
+                        EV<R> f[NP / 2];
+#pragma unroll
+                        for (int k = 0; k < NP / 2; ++k) f[k] = ev_fold(S.lev[0], P[2 * k + 1], P[2 * k]);
+#pragma unroll
+                        for (int l = 1, c = NP / 4; c >= 2; ++l, c >>= 1)
+#pragma unroll
+                            for (int k = 0; k < c; ++k) f[k] = ev_fold(S.lev[l], f[2 * k + 1], f[2 * k]);
+                        const R r0 = im ? ev_end<true>(f[0]) : ev_end<false>(f[0]);
+                        const R r1 = im ? ev_end<true>(f[1]) : ev_end<false>(f[1]);
+                        const uint32_t sg = (mask >> (i - F.i_begin)) & 1u;
+                        const R w0 = ev_sign(r0 + r1, sg ^ (S.neg & 1u)), w1 = ev_sign(r0 - r1, sg ^ (S.neg >> 1));
+                        if (pend == 0xFFFFFFFFu) {
+                            v0 = w0;
+                            v1 = w1;
+                            pend = S.slots;
+                        } else {
+                            flush(w0, w1, S.slots);
+                        }
+                    }
+                }
+            }
+            if (pend != 0xFFFFFFFFu) flush((R)0, (R)0, 0xFFFFFFFFu);
+        }
+        __syncthreads();
+        if (it + 2 < mine) load(buf + (it & 1) * E, rep_pf);
+        cp_async_commit();
+        rep_pf = walk_next(rep_pf, bw);
+        if constexpr (sizeof(R) == 4) {
+            // the next writes to the slots follow the next coset's barrier
+            if (((it + 1) % kEvcFlush) == 0 || it + 1 == mine) {
+                for (int q = tid; q < nslots; q += NT) {
+                    float f = 0.f;
+                    for (int w = 0; w < 8; ++w) {
+                        f += acc[q * 8 + w];
+                        acc[q * 8 + w] = 0.f;
+                    }
+                    tot64[q] += (double)f;
+                }
+            }
+        }
+    }
+    cp_async_wait0();
+    __syncthreads();
+    // every pair was taken once
+    for (int q = tid; q < nslots; q += NT) {
+        double s = 0.0;
+        if constexpr (sizeof(R) == 4) s = tot64[q];
+        else
+            for (int w = 0; w < 8; ++w) s += acc[q * 8 + w];
+        part[(size_t)blockIdx.x * part_stride + a.s_begin + q] = 2.0 * s;
     }
 }
 
@@ -4526,6 +4813,29 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
     }
 #undef SV_EVC_CASE
     return cudaGetLastError();
+}
+
+bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, int nslots, int nph, int ngroups, int nitems) {
+    const size_t es = dt == SV_C64 ? 8 : 16;
+    const int rb = dt == SV_C64 ? 5 : 4;
+    if (a.kl + a.m != rb + 8 || a.kl < 1) return false;
+    return 2 * (es << (rb + 8)) + evc_reg_layout(a.m, nslots, nph, ngroups, nitems, (int)es / 2).total <=
+           (size_t)smem_optin();
+}
+
+cudaError_t launch_evc_reg(sv_dtype dt, cudaStream_t st, int grid, const void *psi, const CosetArgs &a,
+                           const EvcRegPhase *phases, int nph, const EvcRegGroup *rgroups, int ngroups,
+                           const EvcRegItem *ritems, int nitems, int nslots, double *part, int part_stride) {
+    const size_t es = dt == SV_C64 ? 8 : 16;
+    const size_t sm = 2 * (es << (a.kl + a.m)) + evc_reg_layout(a.m, nslots, nph, ngroups, nitems, (int)es / 2).total;
+    if (dt == SV_C64) {
+        allow_smem(k_evc_reg<float>, sm);
+        return launch(k_evc_reg<float>, grid, 512, sm, st, (const float2 *)psi, a, phases, nph, rgroups, ritems, nslots,
+                      part, part_stride);
+    }
+    allow_smem(k_evc_reg<double>, sm);
+    return launch(k_evc_reg<double>, grid, 512, sm, st, (const double2 *)psi, a, phases, nph, rgroups, ritems, nslots,
+                  part, part_stride);
 }
 
 cudaError_t launch_evc_pass(sv_dtype dt, cudaStream_t st, int grid, const void *psi, const CosetArgs &a,

@@ -897,16 +897,25 @@ void plan_cosets(EvcPlan &P, std::vector<GroupIn> &groups, int klmin, int mmax, 
         cp.g_begin = (int32_t)P.groups.size();
         cp.s_begin = (int32_t)P.strings.size();
         std::vector<char> in(groups.size(), 0);
-        for (int32_t gi : sel) {
-            in[gi] = 1;
-            GroupIn &G = groups[gi];
-            EvcGroup eg;
-            eg.x = G.x;
+        auto offset = [&](const GroupIn &G) {
             uint32_t c = 0;
             const uint64_t h = G.x & ~lowmask;
             for (int j = 0; j < cp.m; ++j)
                 if (h >> sp.pivot[j] & 1) c |= 1u << j;
-            eg.X = (c << kl) | (uint32_t)(G.x & lowmask);
+            return (c << kl) | (uint32_t)(G.x & lowmask);
+        };
+        // the groups that register phases could take first (plan_evc_phases)
+        std::vector<int32_t> ordered(sel);
+        std::stable_partition(ordered.begin(), ordered.end(), [&](int32_t gi) {
+            const int wt = popc(offset(groups[gi]));
+            return wt >= 1 && wt <= 2 && groups[gi].zs.size() < (size_t)kXformMinStrings;
+        });
+        for (int32_t gi : ordered) {
+            in[gi] = 1;
+            GroupIn &G = groups[gi];
+            EvcGroup eg;
+            eg.x = G.x;
+            eg.X = offset(G);
             eg.s_begin = (int32_t)P.strings.size();
             for (size_t s = 0; s < G.zs.size(); ++s) {
                 EvcString es;
@@ -1111,6 +1120,117 @@ std::string tiling_pauli_strings(int n, int nG, const sv_pauli *p, const std::ve
 }
 
 }  // namespace
+
+void plan_evc_phases(EvcPlan &P, int stage, int r) {
+    for (auto &cp : P.passes) {
+        cp.rp_begin = cp.rp_end = (int32_t)P.rphases.size();
+        cp.g_reg = cp.g_begin;
+        cp.s_reg = cp.s_begin;
+        if (cp.kl + cp.m != stage) continue;
+        int ge = cp.g_begin;
+        while (ge < cp.g_end) {
+            const EvcGroup &G = P.groups[ge];
+            const int wt = popc(G.X);
+            if (wt < 1 || wt > 2 || G.s_end - G.s_begin >= kXformMinStrings) break;
+            ++ge;
+        }
+        if (ge - cp.g_begin < kEvcRegMinGroups) continue;
+        uint64_t piv = 0;
+        for (int j = 0; j < cp.m; ++j) piv |= bit(cp.pivot[j]);
+        const uint64_t freemask = ~(piv | (bit(cp.kl) - 1));
+        const size_t np0 = P.rphases.size(), ng0 = P.rgroups.size(), ni0 = P.ritems.size();
+        std::vector<char> done(ge - cp.g_begin, 0);
+        int left = ge - cp.g_begin;
+        bool fits = true;
+        while (left > 0 && fits) {
+            // the register set grows bit by bit from the first remaining group,
+            // by the bit that completes most remaining groups (ties: the bit in
+            // most remaining groups, then the lowest)
+            uint32_t rm = 0;
+            for (size_t i = 0; i < done.size() && !rm; ++i)
+                if (!done[i]) rm = P.groups[cp.g_begin + i].X;
+            while (popc(rm) < r) {
+                int best = -1;
+                int64_t bs = -1;
+                for (int b = 0; b < stage; ++b) {
+                    if (rm >> b & 1u) continue;
+                    int in = 0, has = 0;
+                    for (size_t i = 0; i < done.size(); ++i) {
+                        if (done[i]) continue;
+                        const uint32_t X = P.groups[cp.g_begin + i].X;
+                        if (!(X >> b & 1u)) continue;
+                        ++has;
+                        if (!(X & ~(rm | (1u << b)))) ++in;
+                    }
+                    const int64_t sc = ((int64_t)in << 20) + has;
+                    if (sc > bs) { bs = sc; best = b; }
+                }
+                rm |= 1u << best;
+            }
+            EvcRegPhase F;
+            F.rmask = rm;
+            F.lanes = phase_lanes(rm, stage);
+            F.g_begin = (int32_t)P.rgroups.size();
+            F.i_begin = (int32_t)P.ritems.size();
+            auto reg = [&](int t) { return popc(rm & ((1u << t) - 1u)); };
+            for (size_t i = 0; i < done.size(); ++i) {
+                const EvcGroup &G = P.groups[cp.g_begin + i];
+                if (done[i] || (G.X & ~rm)) continue;
+                const int hb = hibit(G.X), lbit = popc(G.X) == 2 ? lobit(G.X) : lobit(rm & ~G.X);
+                EvcRegGroup rg;
+                rg.code = reg(hb) * 8 + reg(lbit) + (popc(G.X) == 2 ? 0 : 64);
+                rg.i_begin = (int32_t)P.ritems.size();
+                int cnt[2] = {0, 0};
+                std::vector<EvcRegItem> its[2];
+                for (int q = G.s_begin; q < G.s_end; ++q) {
+                    const EvcString &S = P.strings[q];
+                    const uint32_t tau = (uint32_t)(S.z & (bit(cp.kl) - 1)) | (S.bz << cp.kl);
+                    uint32_t w = 0;
+                    int c = 0;
+                    for (uint32_t o = rm & ~((1u << hb) | (1u << lbit)); o; o &= o - 1, ++c)
+                        if (tau >> lobit(o) & 1u) w |= 1u << c;
+                    const int part = S.nY & 1, dif = tau >> lbit & 1u;
+                    const uint32_t neg = (S.nY == 1 || S.nY == 2) ? 1u : 0u;
+                    EvcRegItem *hit = nullptr;
+                    for (auto &it : its[part])
+                        if (it.w == w && it.tau == (tau & ~rm) && ((it.z ^ S.z) & freemask) == 0 &&
+                            (dif ? it.slot_dif : it.slot_sum) < 0) {
+                            hit = &it;
+                            break;
+                        }
+                    if (!hit) {
+                        its[part].push_back(EvcRegItem{S.z & freemask, tau & ~rm, w, -1, -1, 0u, 0u});
+                        hit = &its[part].back();
+                    }
+                    (dif ? hit->slot_dif : hit->slot_sum) = q - cp.s_begin;
+                    hit->neg |= neg << dif;
+                }
+                cnt[0] = (int)its[0].size();
+                cnt[1] = (int)its[1].size();
+                if ((int)P.ritems.size() - F.i_begin + cnt[0] + cnt[1] > kEvcRegItems) continue;   // a later phase's
+                for (auto &v : its) P.ritems.insert(P.ritems.end(), v.begin(), v.end());
+                rg.nre = cnt[0];
+                rg.nim = cnt[1];
+                P.rgroups.push_back(rg);
+                done[i] = 1;
+                --left;
+            }
+            F.g_end = (int32_t)P.rgroups.size();
+            F.i_end = (int32_t)P.ritems.size();
+            P.rphases.push_back(F);
+            if (P.rphases.size() - np0 > (size_t)kEvcRegPhases) fits = false;
+        }
+        if (!fits) {
+            P.rphases.resize(np0);
+            P.rgroups.resize(ng0);
+            P.ritems.resize(ni0);
+            continue;
+        }
+        cp.rp_end = (int32_t)P.rphases.size();
+        cp.g_reg = ge;
+        cp.s_reg = ge < cp.g_end ? P.groups[ge].s_begin : cp.s_end;
+    }
+}
 
 uint64_t hash_bytes(const void *p, size_t n, uint64_t h) {
     const unsigned char *c = (const unsigned char *)p;

@@ -193,12 +193,41 @@ struct EvcGroup {
     uint32_t X;        // partner offset inside the coset tile: (c << kl) | (x & (2^kl - 1))
     int32_t s_begin, s_end;   // strings (slots)
 };
+// Expectation passes over many X/Y masks of one or two staged bits (a
+// Jordan-Wigner Hamiltonian's): register phases.  In a phase a thread holds
+// the 2^r amplitudes spanned by r staged-index bits (rmask), so the pairs of
+// every group whose mask lies in them are pairs of its own registers.
+// A group's pair index p (element v with bit h = 0, partner v ^ x): its top
+// bit is register bit l, the others the remaining register bits ascending.
+// An item is one or two strings (the sum and the difference over the top bit)
+// that share everything else: the part, the frequency w over the other bits,
+// the thread's frequency tau and z on the coset representatives.
+constexpr int kEvcRegPhases = 12;    // phases of one pass (shared-memory tables)
+constexpr int kEvcRegItems = 32;     // items of one phase (one bit each in the thread's sign word)
+struct EvcRegPhase {
+    uint32_t rmask, lanes;           // staged-index bits in registers and in the lane bits (phase_lanes)
+    int32_t g_begin, g_end, i_begin, i_end;
+};
+struct EvcRegGroup {
+    int32_t code;                    // h * 8 + l of x = bits h and l; 64 more when x is bit h alone
+    int32_t nre, nim, i_begin;       // items using Re, then those using Im
+};
+struct EvcRegItem {
+    uint64_t z;
+    uint32_t tau, w;
+    int32_t slot_sum, slot_dif;      // strings of the pass (relative), or -1
+    uint32_t neg;                    // bit 0: the sum's sign, bit 1: the difference's
+    uint32_t pad;
+};
+
 struct CosetPass {
     int32_t kl = 0, m = 0;
     uint64_t basis[kMaxSpan] = {};    // span vectors over bits >= kl, reduced
     int32_t pivot[kMaxSpan] = {};
     int32_t g_begin = 0, g_end = 0;   // groups
     int32_t s_begin = 0, s_end = 0;   // strings (slots), contiguous
+    // register phases (plan_evc_phases): they take the groups before g_reg
+    int32_t rp_begin = 0, rp_end = 0, g_reg = 0, s_reg = 0;
 };
 
 struct EvcPlan {
@@ -210,6 +239,9 @@ struct EvcPlan {
     std::vector<CosetPass> passes;
     std::vector<EvcGroup> groups;
     std::vector<EvcString> strings;   // slots
+    std::vector<EvcRegPhase> rphases;
+    std::vector<EvcRegGroup> rgroups;
+    std::vector<EvcRegItem> ritems;
     std::vector<int32_t> term_slot;   // per input term
     std::vector<int32_t> init_l2p, final_l2p;
     int32_t nqr() const {
@@ -249,6 +281,11 @@ std::string plan_evc(int n, int g, const sv_pauli *p, const double *coeffs, size
 // H|psi> grouping: one tile, no QR, cosets over all n bits.
 std::string plan_hpsi(int n, const sv_pauli *p, const double *coeffs, size_t nterms,
                       const PlanOptions &o, const std::vector<int32_t> &l2p, EvcPlan &out);
+// Register phases of the passes that stage 2^stage amplitudes and hold enough
+// groups of one or two staged bits (fewer than kXformMinStrings strings each).
+void plan_evc_phases(EvcPlan &P, int stage, int r);
+constexpr int kXformMinStrings = 16;  // groups with at least this many strings take the transform path
+constexpr int kEvcRegMinGroups = 6;
 // Write a bit permutation from layout `from` to layout `to` as at most two
 // sets of disjoint physical bit swaps (every permutation is a product of two
 // involutions).
