@@ -144,13 +144,13 @@ struct EvcEntry {
     EvcPlan plan;
     std::vector<CosetArgs> args;
     std::vector<CosetArgs> rest;    // what register phases leave of a pass (g_begin == g_end: nothing)
-    DevBuf groups, strings, term_slot, coeffs, rphases, rgroups, ritems;
+    DevBuf groups, strings, term_slot, coeffs, rphases, ritems;
     int nterms = 0;
     double plan_ms = 0;
     uint64_t last_use = 0;
     void release() {
         groups.release(); strings.release(); term_slot.release(); coeffs.release();
-        rphases.release(); rgroups.release(); ritems.release();
+        rphases.release(); ritems.release();
     }
 };
 
@@ -459,13 +459,6 @@ sv_status get_qsu(sv_handle *h, const sv_gate *gates, size_t m, size_t np, sv_sc
     return SV_OK;
 }
 
-int reg_groups(const EvcPlan &P, const CosetPass &cp) {
-    return P.rphases[cp.rp_end - 1].g_end - P.rphases[cp.rp_begin].g_begin;
-}
-int reg_items(const EvcPlan &P, const CosetPass &cp) {
-    return P.rphases[cp.rp_end - 1].i_end - P.rphases[cp.rp_begin].i_begin;
-}
-
 sv_status evc_entry_upload(sv_handle *h, EvcEntry *ent, const double *coeffs, size_t nterms) {
     std::vector<DevGroup> gs(ent->plan.groups.size());
     for (size_t i = 0; i < gs.size(); ++i) {
@@ -493,14 +486,11 @@ sv_status evc_entry_upload(sv_handle *h, EvcEntry *ent, const double *coeffs, si
     std::vector<double> c(coeffs, coeffs + nterms);
     SV_CK(upload(ent->coeffs, c, h->stream));
     SV_CK(upload(ent->rphases, ent->plan.rphases, h->stream));
-    SV_CK(upload(ent->rgroups, ent->plan.rgroups, h->stream));
     SV_CK(upload(ent->ritems, ent->plan.ritems, h->stream));
     for (auto &cp : ent->plan.passes) {
         ent->args.push_back(coset_args(h->n, cp));
         CosetArgs &a = ent->args.back();
-        if (cp.rp_end > cp.rp_begin &&
-            !evc_reg_fits(h->dt, a, cp.s_reg - cp.s_begin, cp.rp_end - cp.rp_begin, reg_groups(ent->plan, cp),
-                          reg_items(ent->plan, cp))) {
+        if (cp.rp_end > cp.rp_begin && !evc_reg_fits(h->dt, a, cp)) {
             cp.rp_end = cp.rp_begin;
             cp.g_reg = cp.g_begin;
             cp.s_reg = cp.s_begin;
@@ -714,10 +704,8 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
             // masks of one or two staged bits in register phases, the rest of the pass (if any) by the general kernels
             const CosetPass &cp = P.passes[pi];
             if (cp.rp_end > cp.rp_begin) {
-                SV_CK(launch_evc_reg(h->dt, h->stream, grid, h->psi, e->args[pi], e->rphases.as<EvcRegPhase>() + cp.rp_begin,
-                                     cp.rp_end - cp.rp_begin, e->rgroups.as<EvcRegGroup>(), reg_groups(P, cp),
-                                     e->ritems.as<EvcRegItem>(), reg_items(P, cp), cp.s_reg - cp.s_begin,
-                                     h->part.as<double>(), nslots));
+                SV_CK(launch_evc_reg(h->dt, h->stream, grid, h->psi, e->args[pi], cp, e->rphases.as<EvcRegPhase>(),
+                                     e->ritems.as<EvcRegItem>(), h->part.as<double>(), nslots));
                 if (e->rest[pi].g_begin == e->rest[pi].g_end) continue;
             }
             SV_CK(launch_evc_pass(h->dt, h->stream, grid, h->psi, e->rest[pi], e->groups.as<DevGroup>(),

@@ -2467,6 +2467,7 @@ __global__ void __launch_bounds__(512, 1) k_evc_pass(const Cx<R> *__restrict__ p
     coset_span(a, spanv);
     const ThreadCoset tc = thread_coset(a.kl);
     // the transform path needs complex64, 16 per thread, 512 threads, 8192 staged, the scratch
+    const bool use_d = sizeof(R) == 8 && EPT == 8 && blockDim.x == 512 && E == 4096u;
     bool use_x = false;
     float lsg[5] = {1.f, 1.f, 1.f, 1.f, 1.f};
     if constexpr (sizeof(R) == 4 && EPT == 16) {
@@ -2522,7 +2523,30 @@ __global__ void __launch_bounds__(512, 1) k_evc_pass(const Cx<R> *__restrict__ p
             const uint32_t e = threadIdx.x + j * blockDim.x;
             own[j] = e < E ? t[e] : mk<R>(0, 0);
         }
-        for (int gi = a.g_begin; gi < a.g_end; ++gi) {
+        if constexpr (sizeof(R) == 8 && EPT == 8) {
+            // FP64 runs at 1/64 of the FP32 rate: per string the products of the
+            // part it uses, one signed fold and its quarter of a four-value
+            // reduction (12.5 FP64 operations a thread instead of 26); the pairs'
+            // factor is applied at the end
+            for (int q0 = a.s_begin; use_d && q0 < a.s_end; q0 += 4) {
+                R c[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (q0 + k >= a.s_end) continue;
+                    const DevString S = strs[q0 + k];
+                    const PairSel ps = S.X ? pair_split(tc, S.X, a.kl, EPT) : PairSel{-1, 0, 1};
+                    const uint32_t code = (uint32_t)(ps.h + 1) | ((uint32_t)ps.s << 3) | ((uint32_t)(S.nY & 1) << 4);
+                    const R v = evc_fast<R, EPT, 9>(t, own, S.X, code, S.bz >> tc.ash);
+                    const int neg = (__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz) ^
+                                     (S.X ? ((S.nY == 1) | (S.nY == 2)) : 0)) & 1;
+                    c[k] = neg ? -v : v;
+                }
+                const R red = warp_sum4<R>(c[0], c[1], c[2], c[3]);
+                const int q = q0 + (lane >> 3);
+                if ((lane & 7) == 0 && q < a.s_end) acc[(q - a.s_begin) * nwarps + warp] += red;
+            }
+        }
+        for (int gi = use_d ? a.g_end : a.g_begin; gi < a.g_end; ++gi) {
             const DevGroup G = groups[gi];
             if constexpr (sizeof(R) == 4 && EPT == 16) {
                 const int K = G.s_end - G.s_begin;
@@ -2673,6 +2697,10 @@ __global__ void __launch_bounds__(512, 1) k_evc_pass(const Cx<R> *__restrict__ p
         if constexpr (sizeof(R) == 4) tsum = tot64[s];
         else
             for (int w = 0; w < nwarps; ++w) tsum += acc[s * nwarps + w];
+        if (use_d) {
+            const uint32_t X = strs[a.s_begin + s].X;
+            if (X) tsum *= (double)pair_split(tc, X, a.kl, EPT).fac;   // the same in every thread
+        }
         part[(size_t)blockIdx.x * part_stride + a.s_begin + s] = tsum;
     }
 }
@@ -3156,25 +3184,23 @@ __global__ void __launch_bounds__(1 << LOGNT, 1) k_evc_ring(const Cx<R> *__restr
 // their (phase, eighth of the coset) units without barriers; what remains per
 // string is its sign bit and its share of a four-value warp reduction.
 // n = 28, 4096 strings (16 passes): 106 -> see DESIGN.
-template <typename R> struct EvcVal;
-template <> struct EvcVal<float> { using T = unsigned long long; };   // packed halves of the products
-template <> struct EvcVal<double> { using T = double; };
-template <typename R> using EV = typename EvcVal<R>::T;
-
-template <bool IM> __device__ __forceinline__ unsigned long long ev_prod(unsigned long long v, unsigned long long u) {
-    if (!IM) return f2_mul(v, u);
-    const float2 h = f2_unpack(v);
-    return f2_mul(f2_pack(h.y, h.x), u);
+// Products and folds are scalar: packing two of them into f32x2 registers
+// halved the fold but cost more in moves.  The first product of a pair is
+// volatile: the compiler otherwise hoists the products that the codes of the
+// switch have in common, hundreds of them, and spills.
+__device__ __forceinline__ float ev_mul(float a, float b) {
+    float r;
+    asm volatile("mul.rn.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
 }
-template <bool IM> __device__ __forceinline__ double ev_prod(double2 v, double2 u) {
-    return IM ? v.x * u.y - v.y * u.x : v.x * u.x + v.y * u.y;
+__device__ __forceinline__ double ev_mul(double a, double b) {
+    double r;
+    asm volatile("mul.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
 }
-__device__ __forceinline__ unsigned long long ev_fold(unsigned long long s, unsigned long long b, unsigned long long a) {
-    return f2_fma(s, b, a);
+template <typename R, bool IM> __device__ __forceinline__ R ev_prod(Cx<R> v, Cx<R> u) {
+    return IM ? fma(v.x, u.y, -ev_mul(v.y, u.x)) : fma(v.x, u.x, ev_mul(v.y, u.y));
 }
-__device__ __forceinline__ double ev_fold(double s, double b, double a) { return fma(s, b, a); }
-template <bool IM> __device__ __forceinline__ float ev_end(unsigned long long r) { return f2_combine<IM>(r); }
-template <bool IM> __device__ __forceinline__ double ev_end(double r) { return r; }
 __device__ __forceinline__ float ev_sign(float v, uint32_t neg) {
     return __uint_as_float(__float_as_uint(v) ^ (neg << 31));
 }
@@ -3192,42 +3218,55 @@ __host__ __device__ constexpr int ev_elem(int p) {
     return v | (((p >> (RB - 2)) & 1) << L);
 }
 template <typename R, int RB, int H, int L, bool ONE, bool IM>
-__device__ __forceinline__ void ev_products(EV<R> *P, const RA<R> *x) {
+__device__ __forceinline__ void ev_products(R *P, const Cx<R> *x) {
     constexpr int XR = (1 << H) | (ONE ? 0 : 1 << L);
 #pragma unroll
     for (int p = 0; p < (1 << (RB - 1)); ++p) {
         const int v = ev_elem<RB, H, L>(p);
-        P[p] = ev_prod<IM>(x[v ^ XR], x[v]);
+        P[p] = ev_prod<R, IM>(x[v ^ XR], x[v]);
     }
 }
-template <typename R, int RB, bool IM>
-__device__ __forceinline__ void ev_group_products(EV<R> *P, const RA<R> *x, int code) {
-#define SV_EP(H, L)                                                                              \
-    case H * 8 + L: if constexpr (H < RB) ev_products<R, RB, H, L, false, IM>(P, x); break;
-#define SV_EO(H, L)                                                                              \
-    case 64 + H * 8 + L: if constexpr (H < RB) ev_products<R, RB, H, L, true, IM>(P, x); break;
+// products of one part of a group: code = 2 * (index of (h, l)) + (Im: 1)
+__host__ __device__ constexpr int ev_code(int h, int l, bool one) {
+    return one ? 10 + h : h * (h - 1) / 2 + l;
+}
+template <typename R, int RB>
+__device__ __forceinline__ void ev_group_products(R *P, const Cx<R> *x, uint32_t code) {
+#define SV_EP(H, L, ONE)                                                                         \
+    case 2 * ev_code(H, L, ONE): if constexpr (H < RB) ev_products<R, RB, H, L, ONE, false>(P, x); break; \
+    case 2 * ev_code(H, L, ONE) + 1: if constexpr (H < RB) ev_products<R, RB, H, L, ONE, true>(P, x); break;
     switch (code) {
-        SV_EP(1, 0) SV_EP(2, 0) SV_EP(2, 1) SV_EP(3, 0) SV_EP(3, 1) SV_EP(3, 2)
-        SV_EP(4, 0) SV_EP(4, 1) SV_EP(4, 2) SV_EP(4, 3)
-        SV_EO(0, 1) SV_EO(1, 0) SV_EO(2, 0) SV_EO(3, 0) SV_EO(4, 0)
+        SV_EP(1, 0, false) SV_EP(2, 0, false) SV_EP(2, 1, false) SV_EP(3, 0, false) SV_EP(3, 1, false)
+        SV_EP(3, 2, false) SV_EP(4, 0, false) SV_EP(4, 1, false) SV_EP(4, 2, false) SV_EP(4, 3, false)
+        SV_EP(0, 1, true) SV_EP(1, 0, true) SV_EP(2, 0, true) SV_EP(3, 0, true) SV_EP(4, 0, true)
     default: break;
     }
 #undef SV_EP
-#undef SV_EO
 }
 
-template <typename R> struct EvcItemS {
-    EV<R> lev[3];           // signs of the fold's levels
-    uint32_t slots, neg;    // sum slot | difference slot << 16 (0xFFFF: none)
+// Two values reduced over a warp: lanes 0..15 end with the total of v0, 16..31 of v1.
+template <typename R> __device__ __forceinline__ R warp_sum2(R v0, R v1) {
+    const bool hi = threadIdx.x & 16u;
+    R k = hi ? v1 : v0;
+    k += __shfl_xor_sync(0xffffffffu, hi ? v0 : v1, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    return k;
+}
+
+template <typename R> struct __align__(16) EvcItemS {   // 32 bytes, 48 for complex128
+    R lev[4];               // signs of the fold's levels
+    uint32_t slots;         // sum slot | difference slot << 16 (0xFFFF: none)
+    uint32_t ctl;           // bits 0, 1: signs of the two; bits 8..15: code; bit 16: the group's products change
 };
 template <typename R> __host__ __device__ constexpr int evc_reg_bits() { return sizeof(R) == 4 ? 5 : 4; }
 
 // Shared memory beyond the two staged cosets: span table, per string and
 // eighth a partial, FP64 totals (complex64), phases, groups, items.
 struct EvcRegLayout {
-    uint32_t span, acc, tot, phases, prb, pbase, tmask, groups, items, zs, total;
+    uint32_t span, acc, tot, phases, prb, pbase, tmask, items, zs, total;
 };
-__host__ __device__ inline EvcRegLayout evc_reg_layout(int m, int nslots, int nph, int ngr, int nit, int rbytes) {
+__host__ __device__ inline EvcRegLayout evc_reg_layout(int m, int nslots, int nph, int nit, int rbytes) {
     EvcRegLayout L;
     uint32_t o = 0;
     L.span = o;   o = align16u(o + (8u << m));
@@ -3237,8 +3276,7 @@ __host__ __device__ inline EvcRegLayout evc_reg_layout(int m, int nslots, int np
     L.prb = o;    o = align16u(o + 16u * (uint32_t)nph);
     L.pbase = o;  o = align16u(o + 512u * (uint32_t)nph);
     L.tmask = o;  o = align16u(o + 1024u * (uint32_t)nph);
-    L.groups = o; o = align16u(o + 16u * (uint32_t)ngr);
-    L.items = o;  o = align16u(o + 32u * (uint32_t)nit);
+    L.items = o;  o = align16u(o + (rbytes == 4 ? 32u : 48u) * (uint32_t)nit);
     L.zs = o;     o = align16u(o + 8u * (uint32_t)nit);
     L.total = o;
     return L;
@@ -3246,18 +3284,15 @@ __host__ __device__ inline EvcRegLayout evc_reg_layout(int m, int nslots, int np
 
 template <typename R>
 __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ psi, const CosetArgs a,
-                                                    const EvcRegPhase *__restrict__ phases, int nph,
-                                                    const EvcRegGroup *__restrict__ rgroups,
-                                                    const EvcRegItem *__restrict__ ritems, int nslots,
+                                                    const EvcRegPhase *__restrict__ phases, int nph, int nfirst,
+                                                    const EvcRegItem *__restrict__ ritems, int i0, int nit, int nslots,
                                                     double *__restrict__ part, int part_stride) {
     constexpr int RB = evc_reg_bits<R>(), V = 1 << RB, NP = V / 2, LOGE = RB + 8;
     constexpr uint32_t E = 1u << LOGE;
     extern __shared__ __align__(16) unsigned char smem[];
-    RA<R> *buf = reinterpret_cast<RA<R> *>(smem);
+    Cx<R> *buf = reinterpret_cast<Cx<R> *>(smem);
     unsigned char *sm = smem + 2 * (size_t)E * sizeof(Cx<R>);
-    const int g0 = phases[0].g_begin, i0 = phases[0].i_begin;
-    const int ngr = phases[nph - 1].g_end - g0, nit = phases[nph - 1].i_end - i0;
-    const EvcRegLayout L = evc_reg_layout(a.m, nslots, nph, ngr, nit, (int)sizeof(R));
+    const EvcRegLayout L = evc_reg_layout(a.m, nslots, nph, nit, (int)sizeof(R));
     uint64_t *spanv = reinterpret_cast<uint64_t *>(sm + L.span);
     R *acc = reinterpret_cast<R *>(sm + L.acc);
     double *tot64 = reinterpret_cast<double *>(sm + L.tot);
@@ -3265,10 +3300,9 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
     uint16_t *prb = reinterpret_cast<uint16_t *>(sm + L.prb);
     uint16_t *pbase = reinterpret_cast<uint16_t *>(sm + L.pbase);
     uint32_t *tmask = reinterpret_cast<uint32_t *>(sm + L.tmask);
-    EvcRegGroup *grs = reinterpret_cast<EvcRegGroup *>(sm + L.groups);
     EvcItemS<R> *its = reinterpret_cast<EvcItemS<R> *>(sm + L.items);
     uint64_t *zs = reinterpret_cast<uint64_t *>(sm + L.zs);
-    const int tid = threadIdx.x, NT = blockDim.x, warp = tid >> 5, lane = tid & 31, nwarps = NT >> 5;
+    const int tid = threadIdx.x, NT = blockDim.x, warp = tid >> 5, lane = tid & 31;
     for (int j = tid; j < nslots * 8; j += NT) acc[j] = 0;
     if constexpr (sizeof(R) == 4)
         for (int j = tid; j < nslots; j += NT) tot64[j] = 0.0;
@@ -3276,25 +3310,20 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
         EvcRegPhase F = phases[p];
         uint32_t rm = F.rmask;
         for (int i = 0; i < RB; ++i, rm &= rm - 1u) prb[p * 8 + i] = (uint16_t)swz_tile(rm & (0u - rm));
-        F.g_begin -= g0; F.g_end -= g0; F.i_begin -= i0; F.i_end -= i0;
+        F.i_begin -= i0; F.i_end -= i0;
         phs[p] = F;
-    }
-    for (int g = tid; g < ngr; g += NT) {
-        EvcRegGroup G = rgroups[g0 + g];
-        G.i_begin -= i0;
-        grs[g] = G;
     }
     for (int i = tid; i < nit; i += NT) {
         const EvcRegItem t = ritems[i0 + i];
         EvcItemS<R> s;
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
-            const float sg = ((t.w >> l) & 1u) ? -1.f : 1.f;
-            if constexpr (sizeof(R) == 4) s.lev[l] = f2_pack(sg, sg);
-            else s.lev[l] = (double)sg;
+            const R sg = ((t.w >> l) & 1u) ? (R)-1 : (R)1;
+            s.lev[l] = sg;
         }
+        s.lev[3] = 0;
         s.slots = (uint32_t)(t.slot_sum & 0xFFFF) | ((uint32_t)t.slot_dif << 16);
-        s.neg = t.neg;
+        s.ctl = t.ctl;
         its[i] = s;
         zs[i] = t.z;
     }
@@ -3314,7 +3343,7 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
     uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
     const uint32_t lowmask = (1u << a.kl) - 1u;
     constexpr uint32_t PER = 16 / sizeof(Cx<R>);
-    auto load = [&](RA<R> *dst, uint64_t rep) {
+    auto load = [&](Cx<R> *dst, uint64_t rep) {
         for (uint32_t q = tid; q < E / PER; q += (uint32_t)NT) {
             const uint32_t e = q * PER;
             cp_async16(dst + swz_tile(e), psi + (rep ^ spanv[e >> a.kl] ^ (e & lowmask)));
@@ -3330,15 +3359,17 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
     for (uint64_t it = 0; it < mine; ++it) {
         const uint64_t rep = rep_cur;
         rep_cur = walk_next(rep_cur, bw);
-        const RA<R> *t = buf + (it & 1) * E;
+        const Cx<R> *t = buf + (it & 1) * E;
         cp_async_wait1();
         __syncthreads();
-        for (int u = warp; u < nph * 8; u += nwarps) {
-            const int p = u >> 3, wt = u & 7, th = (p << 8) | (wt << 5) | lane;
+        // warps 0..7 take the first phases (split evenly by work), 8..15 the others
+        const int wt = warp & 7;
+        for (int p = warp < 8 ? 0 : nfirst, pe = warp < 8 ? nfirst : nph; p < pe; ++p) {
+            const int th = (p << 8) | (wt << 5) | lane;
             const EvcRegPhase F = phs[p];
             const bool zb = lane < F.i_end - F.i_begin && (__popcll(rep & zs[min(F.i_begin + lane, nit - 1)]) & 1);
             const uint32_t mask = tmask[th] ^ __ballot_sync(0xffffffffu, zb);
-            RA<R> x[V];
+            Cx<R> x[V];
             {
                 const uint4 r = *reinterpret_cast<const uint4 *>(prb + p * 8);
                 const uint32_t rb[5] = {r.x & 0xFFFFu, r.x >> 16, r.y & 0xFFFFu, r.y >> 16, r.z & 0xFFFFu};
@@ -3350,57 +3381,32 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
                 if (sizeof(R) == 4 && (F.rmask & 1u)) {
 #pragma unroll
                     for (int v = 0; v < V; v += 2) {
-                        const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(&t[idx[v]]);
-                        memcpy(&x[v], &w.x, 8);
-                        memcpy(&x[v + 1], &w.y, 8);
+                        const float4 w = *reinterpret_cast<const float4 *>(&t[idx[v]]);
+                        x[v] = mk<R>((R)w.x, (R)w.y);
+                        x[v + 1] = mk<R>((R)w.z, (R)w.w);
                     }
                 } else {
 #pragma unroll
                     for (int v = 0; v < V; ++v) x[v] = t[idx[v]];
                 }
             }
-            // results of two items are reduced together
-            R v0 = 0, v1 = 0;
-            uint32_t pend = 0xFFFFFFFFu;
-            auto flush = [&](R w0, R w1, uint32_t slots) {
-                const R red = warp_sum4<R>(v0, v1, w0, w1);
-                const uint32_t two = (lane & 16) ? slots : pend, sl = (lane & 8) ? two >> 16 : two & 0xFFFFu;
-                if ((lane & 7) == 0 && sl != 0xFFFFu) acc[sl * 8 + wt] += red;
-                pend = 0xFFFFFFFFu;
-            };
-            for (int g = F.g_begin; g < F.g_end; ++g) {
-                const EvcRegGroup G = grs[g];
+            R P[NP];
+            const EvcItemS<R> *ip = its + F.i_begin, *ie = its + F.i_end;
+            for (uint32_t sg = mask; ip < ie; ++ip, sg >>= 1) {
+                const EvcItemS<R> S = *ip;
+                if (S.ctl & 0x10000u) ev_group_products<R, RB>(P, x, (S.ctl >> 8) & 255u);
+                R f[NP / 2];
 #pragma unroll
-                for (int im = 0; im < 2; ++im) {
-                    const int n = im ? G.nim : G.nre, ib = G.i_begin + (im ? G.nre : 0);
-                    if (n == 0) continue;
-                    EV<R> P[NP];
-                    if (im) ev_group_products<R, RB, true>(P, x, G.code);
-                    else ev_group_products<R, RB, false>(P, x, G.code);
-                    for (int i = ib; i < ib + n; ++i) {
-                        const EvcItemS<R> S = its[i];
-                        EV<R> f[NP / 2];
+                for (int k = 0; k < NP / 2; ++k) f[k] = fma(S.lev[0], P[2 * k + 1], P[2 * k]);
 #pragma unroll
-                        for (int k = 0; k < NP / 2; ++k) f[k] = ev_fold(S.lev[0], P[2 * k + 1], P[2 * k]);
+                for (int l = 1, c = NP / 4; c >= 2; ++l, c >>= 1)
 #pragma unroll
-                        for (int l = 1, c = NP / 4; c >= 2; ++l, c >>= 1)
-#pragma unroll
-                            for (int k = 0; k < c; ++k) f[k] = ev_fold(S.lev[l], f[2 * k + 1], f[2 * k]);
-                        const R r0 = im ? ev_end<true>(f[0]) : ev_end<false>(f[0]);
-                        const R r1 = im ? ev_end<true>(f[1]) : ev_end<false>(f[1]);
-                        const uint32_t sg = (mask >> (i - F.i_begin)) & 1u;
-                        const R w0 = ev_sign(r0 + r1, sg ^ (S.neg & 1u)), w1 = ev_sign(r0 - r1, sg ^ (S.neg >> 1));
-                        if (pend == 0xFFFFFFFFu) {
-                            v0 = w0;
-                            v1 = w1;
-                            pend = S.slots;
-                        } else {
-                            flush(w0, w1, S.slots);
-                        }
-                    }
-                }
+                    for (int k = 0; k < c; ++k) f[k] = fma(S.lev[l], f[2 * k + 1], f[2 * k]);
+                const R red = warp_sum2<R>(ev_sign(f[0] + f[1], (sg ^ S.ctl) & 1u),
+                                           ev_sign(f[0] - f[1], (sg ^ (S.ctl >> 1)) & 1u));
+                const uint32_t sl = (lane & 16) ? S.slots >> 16 : S.slots & 0xFFFFu;
+                if ((lane & 15) == 0 && sl != 0xFFFFu) acc[sl * 8 + wt] += red;
             }
-            if (pend != 0xFFFFFFFFu) flush((R)0, (R)0, 0xFFFFFFFFu);
         }
         __syncthreads();
         if (it + 2 < mine) load(buf + (it & 1) * E, rep_pf);
@@ -3485,85 +3491,73 @@ __device__ __forceinline__ void hpsi_fast(Cx<R> *acc, const Cx<R> *t, uint32_t X
     }
 }
 
-// complex64, 16 amplitudes per thread (NT = 512, E = 8192): the signed
-// coefficient of element j is built along a Gray chain written out (each
-// one XOR from an earlier one), and the partner of element j is at byte
-// offset B ^ (j << 12) of the staged coset (B = (t ^ X) * 8) whose shared
-// address is sb.
-template <bool ODD>
-__device__ __forceinline__ void hpsi_gray16(float2 *acc, uint32_t sb, uint32_t B, uint32_t g0, uint32_t w) {
-    const uint32_t F0 = (w & 1u) << 31, F1 = (w & 2u) << 30, F2 = (w & 4u) << 29, F3 = (w & 8u) << 28;
-    const uint32_t g1 = g0 ^ F0, g2 = g0 ^ F1, g3 = g2 ^ F0, g4 = g0 ^ F2, g5 = g4 ^ F0, g6 = g4 ^ F1,
-                   g7 = g6 ^ F0, g8 = g0 ^ F3, g9 = g8 ^ F0, g10 = g8 ^ F1, g11 = g10 ^ F0, g12 = g8 ^ F2,
-                   g13 = g12 ^ F0, g14 = g12 ^ F1, g15 = g14 ^ F0;
-#define SV_HG(J)                                                                                 \
-    {                                                                                            \
-        const float2 v = lds_cx<float>(sb + (B ^ ((uint32_t)(J) << 12)));                        \
-        const float f = __uint_as_float(g##J);                                                   \
-        if (ODD) {                                                                               \
-            acc[J].x = fmaf(-f, v.y, acc[J].x);                                                  \
-            acc[J].y = fmaf(f, v.x, acc[J].y);                                                   \
-        } else {                                                                                 \
-            acc[J].x = fmaf(f, v.x, acc[J].x);                                                   \
-            acc[J].y = fmaf(f, v.y, acc[J].y);                                                   \
-        }                                                                                        \
-    }
-    SV_HG(0) SV_HG(1) SV_HG(2) SV_HG(3) SV_HG(4) SV_HG(5) SV_HG(6) SV_HG(7)
-    SV_HG(8) SV_HG(9) SV_HG(10) SV_HG(11) SV_HG(12) SV_HG(13) SV_HG(14) SV_HG(15)
-#undef SV_HG
+// complex64, 8192 staged, 512 threads: a thread holds the eight element pairs
+// e = 2 tid + 1024 j + {0, 1}, so that partners, old lambda and results move
+// by 16-byte accesses (half the address arithmetic and shared-memory
+// instructions of 16 single elements).  The partners of pair j are pair
+// (2 tid ^ X's thread bits) of row j ^ XR, swapped when X flips bit 0 (SW);
+// its shared address is one register plus an immediate (rows 4..7 from a
+// second base).  The signed coefficients of the 16 elements come from a Gray
+// chain (one XOR each): bit 0 of w is the sign of element bit 0, bits 1..3
+// those of j.
+template <int OFF> __device__ __forceinline__ float4 lds_f4_off(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4+%5];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr), "n"(OFF));
+    return v;
 }
-
-// hpsi_gray16 with the partner's row offset XH = (X >> 9) fixed at compile
-// time: the partner of element j is at Bl + ((j ^ XH) << 12), Bl = shared
-// address of the coset + (t ^ (X & 511)) * 8, so every load is one register
-// plus an immediate (rows 8..15 from Bl + 32 KiB, keeping immediates small).
-template <bool ODD, int XH>
-__device__ __forceinline__ void hpsi_row16(float2 *acc, uint32_t Bl, uint32_t g0, uint32_t w) {
+template <bool ODD>
+__device__ __forceinline__ void hpsi_add(float &ax, float &ay, uint32_t gu, float vx, float vy) {
+    const float f = __uint_as_float(gu);
+    if (ODD) {
+        ax = fmaf(-f, vy, ax);
+        ay = fmaf(f, vx, ay);
+    } else {
+        ax = fmaf(f, vx, ax);
+        ay = fmaf(f, vy, ay);
+    }
+}
+template <bool ODD, int XR, bool SW>
+__device__ __forceinline__ void hpsi_rows(float4 *acc, uint32_t Bl, uint32_t g0, uint32_t w) {
     const uint32_t Bh = Bl + 32768u;
     const uint32_t F0 = (w & 1u) << 31, F1 = (w & 2u) << 30, F2 = (w & 4u) << 29, F3 = (w & 8u) << 28;
-    const uint32_t g1 = g0 ^ F0, g2 = g0 ^ F1, g3 = g2 ^ F0, g4 = g0 ^ F2, g5 = g4 ^ F0, g6 = g4 ^ F1,
-                   g7 = g6 ^ F0, g8 = g0 ^ F3, g9 = g8 ^ F0, g10 = g8 ^ F1, g11 = g10 ^ F0, g12 = g8 ^ F2,
-                   g13 = g12 ^ F0, g14 = g12 ^ F1, g15 = g14 ^ F0;
+    const uint32_t h0 = g0, h1 = g0 ^ F1, h2 = g0 ^ F2, h3 = h2 ^ F1, h4 = g0 ^ F3, h5 = h4 ^ F1, h6 = h4 ^ F2,
+                   h7 = h6 ^ F1;
 #define SV_HR(J)                                                                                 \
     {                                                                                            \
-        const float2 v = (((J) ^ XH) < 8) ? lds_f2_off<(((J) ^ XH) & 7) << 12>(Bl)               \
-                                          : lds_f2_off<(((J) ^ XH) & 7) << 12>(Bh);              \
-        const float f = __uint_as_float(g##J);                                                   \
-        if (ODD) {                                                                               \
-            acc[J].x = fmaf(-f, v.y, acc[J].x);                                                  \
-            acc[J].y = fmaf(f, v.x, acc[J].y);                                                   \
-        } else {                                                                                 \
-            acc[J].x = fmaf(f, v.x, acc[J].x);                                                   \
-            acc[J].y = fmaf(f, v.y, acc[J].y);                                                   \
-        }                                                                                        \
+        const float4 v = (((J) ^ XR) < 4) ? lds_f4_off<(((J) ^ XR) & 3) << 13>(Bl)               \
+                                          : lds_f4_off<(((J) ^ XR) & 3) << 13>(Bh);              \
+        hpsi_add<ODD>(acc[J].x, acc[J].y, h##J, SW ? v.z : v.x, SW ? v.w : v.y);                 \
+        hpsi_add<ODD>(acc[J].z, acc[J].w, h##J ^ F0, SW ? v.x : v.z, SW ? v.y : v.w);            \
     }
     SV_HR(0) SV_HR(1) SV_HR(2) SV_HR(3) SV_HR(4) SV_HR(5) SV_HR(6) SV_HR(7)
-    SV_HR(8) SV_HR(9) SV_HR(10) SV_HR(11) SV_HR(12) SV_HR(13) SV_HR(14) SV_HR(15)
 #undef SV_HR
 }
 
-// Strings of one H|psi> pass staged once per launch (complex64, 16 amplitudes
-// per thread, 512 threads, at most kHpsiTab strings): per string the signed
-// coefficient, X (bit 31: nY odd), w and z; per thread the coset-independent
-// sign bits parity(l & z) ^ parity(a0 & bz) ^ nY of every string.  Per coset
-// one ballot gives parity(rep & z) of every string.
-constexpr int kHpsiTab = 32;
-// The same for passes with more strings (several per X/Y mask), in dynamic
-// shared memory; tz gives the coset-independent sign, parity(tid & tz).
+// A string of such a pass: coefficient with its constant sign, code (row XR |
+// swap << 3 | odd << 4) with X's thread bits above it, w as above, the
+// thread's sign mask (parity(2 tid & tz)) and z on the coset representatives.
 struct HpsiStr {
     uint64_t z;
-    uint32_t X, g, w, tz;
+    uint32_t g, xc, w, tz;
 };
 static_assert(sizeof(HpsiStr) == 24, "HpsiStr layout");
-struct HpsiTab {
-    uint64_t z[kHpsiTab];
-    uint32_t X[kHpsiTab], g[kHpsiTab], w[kHpsiTab];
-};
-
-__device__ __forceinline__ void hpsi_string(float2 *acc, uint32_t Xo, uint32_t g0, uint32_t w, uint32_t sb) {
-    const uint32_t Bl = sb + ((threadIdx.x ^ (Xo & 511u)) << 3);
-    switch (((Xo >> 9) & 15u) | ((Xo >> 31) << 4)) {
-#define SV_HC(C) case C: hpsi_row16<((C) >> 4) != 0, (C) & 15>(acc, Bl, g0, w); break;
+constexpr int kHpsiTab = 32;   // strings whose signs fit one word per thread
+__device__ __forceinline__ HpsiStr hpsi_str(const DevString &S, int kl) {
+    const uint32_t tau = (uint32_t)(S.z & ((1ull << kl) - 1ull)) | (S.bz << kl);
+    HpsiStr h;
+    h.z = S.z & ~((1ull << kl) - 1ull);
+    const bool neg = ((S.nY >> 1) ^ S.nY) & 1;      // i^nY (-1)^{|(b ^ x) & z|}: (-1)^{nY / 2} and (-1)^nY
+    h.g = __float_as_uint(neg ? -(float)S.coef : (float)S.coef);
+    h.xc = (S.X >> 10) | ((S.X & 1u) << 3) | ((uint32_t)(S.nY & 1) << 4) | ((S.X & 1022u) << 8);
+    h.w = (tau & 1u) | ((tau >> 10) << 1);
+    h.tz = tau & 1022u;
+    return h;
+}
+__device__ __forceinline__ void hpsi_string(float4 *acc, uint32_t xc, uint32_t g0, uint32_t w, uint32_t sb) {
+    const uint32_t Bl = sb + ((2u * threadIdx.x ^ (xc >> 8)) << 3);
+    switch (xc & 31u) {
+#define SV_HC(C) case C: hpsi_rows<((C) >> 4) != 0, (C) & 7, (((C) >> 3) & 1) != 0>(acc, Bl, g0, w); break;
         SV_HC(0) SV_HC(1) SV_HC(2) SV_HC(3) SV_HC(4) SV_HC(5) SV_HC(6) SV_HC(7)
         SV_HC(8) SV_HC(9) SV_HC(10) SV_HC(11) SV_HC(12) SV_HC(13) SV_HC(14) SV_HC(15)
         SV_HC(16) SV_HC(17) SV_HC(18) SV_HC(19) SV_HC(20) SV_HC(21) SV_HC(22) SV_HC(23)
@@ -3572,14 +3566,118 @@ __device__ __forceinline__ void hpsi_string(float2 *acc, uint32_t Xo, uint32_t g
     default: break;
     }
 }
-__device__ __forceinline__ void hpsi_tab_string(float2 *acc, const HpsiTab &T, int k, uint32_t sb, uint32_t bmask) {
-    hpsi_string(acc, T.X[k], T.g[k] ^ (((bmask >> k) & 1u) << 31), T.w[k], sb);
+
+// K-HPSI, complex64 with 8192 staged.  MANY: more than kHpsiTab strings (a
+// variant of its own: both string loops in one kernel cost the passes of few
+// strings 4 %); else one ballot per coset gives every string's sign.
+template <bool MANY>
+__global__ void __launch_bounds__(512, 1) k_hpsi_vec(const float2 *__restrict__ psi, float2 *__restrict__ lam,
+                                                     const CosetArgs a, const DevString *__restrict__ strs, int first,
+                                                     int last, double *__restrict__ epart) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr uint32_t E = 8192;
+    float2 *buf = reinterpret_cast<float2 *>(smem);
+    uint64_t *spanv = reinterpret_cast<uint64_t *>(buf + 2 * E);
+    HpsiStr *tab = reinterpret_cast<HpsiStr *>(spanv + (1u << a.m));
+    __shared__ double wsum[16];
+    coset_span(a, spanv);
+    const uint32_t lowmask = (1u << a.kl) - 1u;
+    const uint64_t ncos = 1ull << a.nfree;
+    const uint64_t mine = blockIdx.x < ncos ? (ncos - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    // coset representatives walked with masked additions: rep_cur of the
+    // current iteration, rep_pf of the one two ahead (the next copy issued)
+    const BitWalk bw = bit_walk(a.freeb, a.nfree, gridDim.x);
+    uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
+    const int ns = a.s_end - a.s_begin, lane = threadIdx.x & 31;
+    for (int q = (int)threadIdx.x; q < ns; q += 512) tab[q] = hpsi_str(strs[a.s_begin + q], a.kl);
+    __syncthreads();
+    uint32_t tmask = 0;
+    if constexpr (!MANY)
+        for (int q = 0; q < ns; ++q) tmask |= (uint32_t)(__popc(2u * threadIdx.x & tab[q].tz) & 1) << q;
+    // the thread's first pair and the distance of its rows in the span
+    const uint32_t e0 = 2u * threadIdx.x;
+    const uint64_t off0 = spanv[e0 >> a.kl] ^ (e0 & lowmask);
+    const uint64_t *row = spanv;                        // spanv[(1024 >> kl) j]: the span is linear
+    const uint32_t rstep = 1024u >> a.kl;
+    pdl_wait();
+    pdl_next();
+    for (uint64_t k = 0; k < 2; ++k) {
+        if (k < mine) load_coset<float>(buf + k * E, psi, rep_pf, spanv, a.kl, E);
+        cp_async_commit();
+        rep_pf = walk_next(rep_pf, bw);
+    }
+    double eacc = 0.0;
+    float eblk = 0.f;
+    for (uint64_t it = 0; it < mine; ++it) {
+        const uint64_t rep = rep_cur;
+        rep_cur = walk_next(rep_cur, bw);
+        const float2 *t = buf + (it & 1) * E;
+        float4 acc[8], old[8];
+        float2 *lp = lam;
+        const uint64_t base = rep ^ off0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            old[j] = acc[j];
+            if (!first) old[j] = *reinterpret_cast<const float4 *>(lp + (base ^ row[rstep * j]));
+        }
+        cp_async_wait1();
+        __syncthreads();
+        const uint32_t sb = smem_u32(t);
+        if constexpr (MANY) {
+            for (int k = 0; k < ns; ++k) {
+                const HpsiStr h = tab[k];
+                const uint32_t neg = (uint32_t)(__popcll(rep & h.z) ^ __popc(e0 & h.tz)) & 1u;
+                hpsi_string(acc, h.xc, h.g ^ (neg << 31), h.w, sb);
+            }
+        } else {
+            const uint32_t bmask =
+                tmask ^ __ballot_sync(0xffffffffu, lane < ns && (__popcll(rep & tab[min(lane, ns - 1)].z) & 1));
+            for (int k = 0; k < ns; ++k)
+                hpsi_string(acc, tab[k].xc, tab[k].g ^ (((bmask >> k) & 1u) << 31), tab[k].w, sb);
+        }
+        float eloc = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            acc[j].x += old[j].x;
+            acc[j].y += old[j].y;
+            acc[j].z += old[j].z;
+            acc[j].w += old[j].w;
+            *reinterpret_cast<float4 *>(lp + (base ^ row[rstep * j])) = acc[j];
+            if (last) {
+                const float4 p = *reinterpret_cast<const float4 *>(t + e0 + 1024 * j);
+                eloc += p.x * acc[j].x + p.y * acc[j].y;
+                eloc += p.z * acc[j].z + p.w * acc[j].w;
+            }
+        }
+        if (last) {
+            // FP32 over up to 64 cosets, then FP64 (1/64 of the FP32 rate here)
+            eblk += eloc;
+            if (((it + 1) & 63) == 0) {
+                eacc += (double)eblk;
+                eblk = 0.f;
+            }
+        }
+        __syncthreads();
+        if (it + 2 < mine) load_coset<float>(buf + (it & 1) * E, psi, rep_pf, spanv, a.kl, E);
+        cp_async_commit();
+        rep_pf = walk_next(rep_pf, bw);
+    }
+    if (last) {
+        double v = eacc + (double)eblk;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) wsum[threadIdx.x >> 5] = v;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double tsum = 0.0;
+            for (int w = 0; w < 16; ++w) tsum += wsum[w];
+            epart[blockIdx.x] = tsum;
+        }
+    }
 }
 
-// MANY: complex64 passes of 8192 staged with more than kHpsiTab strings (a
-// variant of its own: the two string loops in one kernel cost the passes of
-// few strings 4 %).
-template <typename R, int EPT, bool MANY>
+// K-HPSI, the other layouts
+template <typename R, int EPT>
 __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam,
                                                       const CosetArgs a, const DevGroup *__restrict__ groups,
                                                       const DevString *__restrict__ strs, int first, int last,
@@ -3589,7 +3687,6 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
     const uint32_t E = 1u << (a.kl + a.m);
     Cx<R> *buf = reinterpret_cast<Cx<R> *>(smem);
     uint64_t *spanv = reinterpret_cast<uint64_t *>(buf + 2 * E);
-    HpsiStr *many = reinterpret_cast<HpsiStr *>(spanv + (1u << a.m));   // passes of more than kHpsiTab strings
     __shared__ double wsum[32];
     coset_span(a, spanv);
     const ThreadCoset tc = thread_coset(a.kl);
@@ -3608,39 +3705,6 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
         cp_async_commit();
         rep_pf = walk_next(rep_pf, bw);
     }
-    // string table (complex64, 16 per thread, 512 threads, few strings)
-    __shared__ HpsiTab tabs;
-    int ns = 0;
-    uint32_t tmask = 0;
-    if constexpr (sizeof(R) == 4 && EPT == 16) {
-        if (fast) {
-            ns = a.s_end - a.s_begin;
-            for (int q = (int)threadIdx.x; q < ns; q += 512) {
-                const DevString S = strs[a.s_begin + q];
-                const float g = (S.nY & 2) ? -(float)S.coef : (float)S.coef;
-                if constexpr (MANY) {
-                    many[q].z = S.z;
-                    many[q].X = S.X | ((uint32_t)(S.nY & 1) << 31);
-                    many[q].g = __float_as_uint((S.nY & 1) ? -g : g);
-                    many[q].w = S.bz >> tc.ash;
-                    many[q].tz = (uint32_t)(S.z & ((1ull << a.kl) - 1ull)) | ((S.bz & ((1u << tc.ash) - 1u)) << a.kl);
-                } else {
-                    tabs.z[q] = S.z;
-                    tabs.X[q] = S.X | ((uint32_t)(S.nY & 1) << 31);
-                    tabs.g[q] = __float_as_uint(g);
-                    tabs.w[q] = S.bz >> tc.ash;
-                }
-            }
-            if constexpr (!MANY)
-                for (int q = 0; q < ns; ++q) {
-                    const DevString S = strs[a.s_begin + q];
-                    tmask |= (uint32_t)((__popcll(tc.l & S.z) ^ __popc(tc.a0 & S.bz) ^ S.nY) & 1) << q;
-                }
-            __syncthreads();
-        }
-    }
-    const bool tabbed = ns > 0;
-    const int lane = threadIdx.x & 31;
     double eacc = 0.0;
     R eblk = 0;
     for (uint64_t it = 0; it < mine; ++it) {
@@ -3657,23 +3721,7 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_pass(const Cx<R> *__restrict__ 
         }
         cp_async_wait1();
         __syncthreads();
-        if constexpr (sizeof(R) == 4 && EPT == 16 && MANY) {
-            const uint32_t sb = smem_u32(t);
-            for (int k = 0; k < ns; ++k) {
-                const HpsiStr h = many[k];
-                const uint32_t neg = (uint32_t)(__popcll(rep & h.z) ^ __popc(threadIdx.x & h.tz)) & 1u;
-                hpsi_string(reinterpret_cast<float2 *>(acc), h.X, h.g ^ (neg << 31), h.w, sb);
-            }
-        } else if constexpr (sizeof(R) == 4 && EPT == 16) {
-            if (tabbed) {
-                const bool pb = lane < ns && ((__popcll(rep & tabs.z[lane < ns ? lane : 0]) & 1) != 0);
-                const uint32_t bmask = tmask ^ __ballot_sync(0xffffffffu, pb);
-                const uint32_t sb = smem_u32(t);
-                for (int k = 0; k < ns; ++k)
-                    hpsi_tab_string(reinterpret_cast<float2 *>(acc), tabs, k, sb, bmask);
-            }
-        }
-        for (int gi = tabbed ? a.g_end : a.g_begin; gi < a.g_end; ++gi) {
+        for (int gi = a.g_begin; gi < a.g_end; ++gi) {
             const DevGroup G = groups[gi];
             for (int s = G.s_begin; s < G.s_end; ++s) {
                 const DevString S = strs[s];
@@ -4064,7 +4112,6 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
     R *coef = reinterpret_cast<R *>(opbase + (size_t)kBatchMaxOps * nwarps * 8);     // [2 * kBatchMaxGates]
     __shared__ int s_state;
     __shared__ double s_red[32];
-    __shared__ HpsiTab tabs;
     const size_t N = (size_t)1 << a.n;
     Cx<R> *psi = reinterpret_cast<Cx<R> *>(a.work) + (size_t)blockIdx.x * 2 * N;
     Cx<R> *lam = psi + N;
@@ -4146,31 +4193,19 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
             const ThreadCoset tc = thread_coset(C.kl);
             const uint64_t ncos = 1ull << C.nfree;
             const bool fast = (NT == 512) && (E == (uint32_t)EPT * 512u);
-            // the pass's strings staged once (as in k_hpsi_pass); the table of
-            // the previous pass is no longer read (barrier at its end)
-            int ns = 0;
-            uint32_t tmask = 0;
-            if constexpr (sizeof(R) == 4 && EPT == 16) {
-                if (fast) {
-                    for (int gi = C.g_begin; gi < C.g_end; ++gi) {
-                        const DevGroup G = a.groups[gi];
-                        for (int sidx = G.s_begin; sidx < G.s_end; ++sidx, ++ns) {
-                            if (ns >= kHpsiTab) continue;
-                            const DevString S = a.strs[sidx];
-                            tmask |= (uint32_t)((__popcll(tc.l & S.z) ^ __popc(tc.a0 & S.bz) ^ S.nY) & 1) << ns;
-                            if (threadIdx.x == 0) {
-                                const float gf = (S.nY & 2) ? -(float)S.coef : (float)S.coef;
-                                tabs.z[ns] = S.z;
-                                tabs.X[ns] = G.X | ((uint32_t)(S.nY & 1) << 31);
-                                tabs.g[ns] = __float_as_uint(gf);
-                                tabs.w[ns] = S.bz >> tc.ash;
-                            }
-                        }
-                    }
-                }
-            }
-            const bool tabbed = ns > 0 && ns <= kHpsiTab;
+            // complex64 with 8192 staged: element pairs and the pass's strings
+            // staged once, as in k_hpsi_vec; the table lies behind the gradient
+            // slots, which are half as wide as their room (and the previous
+            // pass's is no longer read: barrier at its end)
+            HpsiStr *tab = reinterpret_cast<HpsiStr *>(opbase + (size_t)kBatchMaxOps * nwarps * 4);
+            const int ns = C.s_end - C.s_begin;
+            const bool vec = sizeof(R) == 4 && EPT == 16 && fast && C.kl >= 1 && C.kl <= 10;
+            if (vec)
+                for (int q = (int)threadIdx.x; q < ns; q += NT) tab[q] = hpsi_str(a.strs[C.s_begin + q], C.kl);
             __syncthreads();
+            uint32_t tmask = 0;
+            if (vec && ns <= kHpsiTab)
+                for (int q = 0; q < ns; ++q) tmask |= (uint32_t)(__popc(2u * threadIdx.x & tab[q].tz) & 1) << q;
             // cosets alternate between the two buffers (lambda's buffer is free
             // here); the next one streams in while the current one is used
             load_coset<R>(tp, psi, deposit(0, C.freeb, C.nfree), spanv, C.kl, E);
@@ -4180,6 +4215,42 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
                 Cx<R> *cur = (ci & 1) ? tl : tp;
                 if (ci + 1 < ncos) load_coset<R>((ci & 1) ? tp : tl, psi, deposit(ci + 1, C.freeb, C.nfree), spanv, C.kl, E);
                 cp_async_commit();
+                R el = 0;
+                if constexpr (sizeof(R) == 4 && EPT == 16) {
+                    if (vec) {
+                        const uint32_t e0 = 2u * threadIdx.x, rstep = 1024u >> C.kl;
+                        float2 *lp = reinterpret_cast<float2 *>(lam);
+                        const uint64_t base = rep ^ spanv[e0 >> C.kl] ^ (e0 & lm);
+                        float4 acc[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            acc[j] = hp > 0 ? *reinterpret_cast<const float4 *>(lp + (base ^ spanv[rstep * j]))
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+                        cp_async_wait1();
+                        __syncthreads();
+                        const uint32_t sb = smem_u32(cur);
+                        uint32_t bmask = 0;
+                        if (ns <= kHpsiTab)
+                            bmask = tmask ^ __ballot_sync(0xffffffffu, lane < ns && (__popcll(rep & tab[min(lane, ns - 1)].z) & 1));
+                        for (int k = 0; k < ns; ++k) {
+                            const HpsiStr h = tab[k];
+                            const uint32_t neg = ns <= kHpsiTab
+                                                     ? (bmask >> k) & 1u
+                                                     : (uint32_t)(__popcll(rep & h.z) ^ __popc(e0 & h.tz)) & 1u;
+                            hpsi_string(acc, h.xc, h.g ^ (neg << 31), h.w, sb);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            *reinterpret_cast<float4 *>(lp + (base ^ spanv[rstep * j])) = acc[j];
+                            const float4 p = *reinterpret_cast<const float4 *>(cur + e0 + 1024 * j);
+                            el += p.x * acc[j].x + p.y * acc[j].y;
+                            el += p.z * acc[j].z + p.w * acc[j].w;
+                        }
+                        if (hp == a.nhpass - 1) eacc += (double)el;
+                        __syncthreads();
+                        continue;
+                    }
+                }
                 Cx<R> acc[EPT];
 #pragma unroll
                 for (int j = 0; j < EPT; ++j) {
@@ -4189,33 +4260,12 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
                 }
                 cp_async_wait1();
                 __syncthreads();
-                if constexpr (sizeof(R) == 4 && EPT == 16) {
-                    if (tabbed) {
-                        const bool pb = lane < ns && ((__popcll(rep & tabs.z[lane < ns ? lane : 0]) & 1) != 0);
-                        const uint32_t bmask = tmask ^ __ballot_sync(0xffffffffu, pb);
-                        const uint32_t sb = smem_u32(cur);
-                        for (int k = 0; k < ns; ++k)
-                            hpsi_tab_string(reinterpret_cast<float2 *>(acc), tabs, k, sb, bmask);
-                    }
-                }
-                for (int gi = tabbed ? C.g_end : C.g_begin; gi < C.g_end; ++gi) {
+                for (int gi = C.g_begin; gi < C.g_end; ++gi) {
                     const DevGroup G = a.groups[gi];
                     for (int s = G.s_begin; s < G.s_end; ++s) {
                         const DevString S = a.strs[s];
                         const int base = (__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz) ^ S.nY) & 1;
                         const R g = (S.nY & 2) ? -(R)S.coef : (R)S.coef;
-                        if constexpr (sizeof(R) == 4 && EPT == 16) {
-                            if (fast) {
-                                const uint32_t g0 = __float_as_uint((float)g) ^ ((uint32_t)base << 31);
-                                const uint32_t B = (threadIdx.x ^ G.X) * 8u;
-                                const uint32_t sb = smem_u32(cur);
-                                if (S.nY & 1)
-                                    hpsi_gray16<true>(reinterpret_cast<float2 *>(acc), sb, B, g0, S.bz >> tc.ash);
-                                else
-                                    hpsi_gray16<false>(reinterpret_cast<float2 *>(acc), sb, B, g0, S.bz >> tc.ash);
-                                continue;
-                            }
-                        }
                         const uint32_t jm = walsh_mask(S.bz >> tc.ash);
                         if (fast) {
                             const uint32_t sm = base ? ~jm : jm;
@@ -4228,7 +4278,6 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
                         }
                     }
                 }
-                R el = 0;
 #pragma unroll
                 for (int j = 0; j < EPT; ++j) {
                     const uint32_t e = threadIdx.x + j * NT;
@@ -4815,27 +4864,32 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
     return cudaGetLastError();
 }
 
-bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, int nslots, int nph, int ngroups, int nitems) {
+bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, const CosetPass &cp) {
+    const int nph = cp.rp_end - cp.rp_begin, nitems = cp.ri_end - cp.ri_begin;
+    const int nslots = cp.s_reg - cp.s_begin;
     const size_t es = dt == SV_C64 ? 8 : 16;
     const int rb = dt == SV_C64 ? 5 : 4;
     if (a.kl + a.m != rb + 8 || a.kl < 1) return false;
-    return 2 * (es << (rb + 8)) + evc_reg_layout(a.m, nslots, nph, ngroups, nitems, (int)es / 2).total <=
+    return 2 * (es << (rb + 8)) + evc_reg_layout(a.m, nslots, nph, nitems, (int)es / 2).total <=
            (size_t)smem_optin();
 }
 
 cudaError_t launch_evc_reg(sv_dtype dt, cudaStream_t st, int grid, const void *psi, const CosetArgs &a,
-                           const EvcRegPhase *phases, int nph, const EvcRegGroup *rgroups, int ngroups,
-                           const EvcRegItem *ritems, int nitems, int nslots, double *part, int part_stride) {
+                           const CosetPass &cp, const EvcRegPhase *phases, const EvcRegItem *ritems,
+                           double *part, int part_stride) {
     const size_t es = dt == SV_C64 ? 8 : 16;
-    const size_t sm = 2 * (es << (a.kl + a.m)) + evc_reg_layout(a.m, nslots, nph, ngroups, nitems, (int)es / 2).total;
+    const int nph = cp.rp_end - cp.rp_begin, nit = cp.ri_end - cp.ri_begin;
+    const int nslots = cp.s_reg - cp.s_begin;
+    const size_t sm = 2 * (es << (a.kl + a.m)) + evc_reg_layout(a.m, nslots, nph, nit, (int)es / 2).total;
+    phases += cp.rp_begin;
     if (dt == SV_C64) {
         allow_smem(k_evc_reg<float>, sm);
-        return launch(k_evc_reg<float>, grid, 512, sm, st, (const float2 *)psi, a, phases, nph, rgroups, ritems, nslots,
-                      part, part_stride);
+        return launch(k_evc_reg<float>, grid, 512, sm, st, (const float2 *)psi, a, phases, nph, cp.rp_first,
+                      ritems, cp.ri_begin, nit, nslots, part, part_stride);
     }
     allow_smem(k_evc_reg<double>, sm);
-    return launch(k_evc_reg<double>, grid, 512, sm, st, (const double2 *)psi, a, phases, nph, rgroups, ritems, nslots,
-                  part, part_stride);
+    return launch(k_evc_reg<double>, grid, 512, sm, st, (const double2 *)psi, a, phases, nph, cp.rp_first,
+                  ritems, cp.ri_begin, nit, nslots, part, part_stride);
 }
 
 cudaError_t launch_evc_pass(sv_dtype dt, cudaStream_t st, int grid, const void *psi, const CosetArgs &a,
@@ -4850,24 +4904,31 @@ cudaError_t hpsi_dispatch(cudaStream_t st, int grid, const void *psi, void *lam,
                           const DevGroup *groups, const DevString *strs, int first, int last, double *epart,
                           int *status, long long limit) {
     const int E = 1 << (a.kl + a.m);
-    const size_t sm = 2 * (size_t)E * sizeof(Cx<R>) + ((size_t)1 << a.m) * 8 +
-                      (a.s_end - a.s_begin > kHpsiTab ? (size_t)(a.s_end - a.s_begin) * sizeof(HpsiStr) : 0);
+    const size_t sm = 2 * (size_t)E * sizeof(Cx<R>) + ((size_t)1 << a.m) * 8;
     // a multiple of the run length, at least one warp, at most 512
     const int threads = std::max(std::max(32, 1 << a.kl), std::min(E, 512));
     const int ept = std::max(1, E / threads);
-    // eight strings or so per pass are random masks, hundreds Jordan-Wigner ones
     if constexpr (sizeof(R) == 4) {
-        if (ept == 16 && threads == 512 && a.s_end - a.s_begin > kHpsiTab) {
-            allow_smem(k_hpsi_pass<R, 16, true>, sm);
-            return launch(k_hpsi_pass<R, 16, true>, grid, threads, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, groups,
-                          strs, first, last, epart, status, limit);
+        // runs of at least a pair, at most a row (1024 elements)
+        if (E == 8192 && a.kl >= 1 && a.kl <= 10) {
+            const int ns = a.s_end - a.s_begin;
+            const size_t smv = sm + (size_t)ns * sizeof(HpsiStr);
+            // about eight strings a pass are random masks, hundreds Jordan-Wigner ones
+            if (ns > kHpsiTab) {
+                allow_smem(k_hpsi_vec<true>, smv);
+                return launch(k_hpsi_vec<true>, grid, 512, smv, st, (const float2 *)psi, (float2 *)lam, a, strs, first,
+                              last, epart);
+            }
+            allow_smem(k_hpsi_vec<false>, smv);
+            return launch(k_hpsi_vec<false>, grid, 512, smv, st, (const float2 *)psi, (float2 *)lam, a, strs, first,
+                          last, epart);
         }
     }
 #define SV_HPSI_CASE(N)                                                                                      \
     case N:                                                                                                  \
-        allow_smem(k_hpsi_pass<R, N, false>, sm);                                                            \
-        return launch(k_hpsi_pass<R, N, false>, grid, threads, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a,  \
-                      groups, strs, first, last, epart, status, limit);
+        allow_smem(k_hpsi_pass<R, N>, sm);                                                                   \
+        return launch(k_hpsi_pass<R, N>, grid, threads, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, groups, \
+                      strs, first, last, epart, status, limit);
     switch (ept) {
         SV_HPSI_CASE(1)
         SV_HPSI_CASE(2)

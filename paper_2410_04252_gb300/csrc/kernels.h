@@ -129,12 +129,10 @@ cudaError_t launch_evc_pass(sv_dtype dt, cudaStream_t st, int grid, const void *
 cudaError_t launch_hpsi_pass(sv_dtype dt, cudaStream_t st, int grid, const void *psi, void *lam,
                              const CosetArgs &a, const DevGroup *groups, const DevString *strs,
                              int first, int last, double *epart, int *status, long long limit);
-// Register phases of an expectation pass (plan_evc_phases): nslots strings
-// from a.s_begin; ngroups and nitems count those of the nph phases.
-bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, int nslots, int nph, int ngroups, int nitems);
+// Register phases of an expectation pass (plan_evc_phases).
+bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, const CosetPass &cp);
 cudaError_t launch_evc_reg(sv_dtype dt, cudaStream_t st, int grid, const void *psi, const CosetArgs &a,
-                           const EvcRegPhase *phases, int nph, const EvcRegGroup *rgroups, int ngroups,
-                           const EvcRegItem *ritems, int nitems, int nslots, double *part, int part_stride);
+                           const CosetPass &cp, const EvcRegPhase *phases, const EvcRegItem *ritems, double *part, int part_stride);
 // Few cosets (coset_slices_pay): several CTAs share a coset.  Expectation:
 // part rows are the 2^nfree cosets; H|psi>: *rows energy partials.
 bool coset_slices_pay(sv_dtype dt, const CosetArgs &a);

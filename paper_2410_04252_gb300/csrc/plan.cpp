@@ -1138,7 +1138,7 @@ void plan_evc_phases(EvcPlan &P, int stage, int r) {
         uint64_t piv = 0;
         for (int j = 0; j < cp.m; ++j) piv |= bit(cp.pivot[j]);
         const uint64_t freemask = ~(piv | (bit(cp.kl) - 1));
-        const size_t np0 = P.rphases.size(), ng0 = P.rgroups.size(), ni0 = P.ritems.size();
+        const size_t np0 = P.rphases.size(), ni0 = P.ritems.size();
         std::vector<char> done(ge - cp.g_begin, 0);
         int left = ge - cp.g_begin;
         bool fits = true;
@@ -1170,17 +1170,14 @@ void plan_evc_phases(EvcPlan &P, int stage, int r) {
             EvcRegPhase F;
             F.rmask = rm;
             F.lanes = phase_lanes(rm, stage);
-            F.g_begin = (int32_t)P.rgroups.size();
             F.i_begin = (int32_t)P.ritems.size();
             auto reg = [&](int t) { return popc(rm & ((1u << t) - 1u)); };
             for (size_t i = 0; i < done.size(); ++i) {
                 const EvcGroup &G = P.groups[cp.g_begin + i];
                 if (done[i] || (G.X & ~rm)) continue;
                 const int hb = hibit(G.X), lbit = popc(G.X) == 2 ? lobit(G.X) : lobit(rm & ~G.X);
-                EvcRegGroup rg;
-                rg.code = reg(hb) * 8 + reg(lbit) + (popc(G.X) == 2 ? 0 : 64);
-                rg.i_begin = (int32_t)P.ritems.size();
-                int cnt[2] = {0, 0};
+                const int h = reg(hb), l = reg(lbit);
+                const uint32_t code = 2u * (uint32_t)(popc(G.X) == 2 ? h * (h - 1) / 2 + l : 10 + h);
                 std::vector<EvcRegItem> its[2];
                 for (int q = G.s_begin; q < G.s_end; ++q) {
                     const EvcString &S = P.strings[q];
@@ -1199,34 +1196,47 @@ void plan_evc_phases(EvcPlan &P, int stage, int r) {
                             break;
                         }
                     if (!hit) {
-                        its[part].push_back(EvcRegItem{S.z & freemask, tau & ~rm, w, -1, -1, 0u, 0u});
+                        its[part].push_back(EvcRegItem{S.z & freemask, tau & ~rm, w, -1, -1, (code + (uint32_t)part) << 8, 0u});
                         hit = &its[part].back();
                     }
                     (dif ? hit->slot_dif : hit->slot_sum) = q - cp.s_begin;
-                    hit->neg |= neg << dif;
+                    hit->ctl |= neg << dif;
                 }
-                cnt[0] = (int)its[0].size();
-                cnt[1] = (int)its[1].size();
-                if ((int)P.ritems.size() - F.i_begin + cnt[0] + cnt[1] > kEvcRegItems) continue;   // a later phase's
-                for (auto &v : its) P.ritems.insert(P.ritems.end(), v.begin(), v.end());
-                rg.nre = cnt[0];
-                rg.nim = cnt[1];
-                P.rgroups.push_back(rg);
+                if (P.ritems.size() - F.i_begin + its[0].size() + its[1].size() > (size_t)kEvcRegItems)
+                    continue;   // a later phase's
+                for (auto &v : its) {
+                    if (!v.empty()) v[0].ctl |= 0x10000u;
+                    P.ritems.insert(P.ritems.end(), v.begin(), v.end());
+                }
                 done[i] = 1;
                 --left;
             }
-            F.g_end = (int32_t)P.rgroups.size();
             F.i_end = (int32_t)P.ritems.size();
             P.rphases.push_back(F);
             if (P.rphases.size() - np0 > (size_t)kEvcRegPhases) fits = false;
         }
         if (!fits) {
             P.rphases.resize(np0);
-            P.rgroups.resize(ng0);
             P.ritems.resize(ni0);
             continue;
         }
         cp.rp_end = (int32_t)P.rphases.size();
+        cp.ri_begin = (int32_t)ni0;
+        cp.ri_end = (int32_t)P.ritems.size();
+        // two halves of about the same work: the largest phase left to the half
+        // with less so far (a gather weighs about an item and a half)
+        auto work = [&](const EvcRegPhase &F) { return 3 + 2 * (F.i_end - F.i_begin); };
+        std::vector<EvcRegPhase> all(P.rphases.begin() + np0, P.rphases.end()), half[2];
+        std::stable_sort(all.begin(), all.end(), [&](const EvcRegPhase &x, const EvcRegPhase &y) { return work(x) > work(y); });
+        int64_t sum[2] = {0, 0};
+        for (auto &F : all) {
+            const int k = sum[1] < sum[0];
+            half[k].push_back(F);
+            sum[k] += work(F);
+        }
+        std::copy(half[0].begin(), half[0].end(), P.rphases.begin() + np0);
+        std::copy(half[1].begin(), half[1].end(), P.rphases.begin() + np0 + half[0].size());
+        cp.rp_first = (int32_t)half[0].size();
         cp.g_reg = ge;
         cp.s_reg = ge < cp.g_end ? P.groups[ge].s_begin : cp.s_end;
     }

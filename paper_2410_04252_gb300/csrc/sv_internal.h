@@ -206,17 +206,14 @@ constexpr int kEvcRegPhases = 12;    // phases of one pass (shared-memory tables
 constexpr int kEvcRegItems = 32;     // items of one phase (one bit each in the thread's sign word)
 struct EvcRegPhase {
     uint32_t rmask, lanes;           // staged-index bits in registers and in the lane bits (phase_lanes)
-    int32_t g_begin, g_end, i_begin, i_end;
-};
-struct EvcRegGroup {
-    int32_t code;                    // h * 8 + l of x = bits h and l; 64 more when x is bit h alone
-    int32_t nre, nim, i_begin;       // items using Re, then those using Im
+    int32_t i_begin, i_end;
 };
 struct EvcRegItem {
     uint64_t z;
     uint32_t tau, w;
     int32_t slot_sum, slot_dif;      // strings of the pass (relative), or -1
-    uint32_t neg;                    // bit 0: the sum's sign, bit 1: the difference's
+    uint32_t ctl;                    // bits 0, 1: signs of the sum and the difference; bits 8..15: pair code (2 *
+                                     // place of (h, l), plus 1 for Im); bit 16: first item of its group and part
     uint32_t pad;
 };
 
@@ -227,7 +224,9 @@ struct CosetPass {
     int32_t g_begin = 0, g_end = 0;   // groups
     int32_t s_begin = 0, s_end = 0;   // strings (slots), contiguous
     // register phases (plan_evc_phases): they take the groups before g_reg
-    int32_t rp_begin = 0, rp_end = 0, g_reg = 0, s_reg = 0;
+    // (half of the warps run phases [rp_begin, rp_begin + rp_first), the others the rest)
+    int32_t rp_begin = 0, rp_end = 0, rp_first = 0, g_reg = 0, s_reg = 0;
+    int32_t ri_begin = 0, ri_end = 0;
 };
 
 struct EvcPlan {
@@ -240,7 +239,6 @@ struct EvcPlan {
     std::vector<EvcGroup> groups;
     std::vector<EvcString> strings;   // slots
     std::vector<EvcRegPhase> rphases;
-    std::vector<EvcRegGroup> rgroups;
     std::vector<EvcRegItem> ritems;
     std::vector<int32_t> term_slot;   // per input term
     std::vector<int32_t> init_l2p, final_l2p;
