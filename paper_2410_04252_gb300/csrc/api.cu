@@ -144,13 +144,13 @@ struct EvcEntry {
     EvcPlan plan;
     std::vector<CosetArgs> args;
     std::vector<CosetArgs> rest;    // what register phases leave of a pass (g_begin == g_end: nothing)
-    DevBuf groups, strings, term_slot, coeffs, rphases, ritems;
+    DevBuf groups, strings, term_slot, coeffs, rphases, ritems, uitems;
     int nterms = 0;
     double plan_ms = 0;
     uint64_t last_use = 0;
     void release() {
         groups.release(); strings.release(); term_slot.release(); coeffs.release();
-        rphases.release(); ritems.release();
+        rphases.release(); ritems.release(); uitems.release();
     }
 };
 
@@ -487,10 +487,12 @@ sv_status evc_entry_upload(sv_handle *h, EvcEntry *ent, const double *coeffs, si
     SV_CK(upload(ent->coeffs, c, h->stream));
     SV_CK(upload(ent->rphases, ent->plan.rphases, h->stream));
     SV_CK(upload(ent->ritems, ent->plan.ritems, h->stream));
+    SV_CK(upload(ent->uitems, ent->plan.uitems, h->stream));
     for (auto &cp : ent->plan.passes) {
         ent->args.push_back(coset_args(h->n, cp));
         CosetArgs &a = ent->args.back();
-        if (cp.rp_end > cp.rp_begin && !evc_reg_fits(h->dt, a, cp)) {
+        // single strings keep per-thread partials in the kernels for few strings
+        if (cp.rp_end > cp.rp_begin && (a.few || !evc_reg_fits(h->dt, a, cp))) {
             cp.rp_end = cp.rp_begin;
             cp.g_reg = cp.g_begin;
             cp.s_reg = cp.s_begin;
@@ -554,6 +556,7 @@ sv_status get_evc(sv_handle *h, const sv_pauli *p, const double *c, size_t nterm
     if (!hpsi) {
         const int r = h->dt == SV_C64 ? 5 : 4;
         plan_evc_phases(ent->plan, r + 8, r);
+        if (h->dt == SV_C64) plan_evc_units(ent->plan);
     }
     ent->plan_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     ent->key = key;
@@ -703,6 +706,11 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
             }
             // masks of one or two staged bits in register phases, the rest of the pass (if any) by the general kernels
             const CosetPass &cp = P.passes[pi];
+            if (cp.u_end > cp.u_begin) {
+                SV_CK(launch_evc_unit(h->stream, grid, h->psi, e->args[pi], cp, e->uitems.as<EvcUnitItem>(),
+                                      h->part.as<double>(), nslots));
+                continue;
+            }
             if (cp.rp_end > cp.rp_begin) {
                 SV_CK(launch_evc_reg(h->dt, h->stream, grid, h->psi, e->args[pi], cp, e->rphases.as<EvcRegPhase>(),
                                      e->ritems.as<EvcRegItem>(), h->part.as<double>(), nslots));

@@ -3226,15 +3226,14 @@ __device__ __forceinline__ void ev_products(R *P, const Cx<R> *x) {
         P[p] = ev_prod<R, IM>(x[v ^ XR], x[v]);
     }
 }
-// products of one part of a group: code = 2 * (index of (h, l)) + (Im: 1)
+// products of one part of a group: code = index of (h, l)
 __host__ __device__ constexpr int ev_code(int h, int l, bool one) {
     return one ? 10 + h : h * (h - 1) / 2 + l;
 }
-template <typename R, int RB>
+template <typename R, int RB, bool IM>
 __device__ __forceinline__ void ev_group_products(R *P, const Cx<R> *x, uint32_t code) {
 #define SV_EP(H, L, ONE)                                                                         \
-    case 2 * ev_code(H, L, ONE): if constexpr (H < RB) ev_products<R, RB, H, L, ONE, false>(P, x); break; \
-    case 2 * ev_code(H, L, ONE) + 1: if constexpr (H < RB) ev_products<R, RB, H, L, ONE, true>(P, x); break;
+    case ev_code(H, L, ONE): if constexpr (H < RB) ev_products<R, RB, H, L, ONE, IM>(P, x); break;
     switch (code) {
         SV_EP(1, 0, false) SV_EP(2, 0, false) SV_EP(2, 1, false) SV_EP(3, 0, false) SV_EP(3, 1, false)
         SV_EP(3, 2, false) SV_EP(4, 0, false) SV_EP(4, 1, false) SV_EP(4, 2, false) SV_EP(4, 3, false)
@@ -3244,20 +3243,28 @@ __device__ __forceinline__ void ev_group_products(R *P, const Cx<R> *x, uint32_t
 #undef SV_EP
 }
 
-// Two values reduced over a warp: lanes 0..15 end with the total of v0, 16..31 of v1.
-template <typename R> __device__ __forceinline__ R warp_sum2(R v0, R v1) {
-    const bool hi = threadIdx.x & 16u;
-    R k = hi ? v1 : v0;
-    k += __shfl_xor_sync(0xffffffffu, hi ? v0 : v1, 16);
+// the signed sum of the pair terms over all but the pair index's top bit: r[0], r[1]
+template <typename R, int NP>
+__device__ __forceinline__ void ev_fold(const R *P, const R *lev, R *r) {
+    R f[NP / 2];
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-    return k;
+    for (int k = 0; k < NP / 2; ++k) f[k] = fma(lev[0], P[2 * k + 1], P[2 * k]);
+#pragma unroll
+    for (int l = 1, c = NP / 4; c >= 2; ++l, c >>= 1)
+#pragma unroll
+        for (int k = 0; k < c; ++k) f[k] = fma(lev[l], f[2 * k + 1], f[2 * k]);
+    r[0] = f[0];
+    r[1] = f[1];
 }
 
-template <typename R> struct __align__(16) EvcItemS {   // 32 bytes, 48 for complex128
-    R lev[4];               // signs of the fold's levels
-    uint32_t slots;         // sum slot | difference slot << 16 (0xFFFF: none)
-    uint32_t ctl;           // bits 0, 1: signs of the two; bits 8..15: code; bit 16: the group's products change
+// An item of the Re part and one of the Im part of the same group (either may
+// be missing), so that four results share one warp reduction.
+template <typename R> struct __align__(16) EvcItemS {   // 48 bytes, 64 for complex128
+    R lev[2][3];            // signs of the folds' levels
+    uint32_t slots[2];      // per part: sum slot | difference slot << 16 (0xFFFF: none)
+    uint32_t ctl;           // bits 0..3: signs of the four; bits 8..15: code; bit 16, 17: the part is there;
+                            // bit 18: the group's Re products are still held
+    uint32_t pad;
 };
 template <typename R> __host__ __device__ constexpr int evc_reg_bits() { return sizeof(R) == 4 ? 5 : 4; }
 
@@ -3276,8 +3283,8 @@ __host__ __device__ inline EvcRegLayout evc_reg_layout(int m, int nslots, int np
     L.prb = o;    o = align16u(o + 16u * (uint32_t)nph);
     L.pbase = o;  o = align16u(o + 512u * (uint32_t)nph);
     L.tmask = o;  o = align16u(o + 1024u * (uint32_t)nph);
-    L.items = o;  o = align16u(o + (rbytes == 4 ? 32u : 48u) * (uint32_t)nit);
-    L.zs = o;     o = align16u(o + 8u * (uint32_t)nit);
+    L.items = o;  o = align16u(o + (rbytes == 4 ? 48u : 64u) * (uint32_t)nit);
+    L.zs = o;     o = align16u(o + 16u * (uint32_t)nit);
     L.total = o;
     return L;
 }
@@ -3317,15 +3324,16 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
         const EvcRegItem t = ritems[i0 + i];
         EvcItemS<R> s;
 #pragma unroll
-        for (int l = 0; l < 3; ++l) {
-            const R sg = ((t.w >> l) & 1u) ? (R)-1 : (R)1;
-            s.lev[l] = sg;
+        for (int p = 0; p < 2; ++p) {
+#pragma unroll
+            for (int l = 0; l < 3; ++l) s.lev[p][l] = ((t.w[p] >> l) & 1u) ? (R)-1 : (R)1;
+            s.slots[p] = (uint32_t)(t.slot_sum[p] & 0xFFFF) | ((uint32_t)t.slot_dif[p] << 16);
         }
-        s.lev[3] = 0;
-        s.slots = (uint32_t)(t.slot_sum & 0xFFFF) | ((uint32_t)t.slot_dif << 16);
         s.ctl = t.ctl;
+        s.pad = 0;
         its[i] = s;
-        zs[i] = t.z;
+        zs[2 * i] = t.z[0];
+        zs[2 * i + 1] = t.z[1];
     }
     coset_span(a, spanv);
     for (int e = tid; e < nph * 256; e += NT) {
@@ -3333,7 +3341,8 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
         const uint32_t base = phase_base(F.rmask, F.lanes, LOGE, (uint32_t)e & 255u);
         uint32_t m = 0;
         for (int i = F.i_begin; i < F.i_end; ++i)
-            m |= (uint32_t)(__popc(base & ritems[i0 + i].tau) & 1) << (i - F.i_begin);
+            for (int p = 0; p < 2; ++p)
+                m |= (uint32_t)(__popc(base & ritems[i0 + i].tau[p]) & 1) << (2 * (i - F.i_begin) + p);
         pbase[e] = (uint16_t)base;
         tmask[e] = m;
     }
@@ -3341,13 +3350,16 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
     const uint64_t mine = blockIdx.x < ncos ? (ncos - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
     const BitWalk bw = bit_walk(a.freeb, a.nfree, gridDim.x);
     uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
-    const uint32_t lowmask = (1u << a.kl) - 1u;
-    constexpr uint32_t PER = 16 / sizeof(Cx<R>);
+    // copies: piece i of a thread is element e0 + i ROW; the span and the
+    // swizzle are linear, so its places are the thread's XOR a constant
+    // (runs of 2^kl elements, kl at most log2(ROW): host rule)
+    constexpr uint32_t PER = 16 / sizeof(Cx<R>), ROW = 512u * PER;
+    const uint32_t e0 = (uint32_t)tid * PER, slot0 = swz_tile(e0), rstep = ROW >> a.kl;
+    const uint64_t off0 = spanv[e0 >> a.kl] ^ (e0 & ((1u << a.kl) - 1u));
     auto load = [&](Cx<R> *dst, uint64_t rep) {
-        for (uint32_t q = tid; q < E / PER; q += (uint32_t)NT) {
-            const uint32_t e = q * PER;
-            cp_async16(dst + swz_tile(e), psi + (rep ^ spanv[e >> a.kl] ^ (e & lowmask)));
-        }
+#pragma unroll
+        for (uint32_t i = 0; i < E / ROW; ++i)
+            cp_async16(dst + (slot0 ^ swz_tile(i * ROW)), psi + (rep ^ off0 ^ spanv[rstep * i]));
     };
     pdl_wait();
     pdl_next();
@@ -3367,7 +3379,7 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
         for (int p = warp < 8 ? 0 : nfirst, pe = warp < 8 ? nfirst : nph; p < pe; ++p) {
             const int th = (p << 8) | (wt << 5) | lane;
             const EvcRegPhase F = phs[p];
-            const bool zb = lane < F.i_end - F.i_begin && (__popcll(rep & zs[min(F.i_begin + lane, nit - 1)]) & 1);
+            const bool zb = lane < 2 * (F.i_end - F.i_begin) && (__popcll(rep & zs[min(2 * F.i_begin + lane, 2 * nit - 1)]) & 1);
             const uint32_t mask = tmask[th] ^ __ballot_sync(0xffffffffu, zb);
             Cx<R> x[V];
             {
@@ -3392,20 +3404,24 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
             }
             R P[NP];
             const EvcItemS<R> *ip = its + F.i_begin, *ie = its + F.i_end;
-            for (uint32_t sg = mask; ip < ie; ++ip, sg >>= 1) {
+            for (uint32_t sg = mask; ip < ie; ++ip, sg >>= 2) {
                 const EvcItemS<R> S = *ip;
-                if (S.ctl & 0x10000u) ev_group_products<R, RB>(P, x, (S.ctl >> 8) & 255u);
-                R f[NP / 2];
-#pragma unroll
-                for (int k = 0; k < NP / 2; ++k) f[k] = fma(S.lev[0], P[2 * k + 1], P[2 * k]);
-#pragma unroll
-                for (int l = 1, c = NP / 4; c >= 2; ++l, c >>= 1)
-#pragma unroll
-                    for (int k = 0; k < c; ++k) f[k] = fma(S.lev[l], f[2 * k + 1], f[2 * k]);
-                const R red = warp_sum2<R>(ev_sign(f[0] + f[1], (sg ^ S.ctl) & 1u),
-                                           ev_sign(f[0] - f[1], (sg ^ (S.ctl >> 1)) & 1u));
-                const uint32_t sl = (lane & 16) ? S.slots >> 16 : S.slots & 0xFFFFu;
-                if ((lane & 15) == 0 && sl != 0xFFFFu) acc[sl * 8 + wt] += red;
+                R r[2] = {0, 0}, q[2] = {0, 0};
+                if (S.ctl & 0x10000u) {
+                    if (!(S.ctl & 0x40000u)) ev_group_products<R, RB, false>(P, x, (S.ctl >> 8) & 255u);
+                    ev_fold<R, NP>(P, S.lev[0], r);
+                }
+                if (S.ctl & 0x20000u) {
+                    ev_group_products<R, RB, true>(P, x, (S.ctl >> 8) & 255u);
+                    ev_fold<R, NP>(P, S.lev[1], q);
+                }
+                const uint32_t s1 = sg >> 1;
+                const R red = warp_sum4<R>(ev_sign(r[0] + r[1], (sg ^ S.ctl) & 1u),
+                                           ev_sign(r[0] - r[1], (sg ^ (S.ctl >> 1)) & 1u),
+                                           ev_sign(q[0] + q[1], (s1 ^ (S.ctl >> 2)) & 1u),
+                                           ev_sign(q[0] - q[1], (s1 ^ (S.ctl >> 3)) & 1u));
+                const uint32_t two = (lane & 16) ? S.slots[1] : S.slots[0], sl = (lane & 8) ? two >> 16 : two & 0xFFFFu;
+                if ((lane & 7) == 0 && sl != 0xFFFFu) acc[sl * 8 + wt] += red;
             }
         }
         __syncthreads();
@@ -3435,6 +3451,168 @@ __global__ void __launch_bounds__(512, 1) k_evc_reg(const Cx<R> *__restrict__ ps
         else
             for (int w = 0; w < 8; ++w) s += acc[q * 8 + w];
         part[(size_t)blockIdx.x * part_stride + a.s_begin + q] = 2.0 * s;
+    }
+}
+
+// ---- K-EVC of few strings whose masks are the span basis (complex64) ----
+// Random strings: one per mask, eight or so in a span.  The ring kernel read
+// each string's partners from shared memory (with the copies 3072 clocks of
+// its bandwidth per 64 KB coset at eight strings, as much as HBM needs, and
+// the two did not overlap: 0.6 of HBM).  With the masks as the span's basis a
+// string's pairs differ in one span bit, so the warps that hold that bit in
+// registers need no partner reads: two gathers of the coset in all.  Partials
+// stay per thread, FP32 over at most 64 cosets, then FP64.
+template <int H, bool B0, bool IM>
+__device__ __forceinline__ void eu_products(float *P, const float2 *x) {
+    constexpr int XR = (1 << H) | (B0 ? 1 : 0);
+#pragma unroll
+    for (int p = 0; p < 16; ++p) {
+        const int v = ((p >> H) << (H + 1)) | (p & ((1 << H) - 1));
+        P[p] = ev_prod<float, IM>(x[v ^ XR], x[v]);
+    }
+}
+struct __align__(16) EvcUnitS {
+    float lev[4];
+    uint32_t code, sX;       // sX: swizzled slot of X
+    float last;              // code 16, 17: the fifth sign
+    float fac;               // 2 when each pair is taken once
+};
+
+__global__ void __launch_bounds__(512, 1) k_evc_unit(const float2 *__restrict__ psi, const CosetArgs a,
+                                                     const EvcUnitItem *__restrict__ items, int u_mid, int nu,
+                                                     double *__restrict__ part, int part_stride) {
+    constexpr uint32_t E = 8192, KL = kEvcUnitRun;
+    extern __shared__ __align__(16) unsigned char smem[];
+    float2 *buf = reinterpret_cast<float2 *>(smem);
+    uint64_t *spanv = reinterpret_cast<uint64_t *>(buf + 3 * E);
+    float *acc = reinterpret_cast<float *>(spanv + (1u << kEvcUnitSpan));      // [string of the half][thread]
+    __shared__ EvcUnitS its[2 * kEvcUnitMax];
+    __shared__ uint64_t zs[2 * kEvcUnitMax];
+    __shared__ double wsum[kEvcUnitMax][16];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = warp >> 3;
+    const int ub = half ? u_mid : 0, n = half ? nu - u_mid : u_mid;
+    for (int i = tid; i < nu; i += 512) {
+        const EvcUnitItem t = items[i];
+        EvcUnitS s;
+#pragma unroll
+        for (int l = 0; l < 4; ++l) s.lev[l] = ((t.w >> l) & 1u) ? -1.f : 1.f;
+        s.code = t.code;
+        s.sX = swz_tile(t.X);
+        s.last = ((t.w >> 4) & 1u) ? -1.f : 1.f;
+        s.fac = t.code < 16u ? 2.f : 1.f;
+        its[i] = s;
+        zs[i] = t.z;
+    }
+    coset_span(a, spanv);
+    // the half's registers: bit 0 and its four span bits
+    const uint32_t rmask = 1u | (15u << (KL + 4 * half));
+    uint32_t rest = (uint32_t)(tid & 255), base = 0;
+    // lanes: run bits 1..4 and the lowest span bit of the other half (their
+    // slots differ in bits 1..3, so 16-byte gathers are conflict-free)
+    for (uint32_t m = (E - 1u) & ~rmask; m; m &= m - 1u, rest >>= 1)
+        if (rest & 1u) base |= m & (0u - m);
+    uint32_t tmask = 0;
+    for (int i = 0; i < n; ++i) {
+        const EvcUnitItem t = items[ub + i];
+        tmask |= (((uint32_t)__popc(base & t.tau) ^ t.neg) & 1u) << i;
+        acc[i * 512 + tid] = 0.f;
+    }
+    for (int j = tid; j < kEvcUnitMax * 16; j += 512) wsum[j / 16][j % 16] = 0.0;
+    const uint32_t sbase = swz_tile(base);
+    uint32_t rb[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) rb[i] = swz_tile(1u << (KL + 4 * half + i));
+    const uint64_t ncos = 1ull << a.nfree;
+    const uint64_t mine = blockIdx.x < ncos ? (ncos - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    const BitWalk bw = bit_walk(a.freeb, a.nfree, gridDim.x);
+    uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
+    const uint32_t e0 = 2u * (uint32_t)tid, slot0 = swz_tile(e0);
+    const uint64_t off0 = spanv[e0 >> KL] ^ (e0 & ((1u << KL) - 1u));
+    auto load = [&](float2 *dst, uint64_t rep) {
+#pragma unroll
+        for (uint32_t i = 0; i < 8; ++i)
+            cp_async16(dst + (slot0 ^ swz_tile(i * 1024u)), psi + (rep ^ off0 ^ spanv[(1024u >> KL) * i]));
+    };
+    __syncthreads();
+    pdl_wait();
+    pdl_next();
+    for (uint64_t k = 0; k < 2; ++k) {
+        if (k < mine) load(buf + k * E, rep_pf);
+        cp_async_commit();
+        rep_pf = walk_next(rep_pf, bw);
+    }
+    for (uint64_t it = 0; it < mine; ++it) {
+        const uint64_t rep = rep_cur;
+        rep_cur = walk_next(rep_cur, bw);
+        cp_async_wait1();
+        __syncthreads();
+        // coset it + 2 into the buffer of coset it - 1 (every thread is past it)
+        if (it + 2 < mine) load(buf + ((it + 2) % 3) * E, rep_pf);
+        cp_async_commit();
+        rep_pf = walk_next(rep_pf, bw);
+        const float2 *t = buf + (it % 3) * E;
+        const uint32_t mask = tmask ^ __ballot_sync(0xffffffffu, lane < n && (__popcll(rep & zs[min(ub + lane, nu - 1)]) & 1));
+        float2 x[32];
+        uint32_t idx[16];
+        idx[0] = sbase;
+#pragma unroll
+        for (int v = 1; v < 16; ++v) idx[v] = idx[v & (v - 1)] ^ rb[(v & 1) ? 0 : (v & 2) ? 1 : (v & 4) ? 2 : 3];
+#pragma unroll
+        for (int v = 0; v < 16; ++v) {
+            const float4 w = *reinterpret_cast<const float4 *>(&t[idx[v]]);
+            x[2 * v] = make_float2(w.x, w.y);
+            x[2 * v + 1] = make_float2(w.z, w.w);
+        }
+        for (int i = 0; i < n; ++i) {
+            const EvcUnitS S = its[ub + i];
+            float P[16];
+            switch (S.code) {
+#define SV_EU(H)                                                                                 \
+    case 4 * (H - 1): eu_products<H, false, false>(P, x); break;                                 \
+    case 4 * (H - 1) + 1: eu_products<H, false, true>(P, x); break;                              \
+    case 4 * (H - 1) + 2: eu_products<H, true, false>(P, x); break;                              \
+    case 4 * (H - 1) + 3: eu_products<H, true, true>(P, x); break;
+                SV_EU(1) SV_EU(2) SV_EU(3) SV_EU(4)
+#undef SV_EU
+            default: {
+                // partners from shared memory, every element; the register
+                // bits' signs: pairs (v, v + 16) fold into P by the fifth
+                const uint32_t sx = S.sX;
+                const bool im = S.code & 1u;
+#pragma unroll
+                for (int v = 0; v < 16; ++v) {
+                    const uint32_t lo = idx[v >> 1] ^ (uint32_t)(v & 1), hi = idx[(v + 16) >> 1] ^ (uint32_t)(v & 1);
+                    const float2 a0 = t[lo ^ sx], a1 = t[hi ^ sx];
+                    const float p0 = im ? a0.x * x[v].y - a0.y * x[v].x : a0.x * x[v].x + a0.y * x[v].y;
+                    const float p1 = im ? a1.x * x[v + 16].y - a1.y * x[v + 16].x
+                                        : a1.x * x[v + 16].x + a1.y * x[v + 16].y;
+                    P[v] = fmaf(S.last, p1, p0);
+                }
+                break;
+            }
+            }
+            float r[2];
+            ev_fold<float, 16>(P, S.lev, r);
+            const float v = fmaf(S.lev[3], r[1], r[0]);
+            acc[i * 512 + tid] += ev_sign(v, (mask >> i) & 1u);
+        }
+        if ((it & 63) == 63 || it + 1 == mine) {
+            // flush: FP64 warp sums into the per-warp slots (fixed order)
+            for (int i = 0; i < n; ++i) {
+                double v = (double)acc[i * 512 + tid] * (double)its[ub + i].fac;
+                acc[i * 512 + tid] = 0.f;
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane == 0) wsum[i][warp] += v;
+            }
+        }
+    }
+    cp_async_wait0();
+    __syncthreads();
+    if (tid < nu) {
+        const bool second = tid >= u_mid;
+        double s = 0.0;
+        for (int w = 0; w < 8; ++w) s += wsum[second ? tid - u_mid : tid][second ? 8 + w : w];
+        part[(size_t)blockIdx.x * part_stride + a.s_begin + items[tid].slot] = s;
     }
 }
 
@@ -3599,10 +3777,14 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_vec(const float2 *__restrict__ 
     const uint64_t off0 = spanv[e0 >> a.kl] ^ (e0 & lowmask);
     const uint64_t *row = spanv;                        // spanv[(1024 >> kl) j]: the span is linear
     const uint32_t rstep = 1024u >> a.kl;
+    auto load = [&](float2 *dst, uint64_t rep) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) cp_async16(dst + e0 + 1024 * j, psi + (rep ^ off0 ^ row[rstep * j]));
+    };
     pdl_wait();
     pdl_next();
     for (uint64_t k = 0; k < 2; ++k) {
-        if (k < mine) load_coset<float>(buf + k * E, psi, rep_pf, spanv, a.kl, E);
+        if (k < mine) load(buf + k * E, rep_pf);
         cp_async_commit();
         rep_pf = walk_next(rep_pf, bw);
     }
@@ -3659,7 +3841,7 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_vec(const float2 *__restrict__ 
             }
         }
         __syncthreads();
-        if (it + 2 < mine) load_coset<float>(buf + (it & 1) * E, psi, rep_pf, spanv, a.kl, E);
+        if (it + 2 < mine) load(buf + (it & 1) * E, rep_pf);
         cp_async_commit();
         rep_pf = walk_next(rep_pf, bw);
     }
@@ -4869,9 +5051,17 @@ bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, const CosetPass &cp) {
     const int nslots = cp.s_reg - cp.s_begin;
     const size_t es = dt == SV_C64 ? 8 : 16;
     const int rb = dt == SV_C64 ? 5 : 4;
-    if (a.kl + a.m != rb + 8 || a.kl < 1) return false;
+    if (a.kl + a.m != rb + 8 || a.kl < 1 || a.kl > 9) return false;
     return 2 * (es << (rb + 8)) + evc_reg_layout(a.m, nslots, nph, nitems, (int)es / 2).total <=
            (size_t)smem_optin();
+}
+
+cudaError_t launch_evc_unit(cudaStream_t st, int grid, const void *psi, const CosetArgs &a, const CosetPass &cp,
+                            const EvcUnitItem *uitems, double *part, int part_stride) {
+    const size_t sm = 3 * 8192 * sizeof(float2) + ((size_t)8 << kEvcUnitSpan) + kEvcUnitMax * 512 * sizeof(float);
+    allow_smem(k_evc_unit, sm);
+    return launch(k_evc_unit, grid, 512, sm, st, (const float2 *)psi, a, uitems + cp.u_begin, cp.u_mid - cp.u_begin,
+                  cp.u_end - cp.u_begin, part, part_stride);
 }
 
 cudaError_t launch_evc_reg(sv_dtype dt, cudaStream_t st, int grid, const void *psi, const CosetArgs &a,

@@ -133,6 +133,9 @@ cudaError_t launch_hpsi_pass(sv_dtype dt, cudaStream_t st, int grid, const void 
 bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, const CosetPass &cp);
 cudaError_t launch_evc_reg(sv_dtype dt, cudaStream_t st, int grid, const void *psi, const CosetArgs &a,
                            const CosetPass &cp, const EvcRegPhase *phases, const EvcRegItem *ritems, double *part, int part_stride);
+// Few strings with their masks as the span basis (plan_evc_units; complex64).
+cudaError_t launch_evc_unit(cudaStream_t st, int grid, const void *psi, const CosetArgs &a, const CosetPass &cp,
+                            const EvcUnitItem *uitems, double *part, int part_stride);
 // Few cosets (coset_slices_pay): several CTAs share a coset.  Expectation:
 // part rows are the 2^nfree cosets; H|psi>: *rows energy partials.
 bool coset_slices_pay(sv_dtype dt, const CosetArgs &a);

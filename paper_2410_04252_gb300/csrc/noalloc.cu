@@ -106,6 +106,7 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
     sv::EvcPlan P;
     std::string err = sv::plan_hpsi(n, paulis, coeffs, nterms, po, l2p, P);
     if (!err.empty()) return noalloc_fail(SV_EINVAL, "plan: " + err);
+    if (dt == SV_C64) sv::plan_evc_units(P);
     const int nslots = (int)P.strings.size();
     const int ngroups = (int)P.groups.size();
 
@@ -134,6 +135,8 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
     size_t off = 0;
     sv::DevGroup *d_groups = (sv::DevGroup *)(p + off); off = align256(off + ngroups * sizeof(sv::DevGroup));
     sv::DevString *d_strs = (sv::DevString *)(p + off); off = align256(off + nslots * sizeof(sv::DevString));
+    sv::EvcUnitItem *d_units = (sv::EvcUnitItem *)(p + off);
+    off = align256(off + P.uitems.size() * sizeof(sv::EvcUnitItem));
     int32_t *d_term_slot = (int32_t *)(p + off); off = align256(off + nterms * sizeof(int32_t));
     double *d_coeffs = (double *)(p + off); off = align256(off + nterms * sizeof(double));
     double *d_slotval = (double *)(p + off); off = align256(off + nslots * sizeof(double));
@@ -188,8 +191,15 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
     NOALLOC_CK(cudaMemcpyAsync(d_strs, ss.data(), nslots * sizeof(sv::DevString), cudaMemcpyHostToDevice, st));
     NOALLOC_CK(cudaMemcpyAsync(d_term_slot, P.term_slot.data(), nterms * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     NOALLOC_CK(cudaMemcpyAsync(d_coeffs, coeffs, nterms * sizeof(double), cudaMemcpyHostToDevice, st));
-    for (auto &a : args) {
-        if (slices)
+    if (!P.uitems.empty())
+        NOALLOC_CK(cudaMemcpyAsync(d_units, P.uitems.data(), P.uitems.size() * sizeof(sv::EvcUnitItem),
+                                   cudaMemcpyHostToDevice, st));
+    for (size_t i = 0; i < args.size(); ++i) {
+        const sv::CosetArgs &a = args[i];
+        const sv::CosetPass &cp = P.passes[i];
+        if (!slices && cp.u_end > cp.u_begin)
+            NOALLOC_CK(sv::launch_evc_unit(st, grid, state, a, cp, d_units, d_part, nslots));
+        else if (slices)
             NOALLOC_CK(sv::launch_evc_slice(dt, st, state, a, d_strs, d_part, nslots));
         else
             NOALLOC_CK(sv::launch_evc_pass(dt, st, grid, state, a, d_groups, d_strs, d_part, nslots, d_status,

@@ -894,15 +894,48 @@ void plan_cosets(EvcPlan &P, std::vector<GroupIn> &groups, int klmin, int mmax, 
         cp.kl = kl;
         cp.m = (int32_t)sp.basis.size();
         for (int j = 0; j < cp.m; ++j) { cp.basis[j] = sp.basis[j]; cp.pivot[j] = sp.pivot[j]; }
+        // Few single strings: the basis becomes their own masks (with the run
+        // bits above bit 0, which keeps 16-byte copies whole), as far as they
+        // are independent, so that a string flips one span bit.  Same span,
+        // same representatives (pivots).
+        bool units = !useA && kl >= 1 && sel.size() <= 16;
+        for (int32_t gi : sel) units = units && groups[gi].zs.size() == 1;
+        if (units) {
+            Span ind;
+            std::vector<uint64_t> own;
+            auto take = [&](uint64_t v) {
+                if ((int)own.size() < cp.m && ind.reduce(v & ~lowmask)) {
+                    ind.insert(v & ~lowmask);
+                    own.push_back(v);
+                }
+            };
+            for (int32_t gi : sel) take(groups[gi].x & ~1ull);
+            for (uint64_t v : sp.basis) take(v);
+            for (int j = 0; j < cp.m; ++j) cp.basis[j] = own[j];
+        }
         cp.g_begin = (int32_t)P.groups.size();
         cp.s_begin = (int32_t)P.strings.size();
         std::vector<char> in(groups.size(), 0);
+        // coordinates over cp.basis: its high parts, reduced, with the members each is made of
+        std::vector<uint64_t> red;
+        std::vector<uint32_t> made;
+        for (int j = 0; j < cp.m; ++j) {
+            uint64_t v = cp.basis[j] & ~lowmask;
+            uint32_t c = 1u << j;
+            for (size_t i = 0; i < red.size(); ++i)
+                if (v >> hibit(red[i]) & 1) { v ^= red[i]; c ^= made[i]; }
+            red.push_back(v);
+            made.push_back(c);
+        }
         auto offset = [&](const GroupIn &G) {
+            uint64_t h = G.x & ~lowmask;
             uint32_t c = 0;
-            const uint64_t h = G.x & ~lowmask;
+            for (size_t i = 0; i < red.size(); ++i)
+                if (h >> hibit(red[i]) & 1) { h ^= red[i]; c ^= made[i]; }
+            uint64_t low = G.x & lowmask;
             for (int j = 0; j < cp.m; ++j)
-                if (h >> sp.pivot[j] & 1) c |= 1u << j;
-            return (c << kl) | (uint32_t)(G.x & lowmask);
+                if (c >> j & 1u) low ^= cp.basis[j] & lowmask;
+            return (c << kl) | (uint32_t)low;
         };
         // the groups that register phases could take first (plan_evc_phases)
         std::vector<int32_t> ordered(sel);
@@ -924,7 +957,7 @@ void plan_cosets(EvcPlan &P, std::vector<GroupIn> &groups, int klmin, int mmax, 
                 es.coef = G.zs[s].second;
                 es.bz = 0;
                 for (int j = 0; j < cp.m; ++j)
-                    if (popc(sp.basis[j] & es.z) & 1) es.bz |= 1u << j;
+                    if (popc(cp.basis[j] & es.z) & 1) es.bz |= 1u << j;
                 for (int32_t t : G.terms[s]) P.term_slot[t] = (int32_t)P.strings.size();
                 P.strings.push_back(es);
             }
@@ -1177,8 +1210,14 @@ void plan_evc_phases(EvcPlan &P, int stage, int r) {
                 if (done[i] || (G.X & ~rm)) continue;
                 const int hb = hibit(G.X), lbit = popc(G.X) == 2 ? lobit(G.X) : lobit(rm & ~G.X);
                 const int h = reg(hb), l = reg(lbit);
-                const uint32_t code = 2u * (uint32_t)(popc(G.X) == 2 ? h * (h - 1) / 2 + l : 10 + h);
-                std::vector<EvcRegItem> its[2];
+                const uint32_t code = (uint32_t)(popc(G.X) == 2 ? h * (h - 1) / 2 + l : 10 + h);
+                struct One {
+                    uint64_t z;
+                    uint32_t tau, w;
+                    int32_t slot_sum, slot_dif;
+                    uint32_t neg;
+                };
+                std::vector<One> its[2];
                 for (int q = G.s_begin; q < G.s_end; ++q) {
                     const EvcString &S = P.strings[q];
                     const uint32_t tau = (uint32_t)(S.z & (bit(cp.kl) - 1)) | (S.bz << cp.kl);
@@ -1188,7 +1227,7 @@ void plan_evc_phases(EvcPlan &P, int stage, int r) {
                         if (tau >> lobit(o) & 1u) w |= 1u << c;
                     const int part = S.nY & 1, dif = tau >> lbit & 1u;
                     const uint32_t neg = (S.nY == 1 || S.nY == 2) ? 1u : 0u;
-                    EvcRegItem *hit = nullptr;
+                    One *hit = nullptr;
                     for (auto &it : its[part])
                         if (it.w == w && it.tau == (tau & ~rm) && ((it.z ^ S.z) & freemask) == 0 &&
                             (dif ? it.slot_dif : it.slot_sum) < 0) {
@@ -1196,17 +1235,36 @@ void plan_evc_phases(EvcPlan &P, int stage, int r) {
                             break;
                         }
                     if (!hit) {
-                        its[part].push_back(EvcRegItem{S.z & freemask, tau & ~rm, w, -1, -1, (code + (uint32_t)part) << 8, 0u});
+                        its[part].push_back(One{S.z & freemask, tau & ~rm, w, -1, -1, 0u});
                         hit = &its[part].back();
                     }
                     (dif ? hit->slot_dif : hit->slot_sum) = q - cp.s_begin;
-                    hit->ctl |= neg << dif;
+                    hit->neg |= neg << dif;
                 }
-                if (P.ritems.size() - F.i_begin + its[0].size() + its[1].size() > (size_t)kEvcRegItems)
-                    continue;   // a later phase's
-                for (auto &v : its) {
-                    if (!v.empty()) v[0].ctl |= 0x10000u;
-                    P.ritems.insert(P.ritems.end(), v.begin(), v.end());
+                const size_t cnt = std::max(its[0].size(), its[1].size());
+                if (P.ritems.size() - F.i_begin + cnt > (size_t)kEvcRegItems) continue;   // a later phase's
+                // the shorter list stands at the end, so that Re products held
+                // from one item to the next are not overwritten by Im products
+                for (size_t u = 0; u < cnt; ++u) {
+                    EvcRegItem it{};
+                    it.ctl = code << 8;
+                    for (int part = 0; part < 2; ++part) {
+                        it.slot_sum[part] = it.slot_dif[part] = -1;
+                        const size_t skip = cnt - its[part].size();
+                        if (u < skip) continue;
+                        const One &o = its[part][u - skip];
+                        it.z[part] = o.z;
+                        it.tau[part] = o.tau;
+                        it.w[part] = o.w;
+                        it.slot_sum[part] = o.slot_sum;
+                        it.slot_dif[part] = o.slot_dif;
+                        it.ctl |= (o.neg << (2 * part)) | (1u << (16 + part));
+                    }
+                    if (u > 0) {
+                        const uint32_t before = P.ritems.back().ctl;
+                        if ((before & 0x10000u) && !(before & 0x20000u)) it.ctl |= 0x40000u;
+                    }
+                    P.ritems.push_back(it);
                 }
                 done[i] = 1;
                 --left;
@@ -1239,6 +1297,54 @@ void plan_evc_phases(EvcPlan &P, int stage, int r) {
         cp.rp_first = (int32_t)half[0].size();
         cp.g_reg = ge;
         cp.s_reg = ge < cp.g_end ? P.groups[ge].s_begin : cp.s_end;
+    }
+}
+
+void plan_evc_units(EvcPlan &P) {
+    for (auto &cp : P.passes) {
+        cp.u_begin = cp.u_mid = cp.u_end = (int32_t)P.uitems.size();
+        const int ns = cp.s_end - cp.s_begin;
+        if (cp.kl != kEvcUnitRun || cp.m != kEvcUnitSpan || ns != cp.g_end - cp.g_begin || ns > 2 * kEvcUnitMax) continue;
+        const uint32_t mask[2] = {1u | (15u << cp.kl), 1u | (15u << (cp.kl + 4))};
+        uint64_t piv = 0;
+        for (int j = 0; j < cp.m; ++j) piv |= bit(cp.pivot[j]);
+        const uint64_t freemask = ~(piv | (bit(cp.kl) - 1));
+        std::vector<EvcUnitItem> half[2], other;
+        bool ok = true;
+        for (int g = cp.g_begin; g < cp.g_end; ++g) {
+            const EvcGroup &G = P.groups[g];
+            const EvcString &S = P.strings[G.s_begin];
+            if (!G.X) ok = false;                            // |psi|^2: the other kernels
+            EvcUnitItem it{};
+            it.z = S.z & freemask;
+            it.tau = (uint32_t)(S.z & (bit(cp.kl) - 1)) | (S.bz << cp.kl);
+            it.X = G.X;
+            it.neg = (S.nY == 1 || S.nY == 2) ? 1u : 0u;
+            it.slot = G.s_begin - cp.s_begin;
+            const int hi = popc(G.X & ~1u) == 1 ? lobit(G.X & ~1u) - cp.kl : -1;
+            it.code = 16u + (S.nY & 1);
+            if (hi >= 0) it.code = 4u * (hi & 3) + 2u * (G.X & 1u) + (S.nY & 1);
+            if (hi < 0) other.push_back(it);
+            else half[hi >> 2].push_back(it);
+        }
+        for (auto &it : other) half[half[1].size() < half[0].size()].push_back(it);
+        if (!ok || half[0].size() > (size_t)kEvcUnitMax || half[1].size() > (size_t)kEvcUnitMax) continue;
+        for (int k = 0; k < 2; ++k) {
+            for (auto &it : half[k]) {
+                // frequency over the half's register bits: bit 0, then the four span bits
+                const uint32_t f = (it.tau & 1u) | ((it.tau >> (cp.kl + 4 * k) & 15u) << 1);
+                if (it.code >= 16) {
+                    it.w = f;
+                } else {
+                    const int h = 1 + (int)(it.code >> 2);
+                    it.w = (f & ((1u << h) - 1u)) | ((f >> (h + 1)) << h);
+                }
+                it.tau &= ~mask[k];
+                P.uitems.push_back(it);
+            }
+            if (k == 0) cp.u_mid = (int32_t)P.uitems.size();
+        }
+        cp.u_end = (int32_t)P.uitems.size();
     }
 }
 

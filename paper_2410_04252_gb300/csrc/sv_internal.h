@@ -203,18 +203,36 @@ struct EvcGroup {
 // that share everything else: the part, the frequency w over the other bits,
 // the thread's frequency tau and z on the coset representatives.
 constexpr int kEvcRegPhases = 12;    // phases of one pass (shared-memory tables)
-constexpr int kEvcRegItems = 32;     // items of one phase (one bit each in the thread's sign word)
+constexpr int kEvcRegItems = 16;     // items of one phase (two bits each in the thread's sign word)
 struct EvcRegPhase {
     uint32_t rmask, lanes;           // staged-index bits in registers and in the lane bits (phase_lanes)
     int32_t i_begin, i_end;
 };
-struct EvcRegItem {
-    uint64_t z;
-    uint32_t tau, w;
-    int32_t slot_sum, slot_dif;      // strings of the pass (relative), or -1
-    uint32_t ctl;                    // bits 0, 1: signs of the sum and the difference; bits 8..15: pair code (2 *
-                                     // place of (h, l), plus 1 for Im); bit 16: first item of its group and part
+struct EvcRegItem {                  // an item of the Re part and one of the Im part of a group
+    uint64_t z[2];
+    uint32_t tau[2], w[2];
+    int32_t slot_sum[2], slot_dif[2];   // strings of the pass (relative), or -1
+    uint32_t ctl;                    // bits 0..3: signs (Re sum, difference, Im sum, difference); bits 8..15: place
+                                     // of (h, l); bits 16, 17: the part is there; bit 18: another item of the group
+                                     // came before without an Im part, its Re products are still held
     uint32_t pad;
+};
+
+// Passes of few strings, one per X/Y mask (random strings), whose span basis
+// is the masks themselves: a string then flips one span bit (and perhaps bit
+// 0) of the staged index.  Half of the warps hold bit 0 and the first four
+// span bits in registers, half bit 0 and the other four, and every string
+// goes to the half that holds its pairs; the strings that neither half holds
+// (masks inside the span of the others) read their partners.
+constexpr int kEvcUnitSpan = 8, kEvcUnitRun = 5, kEvcUnitMax = 8;   // span bits, run bits, strings per half
+struct EvcUnitItem {
+    uint64_t z;                      // on the coset representatives
+    uint32_t tau;                    // staged-index frequency
+    uint32_t w;                      // of it, the four register bits besides the flipped span bit (all five: code 16)
+    uint32_t X;
+    uint32_t code;                   // 4 * (register bit h - 1) + 2 * (bit 0 flips) + (Im: 1); 16, 17: partners read
+    uint32_t neg;
+    int32_t slot;                    // string of the pass (relative)
 };
 
 struct CosetPass {
@@ -227,6 +245,8 @@ struct CosetPass {
     // (half of the warps run phases [rp_begin, rp_begin + rp_first), the others the rest)
     int32_t rp_begin = 0, rp_end = 0, rp_first = 0, g_reg = 0, s_reg = 0;
     int32_t ri_begin = 0, ri_end = 0;
+    // plan_evc_units: strings of the first and of the second half of the warps
+    int32_t u_begin = 0, u_mid = 0, u_end = 0;
 };
 
 struct EvcPlan {
@@ -240,6 +260,7 @@ struct EvcPlan {
     std::vector<EvcString> strings;   // slots
     std::vector<EvcRegPhase> rphases;
     std::vector<EvcRegItem> ritems;
+    std::vector<EvcUnitItem> uitems;
     std::vector<int32_t> term_slot;   // per input term
     std::vector<int32_t> init_l2p, final_l2p;
     int32_t nqr() const {
@@ -282,6 +303,8 @@ std::string plan_hpsi(int n, const sv_pauli *p, const double *coeffs, size_t nte
 // Register phases of the passes that stage 2^stage amplitudes and hold enough
 // groups of one or two staged bits (fewer than kXformMinStrings strings each).
 void plan_evc_phases(EvcPlan &P, int stage, int r);
+// The passes that k_evc_unit takes (complex64: 2^13 staged, runs of 2^5).
+void plan_evc_units(EvcPlan &P);
 constexpr int kXformMinStrings = 16;  // groups with at least this many strings take the transform path
 constexpr int kEvcRegMinGroups = 6;
 // Write a bit permutation from layout `from` to layout `to` as at most two
