@@ -96,6 +96,7 @@ GatePassArgs gate_args(int n, const GatePass &gp) {
     a.mem_begin = gp.mem_begin;
     a.mem_end = gp.mem_end;
     a.dense = gp.dense;
+    a.mat1 = gp.mat1;
     return a;
 }
 

@@ -1005,13 +1005,16 @@ __device__ __forceinline__ R ra_ry_grad(const RA<R> *p, const RA<R> *l) {
         const float2 a = f2_unpack(P), b = f2_unpack(M);
         return (a.x + a.y) - (b.x + b.y);
     } else {
-        double g = 0;
+        // one fused multiply-add per product (FP64 is what bounds complex128)
+        double g = 0, h = 0;
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             if (v & (1 << B)) continue;
             const int w = v | (1 << B);
-            g += (l[w].x * p[v].x + l[w].y * p[v].y) - (l[v].x * p[w].x + l[v].y * p[w].y);
+            g = fma(l[w].x, p[v].x, fma(l[w].y, p[v].y, g));
+            h = fma(l[v].x, p[w].x, fma(l[v].y, p[w].y, h));
         }
+        g -= h;
         return g;
     }
 }
@@ -1572,16 +1575,16 @@ __device__ __forceinline__ void reg_image_load(unsigned char *sm, const unsigned
 
 // x[v] *= the block's factor (register block: table entry [v][zm]; thread block: one factor)
 template <typename R, int RB>
-__device__ __forceinline__ void reg_diag(RA<R> *x, const DiagBlock &B, const unsigned char *area) {
+__device__ __forceinline__ void reg_diag(RA<R> *x, const DiagBlock &B, const unsigned char *area, uint32_t thread) {
     constexpr int V = 1 << RB;
     if (B.kind == 0) {
         const Cx<R> *tab = reinterpret_cast<const Cx<R> *>(area + B.smem);
-        const uint32_t zm = area[B.smem + V * V * (int)sizeof(Cx<R>) + threadIdx.x];
+        const uint32_t zm = area[B.smem + V * V * (int)sizeof(Cx<R>) + thread];
         const Cx<R> *col = tab + zm;
 #pragma unroll
         for (int v = 0; v < V; ++v) x[v] = ra_cmul<R>(x[v], col[v * V]);
     } else {
-        const Cx<R> w = reinterpret_cast<const Cx<R> *>(area + B.smem)[threadIdx.x];
+        const Cx<R> w = reinterpret_cast<const Cx<R> *>(area + B.smem)[thread];
 #pragma unroll
         for (int v = 0; v < V; ++v) x[v] = ra_cmul<R>(x[v], w);
     }
@@ -1748,7 +1751,7 @@ k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *_
                         ra_rotf_bit<R, V, RB>(x, b, (S.a >> (8 + b)) & 1, rotf<R>(k.x));
                     }
                 } else if (S.type == SV_STEP_DIAG) {
-                    reg_diag<R, RB>(x, bl[S.a - a.db_begin], area);
+                    reg_diag<R, RB>(x, bl[S.a - a.db_begin], area, threadIdx.x);
                 } else {
                     reg_op<R, true>(x, (uint32_t)S.a, F.rmask, base, gbase, cs[S.op_begin], pmats + S.op_end);
                 }
@@ -1761,6 +1764,92 @@ k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *_
         if (it + 2 < mine) reg_tile_load<R>(tile, mypsi + base_pf, chunk, slot);
         cp_async_commit();
         base_pf = walk_next(base_pf, bw);
+    }
+}
+
+// The same pass with two tiles in work per CTA (complex64, no dense matrices):
+// two groups of 2^(k - 4) threads, each with a tile of its own and a barrier
+// of its own, so that one group's gathers and scatters run under the other's
+// arithmetic.  With one tile all warps meet the shared-memory pipe and then
+// the issue slots together: a phase of an n = 26 brick pass took 2900 clocks,
+// of which 1024 are shared memory and 1280 issue.  The second tile's room is
+// the first kernel's prefetch buffer, so the passes of few phases, which HBM
+// bounds, stay with that one (gate_two_pays).
+template <typename R>
+__global__ void __launch_bounds__(1024, 1)
+k_gate_two(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *__restrict__ image, int early) {
+    constexpr int RB = kRegBits, V = 1 << RB;
+    constexpr uint32_t P = 16 / sizeof(Cx<R>);
+    extern __shared__ __align__(16) unsigned char smem[];
+    const uint32_t T = 1u << a.k, NT = T >> RB;
+    const uint32_t grp = threadIdx.x >> (a.k - RB), th = threadIdx.x & (NT - 1u);
+    RA<R> *tile = reinterpret_cast<RA<R> *>(smem) + grp * T;
+    unsigned char *sm = smem + 2 * T * sizeof(RA<R>);
+    const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), false);
+    if (!early) pdl_wait();
+    reg_image_load(sm, image, L.image);
+    pdl_wait();
+    pdl_next();
+    const R ftot = reinterpret_cast<const R *>(sm + L.sc)[a.st_end - a.st_begin];   // product of the RY factors
+    const uint64_t *hioff = reinterpret_cast<const uint64_t *>(sm + L.hioff);
+    const ChunkOff *chunk = reinterpret_cast<const ChunkOff *>(sm + L.chunk);
+    const Cx<R> *cs = reinterpret_cast<const Cx<R> *>(sm + L.cs);
+    const RegStep *st = reinterpret_cast<const RegStep *>(sm + L.steps);
+    const DiagBlock *bl = reinterpret_cast<const DiagBlock *>(sm + L.blocks);
+    const PhaseS *phs = reinterpret_cast<const PhaseS *>(sm + L.phases);
+    const uint16_t *pbase = reinterpret_cast<const uint16_t *>(sm + L.pbase);
+    const uint16_t *prb = reinterpret_cast<const uint16_t *>(sm + L.prb);
+    const unsigned char *area = sm + L.area;
+    const int nph = a.ph_end - a.ph_begin;
+    const uint64_t ntiles = 1ull << a.nout, first = blockIdx.x + (uint64_t)gridDim.x * grp, stride = 2ull * gridDim.x;
+    const uint64_t mine = first < ntiles ? (ntiles - first + stride - 1) / stride : 0;
+    const uint32_t j0 = P * th, slot = swz_tile(j0);
+    Cx<R> *mypsi = psi + (hioff[j0 >> a.nlow] | (j0 & ((1u << a.nlow) - 1u)));
+    const BitWalk bw = bit_walk(a.out, a.nout, stride);
+    uint64_t gbase = deposit(first, a.out, a.nout);
+    auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1u + grp), "r"(NT) : "memory"); };
+    for (uint64_t it = 0; it < mine; ++it) {
+        // a thread's pieces go to the slots that it stored from last
+        reg_tile_load<R>(tile, mypsi + gbase, chunk, slot);
+        cp_async_commit();
+        cp_async_wait0();
+        group_sync();
+        for (int ph = 0; ph < nph; ++ph) {
+            const PhaseS F = phs[ph];
+            const uint32_t base = pbase[ph * NT + th];
+            RA<R> x[V];
+            {
+                uint32_t idx[V];
+                phase_slots16(idx, base, prb + ph * 4);
+                phase_gather<R>(x, tile, idx, F.rmask & 1u);
+            }
+            for (int s = F.st_begin; s < F.st_end; ++s) {
+                const RegStep S = st[s];
+                if (S.type == SV_STEP_ROT) {
+                    // factored RYs (t, factor): the factors are applied at the store
+                    const Cx<R> *c = cs + (S.op_begin - a.op_begin);
+#pragma unroll
+                    for (int b = 0; b < RB; ++b) {
+                        if (!((S.a >> b) & 1)) continue;
+                        const Cx<R> k = *c++;
+                        ra_rotf_bit<R, V, RB>(x, b, (S.a >> (8 + b)) & 1, rotf<R>(k.x));
+                    }
+                } else if (S.type == SV_STEP_DIAG) {
+                    reg_diag<R, RB>(x, bl[S.a - a.db_begin], area, th);
+                } else {
+                    reg_op<R, false>(x, (uint32_t)S.a, F.rmask, base, gbase, cs[S.op_begin], nullptr);
+                }
+            }
+            {
+                // the slots again (fewer registers live across the steps)
+                uint32_t idx[V];
+                phase_slots16(idx, pbase[ph * NT + th], prb + ph * 4);
+                phase_scatter<R>(x, tile, idx, F.rmask & 1u);
+            }
+            group_sync();
+        }
+        reg_tile_store<R>(mypsi + gbase, tile, chunk, slot, ftot);
+        gbase = walk_next(gbase, bw);
     }
 }
 
@@ -4829,11 +4918,22 @@ size_t adj_reg_smem(sv_dtype dt, const GatePassArgs &a) {
     return 2 * ((size_t)1 << a.k) * amp + reg_layout(a, amp, true).total;
 }
 
+// Two tiles in work per CTA from kTwoPhases phases on (1-qubit matrices may
+// stay, they are one row product): see k_gate_two.
+#ifndef KTWO
+#define KTWO 3
+#endif
+constexpr int kTwoPhases = KTWO;
+static bool gate_two_pays(sv_dtype dt, const GatePassArgs &a) {
+    return dt == SV_C64 && !a.dense && !a.mat1 && a.ph_end - a.ph_begin >= kTwoPhases;
+}
+
 int reg_pass_grid(sv_dtype dt, const GatePassArgs &a, bool adj, int blocks_per_sm) {
     const size_t sm = (adj ? adj_reg_smem(dt, a) : gate_reg_smem(dt, a)) + 1024;
-    const int nt = 1 << (a.k - kRegBits);
+    const bool two = !adj && gate_two_pays(dt, a);
+    const int nt = (two ? 2 : 1) << (a.k - kRegBits);
     // resident CTAs by shared memory, by the launch bound's register share and by the block limit
-    int per = (int)std::min<size_t>((size_t)228 * 1024 / sm, (size_t)((dt == SV_C64 ? 512 : 256) / nt));
+    int per = (int)std::min<size_t>((size_t)228 * 1024 / sm, (size_t)((two ? 1024 : dt == SV_C64 ? 512 : 256) / nt));
     per = std::max(1, std::min(per, 16));
     if (blocks_per_sm > 0) per = std::min(per, blocks_per_sm);
     const uint64_t ntiles = 1ull << a.nout;
@@ -4846,6 +4946,13 @@ cudaError_t gate_reg_dispatch(cudaStream_t st, int grid, void *psi, const GatePa
     const size_t sm = gate_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
     const int nt = 1 << (a.k - kRegBits);
     if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
+    if constexpr (sizeof(R) == 4) {
+        if (gate_two_pays(SV_C64, a)) {
+            allow_smem(k_gate_two<float>, sm);
+            return launch(k_gate_two<float>, grid, 2 * nt, sm, st, (float2 *)psi, a, (const unsigned char *)image,
+                          early ? 1 : 0);
+        }
+    }
     allow_smem(k_gate_reg<R>, sm);
     return launch(k_gate_reg<R>, grid, nt, sm, st, (Cx<R> *)psi, a, (const unsigned char *)image,
                   (const Cx<R> *)pmats, early ? 1 : 0);

@@ -508,6 +508,7 @@ void plan_phases(QsuPlan &P, bool pairs, int threads) {
             const bool pair = kd == SV_GIVENS || kd == SV_DEXC || kd == SV_MAT2 || kd == SV_MAT4;
             if (kd != SV_RY && kd != SV_RZ && kd != SV_CZ && kd != SV_MAT1 && !(pairs && pair)) ok = false;
             if (kd == SV_MAT2 || kd == SV_MAT4) dense = true;
+            if (kd == SV_MAT1) gp.mat1 = 1;
         }
         if (!ok) continue;
         gp.dense = dense;

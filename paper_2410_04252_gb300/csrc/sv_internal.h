@@ -65,6 +65,7 @@ struct GatePass {
     uint64_t bits = 0;                // physical staged bits
     int32_t op_begin = 0, op_end = 0; // into QsuPlan::ops
     int32_t ph_begin = -1, ph_end = -1;  // register phases (register-blocked passes), else -1
+    int32_t mat1 = 0;                    // 1: the phases hold 1-qubit matrices
     int32_t dense = 0;                   // 1: the phases hold 2- or 4-qubit matrices (forward only)
     int32_t db_begin = 0, db_end = 0;    // diagonal blocks of the pass (register-blocked passes)
     int32_t st_begin = 0, st_end = 0;    // steps of the pass's phases
