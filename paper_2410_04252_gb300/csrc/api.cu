@@ -97,6 +97,8 @@ GatePassArgs gate_args(int n, const GatePass &gp) {
     a.mem_end = gp.mem_end;
     a.dense = gp.dense;
     a.mat1 = gp.mat1;
+    a.pairs = gp.pairs;
+    a.others = gp.others;
     return a;
 }
 

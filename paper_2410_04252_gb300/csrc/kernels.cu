@@ -891,35 +891,6 @@ __device__ __forceinline__ RA<R> ra_cmul(RA<R> a, Cx<R> w) {
 template <typename R> struct RotK;
 template <> struct RotK<float> { unsigned long long C, S, NS; };
 template <> struct RotK<double> { double c, s; };
-template <typename R> __device__ __forceinline__ RotK<R> rotk(R c, R s);
-template <> __device__ __forceinline__ RotK<float> rotk<float>(float c, float s) {
-    return {f2_pack(c, c), f2_pack(s, s), f2_pack(-s, -s)};
-}
-template <> __device__ __forceinline__ RotK<double> rotk<double>(double c, double s) { return {c, s}; }
-
-// (u, v) <- (c u - s v, s u + c v) on every pair of register bit B
-template <typename R, int V, int B>
-__device__ __forceinline__ void ra_rot(RA<R> *x, const RotK<R> &k) {
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-        if (v & (1 << B)) continue;
-        const int w = v | (1 << B);
-        if constexpr (sizeof(R) == 4) {
-            unsigned long long t, uu, vv;
-            asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(x[w]), "l"(k.NS));
-            asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(uu) : "l"(x[v]), "l"(k.C), "l"(t));
-            asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(x[w]), "l"(k.C));
-            asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(vv) : "l"(x[v]), "l"(k.S), "l"(t));
-            x[v] = uu;
-            x[w] = vv;
-        } else {
-            const double2 a = x[v], b = x[w];
-            x[v] = make_double2(k.c * a.x - k.s * b.x, k.c * a.y - k.s * b.y);
-            x[w] = make_double2(k.s * a.x + k.c * b.x, k.s * a.y + k.c * b.y);
-        }
-    }
-}
-
 // RY with its larger coefficient factored out (the factor is common to every
 // amplitude of the tile, so a pass carries the product of the factors and
 // applies it once when the tile is stored):
@@ -929,11 +900,19 @@ __device__ __forceinline__ void ra_rot(RA<R> *x, const RotK<R> &k) {
 // costs two fused multiply-adds (form B: plus a sign flip) instead of two
 // products and two fused multiply-adds.
 template <typename R> struct RotF;
-template <> struct RotF<float> { unsigned long long T, NT; };
+template <> struct RotF<float> { unsigned long long T; };
 template <> struct RotF<double> { double t; };
-template <typename R> __device__ __forceinline__ RotF<R> rotf(R t);
-template <> __device__ __forceinline__ RotF<float> rotf<float>(float t) { return {f2_pack(t, t), f2_pack(-t, -t)}; }
-template <> __device__ __forceinline__ RotF<double> rotf<double>(double t) { return {t}; }
+// from the pass's table, where a factored RY stands as (t, t)
+template <typename R> __device__ __forceinline__ RotF<R> rotf(Cx<R> tt);
+template <> __device__ __forceinline__ RotF<float> rotf<float>(float2 tt) { return {f2_pack(tt.x, tt.y)}; }
+template <> __device__ __forceinline__ RotF<double> rotf<double>(double2 tt) { return {tt.x}; }
+// (-a.x, -a.y), exact, on the FMA pipe: two sign flips on the integer pipe,
+// which these kernels use most, cost twice as much
+__device__ __forceinline__ unsigned long long f2_neg(unsigned long long a) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(0xBF800000BF800000ull));
+    return r;
+}
 
 // factored form (t, factor) and form bit of an RY with coefficients (c, s)
 template <typename R> __device__ __forceinline__ Cx<R> ry_factored(R c, R s, int &form_b) {
@@ -944,6 +923,8 @@ template <typename R> __device__ __forceinline__ Cx<R> ry_factored(R c, R s, int
 
 template <typename R, int V, int B, bool FB>
 __device__ __forceinline__ void ra_rotf(RA<R> *x, const RotF<R> &k) {
+    unsigned long long nt = 0;
+    if constexpr (sizeof(R) == 4 && !FB) nt = f2_neg(k.T);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         if (v & (1 << B)) continue;
@@ -951,11 +932,11 @@ __device__ __forceinline__ void ra_rotf(RA<R> *x, const RotF<R> &k) {
         if constexpr (sizeof(R) == 4) {
             unsigned long long uu, vv;
             if (FB) {   // (t u - v, u + t v)
-                const unsigned long long nw = x[w] ^ 0x8000000080000000ull;
+                const unsigned long long nw = f2_neg(x[w]);
                 asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(uu) : "l"(x[v]), "l"(k.T), "l"(nw));
                 asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(vv) : "l"(x[w]), "l"(k.T), "l"(x[v]));
             } else {    // (u - t v, v + t u)
-                asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(uu) : "l"(x[w]), "l"(k.NT), "l"(x[v]));
+                asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(uu) : "l"(x[w]), "l"(nt), "l"(x[v]));
                 asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(vv) : "l"(x[v]), "l"(k.T), "l"(x[w]));
             }
             x[v] = uu;
@@ -1105,12 +1086,9 @@ enum : uint32_t {
     RO_MAT1 = 18,      // + register bit
     RO_MAT2 = 22,      // + index of the bit pair 01 02 03 12 13 23
     RO_MAT4 = 28,
-    RO_RZ = 29,        // + register bit
-    RO_RZ_THREAD = 33, // t0: tile bit
-    RO_CZ = 34,        // t0, t1: tile bits
-    RO_RZ_OUT = 35,    // t0 - kOutTarget: physical bit outside the tile
-    RO_CZ_OUT = 36,    // t0 or t1 (or both) outside the tile
-    RO_NOP = 37
+    RO_RZ = 29,        // t0: tile bit, or kOutTarget + physical bit outside the tile
+    RO_CZ = 30,        // t0, t1 likewise
+    RO_NOP = 31
 };
 #define SV_RO_GIVENS(CALL)                                                                       \
     case 0: CALL(1, 2); break;  case 1: CALL(1, 4); break;  case 2: CALL(1, 8); break;           \
@@ -1185,81 +1163,41 @@ __device__ __forceinline__ void reg_mat4(RA<R> *x, const Cx<R> *M) {
 __device__ __forceinline__ uint32_t reg_bit_mask(uint32_t b) {
     return b == 0 ? 0xAAAAu : b == 1 ? 0xCCCCu : b == 2 ? 0xF0F0u : 0xFF00u;
 }
-// the register amplitudes on which a CZ of in-tile bits t0, t1 is -1
-__device__ __forceinline__ uint32_t cz_negmask(uint32_t t0, uint32_t t1, uint32_t rmask, uint32_t base) {
-    uint32_t m = 0xFFFFu;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const uint32_t t = i ? t1 : t0;
-        if ((rmask >> t) & 1u) m &= reg_bit_mask(__popc(rmask & ((1u << t) - 1u)));
-        else if (!((base >> t) & 1u)) m = 0;
-    }
-    return m;
+// the thread's tile bits outside the register set, from its place in shared memory (the swizzle is its own inverse)
+template <typename R> __device__ __forceinline__ uint32_t phase_bits(uint32_t place) {
+    return swz_tile(place / (uint32_t)sizeof(Cx<R>));
 }
-template <typename R>
-__device__ __forceinline__ void reg_neg_mask(RA<R> *x, uint32_t m) {
-#pragma unroll
-    for (int v = 0; v < (1 << kRegBits); ++v)
-        if ((m >> v) & 1u) x[v] = ra_neg<R>(x[v]);
+// the register amplitudes on which in-tile bit t is 1
+__device__ __forceinline__ uint32_t reg_or_thread_mask(uint32_t t, uint32_t rmask, uint32_t base) {
+    if ((rmask >> t) & 1u) return reg_bit_mask(__popc(rmask & ((1u << t) - 1u)));
+    return ((base >> t) & 1u) ? 0xFFFFu : 0u;
 }
-template <typename R, int B>
-__device__ __forceinline__ void reg_rz_bit(RA<R> *x, Cx<R> k) {
-    const Cx<R> w0 = mk<R>(k.x, -k.y), w1 = mk<R>(k.x, k.y);
-#pragma unroll
-    for (int v = 0; v < (1 << kRegBits); ++v) x[v] = ra_cmul<R>(x[v], ((v >> B) & 1) ? w1 : w0);
-}
-template <typename R>
-__device__ __forceinline__ void reg_phase_all(RA<R> *x, Cx<R> k, bool one) {
-    const Cx<R> w = mk<R>(k.x, one ? k.y : -k.y);
-#pragma unroll
-    for (int v = 0; v < (1 << kRegBits); ++v) x[v] = ra_cmul<R>(x[v], w);
-}
-// sign mask of a CZ with a target outside the tile (constant over the tile)
-__device__ __forceinline__ uint32_t cz_out_negmask(uint32_t t0, uint32_t t1, uint32_t rmask, uint32_t base,
-                                                   uint64_t gbase) {
-    const bool o0 = t0 >= (uint32_t)kOutTarget, o1 = t1 >= (uint32_t)kOutTarget;
-    if (o0 && !((gbase >> (t0 - kOutTarget)) & 1ull)) return 0;
-    if (o1 && !((gbase >> (t1 - kOutTarget)) & 1ull)) return 0;
-    if (o0 && o1) return 0xFFFFu;
-    const uint32_t t = o0 ? t1 : t0;
-    return cz_negmask(t, t, rmask, base);
+// the same for a qubit inside or outside the tile (t >= kOutTarget: constant over the tile)
+__device__ __forceinline__ uint32_t diag_bit_mask(uint32_t t, uint32_t rmask, uint32_t base, uint64_t gbase) {
+    if (t >= (uint32_t)kOutTarget) return ((gbase >> (t - kOutTarget)) & 1ull) ? 0xFFFFu : 0u;
+    return reg_or_thread_mask(t, rmask, base);
 }
 
-// One operation of a step (code and targets packed in `a`: code | t0 << 8 |
-// t1 << 16) on the register amplitudes; k = (cos, sin), sin negated for an
-// inverse; M = the prepared matrix.  DENSE: 2- and 4-qubit matrices too
-// (their reverse passes run in k_adj_pass).
-template <typename R, bool DENSE>
-__device__ __forceinline__ void reg_op(RA<R> *x, uint32_t a, uint32_t rmask, uint32_t base, uint64_t gbase,
-                                       Cx<R> k, const Cx<R> *M) {
-    constexpr int V = 1 << kRegBits;
-    const uint32_t t0 = (a >> 8) & 255u, t1 = (a >> 16) & 255u;
-    const RotK<R> rk = rotk<R>(k.x, k.y);
-    switch (a & 255u) {
-#define SV_C(MU, MV) ra_pair_rot<R, V, MU, MV>(x, rk)
-        SV_RO_GIVENS(SV_C)
-#undef SV_C
-    case RO_MAT1: reg_mat<R, 0, 0>(x, M); break;
-    case RO_MAT1 + 1: reg_mat<R, 1, 1>(x, M); break;
-    case RO_MAT1 + 2: reg_mat<R, 2, 2>(x, M); break;
-    case RO_MAT1 + 3: reg_mat<R, 3, 3>(x, M); break;
-    case RO_MAT2: if constexpr (DENSE) reg_mat<R, 0, 1>(x, M); break;
-    case RO_MAT2 + 1: if constexpr (DENSE) reg_mat<R, 0, 2>(x, M); break;
-    case RO_MAT2 + 2: if constexpr (DENSE) reg_mat<R, 0, 3>(x, M); break;
-    case RO_MAT2 + 3: if constexpr (DENSE) reg_mat<R, 1, 2>(x, M); break;
-    case RO_MAT2 + 4: if constexpr (DENSE) reg_mat<R, 1, 3>(x, M); break;
-    case RO_MAT2 + 5: if constexpr (DENSE) reg_mat<R, 2, 3>(x, M); break;
-    case RO_MAT4: if constexpr (DENSE) reg_mat4<R>(x, M); break;
-    case RO_RZ: reg_rz_bit<R, 0>(x, k); break;
-    case RO_RZ + 1: reg_rz_bit<R, 1>(x, k); break;
-    case RO_RZ + 2: reg_rz_bit<R, 2>(x, k); break;
-    case RO_RZ + 3: reg_rz_bit<R, 3>(x, k); break;
-    case RO_RZ_THREAD: reg_phase_all<R>(x, k, (base >> t0) & 1u); break;
-    case RO_RZ_OUT: reg_phase_all<R>(x, k, (gbase >> (t0 - kOutTarget)) & 1ull); break;
-    case RO_CZ: reg_neg_mask<R>(x, cz_negmask(t0, t1, rmask, base)); break;
-    case RO_CZ_OUT: reg_neg_mask<R>(x, cz_out_negmask(t0, t1, rmask, base, gbase)); break;
-    default: break;
+// A diagonal gate outside the blocks on the register amplitudes, m the
+// amplitudes whose bits are 1: CZ negates them, RZ turns them the other way.
+// One straight-line body each for every place of the targets: the codes of a
+// switch meet in register moves, more of them than arithmetic.
+__device__ __forceinline__ float flip_by(float v, uint32_t m, int b) {
+    return __uint_as_float(__float_as_uint(v) ^ ((m << (31 - b)) & 0x80000000u));
+}
+__device__ __forceinline__ double flip_by(double v, uint32_t m, int b) {
+    return __hiloint2double(__double2hiint(v) ^ (int)((m << (31 - b)) & 0x80000000u), __double2loint(v));
+}
+template <typename R> __device__ __forceinline__ void reg_cz(RA<R> *x, uint32_t m) {
+#pragma unroll
+    for (int v = 0; v < (1 << kRegBits); ++v) {
+        const Cx<R> c = ra_cx<R>(x[v]);
+        x[v] = cx_ra<R>(mk<R>(flip_by(c.x, m, v), flip_by(c.y, m, v)));
     }
+}
+template <typename R> __device__ __forceinline__ void reg_rz(RA<R> *x, Cx<R> k, uint32_t m) {
+#pragma unroll
+    for (int v = 0; v < (1 << kRegBits); ++v) x[v] = ra_cmul<R>(x[v], mk<R>(k.x, flip_by(-k.y, m, v)));
 }
 
 // Im(conj(l) p) per register amplitude
@@ -1269,41 +1207,23 @@ __device__ __forceinline__ R ra_imdot(RA<R> l, RA<R> p) {
     return a.x * b.y - a.y * b.x;
 }
 
-// Adjoint of one operation: gradient part Im<lambda|G|psi> (the subspace Y of
-// a rotation, Z of an RZ), then U^dagger on both register sets.
-__device__ __forceinline__ bool reg_op_param(uint32_t a) {
-    const uint32_t c = a & 255u;
-    return c < RO_MAT1 || (c >= RO_RZ && c <= RO_RZ_THREAD) || c == RO_RZ_OUT;
+// coefficients of pair rotation o of the pass from its table record, and its code
+template <typename R> __device__ __forceinline__ RotK<R> pair_rec(const Cx<R> *rec, uint32_t &code);
+template <> __device__ __forceinline__ RotK<float> pair_rec<float>(const float2 *rec, uint32_t &code) {
+    const ulonglong2 a = reinterpret_cast<const ulonglong2 *>(rec)[0], b = reinterpret_cast<const ulonglong2 *>(rec)[1];
+    code = (uint32_t)b.y;
+    return {a.x, a.y, b.x};
 }
-template <typename R>
-__device__ __forceinline__ R reg_op_adj(RA<R> *p, RA<R> *l, uint32_t a, uint32_t rmask, uint32_t base, uint64_t gbase,
-                                        Cx<R> k, const Cx<R> *M) {
-    constexpr int V = 1 << kRegBits;
-    const uint32_t t0 = (a >> 8) & 255u;
-    const uint32_t c = a & 255u;
-    R g = 0;
-    if (c < RO_MAT1) {
-        switch (c) {
-#define SV_C(MU, MV) g = ra_pair_grad<R, V, MU, MV>(p, l)
-            SV_RO_GIVENS(SV_C)
-#undef SV_C
-        default: break;
-        }
-    } else if (reg_op_param(a)) {
-        // amplitudes on which Z is -1
-        const uint32_t neg = c == RO_RZ_THREAD ? (((base >> t0) & 1u) ? 0xFFFFu : 0u)
-                             : c == RO_RZ_OUT  ? (((gbase >> (t0 - kOutTarget)) & 1ull) ? 0xFFFFu : 0u)
-                                               : reg_bit_mask((c - RO_RZ) & 3u);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const R im = ra_imdot<R>(l[v], p[v]);
-            g += ((neg >> v) & 1u) ? -im : im;
-        }
-    }
-    reg_op<R, false>(p, a, rmask, base, gbase, k, M);
-    reg_op<R, false>(l, a, rmask, base, gbase, k, M);
-    return g;
+template <> __device__ __forceinline__ RotK<double> pair_rec<double>(const double2 *rec, uint32_t &code) {
+    code = (uint32_t)__double_as_longlong(rec[3].x);
+    return {rec[0].x, rec[1].x};
 }
+
+// The step loop of a phase comes in three kinds, chosen per pass by what the
+// pass holds, since the operations it does not hold would cost it register
+// moves where their codes meet: 0 rotations and diagonal gates only
+// (hardware-efficient ansatz), 1 pair rotations only (brick ansatz), 2 all.
+constexpr int kStepsDiag = 0, kStepsPair = 1, kStepsAll = 2;
 
 // Hint: bring [p, p + bytes) into L2 (bytes a multiple of 16, p 16-byte aligned).
 __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
@@ -1331,7 +1251,7 @@ __device__ __forceinline__ void load_tile_async(E *tile, const Cx<R> *psi, uint6
 // Shared-memory layout of a register-blocked pass (both kernels): the tiles,
 // then these tables (offsets in bytes from the end of the tiles).
 struct RegLayout {
-    uint32_t hioff, chunk, cs, steps, blocks, mem, phases, pbase, prb, sc, area, image, acc, tot, total;
+    uint32_t hioff, chunk, cs, steps, blocks, mem, phases, pbase, prb, rk, sc, area, image, acc, tot, total;
 };
 // FP64 is 1/64 of the FP32 rate on this part: per-tile gradient partials stay
 // in FP32 slots and reach FP64 once every kAdjFlush tiles
@@ -1351,7 +1271,9 @@ __host__ __device__ inline RegLayout reg_layout(const GatePassArgs &a, int amp, 
     L.mem = o;   o = align16u(o + (uint32_t)sizeof(DiagMember) * (uint32_t)(a.mem_end - a.mem_begin));
     L.phases = o; o = align16u(o + 16u * nph);
     L.pbase = o; o = align16u(o + 2u * nt * nph);
-    L.prb = o;   o = align16u(o + 8u * nph);
+    L.prb = o;   o = align16u(o + 16u * nph);
+    // pair rotations: coefficients as packed operands (c, c), (s, s), (-s, -s), and the code
+    L.rk = o;    o = align16u(o + (a.pairs ? 4u * (uint32_t)amp * nops : 0u));
     // factored RYs: per step the product of the factors applied before it
     // (adjoint), and the pass's total factor (entry nst)
     L.sc = o;    o = align16u(o + ((uint32_t)amp / 2u) * (nst + 1u));
@@ -1370,7 +1292,7 @@ __host__ __device__ inline RegLayout reg_layout(const GatePassArgs &a, int amp, 
 // thread's XOR / OR these per-chunk constants.
 struct ChunkOff {
     uint64_t g;    // global element offset of tile bits i P NT
-    uint32_t s;    // shared slot of the same
+    uint32_t s;    // shared byte offset of the same
     uint32_t pad;
 };
 struct PhaseS {
@@ -1443,11 +1365,9 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
             } else if (op.kind == SV_MAT4) {
                 code = RO_MAT4;
             } else if (op.kind == SV_RZ) {
-                code = t0 >= (uint32_t)kOutTarget ? (uint32_t)RO_RZ_OUT
-                       : ((rmask >> t0) & 1u)     ? RO_RZ + reg(t0)
-                                                  : (uint32_t)RO_RZ_THREAD;
+                code = RO_RZ;
             } else if (op.kind == SV_CZ) {
-                code = (t0 >= (uint32_t)kOutTarget || t1 >= (uint32_t)kOutTarget) ? RO_CZ_OUT : RO_CZ;
+                code = RO_CZ;
             }
             S.op_begin = S.a - a.op_begin;
             S.a = (int32_t)(code | (t0 << 8) | (t1 << 16));
@@ -1479,9 +1399,24 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
         ChunkOff *chunk = reinterpret_cast<ChunkOff *>(out + L.chunk);
         for (uint32_t i = tid; i < 16u / P; i += nthr) {
             const uint32_t j = i * P * (uint32_t)NT;
-            chunk[i] = {(j & lowmask) | deposit(j >> a.nlow, a.hi, a.nhi), swz_tile(j), 0u};
+            chunk[i] = {(j & lowmask) | deposit(j >> a.nlow, a.hi, a.nhi), swz_tile(j) * (uint32_t)sizeof(Cx<R>), 0u};
         }
-        for (int o = tid; o < a.op_end - a.op_begin; o += nthr) reinterpret_cast<Cx<R> *>(out + L.cs)[o] = cs[o];
+        for (int o = tid; o < a.op_end - a.op_begin; o += nthr) {
+            const Cx<R> k = cs[o];
+            // factored RYs as (t, t): a packed operand as it is loaded
+            reinterpret_cast<Cx<R> *>(out + L.cs)[o] = ops[a.op_begin + o].kind == SV_RY ? mk<R>(k.x, k.x) : k;
+            if (a.pairs) {
+                Cx<R> *rec = reinterpret_cast<Cx<R> *>(out + L.rk) + 4 * o;
+                rec[0] = mk<R>(k.x, k.x);
+                rec[1] = mk<R>(k.y, k.y);
+                rec[2] = mk<R>(-k.y, -k.y);
+            }
+        }
+        // pair rotations carry their code in the record
+        for (int s = tid; a.pairs && s < nst; s += nthr)
+            if (st[s].type == SV_STEP_OP)
+                *reinterpret_cast<uint64_t *>(reinterpret_cast<Cx<R> *>(out + L.rk) + 4 * st[s].op_begin + 3) =
+                    (uint64_t)((uint32_t)st[s].a & 255u);
         for (int s = tid; s < nst; s += nthr) reinterpret_cast<RegStep *>(out + L.steps)[s] = st[s];
         for (int b = a.db_begin + tid; b < a.db_end; b += nthr)
             reinterpret_cast<DiagBlock *>(out + L.blocks)[b - a.db_begin] = dblocks[b];
@@ -1492,7 +1427,7 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
             reinterpret_cast<PhaseS *>(out + L.phases)[q] = {F.rmask, F.st_begin - a.st_begin, F.st_end - a.st_begin, 0u};
             uint32_t rm = F.rmask;
             for (int i = 0; i < RB; ++i, rm &= rm - 1u)
-                reinterpret_cast<uint16_t *>(out + L.prb)[q * 4 + i] = (uint16_t)swz_tile(rm & (0u - rm));
+                reinterpret_cast<uint32_t *>(out + L.prb)[q * 4 + i] = swz_tile(rm & (0u - rm)) * (uint32_t)sizeof(Cx<R>);
         }
         // prefix products of the factors in execution order (forward: ascending
         // steps; adjoint: descending), entry nst = the pass's total factor
@@ -1512,7 +1447,8 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
         const int q = e / NT, t = e % NT;
         if (q % kImageSlices != (int)blockIdx.y) continue;
         const Phase F = phases[a.ph_begin + q];
-        reinterpret_cast<uint16_t *>(out + L.pbase)[e] = (uint16_t)phase_base(F.rmask, F.lanes, a.k, (uint32_t)t);
+        reinterpret_cast<uint16_t *>(out + L.pbase)[e] =
+            (uint16_t)(swz_tile(phase_base(F.rmask, F.lanes, a.k, (uint32_t)t)) * (uint32_t)sizeof(Cx<R>));
     }
     // this slice's diagonal blocks: tables and per-thread data
     unsigned char *area = out + L.area;
@@ -1615,69 +1551,295 @@ __device__ __forceinline__ void reg_diag2(RA<R> *x, RA<R> *y, const DiagBlock &B
     }
 }
 
-// The thread's 16 shared-memory slots of a phase (the swizzle is linear, so
-// slot(base | v) = slot(base) ^ XOR of the register bits' slots), and the
-// gather and scatter of its amplitudes.  A phase that holds tile bit 0 moves
-// complex64 pairs (v, v | 1) by one 16-byte access: with 8-byte accesses its
-// lanes could only reach half of the banks.
-__device__ __forceinline__ void phase_slots16(uint32_t *idx, uint32_t base, const uint16_t *prb) {
-    const ushort4 r = *reinterpret_cast<const ushort4 *>(prb);
+// The thread's 16 shared-memory places of a phase, as byte offsets from the
+// block's shared memory (the tile's included: tiles lie at multiples of their
+// size).  The swizzle is linear, so place(base | v) = place(base) ^ XOR of the
+// register bits' places; the tables hold places, not indices, and no address
+// needs more than its XOR -- the integer pipe runs at half rate and was the
+// busiest unit of these kernels (183 of its instructions per phase and warp in
+// a brick pass, of 377 in all).  A phase that holds tile bit 0 moves complex64
+// pairs (v, v | 1) by one 16-byte access: with 8-byte accesses its lanes could
+// only reach half of the banks.
+__device__ __forceinline__ void phase_slots16(uint32_t *idx, uint32_t base, uint4 r) {
     const uint32_t rb[4] = {r.x, r.y, r.z, r.w};
-    idx[0] = swz_tile(base);
+    idx[0] = base;
 #pragma unroll
     for (int v = 1; v < 16; ++v) idx[v] = idx[v & (v - 1)] ^ rb[(v & 1) ? 0 : (v & 2) ? 1 : (v & 4) ? 2 : 3];
 }
 template <typename R>
-__device__ __forceinline__ void phase_gather(RA<R> *x, const RA<R> *tile, const uint32_t *idx, bool pairs) {
+__device__ __forceinline__ void phase_gather(RA<R> *x, const unsigned char *sm, const uint32_t *idx, bool pairs) {
     if (sizeof(R) == 4 && pairs) {
 #pragma unroll
         for (int v = 0; v < 16; v += 2) {
-            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(&tile[idx[v]]);
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(sm + idx[v]);
             memcpy(&x[v], &w.x, 8);
             memcpy(&x[v + 1], &w.y, 8);
         }
     } else {
 #pragma unroll
-        for (int v = 0; v < 16; ++v) x[v] = tile[idx[v]];
+        for (int v = 0; v < 16; ++v) x[v] = *reinterpret_cast<const RA<R> *>(sm + idx[v]);
     }
 }
 template <typename R>
-__device__ __forceinline__ void phase_scatter(const RA<R> *x, RA<R> *tile, const uint32_t *idx, bool pairs) {
+__device__ __forceinline__ void phase_scatter(const RA<R> *x, unsigned char *sm, const uint32_t *idx, bool pairs) {
     if (sizeof(R) == 4 && pairs) {
 #pragma unroll
         for (int v = 0; v < 16; v += 2) {
             ulonglong2 w;
             memcpy(&w.x, &x[v], 8);
             memcpy(&w.y, &x[v + 1], 8);
-            *reinterpret_cast<ulonglong2 *>(&tile[idx[v]]) = w;
+            *reinterpret_cast<ulonglong2 *>(sm + idx[v]) = w;
         }
     } else {
 #pragma unroll
-        for (int v = 0; v < 16; ++v) tile[idx[v]] = x[v];
+        for (int v = 0; v < 16; ++v) *reinterpret_cast<RA<R> *>(sm + idx[v]) = x[v];
     }
 }
 
 // 16-byte copies of a tile between global memory and its swizzled place
 template <typename R>
-__device__ __forceinline__ void reg_tile_load(RA<R> *tile, const Cx<R> *src, const ChunkOff *chunk, uint32_t slot) {
+__device__ __forceinline__ void reg_tile_load(unsigned char *sm, const Cx<R> *src, const ChunkOff *chunk, uint32_t place) {
     constexpr int C = (int)sizeof(Cx<R>);   // 16 / P chunks
 #pragma unroll
-    for (int i = 0; i < C; ++i) cp_async16(&tile[slot ^ chunk[i].s], src + chunk[i].g);
+    for (int i = 0; i < C; ++i) cp_async16(sm + (place ^ chunk[i].s), src + chunk[i].g);
 }
 template <typename R>
-__device__ __forceinline__ void reg_tile_store(Cx<R> *dst, const RA<R> *tile, const ChunkOff *chunk, uint32_t slot,
+__device__ __forceinline__ void reg_tile_store(Cx<R> *dst, const unsigned char *sm, const ChunkOff *chunk, uint32_t place,
                                                R f) {
     constexpr int C = (int)sizeof(Cx<R>);
 #pragma unroll
     for (int i = 0; i < C; ++i) {
         const ChunkOff c = chunk[i];
         if constexpr (sizeof(R) == 4) {
-            float4 v = *reinterpret_cast<const float4 *>(&tile[slot ^ c.s]);
+            float4 v = *reinterpret_cast<const float4 *>(sm + (place ^ c.s));
             v.x *= f; v.y *= f; v.z *= f; v.w *= f;
             *reinterpret_cast<float4 *>(dst + c.g) = v;
         } else {
-            const double2 v = tile[slot ^ c.s];
+            const double2 v = *reinterpret_cast<const double2 *>(sm + (place ^ c.s));
             dst[c.g] = make_double2(v.x * f, v.y * f);
+        }
+    }
+}
+
+template <typename R, int KIND>
+__device__ __forceinline__ void fwd_steps(RA<R> *x, const PhaseS &F, const GatePassArgs &a, const RegStep *st,
+                                          const Cx<R> *cs, const Cx<R> *rk, const DiagBlock *bl,
+                                          const unsigned char *area, uint32_t thread, uint32_t place, uint64_t gbase,
+                                          const Cx<R> *pmats) {
+    constexpr int RB = kRegBits, V = 1 << RB;
+    if constexpr (KIND == kStepsPair) {
+        for (int i = F.st_begin; i < F.st_end; ++i) {       // step i is operation i of the pass
+            uint32_t code;
+            const RotK<R> k = pair_rec<R>(rk + 4 * i, code);
+            switch (code) {
+#define SV_C(MU, MV) ra_pair_rot<R, V, MU, MV>(x, k)
+                SV_RO_GIVENS(SV_C)
+#undef SV_C
+            default: break;
+            }
+        }
+        return;
+    }
+    for (int s = F.st_begin; s < F.st_end; ++s) {
+        const RegStep S = st[s];
+        if (S.type == SV_STEP_ROT) {
+            // factored RYs (t, t): the factors are applied at the store
+            const Cx<R> *c = cs + (S.op_begin - a.op_begin);
+#pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                if (!((S.a >> b) & 1)) continue;
+                const Cx<R> k = *c++;
+                ra_rotf_bit<R, V, RB>(x, b, (S.a >> (8 + b)) & 1, rotf<R>(k));
+            }
+        } else if (S.type == SV_STEP_DIAG) {
+            reg_diag<R, RB>(x, bl[S.a - a.db_begin], area, thread);
+        } else {
+            const uint32_t code = (uint32_t)S.a & 255u, t0 = ((uint32_t)S.a >> 8) & 255u, t1 = ((uint32_t)S.a >> 16) & 255u;
+            const uint32_t base = phase_bits<R>(place);
+            if (code == RO_RZ) {
+                reg_rz<R>(x, cs[S.op_begin], diag_bit_mask(t0, F.rmask, base, gbase));
+            } else if (code == RO_CZ) {
+                reg_cz<R>(x, diag_bit_mask(t0, F.rmask, base, gbase) & diag_bit_mask(t1, F.rmask, base, gbase));
+            } else if constexpr (KIND == kStepsAll) {
+                const Cx<R> *M = pmats + S.op_end;
+                uint32_t pc = 0;
+                RotK<R> k{};
+                if (code < RO_MAT1) k = pair_rec<R>(rk + 4 * S.op_begin, pc);
+                switch (code) {
+#define SV_C(MU, MV) ra_pair_rot<R, V, MU, MV>(x, k)
+                    SV_RO_GIVENS(SV_C)
+#undef SV_C
+                case RO_MAT1: reg_mat<R, 0, 0>(x, M); break;
+                case RO_MAT1 + 1: reg_mat<R, 1, 1>(x, M); break;
+                case RO_MAT1 + 2: reg_mat<R, 2, 2>(x, M); break;
+                case RO_MAT1 + 3: reg_mat<R, 3, 3>(x, M); break;
+                case RO_MAT2: reg_mat<R, 0, 1>(x, M); break;
+                case RO_MAT2 + 1: reg_mat<R, 0, 2>(x, M); break;
+                case RO_MAT2 + 2: reg_mat<R, 0, 3>(x, M); break;
+                case RO_MAT2 + 3: reg_mat<R, 1, 2>(x, M); break;
+                case RO_MAT2 + 4: reg_mat<R, 1, 3>(x, M); break;
+                case RO_MAT2 + 5: reg_mat<R, 2, 3>(x, M); break;
+                case RO_MAT4: reg_mat4<R>(x, M); break;
+                default: break;
+                }
+            }
+        }
+    }
+}
+
+// The steps of a phase in reverse on psi and lambda: per parametric operation
+// the gradient part Im<lambda|G|psi> (Y of an RY, the subspace Y of a pair
+// rotation, Z of an RZ) into the warp's slot, then U^dagger on both.  Factored
+// RYs: before step s both sets hold the true vectors divided by scf[s].
+template <typename R, int KIND>
+__device__ __forceinline__ void adj_steps(RA<R> *xp, RA<R> *xl, const PhaseS &F, const GatePassArgs &a, const RegStep *st,
+                                          const Cx<R> *cs, const Cx<R> *rk, const DiagBlock *bl, const DiagMember *mem,
+                                          const R *scf, const unsigned char *area, uint32_t place, uint64_t gbase,
+                                          const Cx<R> *pmats, R *acc) {
+    constexpr int RB = kRegBits, V = 1 << RB, AS = kAdjSlotStride;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if constexpr (KIND == kStepsPair) {
+        // four operations' parts share a warp reduction (no factored RYs here)
+        R g0 = 0, g1 = 0, g2 = 0, g3 = 0;
+        int held = 0;
+        for (int i = F.st_end - 1; i >= F.st_begin; --i) {
+            uint32_t code;
+            const RotK<R> k = pair_rec<R>(rk + 4 * i, code);
+            g3 = g2;
+            g2 = g1;
+            g1 = g0;
+            g0 = 0;
+            switch (code) {
+#define SV_C(MU, MV)                                  \
+    g0 = ra_pair_grad<R, V, MU, MV>(xp, xl);          \
+    ra_pair_rot<R, V, MU, MV>(xp, k);                 \
+    ra_pair_rot<R, V, MU, MV>(xl, k)
+                SV_RO_GIVENS(SV_C)
+#undef SV_C
+            default: break;
+            }
+            if (++held == 4 || i == F.st_begin) {
+                const R red = warp_sum4<R>(g0, g1, g2, g3);
+                if ((lane & 7) == 0 && (lane >> 3) < held) acc[(i + (lane >> 3)) * AS + warp] += red;
+                g0 = g1 = g2 = 0;
+                held = 0;
+            }
+        }
+        return;
+    }
+    for (int s = F.st_end - 1; s >= F.st_begin; --s) {
+        const RegStep S = st[s];
+        const R fs = scf[s], fs2 = fs * fs;
+        if (S.type == SV_STEP_ROT) {
+            // every RY of the step: gradient part at the step's end (they commute), then RY^dagger
+            R g[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                if (!((S.a >> b) & 1)) continue;
+                switch (b) {
+                case 0: g[0] = ra_ry_grad<R, V, 0>(xp, xl); break;
+                case 1: g[1] = ra_ry_grad<R, V, 1>(xp, xl); break;
+                case 2: g[2] = ra_ry_grad<R, V, 2>(xp, xl); break;
+                default: g[3] = ra_ry_grad<R, V, 3>(xp, xl); break;
+                }
+            }
+            const R tot = warp_sum4<R>(g[0], g[1], g[2], g[3]) * fs2;
+            const Cx<R> *c = cs + (S.op_begin - a.op_begin);
+            int o = S.op_begin - a.op_begin;
+#pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                if (!((S.a >> b) & 1)) continue;
+                if (lane == 8 * b) acc[o * AS + warp] += tot;
+                ++o;
+                const Cx<R> k = *c++;
+                const RotF<R> rf = rotf<R>(k);
+                const bool fb = (S.a >> (8 + b)) & 1;
+                ra_rotf_bit<R, V, RB>(xp, b, fb, rf);
+                ra_rotf_bit<R, V, RB>(xl, b, fb, rf);
+            }
+        } else if (S.type == SV_STEP_DIAG) {
+            // every RZ member's generator expectation at the block's end (Z
+            // commutes with the block), then D^dagger on both register sets
+            const DiagBlock B = bl[S.a - a.db_begin];
+            R tv[V], tot = 0;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                tv[v] = ra_imdot<R>(xl[v], xp[v]);
+                tot += tv[v];
+            }
+            if (B.kind == 0) {
+                R sb[4] = {0, 0, 0, 0};
+                signed_bit_sums<R, RB>(tv, sb);
+                const R red = warp_sum4<R>(sb[0], sb[1], sb[2], sb[3]) * fs2;
+                for (int mi = B.m_begin; mi < B.m_end; ++mi) {
+                    const DiagMember m = mem[mi - a.mem_begin];
+                    if (m.type == SV_DM_REG_RZ && lane == 8 * m.a) acc[(m.op - a.op_begin) * AS + warp] += red;
+                }
+            } else {
+                // thread RZ members: +-tot by the thread's bit, four at a time
+                const uint32_t base = phase_bits<R>(place);
+                for (int m0 = B.m_begin; m0 < B.m_end; m0 += 4) {
+                    R vals[4] = {0, 0, 0, 0};
+                    int opi[4] = {-1, -1, -1, -1};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (m0 + j < B.m_end) {
+                            const DiagMember m = mem[m0 + j - a.mem_begin];
+                            if (m.type == SV_DM_THR_RZ) {
+                                vals[j] = ((base >> m.a) & 1u) ? -tot : tot;
+                                opi[j] = m.op - a.op_begin;
+                            }
+                        }
+                    }
+                    const R red = warp_sum4<R>(vals[0], vals[1], vals[2], vals[3]) * fs2;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (lane == 8 * j && opi[j] >= 0) acc[opi[j] * AS + warp] += red;
+                }
+            }
+            reg_diag2<R, RB>(xp, xl, B, area);
+        } else {
+            const uint32_t code = (uint32_t)S.a & 255u, t0 = ((uint32_t)S.a >> 8) & 255u, t1 = ((uint32_t)S.a >> 16) & 255u;
+            const uint32_t base = phase_bits<R>(place);
+            if (code == RO_RZ) {
+                const uint32_t m = diag_bit_mask(t0, F.rmask, base, gbase);
+                R g = 0;
+#pragma unroll
+                for (int v = 0; v < V; ++v) g += flip_by(ra_imdot<R>(xl[v], xp[v]), m, v);
+                const Cx<R> k = cs[S.op_begin];
+                reg_rz<R>(xp, k, m);
+                reg_rz<R>(xl, k, m);
+                g = warp_sum<R>(g) * fs2;
+                if (lane == 0) acc[S.op_begin * AS + warp] += g;
+            } else if (code == RO_CZ) {
+                const uint32_t m = diag_bit_mask(t0, F.rmask, base, gbase) & diag_bit_mask(t1, F.rmask, base, gbase);
+                reg_cz<R>(xp, m);
+                reg_cz<R>(xl, m);
+            } else if constexpr (KIND == kStepsAll) {
+                // the prepared matrix is followed by its conjugate transpose (1-qubit matrices: 4 elements)
+                const Cx<R> *M = pmats + S.op_end + 4;
+                uint32_t pc = 0;
+                RotK<R> k{};
+                R g = 0;
+                if (code < RO_MAT1) k = pair_rec<R>(rk + 4 * S.op_begin, pc);
+                switch (code) {
+#define SV_C(MU, MV)                                  \
+    g = ra_pair_grad<R, V, MU, MV>(xp, xl);           \
+    ra_pair_rot<R, V, MU, MV>(xp, k);                 \
+    ra_pair_rot<R, V, MU, MV>(xl, k)
+                    SV_RO_GIVENS(SV_C)
+#undef SV_C
+                case RO_MAT1: reg_mat<R, 0, 0>(xp, M); reg_mat<R, 0, 0>(xl, M); break;
+                case RO_MAT1 + 1: reg_mat<R, 1, 1>(xp, M); reg_mat<R, 1, 1>(xl, M); break;
+                case RO_MAT1 + 2: reg_mat<R, 2, 2>(xp, M); reg_mat<R, 2, 2>(xl, M); break;
+                case RO_MAT1 + 3: reg_mat<R, 3, 3>(xp, M); reg_mat<R, 3, 3>(xl, M); break;
+                default: break;
+                }
+                if (code < RO_MAT1) {
+                    g = warp_sum<R>(g) * fs2;
+                    if (lane == 0) acc[S.op_begin * AS + warp] += g;
+                }
+            }
         }
     }
 }
@@ -1687,7 +1849,7 @@ __device__ __forceinline__ void reg_tile_store(Cx<R> *dst, const RA<R> *tile, co
 // HBM.  So everything that does not depend on the amplitudes is done once per
 // call (k_reg_image) or kept as per-chunk constants, tiles move by 16-byte
 // accesses, and a step's operation is one switch on a decoded code.
-template <typename R>
+template <typename R, int KIND>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256, 1)
 k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *__restrict__ image,
            const Cx<R> *__restrict__ pmats, int early) {
@@ -1695,7 +1857,7 @@ k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *_
     constexpr uint32_t P = 16 / sizeof(Cx<R>);
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t T = 1u << a.k;
-    RA<R> *tiles = reinterpret_cast<RA<R> *>(smem);          // two tiles: the next one streams in
+    const uint32_t tbytes = T * (uint32_t)sizeof(RA<R>);     // two tiles: the next one streams in
     unsigned char *sm = smem + 2 * T * sizeof(RA<R>);
     const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), false);
     // early: the tables were complete before the kernel before this one began
@@ -1711,57 +1873,42 @@ k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *_
     const DiagBlock *bl = reinterpret_cast<const DiagBlock *>(sm + L.blocks);
     const PhaseS *phs = reinterpret_cast<const PhaseS *>(sm + L.phases);
     const uint16_t *pbase = reinterpret_cast<const uint16_t *>(sm + L.pbase);
-    const uint16_t *prb = reinterpret_cast<const uint16_t *>(sm + L.prb);
+    const uint4 *prb = reinterpret_cast<const uint4 *>(sm + L.prb);
+    const Cx<R> *rk = reinterpret_cast<const Cx<R> *>(sm + L.rk);
     const unsigned char *area = sm + L.area;
     const int NT = blockDim.x, nph = a.ph_end - a.ph_begin;
     const uint64_t ntiles = 1ull << a.nout;
     const uint64_t mine = blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-    const uint32_t j0 = P * threadIdx.x, slot = swz_tile(j0);
+    const uint32_t j0 = P * threadIdx.x, slot = swz_tile(j0) * (uint32_t)sizeof(RA<R>);
     Cx<R> *mypsi = psi + (hioff[j0 >> a.nlow] | (j0 & ((1u << a.nlow) - 1u)));
     // tile bases walked with masked additions (current, and two ahead)
     const BitWalk bw = bit_walk(a.out, a.nout, gridDim.x);
     uint64_t base_pf = deposit(blockIdx.x, a.out, a.nout), base_cur = base_pf;
     for (uint64_t k = 0; k < 2; ++k) {
-        if (k < mine) reg_tile_load<R>(tiles + k * T, mypsi + base_pf, chunk, slot);
+        if (k < mine) reg_tile_load<R>(smem, mypsi + base_pf, chunk, slot + (uint32_t)k * tbytes);
         cp_async_commit();
         base_pf = walk_next(base_pf, bw);
     }
     for (uint64_t it = 0; it < mine; ++it) {
         const uint64_t gbase = base_cur;
         base_cur = walk_next(base_cur, bw);
-        RA<R> *tile = tiles + (it & 1) * T;
+        const uint32_t tile = (uint32_t)(it & 1) * tbytes;
         cp_async_wait1();
         __syncthreads();
         for (int ph = 0; ph < nph; ++ph) {
             const PhaseS F = phs[ph];
-            const uint32_t base = pbase[ph * NT + threadIdx.x];
+            const uint32_t place = pbase[ph * NT + threadIdx.x];
             uint32_t idx[V];
-            phase_slots16(idx, base, prb + ph * 4);
+            phase_slots16(idx, place | tile, prb[ph]);
             RA<R> x[V];
-            phase_gather<R>(x, tile, idx, F.rmask & 1u);
-            for (int s = F.st_begin; s < F.st_end; ++s) {
-                const RegStep S = st[s];
-                if (S.type == SV_STEP_ROT) {
-                    // factored RYs (t, factor): the factors are applied at the store
-                    const Cx<R> *c = cs + (S.op_begin - a.op_begin);
-#pragma unroll
-                    for (int b = 0; b < RB; ++b) {
-                        if (!((S.a >> b) & 1)) continue;
-                        const Cx<R> k = *c++;
-                        ra_rotf_bit<R, V, RB>(x, b, (S.a >> (8 + b)) & 1, rotf<R>(k.x));
-                    }
-                } else if (S.type == SV_STEP_DIAG) {
-                    reg_diag<R, RB>(x, bl[S.a - a.db_begin], area, threadIdx.x);
-                } else {
-                    reg_op<R, true>(x, (uint32_t)S.a, F.rmask, base, gbase, cs[S.op_begin], pmats + S.op_end);
-                }
-            }
-            phase_scatter<R>(x, tile, idx, F.rmask & 1u);
+            phase_gather<R>(x, smem, idx, F.rmask & 1u);
+            fwd_steps<R, KIND>(x, F, a, st, cs, rk, bl, area, threadIdx.x, place, gbase, pmats);
+            phase_scatter<R>(x, smem, idx, F.rmask & 1u);
             __syncthreads();
         }
-        reg_tile_store<R>(mypsi + gbase, tile, chunk, slot, ftot);
+        reg_tile_store<R>(mypsi + gbase, smem, chunk, slot + tile, ftot);
         // a thread reloads exactly the slots it has just stored from
-        if (it + 2 < mine) reg_tile_load<R>(tile, mypsi + base_pf, chunk, slot);
+        if (it + 2 < mine) reg_tile_load<R>(smem, mypsi + base_pf, chunk, slot + tile);
         cp_async_commit();
         base_pf = walk_next(base_pf, bw);
     }
@@ -1775,7 +1922,7 @@ k_gate_reg(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *_
 // of which 1024 are shared memory and 1280 issue.  The second tile's room is
 // the first kernel's prefetch buffer, so the passes of few phases, which HBM
 // bounds, stay with that one (gate_two_pays).
-template <typename R>
+template <typename R, int KIND>
 __global__ void __launch_bounds__(1024, 1)
 k_gate_two(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *__restrict__ image, int early) {
     constexpr int RB = kRegBits, V = 1 << RB;
@@ -1783,7 +1930,7 @@ k_gate_two(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *_
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t T = 1u << a.k, NT = T >> RB;
     const uint32_t grp = threadIdx.x >> (a.k - RB), th = threadIdx.x & (NT - 1u);
-    RA<R> *tile = reinterpret_cast<RA<R> *>(smem) + grp * T;
+    const uint32_t tile = grp * T * (uint32_t)sizeof(RA<R>);
     unsigned char *sm = smem + 2 * T * sizeof(RA<R>);
     const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), false);
     if (!early) pdl_wait();
@@ -1798,62 +1945,47 @@ k_gate_two(Cx<R> *__restrict__ psi, const GatePassArgs a, const unsigned char *_
     const DiagBlock *bl = reinterpret_cast<const DiagBlock *>(sm + L.blocks);
     const PhaseS *phs = reinterpret_cast<const PhaseS *>(sm + L.phases);
     const uint16_t *pbase = reinterpret_cast<const uint16_t *>(sm + L.pbase);
-    const uint16_t *prb = reinterpret_cast<const uint16_t *>(sm + L.prb);
+    const uint4 *prb = reinterpret_cast<const uint4 *>(sm + L.prb);
+    const Cx<R> *rk = reinterpret_cast<const Cx<R> *>(sm + L.rk);
     const unsigned char *area = sm + L.area;
     const int nph = a.ph_end - a.ph_begin;
     const uint64_t ntiles = 1ull << a.nout, first = blockIdx.x + (uint64_t)gridDim.x * grp, stride = 2ull * gridDim.x;
     const uint64_t mine = first < ntiles ? (ntiles - first + stride - 1) / stride : 0;
-    const uint32_t j0 = P * th, slot = swz_tile(j0);
+    const uint32_t j0 = P * th, slot = swz_tile(j0) * (uint32_t)sizeof(RA<R>);
     Cx<R> *mypsi = psi + (hioff[j0 >> a.nlow] | (j0 & ((1u << a.nlow) - 1u)));
     const BitWalk bw = bit_walk(a.out, a.nout, stride);
     uint64_t gbase = deposit(first, a.out, a.nout);
     auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1u + grp), "r"(NT) : "memory"); };
     for (uint64_t it = 0; it < mine; ++it) {
         // a thread's pieces go to the slots that it stored from last
-        reg_tile_load<R>(tile, mypsi + gbase, chunk, slot);
+        reg_tile_load<R>(smem, mypsi + gbase, chunk, slot + tile);
         cp_async_commit();
         cp_async_wait0();
         group_sync();
         for (int ph = 0; ph < nph; ++ph) {
             const PhaseS F = phs[ph];
-            const uint32_t base = pbase[ph * NT + th];
+            const uint32_t place = pbase[ph * NT + th];
             RA<R> x[V];
             {
                 uint32_t idx[V];
-                phase_slots16(idx, base, prb + ph * 4);
-                phase_gather<R>(x, tile, idx, F.rmask & 1u);
+                phase_slots16(idx, place | tile, prb[ph]);
+                phase_gather<R>(x, smem, idx, F.rmask & 1u);
             }
-            for (int s = F.st_begin; s < F.st_end; ++s) {
-                const RegStep S = st[s];
-                if (S.type == SV_STEP_ROT) {
-                    // factored RYs (t, factor): the factors are applied at the store
-                    const Cx<R> *c = cs + (S.op_begin - a.op_begin);
-#pragma unroll
-                    for (int b = 0; b < RB; ++b) {
-                        if (!((S.a >> b) & 1)) continue;
-                        const Cx<R> k = *c++;
-                        ra_rotf_bit<R, V, RB>(x, b, (S.a >> (8 + b)) & 1, rotf<R>(k.x));
-                    }
-                } else if (S.type == SV_STEP_DIAG) {
-                    reg_diag<R, RB>(x, bl[S.a - a.db_begin], area, th);
-                } else {
-                    reg_op<R, false>(x, (uint32_t)S.a, F.rmask, base, gbase, cs[S.op_begin], nullptr);
-                }
-            }
+            fwd_steps<R, KIND>(x, F, a, st, cs, rk, bl, area, th, place, gbase, nullptr);
             {
                 // the slots again (fewer registers live across the steps)
                 uint32_t idx[V];
-                phase_slots16(idx, pbase[ph * NT + th], prb + ph * 4);
-                phase_scatter<R>(x, tile, idx, F.rmask & 1u);
+                phase_slots16(idx, pbase[ph * NT + th] | tile, prb[ph]);
+                phase_scatter<R>(x, smem, idx, F.rmask & 1u);
             }
             group_sync();
         }
-        reg_tile_store<R>(mypsi + gbase, tile, chunk, slot, ftot);
+        reg_tile_store<R>(mypsi + gbase, smem, chunk, slot + tile, ftot);
         gbase = walk_next(gbase, bw);
     }
 }
 
-template <typename R>
+template <typename R, int KIND>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256, 1)
 k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam, const GatePassArgs a,
           const unsigned char *__restrict__ image, const Cx<R> *__restrict__ pmats, double *__restrict__ part,
@@ -1863,12 +1995,11 @@ k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam, const GatePassArgs a
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t T = 1u << a.k;
     const int nops = a.op_end - a.op_begin, nph = a.ph_end - a.ph_begin;
-    const int NT = blockDim.x, nwarps = NT >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int NT = blockDim.x, nwarps = NT >> 5;
     // slot row stride 17: the lanes 0, 8, 16, 24 that add the four
     // gradients of a step (ops o .. o+3) hit four different banks
     const int AS = kAdjSlotStride;
-    RA<R> *tl = reinterpret_cast<RA<R> *>(smem);           // lambda tile, then the psi tile
-    RA<R> *tp = tl + T;
+    unsigned char *tl = smem, *tp = smem + T * sizeof(RA<R>);   // lambda tile, then the psi tile
     unsigned char *sm = smem + 2 * T * sizeof(RA<R>);
     const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), true);
     R *acc = reinterpret_cast<R *>(sm + L.acc);
@@ -1893,12 +2024,13 @@ k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam, const GatePassArgs a
     const DiagBlock *bl = reinterpret_cast<const DiagBlock *>(sm + L.blocks);
     const PhaseS *phs = reinterpret_cast<const PhaseS *>(sm + L.phases);
     const uint16_t *pbase = reinterpret_cast<const uint16_t *>(sm + L.pbase);
-    const uint16_t *prb = reinterpret_cast<const uint16_t *>(sm + L.prb);
+    const uint4 *prb = reinterpret_cast<const uint4 *>(sm + L.prb);
+    const Cx<R> *rk = reinterpret_cast<const Cx<R> *>(sm + L.rk);
     const unsigned char *area = sm + L.area;
     const DiagMember *mem = reinterpret_cast<const DiagMember *>(sm + L.mem);
     const uint64_t ntiles = 1ull << a.nout;
     const uint64_t mine = blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-    const uint32_t j0 = P * threadIdx.x, slot = swz_tile(j0);
+    const uint32_t j0 = P * threadIdx.x, slot = swz_tile(j0) * (uint32_t)sizeof(RA<R>);
     const uint64_t toff = hioff[j0 >> a.nlow] | (j0 & ((1u << a.nlow) - 1u));
     const BitWalk bw = bit_walk(a.out, a.nout, gridDim.x);
     uint64_t gnext = deposit(blockIdx.x, a.out, a.nout);
@@ -1922,95 +2054,15 @@ k_adj_reg(Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam, const GatePassArgs a
         __syncthreads();
         for (int ph = nph - 1; ph >= 0; --ph) {
             const PhaseS F = phs[ph];
-            const uint32_t base = pbase[ph * NT + threadIdx.x];
+            const uint32_t place = pbase[ph * NT + threadIdx.x];
             uint32_t idx[V];
-            phase_slots16(idx, base, prb + ph * 4);
+            phase_slots16(idx, place, prb[ph]);
             RA<R> xp[V], xl[V];
             phase_gather<R>(xp, tp, idx, F.rmask & 1u);
             phase_gather<R>(xl, tl, idx, F.rmask & 1u);
-            for (int s = F.st_end - 1; s >= F.st_begin; --s) {
-                const RegStep S = st[s];
-                const R fs = scf[s], fs2 = fs * fs;
-                if (S.type == SV_STEP_ROT) {
-                    // every RY of the step: gradient part at the step's end (they commute), then RY^dagger
-                    R g[4] = {0, 0, 0, 0};
-#pragma unroll
-                    for (int b = 0; b < RB; ++b) {
-                        if (!((S.a >> b) & 1)) continue;
-                        switch (b) {
-                        case 0: g[0] = ra_ry_grad<R, V, 0>(xp, xl); break;
-                        case 1: g[1] = ra_ry_grad<R, V, 1>(xp, xl); break;
-                        case 2: g[2] = ra_ry_grad<R, V, 2>(xp, xl); break;
-                        default: g[3] = ra_ry_grad<R, V, 3>(xp, xl); break;
-                        }
-                    }
-                    const R tot = warp_sum4<R>(g[0], g[1], g[2], g[3]) * fs2;
-                    const Cx<R> *c = cs + (S.op_begin - a.op_begin);
-                    int o = S.op_begin - a.op_begin;
-#pragma unroll
-                    for (int b = 0; b < RB; ++b) {
-                        if (!((S.a >> b) & 1)) continue;
-                        if (lane == 8 * b) acc[o * AS + warp] += tot;
-                        ++o;
-                        const Cx<R> k = *c++;
-                        const RotF<R> rk = rotf<R>(k.x);
-                        const bool fb = (S.a >> (8 + b)) & 1;
-                        ra_rotf_bit<R, V, RB>(xp, b, fb, rk);
-                        ra_rotf_bit<R, V, RB>(xl, b, fb, rk);
-                    }
-                } else if (S.type == SV_STEP_DIAG) {
-                    // every RZ member's generator expectation at the block's end (Z
-                    // commutes with the block), then D^dagger on both register sets
-                    const DiagBlock B = bl[S.a - a.db_begin];
-                    R tv[V], tot = 0;
-#pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        tv[v] = ra_imdot<R>(xl[v], xp[v]);
-                        tot += tv[v];
-                    }
-                    if (B.kind == 0) {
-                        R sb[4] = {0, 0, 0, 0};
-                        signed_bit_sums<R, RB>(tv, sb);
-                        const R red = warp_sum4<R>(sb[0], sb[1], sb[2], sb[3]) * fs2;
-                        for (int mi = B.m_begin; mi < B.m_end; ++mi) {
-                            const DiagMember m = mem[mi - a.mem_begin];
-                            if (m.type == SV_DM_REG_RZ && lane == 8 * m.a)
-                                acc[(m.op - a.op_begin) * AS + warp] += red;
-                        }
-                    } else {
-                        // thread RZ members: +-tot by the thread's bit, four at a time
-                        for (int m0 = B.m_begin; m0 < B.m_end; m0 += 4) {
-                            R vals[4] = {0, 0, 0, 0};
-                            int opi[4] = {-1, -1, -1, -1};
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                if (m0 + j < B.m_end) {
-                                    const DiagMember m = mem[m0 + j - a.mem_begin];
-                                    if (m.type == SV_DM_THR_RZ) {
-                                        vals[j] = ((base >> m.a) & 1u) ? -tot : tot;
-                                        opi[j] = m.op - a.op_begin;
-                                    }
-                                }
-                            }
-                            const R red = warp_sum4<R>(vals[0], vals[1], vals[2], vals[3]) * fs2;
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                if (lane == 8 * j && opi[j] >= 0) acc[opi[j] * AS + warp] += red;
-                        }
-                    }
-                    reg_diag2<R, RB>(xp, xl, B, area);
-                } else {
-                    // the prepared matrix is followed by its conjugate transpose (1-qubit matrices: 4 elements)
-                    R g = reg_op_adj<R>(xp, xl, (uint32_t)S.a, F.rmask, base, gbase, cs[S.op_begin],
-                                        pmats + S.op_end + 4);
-                    if (reg_op_param((uint32_t)S.a)) {
-                        g = warp_sum<R>(g) * fs2;
-                        if (lane == 0) acc[S.op_begin * AS + warp] += g;
-                    }
-                }
-            }
+            adj_steps<R, KIND>(xp, xl, F, a, st, cs, rk, bl, mem, scf, area, place, gbase, pmats, acc);
             // the slots again (fewer registers live across the steps)
-            phase_slots16(idx, pbase[ph * NT + threadIdx.x], prb + ph * 4);
+            phase_slots16(idx, pbase[ph * NT + threadIdx.x], prb[ph]);
             phase_scatter<R>(xp, tp, idx, F.rmask & 1u);
             phase_scatter<R>(xl, tl, idx, F.rmask & 1u);
             __syncthreads();
@@ -4918,14 +4970,15 @@ size_t adj_reg_smem(sv_dtype dt, const GatePassArgs &a) {
     return 2 * ((size_t)1 << a.k) * amp + reg_layout(a, amp, true).total;
 }
 
-// Two tiles in work per CTA from kTwoPhases phases on (1-qubit matrices may
-// stay, they are one row product): see k_gate_two.
-#ifndef KTWO
-#define KTWO 3
-#endif
-constexpr int kTwoPhases = KTWO;
+// the step loop for what a pass holds
+static int steps_kind(const GatePassArgs &a) {
+    if (a.dense || a.mat1) return kStepsAll;
+    return !a.pairs ? kStepsDiag : a.others ? kStepsAll : kStepsPair;
+}
+// Two tiles in work per CTA from this many phases on: see k_gate_two.
+constexpr int kTwoPhases = 3;
 static bool gate_two_pays(sv_dtype dt, const GatePassArgs &a) {
-    return dt == SV_C64 && !a.dense && !a.mat1 && a.ph_end - a.ph_begin >= kTwoPhases;
+    return dt == SV_C64 && steps_kind(a) != kStepsAll && a.ph_end - a.ph_begin >= kTwoPhases;
 }
 
 int reg_pass_grid(sv_dtype dt, const GatePassArgs &a, bool adj, int blocks_per_sm) {
@@ -4946,16 +4999,19 @@ cudaError_t gate_reg_dispatch(cudaStream_t st, int grid, void *psi, const GatePa
     const size_t sm = gate_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
     const int nt = 1 << (a.k - kRegBits);
     if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
+    auto go = [&](auto kernel, int threads, auto... more) {
+        allow_smem(kernel, sm);
+        return launch(kernel, grid, threads, sm, st, (Cx<R> *)psi, a, (const unsigned char *)image, more..., early ? 1 : 0);
+    };
+    const int kind = steps_kind(a);
+    const Cx<R> *pm = (const Cx<R> *)pmats;
     if constexpr (sizeof(R) == 4) {
-        if (gate_two_pays(SV_C64, a)) {
-            allow_smem(k_gate_two<float>, sm);
-            return launch(k_gate_two<float>, grid, 2 * nt, sm, st, (float2 *)psi, a, (const unsigned char *)image,
-                          early ? 1 : 0);
-        }
+        if (gate_two_pays(SV_C64, a))
+            return kind == kStepsPair ? go(k_gate_two<R, kStepsPair>, 2 * nt) : go(k_gate_two<R, kStepsDiag>, 2 * nt);
     }
-    allow_smem(k_gate_reg<R>, sm);
-    return launch(k_gate_reg<R>, grid, nt, sm, st, (Cx<R> *)psi, a, (const unsigned char *)image,
-                  (const Cx<R> *)pmats, early ? 1 : 0);
+    if (kind == kStepsPair) return go(k_gate_reg<R, kStepsPair>, nt, pm);
+    if (kind == kStepsDiag) return go(k_gate_reg<R, kStepsDiag>, nt, pm);
+    return go(k_gate_reg<R, kStepsAll>, nt, pm);
 }
 
 template <typename R>
@@ -4964,9 +5020,15 @@ cudaError_t adj_reg_dispatch(cudaStream_t st, int grid, void *psi, void *lam, co
     const size_t sm = adj_reg_smem(sizeof(R) == 4 ? SV_C64 : SV_C128, a);
     const int nt = 1 << (a.k - kRegBits);
     if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
-    allow_smem(k_adj_reg<R>, sm);
-    return launch(k_adj_reg<R>, grid, nt, sm, st, (Cx<R> *)psi, (Cx<R> *)lam, a, (const unsigned char *)image,
-                  (const Cx<R> *)pmats, part, part_stride, early ? 1 : 0);
+    auto go = [&](auto kernel) {
+        allow_smem(kernel, sm);
+        return launch(kernel, grid, nt, sm, st, (Cx<R> *)psi, (Cx<R> *)lam, a, (const unsigned char *)image,
+                      (const Cx<R> *)pmats, part, part_stride, early ? 1 : 0);
+    };
+    const int kind = steps_kind(a);
+    if (kind == kStepsPair) return go(k_adj_reg<R, kStepsPair>);
+    if (kind == kStepsDiag) return go(k_adj_reg<R, kStepsDiag>);
+    return go(k_adj_reg<R, kStepsAll>);
 }
 
 size_t reg_image_bytes(sv_dtype dt, const GatePassArgs &a) {

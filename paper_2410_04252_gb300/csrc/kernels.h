@@ -20,6 +20,8 @@ struct GatePassArgs {
     int st_begin, st_end;    // steps of the pass's register phases
     int area;                // bytes of the diagonal-block data
     int mem_begin, mem_end;  // diagonal-block members of the pass
+    int pairs;               // the phases hold pair rotations (Givens, double excitations)
+    int others;              // and gates besides pair rotations
     int mat1;                // the phases hold 1-qubit matrices
     int dense;               // the phases hold 2- or 4-qubit matrices (the reverse pass runs in k_adj_pass)
     int8_t hi[40];

@@ -509,6 +509,8 @@ void plan_phases(QsuPlan &P, bool pairs, int threads) {
             if (kd != SV_RY && kd != SV_RZ && kd != SV_CZ && kd != SV_MAT1 && !(pairs && pair)) ok = false;
             if (kd == SV_MAT2 || kd == SV_MAT4) dense = true;
             if (kd == SV_MAT1) gp.mat1 = 1;
+            if (kd == SV_GIVENS || kd == SV_DEXC) gp.pairs = 1;
+            else gp.others = 1;
         }
         if (!ok) continue;
         gp.dense = dense;
@@ -615,7 +617,7 @@ void plan_steps(QsuPlan &P, int max_diag, int amp) {
         gp.db_begin = gp.db_end = (int32_t)P.dblocks.size();
         if (gp.ph_begin < 0) continue;
         const int nops = gp.op_end - gp.op_begin;
-        int budget = kRegSmemLimit - reg_pass_fixed_bytes(gp.k, gp.nlow, nops, nops, gp.ph_end - gp.ph_begin, amp);
+        int budget = kRegSmemLimit - reg_pass_fixed_bytes(gp.k, gp.nlow, nops, nops, gp.ph_end - gp.ph_begin, amp, gp.pairs != 0);
         int area = 0;   // bytes of the pass's block area handed out so far
         auto take_block = [&](int kind) {
             const int need = diag_block_bytes(kind, gp.k, amp);

@@ -65,6 +65,8 @@ struct GatePass {
     uint64_t bits = 0;                // physical staged bits
     int32_t op_begin = 0, op_end = 0; // into QsuPlan::ops
     int32_t ph_begin = -1, ph_end = -1;  // register phases (register-blocked passes), else -1
+    int32_t pairs = 0;                   // 1: the phases hold pair rotations
+    int32_t others = 0;                  // 1: the phases hold gates besides pair rotations
     int32_t mat1 = 0;                    // 1: the phases hold 1-qubit matrices
     int32_t dense = 0;                   // 1: the phases hold 2- or 4-qubit matrices (forward only)
     int32_t db_begin = 0, db_end = 0;    // diagonal blocks of the pass (register-blocked passes)
@@ -147,14 +149,14 @@ inline int diag_block_bytes(int kind, int k, int amp) {
     const int V = 1 << kRegBits, NT = 1 << (k - kRegBits);
     return kind == 0 ? V * V * amp + NT : NT * amp;
 }
-inline int reg_pass_fixed_bytes(int k, int nlow, int nops, int nsteps, int nphases, int amp) {
+inline int reg_pass_fixed_bytes(int k, int nlow, int nops, int nsteps, int nphases, int amp, bool pairs) {
     // adjoint (the larger): psi and lambda tiles, high offsets, chunk offsets,
     // (c, s) per op, steps, block headers and members, phases with their
     // thread bases and register offsets, per-warp gradient slots, the RY
-    // factor per step, alignment
+    // factor per step, pair rotations' coefficients, alignment
     return 2 * (1 << k) * amp + 8 * (1 << (k - nlow)) + 256 + nops * amp + 16 * nsteps + 32 * kMaxPassDiag +
-           16 * nops + nphases * (2 * (1 << (k - kRegBits)) + 8 + 32) + nops * kAdjSlotStride * 8 +
-           8 * (nsteps + 1) + 320;
+           16 * nops + nphases * (2 * (1 << (k - kRegBits)) + 16 + 16) + nops * kAdjSlotStride * 8 +
+           8 * (nsteps + 1) + (pairs ? 4 * amp * nops : 0) + 320;
 }
 struct RegStep {
     int32_t type, a;
