@@ -21,14 +21,17 @@ class VQEEnergy(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, params, sim, circ, ham, schedule, init_index):
-        p = params.detach().to("cpu", torch.float64).numpy()
+        p = params.detach().cpu().numpy().astype(np.float64)
         sim.reset(init_index)
         if isinstance(ham, tuple):
             e, g = sim.grad(circ, p, paulis=ham[0], coeffs=ham[1], schedule=schedule)
         else:
             e, g = sim.grad(circ, p, ham, schedule=schedule)
-        ctx.save_for_backward(torch.from_numpy(np.ascontiguousarray(g)).to(params.device, params.dtype))
-        return params.new_tensor(e)
+        # one copy to the device: the gradient, then the energy (which leaves it
+        # as a tensor of its own)
+        both = torch.from_numpy(np.append(g, e)).to(params.dtype).to(params.device)
+        ctx.save_for_backward(both[:-1])
+        return both[-1].clone()
 
     @staticmethod
     def backward(ctx, grad_output):

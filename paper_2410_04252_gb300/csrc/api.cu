@@ -158,6 +158,7 @@ struct EvcEntry {
 };
 
 constexpr size_t kCacheSize = 6;
+constexpr size_t kResHead = 4;
 
 }  // namespace
 
@@ -176,7 +177,11 @@ struct sv_handle {
     uint64_t tick = 0;
     std::vector<std::unique_ptr<QsuEntry>> qsu;
     std::vector<std::unique_ptr<EvcEntry>> evc, hps;
-    DevBuf params, coef, mats, pmats, images, part, slotval, opval, grad, scal, per_term, status;
+    DevBuf params, coef, mats, pmats, images, part, slotval, opval, res;
+    // res, read back by one copy per call: [0] EVC energy, [1] Re<psi|H|psi>,
+    // [2] the kernels' status word, from [kResHead] on the per-term values or
+    // the gradient of the call
+    std::vector<double> back;
     // forward bookkeeping for SV_FORWARD_DONE
     uint64_t last_qsu_key = 0;
     bool forward_valid = false;
@@ -680,7 +685,33 @@ sv_status run_forward(sv_handle *h, QsuEntry *q, sv_stats *st) {
     return SV_OK;
 }
 
-sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, sv_stats *st) {
+// The result buffer with room for `values` doubles; a new one starts with a
+// clear status word (bounded waits of the coset kernels).
+sv_status res_room(sv_handle *h, size_t values) {
+    const size_t bytes = (kResHead + values) * sizeof(double);
+    if (h->res.p && h->res.cap >= bytes) return SV_OK;
+    SV_CK(h->res.ensure(bytes));
+    SV_CK(cudaMemsetAsync(h->res.p, 0, kResHead * sizeof(double), h->stream));
+    return SV_OK;
+}
+int *res_status(sv_handle *h) { return (int *)(h->res.as<double>() + 2); }
+
+// Waits for the call's work and brings its head and `values` doubles back.
+sv_status read_back(sv_handle *h, size_t values) {
+    h->back.resize(kResHead + values);
+    SV_CK(cudaMemcpyAsync(h->back.data(), h->res.p, h->back.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    SV_CK(cudaStreamSynchronize(h->stream));
+    int v;
+    memcpy(&v, &h->back[2], sizeof(int));
+    if (v) {
+        SV_CK(cudaMemsetAsync(res_status(h), 0, sizeof(int), h->stream));
+        return fail(SV_ETIMEOUT, "a device wait for a bulk copy expired");
+    }
+    return SV_OK;
+}
+
+// energy and per-term values into h->res
+sv_status run_evc(sv_handle *h, EvcEntry *e, sv_stats *st) {
     const EvcPlan &P = e->plan;
     const int nslots = (int)P.strings.size();
     int E = 1;
@@ -691,8 +722,6 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
     const int grid = slices ? 1 << e->args[0].nfree : coset_grid(h->dt, E, h->opt.blocks_per_sm, false);
     SV_CK(h->part.ensure((size_t)grid * std::max(nslots, 1) * sizeof(double)));
     SV_CK(h->slotval.ensure(std::max(nslots, 1) * sizeof(double)));
-    SV_CK(h->scal.ensure(4 * sizeof(double)));
-    SV_CK(h->per_term.ensure(std::max(e->nterms, 1) * sizeof(double)));
     for (size_t t = 0; t < P.tiles.size(); ++t) {
         const Tile &T = P.tiles[t];
         if (!T.pairs.empty()) {
@@ -720,7 +749,7 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
                 if (e->rest[pi].g_begin == e->rest[pi].g_end) continue;
             }
             SV_CK(launch_evc_pass(h->dt, h->stream, grid, h->psi, e->rest[pi], e->groups.as<DevGroup>(),
-                                  e->strings.as<DevString>(), h->part.as<double>(), nslots, h->status.as<int>(),
+                                  e->strings.as<DevString>(), h->part.as<double>(), nslots, res_status(h),
                                   (long long)h->opt.wait_limit));
         }
     }
@@ -731,7 +760,7 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
     {
         Rec r(h, st, SV_K_AUX, 0.0);
         SV_CK(launch_energy(h->stream, h->slotval.as<double>(), e->term_slot.as<int32_t>(), e->coeffs.as<double>(),
-                            e->nterms, h->per_term.as<double>(), h->scal.as<double>()));
+                            e->nterms, h->res.as<double>() + kResHead, h->res.as<double>()));
     }
     if (st) {
         st->evc_tiles = (int32_t)P.tiles.size();
@@ -739,14 +768,10 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, double *energy, double *per_term, s
         st->evc_passes = (int32_t)P.passes.size();
     }
     h->l2p = P.final_l2p;
-    if (energy) SV_CK(cudaMemcpyAsync(energy, h->scal.p, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    if (per_term && e->nterms)
-        SV_CK(cudaMemcpyAsync(per_term, h->per_term.p, e->nterms * sizeof(double), cudaMemcpyDeviceToHost,
-                              h->stream));
     return SV_OK;
 }
 
-// lambda = H psi; energy into h->scal[1] (device).
+// lambda = H psi; energy into h->res[1] (device).
 sv_status run_hpsi(sv_handle *h, EvcEntry *e, sv_stats *st) {
     const EvcPlan &P = e->plan;
     SV_TRY(ensure_lam(h));
@@ -755,11 +780,10 @@ sv_status run_hpsi(sv_handle *h, EvcEntry *e, sv_stats *st) {
     const int grid = coset_grid(h->dt, E, h->opt.blocks_per_sm, true);
     SV_CK(h->part.ensure((size_t)std::max(grid, 2 * device_sms()) * sizeof(double) + 64));
     int rows = grid;         // energy partials of the last pass
-    SV_CK(h->scal.ensure(4 * sizeof(double)));
     const int np = (int)P.passes.size();
     if (np == 0) {
         SV_CK(cudaMemsetAsync(h->lam, 0, h->state_bytes(), h->stream));
-        SV_CK(cudaMemsetAsync(h->scal.as<double>() + 1, 0, sizeof(double), h->stream));
+        SV_CK(cudaMemsetAsync(h->res.as<double>() + 1, 0, sizeof(double), h->stream));
         return SV_OK;
     }
     for (int pi = 0; pi < np; ++pi) {
@@ -771,11 +795,11 @@ sv_status run_hpsi(sv_handle *h, EvcEntry *e, sv_stats *st) {
         }
         SV_CK(launch_hpsi_pass(h->dt, h->stream, grid, h->psi, h->lam, e->args[pi], e->groups.as<DevGroup>(),
                                e->strings.as<DevString>(), pi == 0, pi == np - 1, h->part.as<double>(),
-                               h->status.as<int>(), (long long)h->opt.wait_limit));
+                               res_status(h), (long long)h->opt.wait_limit));
     }
     {
         Rec r(h, st, SV_K_AUX, 0.0);
-        SV_CK(launch_reduce_rows(h->stream, h->part.as<double>(), rows, 1, 0, 1, h->scal.as<double>() + 1));
+        SV_CK(launch_reduce_rows(h->stream, h->part.as<double>(), rows, 1, 0, 1, h->res.as<double>() + 1));
     }
     if (st) st->hpsi_passes = np;
     return SV_OK;
@@ -799,7 +823,6 @@ sv_status run_reverse(sv_handle *h, QsuEntry *q, sv_stats *st) {
     }
     SV_CK(h->part.ensure((size_t)grid * std::max(nops, 1) * sizeof(double)));
     SV_CK(h->opval.ensure(std::max(nops, 1) * sizeof(double)));
-    SV_CK(h->grad.ensure(std::max(q->np, 1) * sizeof(double)));
     int pi = (int)P.passes.size() - 1;
     int launched = 0;    // reverse passes so far (the tables may have been made right before the first)
     for (int t = (int)P.tiles.size() - 1; t >= 0; --t) {
@@ -843,7 +866,7 @@ sv_status run_reverse(sv_handle *h, QsuEntry *q, sv_stats *st) {
     {
         Rec r(h, st, SV_K_AUX, 0.0);
         SV_CK(launch_scatter(h->stream, h->opval.as<double>(), q->csr_off.as<int32_t>(), q->csr_idx.as<int32_t>(),
-                             q->np, h->grad.as<double>()));
+                             q->np, h->res.as<double>() + kResHead));
     }
     h->l2p = P.init_l2p;
     return SV_OK;
@@ -851,20 +874,6 @@ sv_status run_reverse(sv_handle *h, QsuEntry *q, sv_stats *st) {
 
 sv_status check_handle(const sv_handle *h) {
     if (!h) return fail(SV_EINVAL, "null handle");
-    return SV_OK;
-}
-
-// Device status word of the coset kernels (bounded waits): cleared before a
-// call's kernels, read after its synchronisation.
-sv_status status_reset(sv_handle *h) {
-    SV_CK(h->status.ensure(sizeof(int)));
-    SV_CK(cudaMemsetAsync(h->status.p, 0, sizeof(int), h->stream));
-    return SV_OK;
-}
-sv_status status_check(sv_handle *h) {
-    int v = 0;
-    SV_CK(cudaMemcpy(&v, h->status.p, sizeof(int), cudaMemcpyDeviceToHost));
-    if (v) return fail(SV_ETIMEOUT, "a device wait for a bulk copy expired");
     return SV_OK;
 }
 
@@ -919,8 +928,7 @@ void sv_destroy(sv_handle *h) {
     for (auto &e : h->qsu) e->release();
     for (auto &e : h->evc) e->release();
     for (auto &e : h->hps) e->release();
-    for (DevBuf *b : {&h->params, &h->coef, &h->mats, &h->pmats, &h->images, &h->part, &h->slotval, &h->opval, &h->grad, &h->scal,
-                      &h->per_term, &h->status})
+    for (DevBuf *b : {&h->params, &h->coef, &h->mats, &h->pmats, &h->images, &h->part, &h->slotval, &h->opval, &h->res})
         b->release();
     h->drop_ckpts();
     for (auto &p : h->pending) { h->ev_pool.push_back(p.a); h->ev_pool.push_back(p.b); }
@@ -1074,12 +1082,13 @@ sv_status sv_expect(sv_handle *h, const sv_pauli *paulis, const double *coeffs, 
     EvcEntry *e = nullptr;
     SV_TRY(check_sched(sched));
     SV_TRY(get_evc(h, paulis, coeffs, nterms, sched, false, &e, st));
-    SV_TRY(status_reset(h));
-    SV_TRY(run_evc(h, e, energy, per_term, st));
+    SV_TRY(res_room(h, nterms));
+    SV_TRY(run_evc(h, e, st));
     if (flags & SV_KEEP_LAYOUT) SV_TRY(relayout(h, entry, false, st));
     else if (h->l2p != entry) h->forward_valid = false;
-    SV_CK(cudaStreamSynchronize(h->stream));
-    SV_TRY(status_check(h));
+    SV_TRY(read_back(h, per_term ? nterms : 0));
+    if (energy) *energy = h->back[0];
+    if (per_term) std::copy(h->back.begin() + kResHead, h->back.end(), per_term);
     SV_TRY(resolve_profile(h, st));
     return SV_OK;
 }
@@ -1093,12 +1102,11 @@ sv_status sv_apply_hamiltonian(sv_handle *h, const sv_pauli *paulis, const doubl
     SV_TRY(ensure_psi(h));
     EvcEntry *e = nullptr;
     SV_TRY(get_evc(h, paulis, coeffs, nterms, SV_SCHED_LAZY, true, &e, st));
-    SV_TRY(status_reset(h));
+    SV_TRY(res_room(h, 0));
     SV_TRY(run_hpsi(h, e, st));
     if (dst) SV_CK(cudaMemcpyAsync(dst, h->lam, h->state_bytes(), cudaMemcpyDeviceToDevice, h->stream));
-    if (energy) SV_CK(cudaMemcpyAsync(energy, h->scal.as<double>() + 1, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    SV_CK(cudaStreamSynchronize(h->stream));
-    SV_TRY(status_check(h));
+    SV_TRY(read_back(h, 0));
+    if (energy) *energy = h->back[1];
     SV_TRY(resolve_profile(h, st));
     return SV_OK;
 }
@@ -1134,7 +1142,7 @@ sv_status sv_grad(sv_handle *h, const sv_gate *gates, size_t m, const double *pa
     }
     EvcEntry *e = nullptr;
     SV_TRY(get_evc(h, paulis, coeffs, nterms, SV_SCHED_LAZY, true, &e, st));
-    SV_TRY(status_reset(h));
+    SV_TRY(res_room(h, np));
     SV_TRY(run_hpsi(h, e, st));
     SV_TRY(run_reverse(h, q, st));
     h->forward_valid = false;
@@ -1142,10 +1150,9 @@ sv_status sv_grad(sv_handle *h, const sv_gate *gates, size_t m, const double *pa
         SV_CK(cudaStreamSynchronize(h->stream));
         h->drop_ckpts();
     }
-    if (grad && np) SV_CK(cudaMemcpyAsync(grad, h->grad.p, np * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    if (energy) SV_CK(cudaMemcpyAsync(energy, h->scal.as<double>() + 1, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    SV_CK(cudaStreamSynchronize(h->stream));
-    SV_TRY(status_check(h));
+    SV_TRY(read_back(h, grad ? np : 0));
+    if (grad) std::copy(h->back.begin() + kResHead, h->back.end(), grad);
+    if (energy) *energy = h->back[1];
     SV_TRY(resolve_profile(h, st));
     return SV_OK;
 }

@@ -4752,6 +4752,20 @@ __global__ void k_prep(const int32_t *__restrict__ gparam, const double *__restr
     coef[2 * g + 1] = (R)s;
 }
 
+__global__ void k_fill_basis(uint4 *psi, size_t n16, uint64_t at, int single) {
+    pdl_wait();
+    pdl_next();
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (i == at / 16) {
+            if (!single) v.y = 0x3FF00000u;               // 1.0
+            else if (at & 8u) v.z = 0x3F800000u;          // 1.0f
+            else v.x = 0x3F800000u;
+        }
+        psi[i] = v;
+    }
+}
+
 template <typename R>
 __global__ void k_set_one(Cx<R> *psi, uint64_t index) {
     pdl_wait();
@@ -4941,6 +4955,13 @@ cudaError_t launch_prep(sv_dtype dt, cudaStream_t st, const int32_t *gparam, con
 }
 
 cudaError_t launch_set_basis(sv_dtype dt, cudaStream_t st, void *psi, size_t bytes, uint64_t index) {
+    // a small state in one launch (a memset is an operation of its own on the stream)
+    if (bytes <= ((size_t)4 << 20) && bytes >= 16) {
+        const size_t n16 = bytes / 16;
+        const int blocks = (int)std::min<size_t>((n16 + 255) / 256, (size_t)2 * device_sms());
+        const uint64_t at = index * (dt == SV_C64 ? 8 : 16);     // the byte where the real part 1 stands
+        return launch(k_fill_basis, blocks, 256, 0, st, (uint4 *)psi, n16, at, dt == SV_C64 ? 1 : 0);
+    }
     cudaError_t e = cudaMemsetAsync(psi, 0, bytes, st);
     if (e != cudaSuccess) return e;
     if (dt == SV_C64) return launch(k_set_one<float>, 1, 1, 0, st, (float2 *)psi, index);
