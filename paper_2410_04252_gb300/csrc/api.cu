@@ -1339,9 +1339,7 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
     const int kmax = o.tile_bits;
     const int hio = std::max(8, kmax - o.low_bits);
     PlanOptions po = plan_options(o);
-    po.max_diag = 0;                     // the batched kernel applies RZ / CZ one by one
-    po.reg_threads = 512;
-    po.reg_pairs = false;                // and runs register phases of RY / RZ / CZ / 1-qubit matrices only
+    po.amp_bytes = dt == SV_C64 ? 8 : 16;
     std::vector<int32_t> l2p(n);
     for (int q = 0; q < n; ++q) l2p[q] = q;
     // one plan per distinct circuit
@@ -1351,7 +1349,23 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
     std::vector<DevOp> ops;
     std::vector<uint64_t> plan_keys;
     std::vector<int32_t> gsize(batch);
+    std::vector<BatchStepOff> step_off;
+    std::vector<RegStep> steps;
+    std::vector<DiagBlock> dblocks;
+    std::vector<DiagMember> dmembers;
     auto t0 = std::chrono::steady_clock::now();
+    // step loops where the kernel has them and the tables fit, else gate by gate
+    bool stepped = dt == SV_C64 && kmax == 13 && o.threads == 512 && n >= 13;
+    size_t step_smem = 0;
+    for (;;) {
+    po.reg_threads = stepped ? 0 : 512;
+    po.reg_pairs = stepped;                // gate by gate, phases hold RY / RZ / CZ only
+    po.max_diag = stepped ? kMaxPassDiag : 0;
+    po.image_limit = stepped ? batch_table_room() : 0;
+    plan_pass_off = {0};
+    plan_op_off = {0};
+    gparam.clear(); passes.clear(); phases.clear(); ops.clear(); plan_keys.clear();
+    step_off.clear(); steps.clear(); dblocks.clear(); dmembers.clear();
     for (int b = 0; b < batch; ++b) {
         const int gb = gate_off[b], ge = gate_off[b + 1];
         const int pb = param_off[b], pe = param_off[b + 1];
@@ -1378,22 +1392,30 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
             if ((int)P.ops.size() > batch_max_ops()) return fail(SV_EINVAL, "sv_batch_run: more than 512 gates in a state");
             const int obase = (int)ops.size();
             const int pbase = (int)phases.size();
+            step_off.push_back({pbase, (int32_t)steps.size(), (int32_t)dblocks.size(), (int32_t)dmembers.size()});
             for (auto &gp : P.passes) {
                 GatePassArgs a = gate_args(n, gp);
-                a.op_begin += obase;
-                a.op_end += obase;
-                if (a.ph_begin >= 0) {
-                    a.ph_begin += pbase;
-                    a.ph_end += pbase;
+                if (!stepped) {
+                    a.op_begin += obase;
+                    a.op_end += obase;
+                    if (a.ph_begin >= 0) {
+                        a.ph_begin += pbase;
+                        a.ph_end += pbase;
+                    }
+                    a.db_begin = a.db_end = 0;
                 }
-                a.db_begin = a.db_end = 0;
                 passes.push_back(a);
             }
             for (Phase f : P.phases) {
-                f.op_begin += obase;
-                f.op_end += obase;
+                if (!stepped) {
+                    f.op_begin += obase;
+                    f.op_end += obase;
+                }
                 phases.push_back(f);
             }
+            steps.insert(steps.end(), P.steps.begin(), P.steps.end());
+            dblocks.insert(dblocks.end(), P.dblocks.begin(), P.dblocks.end());
+            dmembers.insert(dmembers.end(), P.dmembers.begin(), P.dmembers.end());
             ops.insert(ops.end(), P.ops.begin(), P.ops.end());
             plan_pass_off.push_back((int32_t)passes.size());
             plan_op_off.push_back((int32_t)ops.size());
@@ -1401,6 +1423,11 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
             plan_keys.push_back(key);
         }
         state_plan[b] = pi;
+    }
+    if (!stepped) break;
+    step_smem = batch_step_bytes(dt, n, kmax, o.threads, passes);
+    if (step_smem) break;
+    stepped = false;
     }
     EvcPlan H;
     std::string err = plan_hpsi(n, paulis, coeffs, nterms, po, l2p, H);
@@ -1437,7 +1464,7 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
     if (occ < 1) return fail(SV_EINVAL, "sv_batch_run: the batched kernel does not fit an SM with these options");
     const int grid = std::min(batch, device_sms() * occ);
     const size_t es = dt == SV_C64 ? 8 : 16;
-    std::vector<DevBuf> bufs(17);
+    std::vector<DevBuf> bufs(21);
     auto up = [&](int i, const void *src, size_t bytes) -> cudaError_t {
         cudaError_t e = bufs[i].ensure(std::max<size_t>(bytes, 16));
         if (e != cudaSuccess || !bytes) return e;
@@ -1470,6 +1497,12 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
     SV_BCK(up(11, gs.data(), gs.size() * sizeof(DevGroup)));
     SV_BCK(up(12, ss.data(), ss.size() * sizeof(DevString)));
     SV_BCK(up(16, phases.data(), phases.size() * sizeof(Phase)));
+    if (stepped) {
+        SV_BCK(up(17, step_off.data(), step_off.size() * sizeof(BatchStepOff)));
+        SV_BCK(up(18, steps.data(), steps.size() * sizeof(RegStep)));
+        SV_BCK(up(19, dblocks.data(), dblocks.size() * sizeof(DiagBlock)));
+        SV_BCK(up(20, dmembers.data(), dmembers.size() * sizeof(DiagMember)));
+    }
     SV_BCK(bufs[13].ensure((size_t)grid * 2 * ((size_t)1 << n) * es));
     SV_BCK(bufs[14].ensure((batch + nparams + 2 * (size_t)batch) * 8 + 64));
     double *d_energy = bufs[14].as<double>();
@@ -1504,6 +1537,11 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
     a.t_start = d_t;
     a.t_end = d_t + batch;
     a.counter = bufs[15].as<int>();
+    a.step_smem = stepped ? step_smem : 0;
+    a.step = bufs[17].as<BatchStepOff>();
+    a.steps = bufs[18].as<RegStep>();
+    a.dblocks = bufs[19].as<DiagBlock>();
+    a.dmembers = bufs[20].as<DiagMember>();
     // one graph: reset the work counter, then the persistent launch
     SV_BCK(cudaStreamSynchronize(s0));
     cudaStream_t cs = nullptr;

@@ -1222,8 +1222,13 @@ template <> __device__ __forceinline__ RotK<double> pair_rec<double>(const doubl
 // The step loop of a phase comes in three kinds, chosen per pass by what the
 // pass holds, since the operations it does not hold would cost it register
 // moves where their codes meet: 0 rotations and diagonal gates only
-// (hardware-efficient ansatz), 1 pair rotations only (brick ansatz), 2 all.
-constexpr int kStepsDiag = 0, kStepsPair = 1, kStepsAll = 2;
+// (hardware-efficient ansatz), 1 pair rotations only (brick ansatz), 3 both,
+// 2 matrices too.
+constexpr int kStepsDiag = 0, kStepsPair = 1, kStepsAll = 2, kStepsMixed = 3;
+__host__ __device__ inline int steps_kind(const GatePassArgs &a) {
+    if (a.dense || a.mat1) return kStepsAll;
+    return !a.pairs ? kStepsDiag : a.others ? kStepsMixed : kStepsPair;
+}
 
 // Hint: bring [p, p + bytes) into L2 (bytes a multiple of 16, p 16-byte aligned).
 __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
@@ -1313,29 +1318,18 @@ struct PhaseS {
 // every CTA of every pass repeated them.  Block (pass, slice, direction): the
 // slices share a pass's phases and blocks, slice 0 writes the rest.
 constexpr int kImageSlices = 8;
+// `out` in shared or global memory; cs and st: shared room for the pass's
+// operations and steps; slice 0 of nslices writes what the slices don't share.
 template <typename R>
-__global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restrict__ pargs,
-                                                   const uint64_t *__restrict__ offs, const DevOp *__restrict__ ops,
-                                                   const Phase *__restrict__ phases,
-                                                   const RegStep *__restrict__ steps, const R *__restrict__ coef,
-                                                   const DiagBlock *__restrict__ dblocks,
-                                                   const DiagMember *__restrict__ dmem, unsigned char *out0,
-                                                   uint64_t dir_stride, int dir0) {
+__device__ __forceinline__ void reg_tables(unsigned char *out, const RegLayout &L, const GatePassArgs &a,
+                                           const DevOp *ops, const Phase *phases, const RegStep *steps, const R *coef,
+                                           const DiagBlock *dblocks, const DiagMember *dmem, bool adj, Cx<R> *cs,
+                                           RegStep *st, int slice, int nslices) {
     constexpr int RB = kRegBits, V = 1 << RB;
     constexpr uint32_t P = 16 / sizeof(Cx<R>);
-    __shared__ GatePassArgs a;
-    __shared__ Cx<R> cs[kMaxPassOps];
-    __shared__ RegStep st[kMaxPassOps];
     const int tid = threadIdx.x, nthr = blockDim.x;
-    const bool adj = (int)blockIdx.z + dir0 != 0, first = blockIdx.y == 0;
-    for (int i = tid; i < (int)(sizeof(GatePassArgs) / 4); i += nthr)
-        reinterpret_cast<uint32_t *>(&a)[i] = reinterpret_cast<const uint32_t *>(pargs + blockIdx.x)[i];
-    __syncthreads();
-    unsigned char *out = out0 + (adj ? dir_stride : 0) + offs[blockIdx.x];
-    const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), adj);
+    const bool first = slice == 0;
     const int NT = 1 << (a.k - RB), nph = a.ph_end - a.ph_begin, nst = a.st_end - a.st_begin;
-    pdl_wait();
-    pdl_next();
     for (int o = a.op_begin + tid; o < a.op_end; o += nthr) {
         const int gi = ops[o].gate;
         cs[o - a.op_begin] = mk<R>(coef[2 * gi], adj ? -coef[2 * gi + 1] : coef[2 * gi + 1]);
@@ -1445,14 +1439,14 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
     // this slice's phases: the tile bits of every thread
     for (int e = tid; e < nph * NT; e += nthr) {
         const int q = e / NT, t = e % NT;
-        if (q % kImageSlices != (int)blockIdx.y) continue;
+        if (q % nslices != slice) continue;
         const Phase F = phases[a.ph_begin + q];
         reinterpret_cast<uint16_t *>(out + L.pbase)[e] =
             (uint16_t)(swz_tile(phase_base(F.rmask, F.lanes, a.k, (uint32_t)t)) * (uint32_t)sizeof(Cx<R>));
     }
     // this slice's diagonal blocks: tables and per-thread data
     unsigned char *area = out + L.area;
-    for (int b = (int)blockIdx.y; b < a.db_end - a.db_begin; b += kImageSlices) {
+    for (int b = slice; b < a.db_end - a.db_begin; b += nslices) {
         const DiagBlock B = dblocks[a.db_begin + b];
         const DiagMember *mb = dmem + B.m_begin;
         const int nm = B.m_end - B.m_begin;
@@ -1499,6 +1493,28 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
             }
         }
     }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restrict__ pargs,
+                                                   const uint64_t *__restrict__ offs, const DevOp *__restrict__ ops,
+                                                   const Phase *__restrict__ phases,
+                                                   const RegStep *__restrict__ steps, const R *__restrict__ coef,
+                                                   const DiagBlock *__restrict__ dblocks,
+                                                   const DiagMember *__restrict__ dmem, unsigned char *out0,
+                                                   uint64_t dir_stride, int dir0) {
+    __shared__ GatePassArgs a;
+    __shared__ Cx<R> cs[kMaxPassOps];
+    __shared__ RegStep st[kMaxPassOps];
+    const bool adj = (int)blockIdx.z + dir0 != 0;
+    for (int i = threadIdx.x; i < (int)(sizeof(GatePassArgs) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t *>(&a)[i] = reinterpret_cast<const uint32_t *>(pargs + blockIdx.x)[i];
+    __syncthreads();
+    const RegLayout L = reg_layout(a, (int)sizeof(Cx<R>), adj);
+    pdl_wait();
+    pdl_next();
+    reg_tables<R>(out0 + (adj ? dir_stride : 0) + offs[blockIdx.x], L, a, ops, phases, steps, coef, dblocks, dmem, adj,
+                  cs, st, (int)blockIdx.y, kImageSlices);
 }
 
 // A pass's tables from global into shared memory (16 bytes at a time)
@@ -1660,7 +1676,7 @@ __device__ __forceinline__ void fwd_steps(RA<R> *x, const PhaseS &F, const GateP
                 reg_rz<R>(x, cs[S.op_begin], diag_bit_mask(t0, F.rmask, base, gbase));
             } else if (code == RO_CZ) {
                 reg_cz<R>(x, diag_bit_mask(t0, F.rmask, base, gbase) & diag_bit_mask(t1, F.rmask, base, gbase));
-            } else if constexpr (KIND == kStepsAll) {
+            } else if constexpr (KIND == kStepsAll || KIND == kStepsMixed) {
                 const Cx<R> *M = pmats + S.op_end;
                 uint32_t pc = 0;
                 RotK<R> k{};
@@ -1669,17 +1685,17 @@ __device__ __forceinline__ void fwd_steps(RA<R> *x, const PhaseS &F, const GateP
 #define SV_C(MU, MV) ra_pair_rot<R, V, MU, MV>(x, k)
                     SV_RO_GIVENS(SV_C)
 #undef SV_C
-                case RO_MAT1: reg_mat<R, 0, 0>(x, M); break;
-                case RO_MAT1 + 1: reg_mat<R, 1, 1>(x, M); break;
-                case RO_MAT1 + 2: reg_mat<R, 2, 2>(x, M); break;
-                case RO_MAT1 + 3: reg_mat<R, 3, 3>(x, M); break;
-                case RO_MAT2: reg_mat<R, 0, 1>(x, M); break;
-                case RO_MAT2 + 1: reg_mat<R, 0, 2>(x, M); break;
-                case RO_MAT2 + 2: reg_mat<R, 0, 3>(x, M); break;
-                case RO_MAT2 + 3: reg_mat<R, 1, 2>(x, M); break;
-                case RO_MAT2 + 4: reg_mat<R, 1, 3>(x, M); break;
-                case RO_MAT2 + 5: reg_mat<R, 2, 3>(x, M); break;
-                case RO_MAT4: reg_mat4<R>(x, M); break;
+                case RO_MAT1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 0>(x, M); } break;
+                case RO_MAT1 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 1>(x, M); } break;
+                case RO_MAT1 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 2>(x, M); } break;
+                case RO_MAT1 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 3, 3>(x, M); } break;
+                case RO_MAT2: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 1>(x, M); } break;
+                case RO_MAT2 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 2>(x, M); } break;
+                case RO_MAT2 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 3>(x, M); } break;
+                case RO_MAT2 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 2>(x, M); } break;
+                case RO_MAT2 + 4: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 3>(x, M); } break;
+                case RO_MAT2 + 5: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 3>(x, M); } break;
+                case RO_MAT4: if constexpr (KIND == kStepsAll) { reg_mat4<R>(x, M); } break;
                 default: break;
                 }
             }
@@ -1815,7 +1831,7 @@ __device__ __forceinline__ void adj_steps(RA<R> *xp, RA<R> *xl, const PhaseS &F,
                 const uint32_t m = diag_bit_mask(t0, F.rmask, base, gbase) & diag_bit_mask(t1, F.rmask, base, gbase);
                 reg_cz<R>(xp, m);
                 reg_cz<R>(xl, m);
-            } else if constexpr (KIND == kStepsAll) {
+            } else if constexpr (KIND == kStepsAll || KIND == kStepsMixed) {
                 // the prepared matrix is followed by its conjugate transpose (1-qubit matrices: 4 elements)
                 const Cx<R> *M = pmats + S.op_end + 4;
                 uint32_t pc = 0;
@@ -1829,10 +1845,10 @@ __device__ __forceinline__ void adj_steps(RA<R> *xp, RA<R> *xl, const PhaseS &F,
     ra_pair_rot<R, V, MU, MV>(xl, k)
                     SV_RO_GIVENS(SV_C)
 #undef SV_C
-                case RO_MAT1: reg_mat<R, 0, 0>(xp, M); reg_mat<R, 0, 0>(xl, M); break;
-                case RO_MAT1 + 1: reg_mat<R, 1, 1>(xp, M); reg_mat<R, 1, 1>(xl, M); break;
-                case RO_MAT1 + 2: reg_mat<R, 2, 2>(xp, M); reg_mat<R, 2, 2>(xl, M); break;
-                case RO_MAT1 + 3: reg_mat<R, 3, 3>(xp, M); reg_mat<R, 3, 3>(xl, M); break;
+                case RO_MAT1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 0>(xp, M); reg_mat<R, 0, 0>(xl, M); } break;
+                case RO_MAT1 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 1>(xp, M); reg_mat<R, 1, 1>(xl, M); } break;
+                case RO_MAT1 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 2>(xp, M); reg_mat<R, 2, 2>(xl, M); } break;
+                case RO_MAT1 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 3, 3>(xp, M); reg_mat<R, 3, 3>(xl, M); } break;
                 default: break;
                 }
                 if (code < RO_MAT1) {
@@ -4417,10 +4433,132 @@ __device__ __noinline__ void batch_reg_adjoint(Cx<R> *tp, Cx<R> *tl, const GateP
     }
 }
 
+// Gate passes of the batched kernel by the register passes' step loops
+// (complex64, tiles of 2^13, 512 threads): a state's tables of a pass are made
+// in shared memory by the CTA that runs it (a few microseconds against the
+// pass's 32 tiles at n = 18), so that rotations run factored and diagonal
+// gates in blocks instead of one gate after the other.
+struct BatchPass {
+    const GatePassArgs *a;
+    const RegLayout *L;
+    const unsigned char *sm;     // the pass's tables
+};
+template <int KIND>
+__device__ __noinline__ void batch_fwd(unsigned char *smem, const BatchPass &B, float2 *psi) {
+    const GatePassArgs &a = *B.a;
+    const RegLayout &L = *B.L;
+    const unsigned char *sm = B.sm;
+    constexpr uint32_t tbytes = 65536;
+    const float ftot = reinterpret_cast<const float *>(sm + L.sc)[a.st_end - a.st_begin];
+    const uint64_t *hioff = reinterpret_cast<const uint64_t *>(sm + L.hioff);
+    const ChunkOff *chunk = reinterpret_cast<const ChunkOff *>(sm + L.chunk);
+    const PhaseS *phs = reinterpret_cast<const PhaseS *>(sm + L.phases);
+    const uint16_t *pbase = reinterpret_cast<const uint16_t *>(sm + L.pbase);
+    const uint4 *prb = reinterpret_cast<const uint4 *>(sm + L.prb);
+    const int nph = a.ph_end - a.ph_begin;
+    const uint32_t j0 = 2u * threadIdx.x, slot = swz_tile(j0) * 8u;
+    float2 *mypsi = psi + (hioff[j0 >> a.nlow] | (j0 & ((1u << a.nlow) - 1u)));
+    const uint64_t ntiles = 1ull << a.nout;
+    for (uint64_t k = 0; k < 2; ++k) {
+        if (k < ntiles)
+            reg_tile_load<float>(smem, mypsi + deposit(k, a.out, a.nout), chunk, slot + (uint32_t)k * tbytes);
+        cp_async_commit();
+    }
+    for (uint64_t it = 0; it < ntiles; ++it) {
+        const uint64_t gbase = deposit(it, a.out, a.nout);
+        const uint32_t tile = (uint32_t)(it & 1) * tbytes;
+        cp_async_wait1();
+        __syncthreads();
+        for (int ph = 0; ph < nph; ++ph) {
+            const PhaseS F = phs[ph];
+            const uint32_t place = pbase[ph * 512 + threadIdx.x];
+            uint32_t idx[16];
+            phase_slots16(idx, place | tile, prb[ph]);
+            RA<float> x[16];
+            phase_gather<float>(x, smem, idx, F.rmask & 1u);
+            fwd_steps<float, KIND>(x, F, a, reinterpret_cast<const RegStep *>(sm + L.steps),
+                                   reinterpret_cast<const float2 *>(sm + L.cs),
+                                   reinterpret_cast<const float2 *>(sm + L.rk),
+                                   reinterpret_cast<const DiagBlock *>(sm + L.blocks), sm + L.area, threadIdx.x, place,
+                                   gbase, nullptr);
+            phase_scatter<float>(x, smem, idx, F.rmask & 1u);
+            __syncthreads();
+        }
+        reg_tile_store<float>(mypsi + gbase, smem, chunk, slot + tile, ftot);
+        if (it + 2 < ntiles)
+            reg_tile_load<float>(smem, mypsi + deposit(it + 2, a.out, a.nout), chunk, slot + tile);
+        cp_async_commit();
+    }
+    cp_async_wait0();
+    __syncthreads();
+}
+template <int KIND>
+__device__ __noinline__ void batch_adj(unsigned char *smem, const BatchPass &B, float2 *psi, float2 *lam, float *acc) {
+    const GatePassArgs &a = *B.a;
+    const RegLayout &L = *B.L;
+    const unsigned char *sm = B.sm;
+    unsigned char *tl = smem, *tp = smem + 65536;
+    const float *scf = reinterpret_cast<const float *>(sm + L.sc);
+    const float ftot = scf[a.st_end - a.st_begin];
+    const uint64_t *hioff = reinterpret_cast<const uint64_t *>(sm + L.hioff);
+    const ChunkOff *chunk = reinterpret_cast<const ChunkOff *>(sm + L.chunk);
+    const PhaseS *phs = reinterpret_cast<const PhaseS *>(sm + L.phases);
+    const uint16_t *pbase = reinterpret_cast<const uint16_t *>(sm + L.pbase);
+    const uint4 *prb = reinterpret_cast<const uint4 *>(sm + L.prb);
+    const int nph = a.ph_end - a.ph_begin;
+    const uint32_t j0 = 2u * threadIdx.x, slot = swz_tile(j0) * 8u;
+    const uint64_t toff = hioff[j0 >> a.nlow] | (j0 & ((1u << a.nlow) - 1u));
+    const uint64_t ntiles = 1ull << a.nout;
+    for (uint64_t it = 0; it < ntiles; ++it) {
+        const uint64_t gbase = deposit(it, a.out, a.nout);
+        reg_tile_load<float>(tp, psi + (gbase | toff), chunk, slot);
+        reg_tile_load<float>(tl, lam + (gbase | toff), chunk, slot);
+        cp_async_commit();
+        if (it + 1 < ntiles) {
+            const uint64_t gn = deposit(it + 1, a.out, a.nout);
+            for (uint32_t j = threadIdx.x; j < (1u << (a.k - a.nlow)); j += 512u) {
+                prefetch_l2(psi + (gn | hioff[j]), 8u << a.nlow);
+                prefetch_l2(lam + (gn | hioff[j]), 8u << a.nlow);
+            }
+        }
+        cp_async_wait0();
+        __syncthreads();
+        for (int ph = nph - 1; ph >= 0; --ph) {
+            const PhaseS F = phs[ph];
+            const uint32_t place = pbase[ph * 512 + threadIdx.x];
+            uint32_t idx[16];
+            phase_slots16(idx, place, prb[ph]);
+            RA<float> xp[16], xl[16];
+            phase_gather<float>(xp, tp, idx, F.rmask & 1u);
+            phase_gather<float>(xl, tl, idx, F.rmask & 1u);
+            adj_steps<float, KIND>(xp, xl, F, a, reinterpret_cast<const RegStep *>(sm + L.steps),
+                                   reinterpret_cast<const float2 *>(sm + L.cs),
+                                   reinterpret_cast<const float2 *>(sm + L.rk),
+                                   reinterpret_cast<const DiagBlock *>(sm + L.blocks),
+                                   reinterpret_cast<const DiagMember *>(sm + L.mem), scf, sm + L.area, place, gbase,
+                                   nullptr, acc);
+            phase_slots16(idx, pbase[ph * 512 + threadIdx.x], prb[ph]);
+            phase_scatter<float>(xp, tp, idx, F.rmask & 1u);
+            phase_scatter<float>(xl, tl, idx, F.rmask & 1u);
+            __syncthreads();
+        }
+        reg_tile_store<float>(psi + (gbase | toff), tp, chunk, slot, ftot);
+        reg_tile_store<float>(lam + (gbase | toff), tl, chunk, slot, ftot);
+    }
+    __syncthreads();
+}
+
+// Shared memory of the batched kernel with step loops, behind the two tiles:
+// span table, gradient slots of a pass, gradient per operation, coefficients,
+// then the tables of a pass (or of an H|psi> pass's strings).
+constexpr uint32_t kBsSpan = 131072, kBsAcc = kBsSpan + 2048, kBsTot = kBsAcc + 4 * kAdjSlotStride * kMaxPassOps,
+                   kBsCoef = kBsTot + 8 * 512, kBsTab = kBsCoef + 8 * 1024;
+
 constexpr int kBatchMaxOps = 512;      // gate operations per state (smem accumulators)
 constexpr int kBatchMaxGates = 1024;
 
-template <typename R, int EPT>
+// STEP: gate passes by batch_fwd / batch_adj (a.step: per-plan steps and blocks)
+template <typename R, int EPT, bool STEP>
 __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int NT = blockDim.x, nwarps = NT >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -4433,6 +4571,38 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
     unsigned char *opbase = reinterpret_cast<unsigned char *>(hioff + (1u << a.hio));
     R *opacc = reinterpret_cast<R *>(opbase);                                        // [kBatchMaxOps][nwarps]
     R *coef = reinterpret_cast<R *>(opbase + (size_t)kBatchMaxOps * nwarps * 8);     // [2 * kBatchMaxGates]
+    HpsiStr *htab = reinterpret_cast<HpsiStr *>(opbase + (size_t)kBatchMaxOps * nwarps * 4);
+    double *optot = nullptr;
+    __shared__ GatePassArgs sP;
+    __shared__ RegLayout sL;
+    if constexpr (STEP) {
+        hioff = reinterpret_cast<uint64_t *>(smem + kBsSpan);
+        opacc = reinterpret_cast<R *>(smem + kBsAcc);
+        optot = reinterpret_cast<double *>(smem + kBsTot);
+        coef = reinterpret_cast<R *>(smem + kBsCoef);
+        htab = reinterpret_cast<HpsiStr *>(smem + kBsTab);
+    }
+    // the tables of a pass of plan `plan` (the scratch lies in the gradient slots)
+    auto tables = [&](int plan, int pi, bool adj) {
+        if constexpr (STEP) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < (int)(sizeof(GatePassArgs) / 4); i += NT)
+                reinterpret_cast<uint32_t *>(&sP)[i] = reinterpret_cast<const uint32_t *>(a.passes + pi)[i];
+            __syncthreads();
+            const RegLayout L = reg_layout(sP, (int)sizeof(Cx<R>), adj);
+            if (threadIdx.x == 0) sL = L;
+            Cx<R> *cs = reinterpret_cast<Cx<R> *>(opacc);
+            const BatchStepOff off = a.step[plan];
+            reg_tables<R>(smem + kBsTab, L, sP, a.ops + a.plan_op_off[plan], a.phases + off.ph, a.steps + off.st, coef,
+                          a.dblocks + off.db, a.dmembers + off.dm, adj, cs, reinterpret_cast<RegStep *>(cs + kMaxPassOps),
+                          0, 1);
+            __syncthreads();
+            if (adj) {
+                for (int j = threadIdx.x; j < (sP.op_end - sP.op_begin) * kAdjSlotStride; j += NT) opacc[j] = 0;
+                __syncthreads();
+            }
+        }
+    };
     __shared__ int s_state;
     __shared__ double s_red[32];
     const size_t N = (size_t)1 << a.n;
@@ -4456,11 +4626,21 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
             coef[2 * g] = (R)c;
             coef[2 * g + 1] = (R)sn;
         }
-        for (int j = threadIdx.x; j < nops * nwarps; j += NT) opacc[j] = 0;
+        if constexpr (!STEP)
+            for (int j = threadIdx.x; j < nops * nwarps; j += NT) opacc[j] = 0;
         for (size_t i = threadIdx.x; i < N; i += NT) psi[i] = mk<R>(i == a.init_index ? 1 : 0, 0);
         __syncthreads();
         // ---- QSU
         for (int pi = a.plan_pass_off[plan]; pi < a.plan_pass_off[plan + 1]; ++pi) {
+            if constexpr (STEP) {
+                tables(plan, pi, false);
+                const BatchPass B{&sP, &sL, smem + kBsTab};
+                const int kind = steps_kind(sP);
+                if (kind == kStepsDiag) batch_fwd<kStepsDiag>(smem, B, psi);
+                else if (kind == kStepsPair) batch_fwd<kStepsPair>(smem, B, psi);
+                else batch_fwd<kStepsMixed>(smem, B, psi);
+                continue;
+            }
             const GatePassArgs &P = a.passes[pi];
             const uint32_t T = 1u << P.k, nh = 1u << (P.k - P.nlow), lowmask = (1u << P.nlow) - 1u;
             for (uint32_t j = threadIdx.x; j < nh; j += NT) hioff[j] = deposit(j, P.hi, P.nhi);
@@ -4520,7 +4700,7 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
             // staged once, as in k_hpsi_vec; the table lies behind the gradient
             // slots, which are half as wide as their room (and the previous
             // pass's is no longer read: barrier at its end)
-            HpsiStr *tab = reinterpret_cast<HpsiStr *>(opbase + (size_t)kBatchMaxOps * nwarps * 4);
+            HpsiStr *tab = htab;
             const int ns = C.s_end - C.s_begin;
             const bool vec = sizeof(R) == 4 && EPT == 16 && fast && C.kl >= 1 && C.kl <= 10;
             if (vec)
@@ -4624,6 +4804,20 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
         }
         // ---- adjoint reverse sweep
         for (int pi = a.plan_pass_off[plan + 1] - 1; pi >= a.plan_pass_off[plan]; --pi) {
+            if constexpr (STEP) {
+                tables(plan, pi, true);
+                const BatchPass B{&sP, &sL, smem + kBsTab};
+                const int kind = steps_kind(sP);
+                if (kind == kStepsDiag) batch_adj<kStepsDiag>(smem, B, psi, lam, opacc);
+                else if (kind == kStepsPair) batch_adj<kStepsPair>(smem, B, psi, lam, opacc);
+                else batch_adj<kStepsMixed>(smem, B, psi, lam, opacc);
+                for (int o = threadIdx.x; o < sP.op_end - sP.op_begin; o += NT) {
+                    double v = 0.0;
+                    for (int w = 0; w < nwarps; ++w) v += (double)opacc[o * kAdjSlotStride + w];
+                    optot[sP.op_begin + o] = v;
+                }
+                continue;
+            }
             const GatePassArgs &P = a.passes[pi];
             const uint32_t T = 1u << P.k, nh = 1u << (P.k - P.nlow), lowmask = (1u << P.nlow) - 1u;
             __syncthreads();
@@ -4673,6 +4867,7 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
             }
         }
         // gradient: per op, then per parameter in a fixed order
+        if constexpr (STEP) __syncthreads();
         if (threadIdx.x == 0) {
             for (int p = 0; p < np; ++p) a.grads[p0 + p] = 0.0;
             for (int o = 0; o < nops; ++o) {
@@ -4680,7 +4875,9 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
                 const int p = a.gparam[g0 + op.gate];
                 if (p < 0 || !has_param(op.kind)) continue;
                 double v = 0.0;
-                for (int w = 0; w < nwarps; ++w) v += (double)opacc[o * nwarps + w];
+                if constexpr (STEP) v = optot[o];
+                else
+                    for (int w = 0; w < nwarps; ++w) v += (double)opacc[o * nwarps + w];
                 a.grads[p0 + p] += v;
             }
             a.t_start[st] = t0;
@@ -4991,15 +5188,10 @@ size_t adj_reg_smem(sv_dtype dt, const GatePassArgs &a) {
     return 2 * ((size_t)1 << a.k) * amp + reg_layout(a, amp, true).total;
 }
 
-// the step loop for what a pass holds
-static int steps_kind(const GatePassArgs &a) {
-    if (a.dense || a.mat1) return kStepsAll;
-    return !a.pairs ? kStepsDiag : a.others ? kStepsAll : kStepsPair;
-}
 // Two tiles in work per CTA from this many phases on: see k_gate_two.
 constexpr int kTwoPhases = 3;
 static bool gate_two_pays(sv_dtype dt, const GatePassArgs &a) {
-    return dt == SV_C64 && steps_kind(a) != kStepsAll && a.ph_end - a.ph_begin >= kTwoPhases;
+    return dt == SV_C64 && (steps_kind(a) == kStepsDiag || steps_kind(a) == kStepsPair) && a.ph_end - a.ph_begin >= kTwoPhases;
 }
 
 int reg_pass_grid(sv_dtype dt, const GatePassArgs &a, bool adj, int blocks_per_sm) {
@@ -5032,6 +5224,7 @@ cudaError_t gate_reg_dispatch(cudaStream_t st, int grid, void *psi, const GatePa
     }
     if (kind == kStepsPair) return go(k_gate_reg<R, kStepsPair>, nt, pm);
     if (kind == kStepsDiag) return go(k_gate_reg<R, kStepsDiag>, nt, pm);
+    if (kind == kStepsMixed) return go(k_gate_reg<R, kStepsMixed>, nt, pm);
     return go(k_gate_reg<R, kStepsAll>, nt, pm);
 }
 
@@ -5049,6 +5242,7 @@ cudaError_t adj_reg_dispatch(cudaStream_t st, int grid, void *psi, void *lam, co
     const int kind = steps_kind(a);
     if (kind == kStepsPair) return go(k_adj_reg<R, kStepsPair>);
     if (kind == kStepsDiag) return go(k_adj_reg<R, kStepsDiag>);
+    if (kind == kStepsMixed) return go(k_adj_reg<R, kStepsMixed>);
     return go(k_adj_reg<R, kStepsAll>);
 }
 
@@ -5445,23 +5639,44 @@ int batch_occupancy(sv_dtype dt, int kmax, int hio, int threads) {
     const size_t sm = batch_smem(dt, kmax, hio, threads);
     const int ept = (1 << kmax) / threads;
     int occ = 0;
-#define SV_BOCC(R, E)                       \
-    allow_smem(k_batch<R, E>, sm);          \
-    occ = occupancy(k_batch<R, E>, threads, sm);
+#define SV_BOCC(R, E)                              \
+    allow_smem(k_batch<R, E, false>, sm);          \
+    occ = occupancy(k_batch<R, E, false>, threads, sm);
     if (dt == SV_C64) { SV_BATCH_SWITCH(float, ept, SV_BOCC) }
     else { SV_BATCH_SWITCH(double, ept, SV_BOCC) }
 #undef SV_BOCC
     return occ;
 }
 
+// Step loops in the batched kernel: complex64 tiles of 2^13 with 512 threads
+// whose passes' tables fit beside them (the largest of `passes`; 0: they do
+// not).  Smaller states and the other tile and CTA sizes go gate by gate.
+int batch_table_room() { return smem_optin() - 2048 - (int)kBsTab; }
+size_t batch_step_bytes(sv_dtype dt, int n, int kmax, int threads, const std::vector<GatePassArgs> &passes) {
+    if (dt != SV_C64 || kmax != 13 || threads != 512 || n < 13) return 0;
+    size_t tab = (size_t)kMaxPassStrings * sizeof(HpsiStr);
+    for (auto &a : passes) {
+        if (a.k != 13 || a.ph_begin < 0) return 0;
+        tab = std::max<size_t>(tab, reg_layout(a, 8, true).image);
+    }
+    const size_t sm = kBsTab + tab;
+    return sm + 2048 <= (size_t)smem_optin() ? sm : 0;
+}
+
 cudaError_t launch_batch(sv_dtype dt, cudaStream_t st, int grid, int threads, const BatchArgs &a) {
+    if (a.step_smem) {
+        const cudaError_t e = allow_smem(k_batch<float, 16, true>, a.step_smem);
+        if (e != cudaSuccess) return e;
+        k_batch<float, 16, true><<<grid, 512, a.step_smem, st>>>(a);
+        return cudaGetLastError();
+    }
     if (!batch_supported(dt, a.kmax, threads)) return cudaErrorInvalidValue;
     const size_t sm = batch_smem(dt, a.kmax, a.hio, threads);
     const int ept = (1 << a.kmax) / threads;
     cudaError_t e = cudaSuccess;
 #define SV_BLAUNCH(R, E)                                      \
-    e = allow_smem(k_batch<R, E>, sm);                        \
-    if (e == cudaSuccess) k_batch<R, E><<<grid, threads, sm, st>>>(a);
+    e = allow_smem(k_batch<R, E, false>, sm);                 \
+    if (e == cudaSuccess) k_batch<R, E, false><<<grid, threads, sm, st>>>(a);
     if (dt == SV_C64) { SV_BATCH_SWITCH(float, ept, SV_BLAUNCH) }
     else { SV_BATCH_SWITCH(double, ept, SV_BLAUNCH) }
 #undef SV_BLAUNCH

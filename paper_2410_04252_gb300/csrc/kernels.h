@@ -6,6 +6,8 @@
 
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "sv_internal.h"
 
 namespace sv {
@@ -56,6 +58,12 @@ struct DevString {
 // Few-string expectation passes (every group one string): at most this many groups.
 constexpr int kEvcFew = 8;
 
+// First phase, step, diagonal block and block member of a plan (batched kernel
+// with step loops: indices inside a plan are its own).
+struct BatchStepOff {
+    int32_t ph, st, db, dm;
+};
+
 // Batched kernel arguments (see K-BATCH in kernels.cu).
 struct BatchArgs {
     int n, nstates, nhpass;
@@ -81,6 +89,13 @@ struct BatchArgs {
     double *grads;                   // like params
     unsigned long long *t_start, *t_end;
     int *counter;
+    // step loops (step_smem != 0: shared bytes of that kernel; a pass's operation
+    // indices are then its plan's own)
+    size_t step_smem;
+    const BatchStepOff *step;        // [nplans]
+    const RegStep *steps;
+    const DiagBlock *dblocks;
+    const DiagMember *dmembers;
 };
 
 int device_sms();
@@ -162,6 +177,8 @@ cudaError_t launch_batch(sv_dtype dt, cudaStream_t st, int grid, int threads, co
 // max over (count << 32) | (0xFFFFFFFF - rank); binom is C(a, b) as [(n + 1)][(k + 1)].
 cudaError_t launch_alg6_step(cudaStream_t st, const uint64_t *xs, const int32_t *w, int nx, int n, int k,
                              const int64_t *binom, uint64_t ncand, unsigned long long *best);
+int batch_table_room();   // bytes for a pass's tables beside the tiles
+size_t batch_step_bytes(sv_dtype dt, int n, int kmax, int threads, const std::vector<GatePassArgs> &passes);
 size_t batch_smem(sv_dtype dt, int kmax, int hio, int threads);
 // 0 when (dt, kmax, threads) has no instantiated kernel
 int batch_supported(sv_dtype dt, int kmax, int threads);

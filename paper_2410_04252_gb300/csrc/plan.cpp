@@ -605,7 +605,7 @@ bool diag_run_pays(const std::vector<DevOp> &run) {
     return 4 * rz + cz >= 6;
 }
 
-void plan_steps(QsuPlan &P, int max_diag, int amp) {
+void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
     auto tm = [](const DevOp &d) {
         uint32_t m = 0;
         const int nq = op_qubits(d.kind);
@@ -617,7 +617,8 @@ void plan_steps(QsuPlan &P, int max_diag, int amp) {
         gp.db_begin = gp.db_end = (int32_t)P.dblocks.size();
         if (gp.ph_begin < 0) continue;
         const int nops = gp.op_end - gp.op_begin;
-        int budget = kRegSmemLimit - reg_pass_fixed_bytes(gp.k, gp.nlow, nops, nops, gp.ph_end - gp.ph_begin, amp, gp.pairs != 0);
+        const int limit = image_limit ? 2 * (1 << gp.k) * amp + nops * kAdjSlotStride * 8 + image_limit : kRegSmemLimit;
+        int budget = limit - reg_pass_fixed_bytes(gp.k, gp.nlow, nops, nops, gp.ph_end - gp.ph_begin, amp, gp.pairs != 0);
         int area = 0;   // bytes of the pass's block area handed out so far
         auto take_block = [&](int kind) {
             const int need = diag_block_bytes(kind, gp.k, amp);
@@ -1457,7 +1458,7 @@ std::string plan_qsu(int n, int g, const sv_gate *gates, size_t m, bool lazy, co
     int k = std::max(o.tile_bits, std::min(o.low_bits, P.nL) + 4);
     plan_gate_passes(P, ops, k, o.low_bits, o.fuse_max, o.diag_exempt);
     plan_phases(P, o.reg_pairs, o.reg_threads);
-    plan_steps(P, std::min(o.max_diag, kMaxPassDiag), o.amp_bytes);
+    plan_steps(P, std::min(o.max_diag, kMaxPassDiag), o.amp_bytes, o.image_limit);
     return "";
 }
 

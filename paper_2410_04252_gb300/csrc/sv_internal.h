@@ -282,6 +282,7 @@ struct PlanOptions {
     int max_diag = kMaxPassDiag; // diagonal blocks per register-blocked pass (shared-memory budget)
     int amp_bytes = 8;           // 8 complex64, 16 complex128 (shared-memory budget of the blocks)
     bool reg_pairs = true;       // Givens, double excitations and dense matrices may run in register phases
+    int image_limit = 0;         // bytes for a pass's tables when it is less than the shared memory leaves (0)
     int reg_threads = 0;         // register phases on CTAs of this size (the batched kernel), 0 = 2^(k - kRegBits)
     bool diag_exempt = false;    // QSU: diagonal gates (RZ, CZ) never ask for a QR (per-chunk phases)
     // One greedy step of Alg. 6 done elsewhere (on the device): given the
