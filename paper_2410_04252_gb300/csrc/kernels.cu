@@ -4205,9 +4205,12 @@ __global__ void __launch_bounds__(512) k_evc_slice(const Cx<R> *__restrict__ psi
 // lambda over one coset, the outputs split into S slices of O: with O >= 512
 // a thread holds EPT = O / 512 outputs and takes every string; with fewer,
 // 512 / O groups of warps share the strings and are summed in a fixed order.
-template <typename R> struct HSliceStr { R g; uint32_t X, tau; };   // X bit 31: nY odd
+// GROUPED (Jordan-Wigner strings, about four per mask): the strings of a mask
+// first add up their signed coefficients per output, real part from even nY,
+// imaginary from odd, and the partner is read and multiplied once.
+template <typename R> struct HSliceStr { R g; uint32_t X, tau; };   // X bit 31: nY odd, bit 30: last of its mask
 constexpr int kHSliceTab = 256;                                     // strings staged at a time
-template <typename R, int EPT>
+template <typename R, int EPT, bool GROUPED>
 __global__ void __launch_bounds__(512) k_hpsi_slice(const Cx<R> *__restrict__ psi, Cx<R> *__restrict__ lam,
                                                     const CosetArgs a, const DevString *__restrict__ strs, int first,
                                                     int last, double *__restrict__ epart, int slices) {
@@ -4247,11 +4250,54 @@ __global__ void __launch_bounds__(512) k_hpsi_slice(const Cx<R> *__restrict__ ps
             const bool neg = ((S.nY >> 1) ^ S.nY ^ __popcll(rep & S.z)) & 1;
             h.g = neg ? -(R)S.coef : (R)S.coef;
             h.X = S.X | ((uint32_t)(S.nY & 1) << 31);
+            if (GROUPED && (q + 1 == nq || strs[q0 + q + 1].X != S.X)) h.X |= 1u << 30;
             h.tau = coset_tau(S, a.kl);
             tab[q] = h;
         }
         cp_async_wait0();
         __syncthreads();
+        if constexpr (GROUPED) {
+            // whole masks go round the string groups
+            R fe[EPT], fo[EPT];
+            uint32_t turn = 0, parts = 0;
+#pragma unroll
+            for (int j = 0; j < EPT; ++j) fe[j] = fo[j] = 0;
+            for (int q = 0; q < nq; ++q) {
+                const HSliceStr<R> h = tab[q];
+                if (turn == sgrp) {
+                    const R g = (__popc(e0 & h.tau) & 1) ? -h.g : h.g;
+                    const uint32_t jm = EPT > 1 ? walsh_mask((h.tau >> 9) & (EPT - 1)) : 0u;
+                    if (h.X >> 31) {
+                        parts |= 2u;
+#pragma unroll
+                        for (int j = 0; j < EPT; ++j) fo[j] += ((jm >> j) & 1u) ? -g : g;
+                    } else {
+                        parts |= 1u;
+#pragma unroll
+                        for (int j = 0; j < EPT; ++j) fe[j] += ((jm >> j) & 1u) ? -g : g;
+                    }
+                    if (h.X & (1u << 30)) {
+                        const uint32_t X = h.X & 0x3FFFFFFFu;
+#pragma unroll
+                        for (int j = 0; j < EPT; ++j) {
+                            const Cx<R> v = t[(e0 + j * 512u) ^ X];
+                            if (parts & 1u) {
+                                acc[j].x += fe[j] * v.x;
+                                acc[j].y += fe[j] * v.y;
+                            }
+                            if (parts & 2u) {     // i * f * v
+                                acc[j].x -= fo[j] * v.y;
+                                acc[j].y += fo[j] * v.x;
+                            }
+                            fe[j] = fo[j] = 0;
+                        }
+                        parts = 0;
+                    }
+                }
+                if (h.X & (1u << 30)) turn = turn + 1 == nsg ? 0 : turn + 1;
+            }
+            continue;
+        }
 #pragma unroll 4
         for (int q = (int)sgrp; q < nq; q += (int)nsg) {
             const HSliceStr<R> h = tab[q];
@@ -5549,6 +5595,7 @@ cudaError_t launch_evc_slice(sv_dtype dt, cudaStream_t st, const void *psi, cons
 template <typename R>
 cudaError_t hpsi_slice_dispatch(cudaStream_t st, const void *psi, void *lam, const CosetArgs &a, const DevString *strs,
                                 int first, int last, double *epart, int *rows) {
+    const bool grouped = a.s_end - a.s_begin >= 2 * (a.g_end - a.g_begin);
     const int E = 1 << (a.kl + a.m), ncos = 1 << a.nfree;
     int S = 1;
     while (ncos * S < device_sms() && E / (2 * S) >= 32) S *= 2;
@@ -5558,9 +5605,14 @@ cudaError_t hpsi_slice_dispatch(cudaStream_t st, const void *psi, void *lam, con
     *rows = ncos * S;
 #define SV_HS_CASE(N)                                                                                        \
     case N:                                                                                                  \
-        allow_smem(k_hpsi_slice<R, N>, sm);                                                                  \
-        return launch(k_hpsi_slice<R, N>, ncos * S, 512, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, strs,  \
-                      first, last, epart, S);
+        if (grouped) {                                                                                       \
+            allow_smem(k_hpsi_slice<R, N, true>, sm);                                                        \
+            return launch(k_hpsi_slice<R, N, true>, ncos * S, 512, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, \
+                          a, strs, first, last, epart, S);                                                   \
+        }                                                                                                    \
+        allow_smem(k_hpsi_slice<R, N, false>, sm);                                                           \
+        return launch(k_hpsi_slice<R, N, false>, ncos * S, 512, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, \
+                      strs, first, last, epart, S);
     switch (ept) {
         SV_HS_CASE(1)
         SV_HS_CASE(2)
