@@ -1358,76 +1358,76 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
     bool stepped = dt == SV_C64 && kmax == 13 && o.threads == 512 && n >= 13;
     size_t step_smem = 0;
     for (;;) {
-    po.reg_threads = stepped ? 0 : 512;
-    po.reg_pairs = stepped;                // gate by gate, phases hold RY / RZ / CZ only
-    po.max_diag = stepped ? kMaxPassDiag : 0;
-    po.image_limit = stepped ? batch_table_room() : 0;
-    plan_pass_off = {0};
-    plan_op_off = {0};
-    gparam.clear(); passes.clear(); phases.clear(); ops.clear(); plan_keys.clear();
-    step_off.clear(); steps.clear(); dblocks.clear(); dmembers.clear();
-    for (int b = 0; b < batch; ++b) {
-        const int gb = gate_off[b], ge = gate_off[b + 1];
-        const int pb = param_off[b], pe = param_off[b + 1];
-        if (ge < gb || pe < pb) return fail(SV_EINVAL, "offsets must be non-decreasing");
-        const size_t m = (size_t)(ge - gb), np = (size_t)(pe - pb);
-        if ((int)m > batch_max_gates()) return fail(SV_EINVAL, "sv_batch_run: more than 1024 gates in a state");
-        std::string err = validate_gates(n, gates + gb, m, np, 0);
-        if (!err.empty()) return fail(SV_EINVAL, "state " + std::to_string(b) + ": " + err);
-        for (size_t i = 0; i < np; ++i)
-            if (!std::isfinite(params[pb + i])) return fail(SV_EINVAL, "non-finite parameter");
-        for (size_t i = 0; i < m; ++i) {
-            const int k = gates[gb + i].kind;
-            gparam.push_back((k == SV_RY || k == SV_RZ || k == SV_GIVENS || k == SV_DEXC) ? gates[gb + i].param : -1);
-        }
-        gsize[b] = (int)m;
-        const uint64_t key = hash_bytes(gates + gb, m * sizeof(sv_gate));
-        int pi = -1;
-        for (size_t k = 0; k < plan_keys.size(); ++k)
-            if (plan_keys[k] == key) pi = (int)k;
-        if (pi < 0) {
-            QsuPlan P;
-            err = plan_qsu(n, 0, gates + gb, m, true, po, l2p, P);
+        po.reg_threads = stepped ? 0 : 512;
+        po.reg_pairs = stepped;                // gate by gate, phases hold RY / RZ / CZ only
+        po.max_diag = stepped ? kMaxPassDiag : 0;
+        po.image_limit = stepped ? batch_table_room() : 0;
+        plan_pass_off = {0};
+        plan_op_off = {0};
+        gparam.clear(); passes.clear(); phases.clear(); ops.clear(); plan_keys.clear();
+        step_off.clear(); steps.clear(); dblocks.clear(); dmembers.clear();
+        for (int b = 0; b < batch; ++b) {
+            const int gb = gate_off[b], ge = gate_off[b + 1];
+            const int pb = param_off[b], pe = param_off[b + 1];
+            if (ge < gb || pe < pb) return fail(SV_EINVAL, "offsets must be non-decreasing");
+            const size_t m = (size_t)(ge - gb), np = (size_t)(pe - pb);
+            if ((int)m > batch_max_gates()) return fail(SV_EINVAL, "sv_batch_run: more than 1024 gates in a state");
+            std::string err = validate_gates(n, gates + gb, m, np, 0);
             if (!err.empty()) return fail(SV_EINVAL, "state " + std::to_string(b) + ": " + err);
-            if ((int)P.ops.size() > batch_max_ops()) return fail(SV_EINVAL, "sv_batch_run: more than 512 gates in a state");
-            const int obase = (int)ops.size();
-            const int pbase = (int)phases.size();
-            step_off.push_back({pbase, (int32_t)steps.size(), (int32_t)dblocks.size(), (int32_t)dmembers.size()});
-            for (auto &gp : P.passes) {
-                GatePassArgs a = gate_args(n, gp);
-                if (!stepped) {
-                    a.op_begin += obase;
-                    a.op_end += obase;
-                    if (a.ph_begin >= 0) {
-                        a.ph_begin += pbase;
-                        a.ph_end += pbase;
+            for (size_t i = 0; i < np; ++i)
+                if (!std::isfinite(params[pb + i])) return fail(SV_EINVAL, "non-finite parameter");
+            for (size_t i = 0; i < m; ++i) {
+                const int k = gates[gb + i].kind;
+                gparam.push_back((k == SV_RY || k == SV_RZ || k == SV_GIVENS || k == SV_DEXC) ? gates[gb + i].param : -1);
+            }
+            gsize[b] = (int)m;
+            const uint64_t key = hash_bytes(gates + gb, m * sizeof(sv_gate));
+            int pi = -1;
+            for (size_t k = 0; k < plan_keys.size(); ++k)
+                if (plan_keys[k] == key) pi = (int)k;
+            if (pi < 0) {
+                QsuPlan P;
+                err = plan_qsu(n, 0, gates + gb, m, true, po, l2p, P);
+                if (!err.empty()) return fail(SV_EINVAL, "state " + std::to_string(b) + ": " + err);
+                if ((int)P.ops.size() > batch_max_ops()) return fail(SV_EINVAL, "sv_batch_run: more than 512 gates in a state");
+                const int obase = (int)ops.size();
+                const int pbase = (int)phases.size();
+                step_off.push_back({pbase, (int32_t)steps.size(), (int32_t)dblocks.size(), (int32_t)dmembers.size()});
+                for (auto &gp : P.passes) {
+                    GatePassArgs a = gate_args(n, gp);
+                    if (!stepped) {
+                        a.op_begin += obase;
+                        a.op_end += obase;
+                        if (a.ph_begin >= 0) {
+                            a.ph_begin += pbase;
+                            a.ph_end += pbase;
+                        }
+                        a.db_begin = a.db_end = 0;
                     }
-                    a.db_begin = a.db_end = 0;
+                    passes.push_back(a);
                 }
-                passes.push_back(a);
-            }
-            for (Phase f : P.phases) {
-                if (!stepped) {
-                    f.op_begin += obase;
-                    f.op_end += obase;
+                for (Phase f : P.phases) {
+                    if (!stepped) {
+                        f.op_begin += obase;
+                        f.op_end += obase;
+                    }
+                    phases.push_back(f);
                 }
-                phases.push_back(f);
+                steps.insert(steps.end(), P.steps.begin(), P.steps.end());
+                dblocks.insert(dblocks.end(), P.dblocks.begin(), P.dblocks.end());
+                dmembers.insert(dmembers.end(), P.dmembers.begin(), P.dmembers.end());
+                ops.insert(ops.end(), P.ops.begin(), P.ops.end());
+                plan_pass_off.push_back((int32_t)passes.size());
+                plan_op_off.push_back((int32_t)ops.size());
+                pi = (int)plan_keys.size();
+                plan_keys.push_back(key);
             }
-            steps.insert(steps.end(), P.steps.begin(), P.steps.end());
-            dblocks.insert(dblocks.end(), P.dblocks.begin(), P.dblocks.end());
-            dmembers.insert(dmembers.end(), P.dmembers.begin(), P.dmembers.end());
-            ops.insert(ops.end(), P.ops.begin(), P.ops.end());
-            plan_pass_off.push_back((int32_t)passes.size());
-            plan_op_off.push_back((int32_t)ops.size());
-            pi = (int)plan_keys.size();
-            plan_keys.push_back(key);
+            state_plan[b] = pi;
         }
-        state_plan[b] = pi;
-    }
-    if (!stepped) break;
-    step_smem = batch_step_bytes(dt, n, kmax, o.threads, passes);
-    if (step_smem) break;
-    stepped = false;
+        if (!stepped) break;
+        step_smem = batch_step_bytes(dt, n, kmax, o.threads, passes);
+        if (step_smem) break;
+        stepped = false;
     }
     EvcPlan H;
     std::string err = plan_hpsi(n, paulis, coeffs, nterms, po, l2p, H);

@@ -874,12 +874,6 @@ template <typename R> __device__ __forceinline__ RA<R> cx_ra(Cx<R> a);
 template <> __device__ __forceinline__ unsigned long long cx_ra<float>(float2 a) { return f2_pack(a.x, a.y); }
 template <> __device__ __forceinline__ double2 cx_ra<double>(double2 a) { return a; }
 
-template <typename R> __device__ __forceinline__ RA<R> ra_neg(RA<R> a);
-template <> __device__ __forceinline__ unsigned long long ra_neg<float>(unsigned long long a) {
-    return a ^ 0x8000000080000000ull;
-}
-template <> __device__ __forceinline__ double2 ra_neg<double>(double2 a) { return make_double2(-a.x, -a.y); }
-
 // a * w (complex), or a * conj(w)
 template <typename R>
 __device__ __forceinline__ RA<R> ra_cmul(RA<R> a, Cx<R> w) {
@@ -1654,49 +1648,49 @@ __device__ __forceinline__ void fwd_steps(RA<R> *x, const PhaseS &F, const GateP
             default: break;
             }
         }
-        return;
-    }
-    for (int s = F.st_begin; s < F.st_end; ++s) {
-        const RegStep S = st[s];
-        if (S.type == SV_STEP_ROT) {
-            // factored RYs (t, t): the factors are applied at the store
-            const Cx<R> *c = cs + (S.op_begin - a.op_begin);
+    } else {
+        for (int s = F.st_begin; s < F.st_end; ++s) {
+            const RegStep S = st[s];
+            if (S.type == SV_STEP_ROT) {
+                // factored RYs (t, t): the factors are applied at the store
+                const Cx<R> *c = cs + (S.op_begin - a.op_begin);
 #pragma unroll
-            for (int b = 0; b < RB; ++b) {
-                if (!((S.a >> b) & 1)) continue;
-                const Cx<R> k = *c++;
-                ra_rotf_bit<R, V, RB>(x, b, (S.a >> (8 + b)) & 1, rotf<R>(k));
-            }
-        } else if (S.type == SV_STEP_DIAG) {
-            reg_diag<R, RB>(x, bl[S.a - a.db_begin], area, thread);
-        } else {
-            const uint32_t code = (uint32_t)S.a & 255u, t0 = ((uint32_t)S.a >> 8) & 255u, t1 = ((uint32_t)S.a >> 16) & 255u;
-            const uint32_t base = phase_bits<R>(place);
-            if (code == RO_RZ) {
-                reg_rz<R>(x, cs[S.op_begin], diag_bit_mask(t0, F.rmask, base, gbase));
-            } else if (code == RO_CZ) {
-                reg_cz<R>(x, diag_bit_mask(t0, F.rmask, base, gbase) & diag_bit_mask(t1, F.rmask, base, gbase));
-            } else if constexpr (KIND == kStepsAll || KIND == kStepsMixed) {
-                const Cx<R> *M = pmats + S.op_end;
-                uint32_t pc = 0;
-                RotK<R> k{};
-                if (code < RO_MAT1) k = pair_rec<R>(rk + 4 * S.op_begin, pc);
-                switch (code) {
+                for (int b = 0; b < RB; ++b) {
+                    if (!((S.a >> b) & 1)) continue;
+                    const Cx<R> k = *c++;
+                    ra_rotf_bit<R, V, RB>(x, b, (S.a >> (8 + b)) & 1, rotf<R>(k));
+                }
+            } else if (S.type == SV_STEP_DIAG) {
+                reg_diag<R, RB>(x, bl[S.a - a.db_begin], area, thread);
+            } else {
+                const uint32_t code = (uint32_t)S.a & 255u, t0 = ((uint32_t)S.a >> 8) & 255u, t1 = ((uint32_t)S.a >> 16) & 255u;
+                const uint32_t base = phase_bits<R>(place);
+                if (code == RO_RZ) {
+                    reg_rz<R>(x, cs[S.op_begin], diag_bit_mask(t0, F.rmask, base, gbase));
+                } else if (code == RO_CZ) {
+                    reg_cz<R>(x, diag_bit_mask(t0, F.rmask, base, gbase) & diag_bit_mask(t1, F.rmask, base, gbase));
+                } else if constexpr (KIND == kStepsAll || KIND == kStepsMixed) {
+                    const Cx<R> *M = pmats + S.op_end;
+                    uint32_t pc = 0;
+                    RotK<R> k{};
+                    if (code < RO_MAT1) k = pair_rec<R>(rk + 4 * S.op_begin, pc);
+                    switch (code) {
 #define SV_C(MU, MV) ra_pair_rot<R, V, MU, MV>(x, k)
-                    SV_RO_GIVENS(SV_C)
+                        SV_RO_GIVENS(SV_C)
 #undef SV_C
-                case RO_MAT1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 0>(x, M); } break;
-                case RO_MAT1 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 1>(x, M); } break;
-                case RO_MAT1 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 2>(x, M); } break;
-                case RO_MAT1 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 3, 3>(x, M); } break;
-                case RO_MAT2: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 1>(x, M); } break;
-                case RO_MAT2 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 2>(x, M); } break;
-                case RO_MAT2 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 3>(x, M); } break;
-                case RO_MAT2 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 2>(x, M); } break;
-                case RO_MAT2 + 4: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 3>(x, M); } break;
-                case RO_MAT2 + 5: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 3>(x, M); } break;
-                case RO_MAT4: if constexpr (KIND == kStepsAll) { reg_mat4<R>(x, M); } break;
-                default: break;
+                    case RO_MAT1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 0>(x, M); } break;
+                    case RO_MAT1 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 1>(x, M); } break;
+                    case RO_MAT1 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 2>(x, M); } break;
+                    case RO_MAT1 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 3, 3>(x, M); } break;
+                    case RO_MAT2: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 1>(x, M); } break;
+                    case RO_MAT2 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 2>(x, M); } break;
+                    case RO_MAT2 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 3>(x, M); } break;
+                    case RO_MAT2 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 2>(x, M); } break;
+                    case RO_MAT2 + 4: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 3>(x, M); } break;
+                    case RO_MAT2 + 5: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 3>(x, M); } break;
+                    case RO_MAT4: if constexpr (KIND == kStepsAll) { reg_mat4<R>(x, M); } break;
+                    default: break;
+                    }
                 }
             }
         }
@@ -1741,119 +1735,119 @@ __device__ __forceinline__ void adj_steps(RA<R> *xp, RA<R> *xl, const PhaseS &F,
                 held = 0;
             }
         }
-        return;
-    }
-    for (int s = F.st_end - 1; s >= F.st_begin; --s) {
-        const RegStep S = st[s];
-        const R fs = scf[s], fs2 = fs * fs;
-        if (S.type == SV_STEP_ROT) {
-            // every RY of the step: gradient part at the step's end (they commute), then RY^dagger
-            R g[4] = {0, 0, 0, 0};
+    } else {
+        for (int s = F.st_end - 1; s >= F.st_begin; --s) {
+            const RegStep S = st[s];
+            const R fs = scf[s], fs2 = fs * fs;
+            if (S.type == SV_STEP_ROT) {
+                // every RY of the step: gradient part at the step's end (they commute), then RY^dagger
+                R g[4] = {0, 0, 0, 0};
 #pragma unroll
-            for (int b = 0; b < RB; ++b) {
-                if (!((S.a >> b) & 1)) continue;
-                switch (b) {
-                case 0: g[0] = ra_ry_grad<R, V, 0>(xp, xl); break;
-                case 1: g[1] = ra_ry_grad<R, V, 1>(xp, xl); break;
-                case 2: g[2] = ra_ry_grad<R, V, 2>(xp, xl); break;
-                default: g[3] = ra_ry_grad<R, V, 3>(xp, xl); break;
+                for (int b = 0; b < RB; ++b) {
+                    if (!((S.a >> b) & 1)) continue;
+                    switch (b) {
+                    case 0: g[0] = ra_ry_grad<R, V, 0>(xp, xl); break;
+                    case 1: g[1] = ra_ry_grad<R, V, 1>(xp, xl); break;
+                    case 2: g[2] = ra_ry_grad<R, V, 2>(xp, xl); break;
+                    default: g[3] = ra_ry_grad<R, V, 3>(xp, xl); break;
+                    }
                 }
-            }
-            const R tot = warp_sum4<R>(g[0], g[1], g[2], g[3]) * fs2;
-            const Cx<R> *c = cs + (S.op_begin - a.op_begin);
-            int o = S.op_begin - a.op_begin;
+                const R tot = warp_sum4<R>(g[0], g[1], g[2], g[3]) * fs2;
+                const Cx<R> *c = cs + (S.op_begin - a.op_begin);
+                int o = S.op_begin - a.op_begin;
 #pragma unroll
-            for (int b = 0; b < RB; ++b) {
-                if (!((S.a >> b) & 1)) continue;
-                if (lane == 8 * b) acc[o * AS + warp] += tot;
-                ++o;
-                const Cx<R> k = *c++;
-                const RotF<R> rf = rotf<R>(k);
-                const bool fb = (S.a >> (8 + b)) & 1;
-                ra_rotf_bit<R, V, RB>(xp, b, fb, rf);
-                ra_rotf_bit<R, V, RB>(xl, b, fb, rf);
-            }
-        } else if (S.type == SV_STEP_DIAG) {
-            // every RZ member's generator expectation at the block's end (Z
-            // commutes with the block), then D^dagger on both register sets
-            const DiagBlock B = bl[S.a - a.db_begin];
-            R tv[V], tot = 0;
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                tv[v] = ra_imdot<R>(xl[v], xp[v]);
-                tot += tv[v];
-            }
-            if (B.kind == 0) {
-                R sb[4] = {0, 0, 0, 0};
-                signed_bit_sums<R, RB>(tv, sb);
-                const R red = warp_sum4<R>(sb[0], sb[1], sb[2], sb[3]) * fs2;
-                for (int mi = B.m_begin; mi < B.m_end; ++mi) {
-                    const DiagMember m = mem[mi - a.mem_begin];
-                    if (m.type == SV_DM_REG_RZ && lane == 8 * m.a) acc[(m.op - a.op_begin) * AS + warp] += red;
+                for (int b = 0; b < RB; ++b) {
+                    if (!((S.a >> b) & 1)) continue;
+                    if (lane == 8 * b) acc[o * AS + warp] += tot;
+                    ++o;
+                    const Cx<R> k = *c++;
+                    const RotF<R> rf = rotf<R>(k);
+                    const bool fb = (S.a >> (8 + b)) & 1;
+                    ra_rotf_bit<R, V, RB>(xp, b, fb, rf);
+                    ra_rotf_bit<R, V, RB>(xl, b, fb, rf);
                 }
-            } else {
-                // thread RZ members: +-tot by the thread's bit, four at a time
-                const uint32_t base = phase_bits<R>(place);
-                for (int m0 = B.m_begin; m0 < B.m_end; m0 += 4) {
-                    R vals[4] = {0, 0, 0, 0};
-                    int opi[4] = {-1, -1, -1, -1};
+            } else if (S.type == SV_STEP_DIAG) {
+                // every RZ member's generator expectation at the block's end (Z
+                // commutes with the block), then D^dagger on both register sets
+                const DiagBlock B = bl[S.a - a.db_begin];
+                R tv[V], tot = 0;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        if (m0 + j < B.m_end) {
-                            const DiagMember m = mem[m0 + j - a.mem_begin];
-                            if (m.type == SV_DM_THR_RZ) {
-                                vals[j] = ((base >> m.a) & 1u) ? -tot : tot;
-                                opi[j] = m.op - a.op_begin;
+                for (int v = 0; v < V; ++v) {
+                    tv[v] = ra_imdot<R>(xl[v], xp[v]);
+                    tot += tv[v];
+                }
+                if (B.kind == 0) {
+                    R sb[4] = {0, 0, 0, 0};
+                    signed_bit_sums<R, RB>(tv, sb);
+                    const R red = warp_sum4<R>(sb[0], sb[1], sb[2], sb[3]) * fs2;
+                    for (int mi = B.m_begin; mi < B.m_end; ++mi) {
+                        const DiagMember m = mem[mi - a.mem_begin];
+                        if (m.type == SV_DM_REG_RZ && lane == 8 * m.a) acc[(m.op - a.op_begin) * AS + warp] += red;
+                    }
+                } else {
+                    // thread RZ members: +-tot by the thread's bit, four at a time
+                    const uint32_t base = phase_bits<R>(place);
+                    for (int m0 = B.m_begin; m0 < B.m_end; m0 += 4) {
+                        R vals[4] = {0, 0, 0, 0};
+                        int opi[4] = {-1, -1, -1, -1};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (m0 + j < B.m_end) {
+                                const DiagMember m = mem[m0 + j - a.mem_begin];
+                                if (m.type == SV_DM_THR_RZ) {
+                                    vals[j] = ((base >> m.a) & 1u) ? -tot : tot;
+                                    opi[j] = m.op - a.op_begin;
+                                }
                             }
                         }
+                        const R red = warp_sum4<R>(vals[0], vals[1], vals[2], vals[3]) * fs2;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (lane == 8 * j && opi[j] >= 0) acc[opi[j] * AS + warp] += red;
                     }
-                    const R red = warp_sum4<R>(vals[0], vals[1], vals[2], vals[3]) * fs2;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (lane == 8 * j && opi[j] >= 0) acc[opi[j] * AS + warp] += red;
                 }
-            }
-            reg_diag2<R, RB>(xp, xl, B, area);
-        } else {
-            const uint32_t code = (uint32_t)S.a & 255u, t0 = ((uint32_t)S.a >> 8) & 255u, t1 = ((uint32_t)S.a >> 16) & 255u;
-            const uint32_t base = phase_bits<R>(place);
-            if (code == RO_RZ) {
-                const uint32_t m = diag_bit_mask(t0, F.rmask, base, gbase);
-                R g = 0;
+                reg_diag2<R, RB>(xp, xl, B, area);
+            } else {
+                const uint32_t code = (uint32_t)S.a & 255u, t0 = ((uint32_t)S.a >> 8) & 255u, t1 = ((uint32_t)S.a >> 16) & 255u;
+                const uint32_t base = phase_bits<R>(place);
+                if (code == RO_RZ) {
+                    const uint32_t m = diag_bit_mask(t0, F.rmask, base, gbase);
+                    R g = 0;
 #pragma unroll
-                for (int v = 0; v < V; ++v) g += flip_by(ra_imdot<R>(xl[v], xp[v]), m, v);
-                const Cx<R> k = cs[S.op_begin];
-                reg_rz<R>(xp, k, m);
-                reg_rz<R>(xl, k, m);
-                g = warp_sum<R>(g) * fs2;
-                if (lane == 0) acc[S.op_begin * AS + warp] += g;
-            } else if (code == RO_CZ) {
-                const uint32_t m = diag_bit_mask(t0, F.rmask, base, gbase) & diag_bit_mask(t1, F.rmask, base, gbase);
-                reg_cz<R>(xp, m);
-                reg_cz<R>(xl, m);
-            } else if constexpr (KIND == kStepsAll || KIND == kStepsMixed) {
-                // the prepared matrix is followed by its conjugate transpose (1-qubit matrices: 4 elements)
-                const Cx<R> *M = pmats + S.op_end + 4;
-                uint32_t pc = 0;
-                RotK<R> k{};
-                R g = 0;
-                if (code < RO_MAT1) k = pair_rec<R>(rk + 4 * S.op_begin, pc);
-                switch (code) {
-#define SV_C(MU, MV)                                  \
-    g = ra_pair_grad<R, V, MU, MV>(xp, xl);           \
-    ra_pair_rot<R, V, MU, MV>(xp, k);                 \
-    ra_pair_rot<R, V, MU, MV>(xl, k)
-                    SV_RO_GIVENS(SV_C)
-#undef SV_C
-                case RO_MAT1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 0>(xp, M); reg_mat<R, 0, 0>(xl, M); } break;
-                case RO_MAT1 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 1>(xp, M); reg_mat<R, 1, 1>(xl, M); } break;
-                case RO_MAT1 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 2>(xp, M); reg_mat<R, 2, 2>(xl, M); } break;
-                case RO_MAT1 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 3, 3>(xp, M); reg_mat<R, 3, 3>(xl, M); } break;
-                default: break;
-                }
-                if (code < RO_MAT1) {
+                    for (int v = 0; v < V; ++v) g += flip_by(ra_imdot<R>(xl[v], xp[v]), m, v);
+                    const Cx<R> k = cs[S.op_begin];
+                    reg_rz<R>(xp, k, m);
+                    reg_rz<R>(xl, k, m);
                     g = warp_sum<R>(g) * fs2;
                     if (lane == 0) acc[S.op_begin * AS + warp] += g;
+                } else if (code == RO_CZ) {
+                    const uint32_t m = diag_bit_mask(t0, F.rmask, base, gbase) & diag_bit_mask(t1, F.rmask, base, gbase);
+                    reg_cz<R>(xp, m);
+                    reg_cz<R>(xl, m);
+                } else if constexpr (KIND == kStepsAll || KIND == kStepsMixed) {
+                    // the prepared matrix is followed by its conjugate transpose (1-qubit matrices: 4 elements)
+                    const Cx<R> *M = pmats + S.op_end + 4;
+                    uint32_t pc = 0;
+                    RotK<R> k{};
+                    R g = 0;
+                    if (code < RO_MAT1) k = pair_rec<R>(rk + 4 * S.op_begin, pc);
+                    switch (code) {
+#define SV_C(MU, MV)                                  \
+        g = ra_pair_grad<R, V, MU, MV>(xp, xl);           \
+        ra_pair_rot<R, V, MU, MV>(xp, k);                 \
+        ra_pair_rot<R, V, MU, MV>(xl, k)
+                        SV_RO_GIVENS(SV_C)
+#undef SV_C
+                    case RO_MAT1: if constexpr (KIND == kStepsAll) { reg_mat<R, 0, 0>(xp, M); reg_mat<R, 0, 0>(xl, M); } break;
+                    case RO_MAT1 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 1>(xp, M); reg_mat<R, 1, 1>(xl, M); } break;
+                    case RO_MAT1 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 2>(xp, M); reg_mat<R, 2, 2>(xl, M); } break;
+                    case RO_MAT1 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 3, 3>(xp, M); reg_mat<R, 3, 3>(xl, M); } break;
+                    default: break;
+                    }
+                    if (code < RO_MAT1) {
+                        g = warp_sum<R>(g) * fs2;
+                        if (lane == 0) acc[S.op_begin * AS + warp] += g;
+                    }
                 }
             }
         }
@@ -3340,7 +3334,7 @@ __global__ void __launch_bounds__(1 << LOGNT, 1) k_evc_ring(const Cx<R> *__restr
 // signed sum up to its last level.  The coset is only read, so the warps run
 // their (phase, eighth of the coset) units without barriers; what remains per
 // string is its sign bit and its share of a four-value warp reduction.
-// n = 28, 4096 strings (16 passes): 106 -> see DESIGN.
+// n = 28, 4096 strings (16 passes): 106.8 -> 38.5 ms.
 // Products and folds are scalar: packing two of them into f32x2 registers
 // halved the fold but cost more in moves.  The first product of a pair is
 // volatile: the compiler otherwise hoists the products that the codes of the
@@ -4296,30 +4290,30 @@ __global__ void __launch_bounds__(512) k_hpsi_slice(const Cx<R> *__restrict__ ps
                 }
                 if (h.X & (1u << 30)) turn = turn + 1 == nsg ? 0 : turn + 1;
             }
-            continue;
-        }
+        } else {
 #pragma unroll 4
-        for (int q = (int)sgrp; q < nq; q += (int)nsg) {
-            const HSliceStr<R> h = tab[q];
-            const uint32_t X = h.X & 0x7FFFFFFFu;
-            const R g = (__popc(e0 & h.tau) & 1) ? -h.g : h.g;
-            // parity of j's bits (element bits 9 and up) against tau
-            const uint32_t jm = EPT > 1 ? walsh_mask((h.tau >> 9) & (EPT - 1)) : 0u;
-            if (h.X >> 31) {          // i * f * v
+            for (int q = (int)sgrp; q < nq; q += (int)nsg) {
+                const HSliceStr<R> h = tab[q];
+                const uint32_t X = h.X & 0x7FFFFFFFu;
+                const R g = (__popc(e0 & h.tau) & 1) ? -h.g : h.g;
+                // parity of j's bits (element bits 9 and up) against tau
+                const uint32_t jm = EPT > 1 ? walsh_mask((h.tau >> 9) & (EPT - 1)) : 0u;
+                if (h.X >> 31) {          // i * f * v
 #pragma unroll
-                for (int j = 0; j < EPT; ++j) {
-                    const Cx<R> v = t[(e0 + j * 512u) ^ X];
-                    const R f = ((jm >> j) & 1u) ? -g : g;
-                    acc[j].x -= f * v.y;
-                    acc[j].y += f * v.x;
-                }
-            } else {
+                    for (int j = 0; j < EPT; ++j) {
+                        const Cx<R> v = t[(e0 + j * 512u) ^ X];
+                        const R f = ((jm >> j) & 1u) ? -g : g;
+                        acc[j].x -= f * v.y;
+                        acc[j].y += f * v.x;
+                    }
+                } else {
 #pragma unroll
-                for (int j = 0; j < EPT; ++j) {
-                    const Cx<R> v = t[(e0 + j * 512u) ^ X];
-                    const R f = ((jm >> j) & 1u) ? -g : g;
-                    acc[j].x += f * v.x;
-                    acc[j].y += f * v.y;
+                    for (int j = 0; j < EPT; ++j) {
+                        const Cx<R> v = t[(e0 + j * 512u) ^ X];
+                        const R f = ((jm >> j) & 1u) ? -g : g;
+                        acc[j].x += f * v.x;
+                        acc[j].y += f * v.y;
+                    }
                 }
             }
         }
@@ -5572,8 +5566,10 @@ cudaError_t launch_hpsi_pass(sv_dtype dt, cudaStream_t st, int grid, const void 
 // Slices of a coset for the kernels above: about two CTAs for each SM in all,
 // as far as the strings (a warp each) or the outputs (at least 32) go.  The
 // line between whole cosets and slices is two cosets per SM: with fewer, the
-// double-buffered kernels have nothing to overlap (measured on random strings,
-// complex64, per H|psi> pass: see the kernel's comment).
+// double-buffered kernels have nothing to overlap.  complex64, n = 14, 256
+// random strings (2 cosets): an H|psi> pass 210 -> 12 us.  complex128 is bound
+// by its FP64 arithmetic, which one coset per SM already spreads; from there on
+// slices only repeat the loads (4 % slower at n = 20).
 bool coset_slices_pay(sv_dtype dt, const CosetArgs &a) {
     return a.kl + a.m >= 6 && a.nfree < 16 && (1 << a.nfree) < (dt == SV_C64 ? 2 : 1) * device_sms();
 }
