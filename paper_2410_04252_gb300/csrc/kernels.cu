@@ -3629,6 +3629,20 @@ struct __align__(16) EvcUnitS {
     float fac;               // 2 when each pair is taken once
 };
 
+// The eight rows of a coset's copy in Gray order: neighbours differ by one
+// basis vector, so a row's place is two XORs from the last one's (a table in
+// shared memory cost a load for each row and coset, which the compiler may
+// not keep in registers across the copies).
+__host__ __device__ constexpr int gray(int q) { return q ^ (q >> 1); }
+__device__ __forceinline__ uint64_t gray_basis(int q, uint64_t r1, uint64_t r2, uint64_t r4) {
+    return (q & 1) ? r1 : (q & 2) ? r2 : r4;
+}
+__device__ __forceinline__ void eu_pair(float2 *x, const float2 *at) {
+    const float4 w = *reinterpret_cast<const float4 *>(at);
+    x[0] = make_float2(w.x, w.y);
+    x[1] = make_float2(w.z, w.w);
+}
+
 __global__ void __launch_bounds__(512, 1) k_evc_unit(const float2 *__restrict__ psi, const CosetArgs a,
                                                      const EvcUnitItem *__restrict__ items, int u_mid, int nu,
                                                      double *__restrict__ part, int part_stride) {
@@ -3648,7 +3662,7 @@ __global__ void __launch_bounds__(512, 1) k_evc_unit(const float2 *__restrict__ 
 #pragma unroll
         for (int l = 0; l < 4; ++l) s.lev[l] = ((t.w >> l) & 1u) ? -1.f : 1.f;
         s.code = t.code;
-        s.sX = swz_tile(t.X);
+        s.sX = t.X;
         s.last = ((t.w >> 4) & 1u) ? -1.f : 1.f;
         s.fac = t.code < 16u ? 2.f : 1.f;
         its[i] = s;
@@ -3658,8 +3672,9 @@ __global__ void __launch_bounds__(512, 1) k_evc_unit(const float2 *__restrict__ 
     // the half's registers: bit 0 and its four span bits
     const uint32_t rmask = 1u | (15u << (KL + 4 * half));
     uint32_t rest = (uint32_t)(tid & 255), base = 0;
-    // lanes: run bits 1..4 and the lowest span bit of the other half (their
-    // slots differ in bits 1..3, so 16-byte gathers are conflict-free)
+    // lanes: run bits 1..4 and the lowest span bit of the other half, so
+    // 16-byte gathers are conflict-free in the order of the coset itself, and
+    // a thread's places are one address and constants
     for (uint32_t m = (E - 1u) & ~rmask; m; m &= m - 1u, rest >>= 1)
         if (rest & 1u) base |= m & (0u - m);
     uint32_t tmask = 0;
@@ -3669,20 +3684,20 @@ __global__ void __launch_bounds__(512, 1) k_evc_unit(const float2 *__restrict__ 
         acc[i * 512 + tid] = 0.f;
     }
     for (int j = tid; j < kEvcUnitMax * 16; j += 512) wsum[j / 16][j % 16] = 0.0;
-    const uint32_t sbase = swz_tile(base);
-    uint32_t rb[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) rb[i] = swz_tile(1u << (KL + 4 * half + i));
     const uint64_t ncos = 1ull << a.nfree;
     const uint64_t mine = blockIdx.x < ncos ? (ncos - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
     const BitWalk bw = bit_walk(a.freeb, a.nfree, gridDim.x);
     uint64_t rep_pf = deposit(blockIdx.x, a.freeb, a.nfree), rep_cur = rep_pf;
-    const uint32_t e0 = 2u * (uint32_t)tid, slot0 = swz_tile(e0);
+    const uint32_t e0 = 2u * (uint32_t)tid;
     const uint64_t off0 = spanv[e0 >> KL] ^ (e0 & ((1u << KL) - 1u));
+    const uint64_t r1 = spanv[1024u >> KL], r2 = spanv[2048u >> KL], r4 = spanv[4096u >> KL];
     auto load = [&](float2 *dst, uint64_t rep) {
+        uint64_t x = rep ^ off0;
 #pragma unroll
-        for (uint32_t i = 0; i < 8; ++i)
-            cp_async16(dst + (slot0 ^ swz_tile(i * 1024u)), psi + (rep ^ off0 ^ spanv[(1024u >> KL) * i]));
+        for (int q = 0; q < 8; ++q) {
+            if (q) x ^= gray_basis(q, r1, r2, r4);
+            cp_async16(dst + e0 + 1024 * gray(q), psi + x);
+        }
     };
     __syncthreads();
     pdl_wait();
@@ -3704,15 +3719,13 @@ __global__ void __launch_bounds__(512, 1) k_evc_unit(const float2 *__restrict__ 
         const float2 *t = buf + (it % 3) * E;
         const uint32_t mask = tmask ^ __ballot_sync(0xffffffffu, lane < n && (__popcll(rep & zs[min(ub + lane, nu - 1)]) & 1));
         float2 x[32];
-        uint32_t idx[16];
-        idx[0] = sbase;
+        const float2 *tb = t + base;
+        if (half) {
 #pragma unroll
-        for (int v = 1; v < 16; ++v) idx[v] = idx[v & (v - 1)] ^ rb[(v & 1) ? 0 : (v & 2) ? 1 : (v & 4) ? 2 : 3];
+            for (int v = 0; v < 16; ++v) eu_pair(x + 2 * v, tb + v * (16 << KL));
+        } else {
 #pragma unroll
-        for (int v = 0; v < 16; ++v) {
-            const float4 w = *reinterpret_cast<const float4 *>(&t[idx[v]]);
-            x[2 * v] = make_float2(w.x, w.y);
-            x[2 * v + 1] = make_float2(w.z, w.w);
+            for (int v = 0; v < 16; ++v) eu_pair(x + 2 * v, tb + v * (1 << KL));
         }
         for (int i = 0; i < n; ++i) {
             const EvcUnitS S = its[ub + i];
@@ -3728,12 +3741,15 @@ __global__ void __launch_bounds__(512, 1) k_evc_unit(const float2 *__restrict__ 
             default: {
                 // partners from shared memory, every element; the register
                 // bits' signs: pairs (v, v + 16) fold into P by the fifth
-                const uint32_t sx = S.sX;
                 const bool im = S.code & 1u;
+                const uint32_t bx = base ^ (S.sX & ~rmask);
+                // X's register bits, in the order of v
+                const uint32_t xv = (S.sX & 1u) | (((S.sX >> (KL + 4 * half)) & 15u) << 1);
+                const uint32_t vs = KL + 4 * half - 1;
 #pragma unroll
                 for (int v = 0; v < 16; ++v) {
-                    const uint32_t lo = idx[v >> 1] ^ (uint32_t)(v & 1), hi = idx[(v + 16) >> 1] ^ (uint32_t)(v & 1);
-                    const float2 a0 = t[lo ^ sx], a1 = t[hi ^ sx];
+                    const uint32_t q = v ^ xv, u = q ^ 16u;
+                    const float2 a0 = t[bx | (q & 1u) | ((q & 30u) << vs)], a1 = t[bx | (u & 1u) | ((u & 30u) << vs)];
                     const float p0 = im ? a0.x * x[v].y - a0.y * x[v].x : a0.x * x[v].x + a0.y * x[v].y;
                     const float p1 = im ? a1.x * x[v + 16].y - a1.y * x[v + 16].x
                                         : a1.x * x[v + 16].x + a1.y * x[v + 16].y;
@@ -3926,11 +3942,14 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_vec(const float2 *__restrict__ 
     // the thread's first pair and the distance of its rows in the span
     const uint32_t e0 = 2u * threadIdx.x;
     const uint64_t off0 = spanv[e0 >> a.kl] ^ (e0 & lowmask);
-    const uint64_t *row = spanv;                        // spanv[(1024 >> kl) j]: the span is linear
-    const uint32_t rstep = 1024u >> a.kl;
+    const uint64_t r1 = spanv[1024u >> a.kl], r2 = spanv[2048u >> a.kl], r4 = spanv[4096u >> a.kl];
     auto load = [&](float2 *dst, uint64_t rep) {
+        uint64_t x = rep ^ off0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) cp_async16(dst + e0 + 1024 * j, psi + (rep ^ off0 ^ row[rstep * j]));
+        for (int q = 0; q < 8; ++q) {
+            if (q) x ^= gray_basis(q, r1, r2, r4);
+            cp_async16(dst + e0 + 1024 * gray(q), psi + x);
+        }
     };
     pdl_wait();
     pdl_next();
@@ -3947,12 +3966,14 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_vec(const float2 *__restrict__ 
         const float2 *t = buf + (it & 1) * E;
         float4 acc[8], old[8];
         float2 *lp = lam;
-        const uint64_t base = rep ^ off0;
+        uint64_t x = rep ^ off0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int q = 0; q < 8; ++q) {
+            const int j = gray(q);
+            if (q) x ^= gray_basis(q, r1, r2, r4);
             acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             old[j] = acc[j];
-            if (!first) old[j] = *reinterpret_cast<const float4 *>(lp + (base ^ row[rstep * j]));
+            if (!first) old[j] = *reinterpret_cast<const float4 *>(lp + x);
         }
         cp_async_wait1();
         __syncthreads();
@@ -3970,13 +3991,16 @@ __global__ void __launch_bounds__(512, 1) k_hpsi_vec(const float2 *__restrict__ 
                 hpsi_string(acc, tab[k].xc, tab[k].g ^ (((bmask >> k) & 1u) << 31), tab[k].w, sb);
         }
         float eloc = 0.f;
+        x = rep ^ off0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int q = 0; q < 8; ++q) {
+            const int j = gray(q);
+            if (q) x ^= gray_basis(q, r1, r2, r4);
             acc[j].x += old[j].x;
             acc[j].y += old[j].y;
             acc[j].z += old[j].z;
             acc[j].w += old[j].w;
-            *reinterpret_cast<float4 *>(lp + (base ^ row[rstep * j])) = acc[j];
+            *reinterpret_cast<float4 *>(lp + x) = acc[j];
             if (last) {
                 const float4 p = *reinterpret_cast<const float4 *>(t + e0 + 1024 * j);
                 eloc += p.x * acc[j].x + p.y * acc[j].y;
@@ -5137,6 +5161,17 @@ cudaError_t launch(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cu
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, A(v)...);
 }
+// The same without that attribute: the SMs drain first, so that they can take
+// the split of shared memory and L1 that this kernel asks for.
+template <typename... A, typename... V>
+cudaError_t launch_drained(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st, V... v) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, kernel, A(v)...);
+}
 
 size_t gate_smem(sv_dtype dt, int k, int nlow) {
     const size_t es = dt == SV_C64 ? 8 : 16;
@@ -5527,15 +5562,20 @@ cudaError_t hpsi_dispatch(cudaStream_t st, int grid, const void *psi, void *lam,
         if (E == 8192 && a.kl >= 1 && a.kl <= 10) {
             const int ns = a.s_end - a.s_begin;
             const size_t smv = sm + (size_t)ns * sizeof(HpsiStr);
+            // The old lambda comes through L1: behind gate passes, whose tiles take
+            // all of the SM as shared memory, an overlapped first pass would keep
+            // their split for the whole chain (the loads in flight then have 28 KB
+            // of L1; n = 25, 317 strings: 140 -> 190 us a pass).
+            auto go = [&](auto kernel) {
+                allow_smem(kernel, smv);
+                if (first)
+                    return launch_drained(kernel, grid, 512, smv, st, (const float2 *)psi, (float2 *)lam, a, strs,
+                                          first, last, epart);
+                return launch(kernel, grid, 512, smv, st, (const float2 *)psi, (float2 *)lam, a, strs, first, last,
+                              epart);
+            };
             // about eight strings a pass are random masks, hundreds Jordan-Wigner ones
-            if (ns > kHpsiTab) {
-                allow_smem(k_hpsi_vec<true>, smv);
-                return launch(k_hpsi_vec<true>, grid, 512, smv, st, (const float2 *)psi, (float2 *)lam, a, strs, first,
-                              last, epart);
-            }
-            allow_smem(k_hpsi_vec<false>, smv);
-            return launch(k_hpsi_vec<false>, grid, 512, smv, st, (const float2 *)psi, (float2 *)lam, a, strs, first,
-                          last, epart);
+            return ns > kHpsiTab ? go(k_hpsi_vec<true>) : go(k_hpsi_vec<false>);
         }
     }
 #define SV_HPSI_CASE(N)                                                                                      \
