@@ -499,8 +499,7 @@ sv_status evc_entry_upload(sv_handle *h, EvcEntry *ent, const double *coeffs, si
     for (auto &cp : ent->plan.passes) {
         ent->args.push_back(coset_args(h->n, cp));
         CosetArgs &a = ent->args.back();
-        // single strings keep per-thread partials in the kernels for few strings
-        if (cp.rp_end > cp.rp_begin && (a.few || !evc_reg_fits(h->dt, a, cp))) {
+        if (cp.rp_end > cp.rp_begin && !evc_reg_fits(h->dt, a, cp)) {
             cp.rp_end = cp.rp_begin;
             cp.g_reg = cp.g_begin;
             cp.s_reg = cp.s_begin;

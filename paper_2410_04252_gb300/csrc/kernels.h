@@ -55,8 +55,6 @@ struct DevString {
     uint32_t pad;
 };
 
-// Few-string expectation passes (every group one string): at most this many groups.
-constexpr int kEvcFew = 8;
 
 // First phase, step, diagonal block and block member of a plan (batched kernel
 // with step loops: indices inside a plan are its own).

@@ -106,7 +106,6 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
     sv::EvcPlan P;
     std::string err = sv::plan_hpsi(n, paulis, coeffs, nterms, po, l2p, P);
     if (!err.empty()) return noalloc_fail(SV_EINVAL, "plan: " + err);
-    if (dt == SV_C64) sv::plan_evc_units(P);
     const int nslots = (int)P.strings.size();
     const int ngroups = (int)P.groups.size();
 
@@ -130,21 +129,6 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
     for (auto &g : P.groups)
         for (int32_t q = g.s_begin; q < g.s_end; ++q) ss[q].X = g.X;
 
-    // carve the array: tables, results, then per-CTA partial rows
-    unsigned char *p = (unsigned char *)base;
-    size_t off = 0;
-    sv::DevGroup *d_groups = (sv::DevGroup *)(p + off); off = align256(off + ngroups * sizeof(sv::DevGroup));
-    sv::DevString *d_strs = (sv::DevString *)(p + off); off = align256(off + nslots * sizeof(sv::DevString));
-    sv::EvcUnitItem *d_units = (sv::EvcUnitItem *)(p + off);
-    off = align256(off + P.uitems.size() * sizeof(sv::EvcUnitItem));
-    int32_t *d_term_slot = (int32_t *)(p + off); off = align256(off + nterms * sizeof(int32_t));
-    double *d_coeffs = (double *)(p + off); off = align256(off + nterms * sizeof(double));
-    double *d_slotval = (double *)(p + off); off = align256(off + nslots * sizeof(double));
-    double *d_per_term = (double *)(p + off); off = align256(off + nterms * sizeof(double));
-    double *d_energy = (double *)(p + off); off = align256(off + sizeof(double));
-    int *d_status = (int *)(p + off); off = align256(off + sizeof(int));
-    double *d_part = (double *)(p + off);
-    if (off >= kNoAllocScratchBytes) return noalloc_fail(SV_EINVAL, "scratch array too small for this call");
     int E = 1;
     std::vector<sv::CosetArgs> args;
     for (auto &cp : P.passes) {
@@ -169,14 +153,51 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
         a.few = (cp.g_end - cp.g_begin) <= sv::kEvcFew && (cp.s_end - cp.s_begin) == (cp.g_end - cp.g_begin);
         args.push_back(a);
     }
+    // a small state's cosets are shared by several CTAs, a partial row per
+    // coset (three quarters of the scratch: the tables take far less than the
+    // rest); else few strings go to the unit kernel and Jordan-Wigner masks to
+    // register phases, as in sv_expect (n = 26, 177 strings: 5.0 -> 1.9 ms a call)
+    bool slices = true;
+    for (auto &a : args)
+        slices = slices && sv::coset_slices_pay(dt, a) && a.nfree == args[0].nfree &&
+                 ((size_t)nslots * sizeof(double) << a.nfree) <= kNoAllocScratchBytes / 4 * 3;
+    if (!slices) {
+        const int rb = dt == SV_C64 ? 5 : 4;
+        sv::plan_evc_phases(P, rb + 8, rb);
+        if (dt == SV_C64) sv::plan_evc_units(P);
+        for (size_t i = 0; i < args.size(); ++i) {
+            sv::CosetPass &cp = P.passes[i];
+            if (cp.rp_end > cp.rp_begin && !sv::evc_reg_fits(dt, args[i], cp)) {
+                cp.rp_end = cp.rp_begin;
+                cp.g_reg = cp.g_begin;
+                cp.s_reg = cp.s_begin;
+            }
+        }
+    }
+
+    // carve the array: tables, results, then per-CTA partial rows
+    unsigned char *p = (unsigned char *)base;
+    size_t off = 0;
+    sv::DevGroup *d_groups = (sv::DevGroup *)(p + off); off = align256(off + ngroups * sizeof(sv::DevGroup));
+    sv::DevString *d_strs = (sv::DevString *)(p + off); off = align256(off + nslots * sizeof(sv::DevString));
+    sv::EvcUnitItem *d_units = (sv::EvcUnitItem *)(p + off);
+    off = align256(off + P.uitems.size() * sizeof(sv::EvcUnitItem));
+    sv::EvcRegPhase *d_phases = (sv::EvcRegPhase *)(p + off);
+    off = align256(off + P.rphases.size() * sizeof(sv::EvcRegPhase));
+    sv::EvcRegItem *d_items = (sv::EvcRegItem *)(p + off);
+    off = align256(off + P.ritems.size() * sizeof(sv::EvcRegItem));
+    int32_t *d_term_slot = (int32_t *)(p + off); off = align256(off + nterms * sizeof(int32_t));
+    double *d_coeffs = (double *)(p + off); off = align256(off + nterms * sizeof(double));
+    double *d_slotval = (double *)(p + off); off = align256(off + nslots * sizeof(double));
+    double *d_per_term = (double *)(p + off); off = align256(off + nterms * sizeof(double));
+    double *d_energy = (double *)(p + off); off = align256(off + sizeof(double));
+    int *d_status = (int *)(p + off); off = align256(off + sizeof(int));
+    double *d_part = (double *)(p + off);
+    if (off >= kNoAllocScratchBytes) return noalloc_fail(SV_EINVAL, "scratch array too small for this call");
     int grid = sv::coset_grid(dt, E, 0, false);
     const size_t rows = (kNoAllocScratchBytes - off) / ((size_t)nslots * sizeof(double));
     if (rows < 1) return noalloc_fail(SV_EINVAL, "scratch array too small for this call");
     if ((size_t)grid > rows) grid = (int)rows;
-    // a small state's cosets are shared by several CTAs, a partial row per coset
-    bool slices = true;
-    for (auto &a : args)
-        slices = slices && sv::coset_slices_pay(dt, a) && a.nfree == args[0].nfree && ((size_t)1 << a.nfree) <= rows;
     if (slices) grid = 1 << args[0].nfree;
 
     cudaStream_t st = (cudaStream_t)stream;
@@ -194,16 +215,33 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
     if (!P.uitems.empty())
         NOALLOC_CK(cudaMemcpyAsync(d_units, P.uitems.data(), P.uitems.size() * sizeof(sv::EvcUnitItem),
                                    cudaMemcpyHostToDevice, st));
+    if (!P.rphases.empty()) {
+        NOALLOC_CK(cudaMemcpyAsync(d_phases, P.rphases.data(), P.rphases.size() * sizeof(sv::EvcRegPhase),
+                                   cudaMemcpyHostToDevice, st));
+        NOALLOC_CK(cudaMemcpyAsync(d_items, P.ritems.data(), P.ritems.size() * sizeof(sv::EvcRegItem),
+                                   cudaMemcpyHostToDevice, st));
+    }
     for (size_t i = 0; i < args.size(); ++i) {
-        const sv::CosetArgs &a = args[i];
+        sv::CosetArgs a = args[i];
         const sv::CosetPass &cp = P.passes[i];
-        if (!slices && cp.u_end > cp.u_begin)
-            NOALLOC_CK(sv::launch_evc_unit(st, grid, state, a, cp, d_units, d_part, nslots));
-        else if (slices)
+        if (slices) {
             NOALLOC_CK(sv::launch_evc_slice(dt, st, state, a, d_strs, d_part, nslots));
-        else
-            NOALLOC_CK(sv::launch_evc_pass(dt, st, grid, state, a, d_groups, d_strs, d_part, nslots, d_status,
-                                           (long long)o.wait_limit));
+            continue;
+        }
+        if (cp.u_end > cp.u_begin) {
+            NOALLOC_CK(sv::launch_evc_unit(st, grid, state, a, cp, d_units, d_part, nslots));
+            continue;
+        }
+        if (cp.rp_end > cp.rp_begin) {
+            NOALLOC_CK(sv::launch_evc_reg(dt, st, grid, state, a, cp, d_phases, d_items, d_part, nslots));
+            if (cp.g_reg == cp.g_end) continue;
+        }
+        // the rest of the pass by the general kernels
+        a.g_begin = cp.g_reg;
+        a.s_begin = cp.s_reg;
+        a.few = (a.g_end - a.g_begin) <= sv::kEvcFew && (a.s_end - a.s_begin) == (a.g_end - a.g_begin);
+        NOALLOC_CK(sv::launch_evc_pass(dt, st, grid, state, a, d_groups, d_strs, d_part, nslots, d_status,
+                                       (long long)o.wait_limit));
     }
     NOALLOC_CK(sv::launch_reduce_rows(st, d_part, grid, nslots, 0, nslots, d_slotval));
     NOALLOC_CK(sv::launch_energy(st, d_slotval, d_term_slot, d_coeffs, (int)nterms, d_per_term, d_energy));

@@ -1184,6 +1184,9 @@ void plan_evc_phases(EvcPlan &P, int stage, int r) {
         cp.g_reg = cp.g_begin;
         cp.s_reg = cp.s_begin;
         if (cp.kl + cp.m != stage) continue;
+        // few single strings keep per-thread partials in the kernels for them
+        const int ng = cp.g_end - cp.g_begin;
+        if (ng <= kEvcFew && cp.s_end - cp.s_begin == ng) continue;
         int ge = cp.g_begin;
         while (ge < cp.g_end) {
             const EvcGroup &G = P.groups[ge];

@@ -183,6 +183,9 @@ struct QsuPlan {
     }
 };
 
+// Few-string expectation passes (every group one string): at most this many groups.
+constexpr int kEvcFew = 8;
+
 // EVC / H|psi>: strings grouped by physical X/Y mask, groups packed into
 // coset passes (see kernels).
 struct EvcString {
