@@ -156,7 +156,7 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
     // a small state's cosets are shared by several CTAs, a partial row per
     // coset (three quarters of the scratch: the tables take far less than the
     // rest); else few strings go to the unit kernel and Jordan-Wigner masks to
-    // register phases, as in sv_expect (n = 26, 177 strings: 5.0 -> 2.3 ms a call)
+    // register phases, as in sv_expect (n = 26, 177 strings: 5.0 -> 2.5 ms a call)
     bool slices = true;
     for (auto &a : args)
         slices = slices && sv::coset_slices_pay(dt, a) && a.nfree == args[0].nfree &&
