@@ -55,7 +55,6 @@ struct DevString {
     uint32_t pad;
 };
 
-
 // First phase, step, diagonal block and block member of a plan (batched kernel
 // with step loops: indices inside a plan are its own).
 struct BatchStepOff {
