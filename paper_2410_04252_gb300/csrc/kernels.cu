@@ -5135,6 +5135,7 @@ cudaError_t allow_smem_of(const void *kernel, size_t smem) {
     if (smem <= have) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) have = smem;
+    else cudaGetLastError();      // reported here, not by the next launch
     return e;
 }
 template <typename... A>
@@ -5146,9 +5147,10 @@ cudaError_t allow_smem(void (*kernel)(A...), size_t smem) {
 // A launch whose set-up may overlap the kernel before it on the stream
 // (programmatic dependent launch): every kernel launched so runs pdl_wait()
 // in all threads before it touches anything that earlier work on the stream
-// reads or writes.
+// reads or writes.  More shared memory than a block may have is an error here.
 template <typename... A, typename... V>
 cudaError_t launch(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st, V... v) {
+    if (const cudaError_t e = allow_smem(kernel, smem)) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
@@ -5165,6 +5167,7 @@ cudaError_t launch(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cu
 // the split of shared memory and L1 that this kernel asks for.
 template <typename... A, typename... V>
 cudaError_t launch_drained(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st, V... v) {
+    if (const cudaError_t e = allow_smem(kernel, smem)) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
@@ -5244,11 +5247,9 @@ cudaError_t launch_gate_pass(sv_dtype dt, cudaStream_t st, int grid, int threads
                              const GatePassArgs &a, const DevOp *ops, const void *coef, const void *mats) {
     size_t sm = gate_smem(dt, a.k, a.nlow);
     if (dt == SV_C64) {
-        allow_smem(k_gate_pass<float>, sm);
         return launch(k_gate_pass<float>, grid, threads, sm, st, (float2 *)psi, a, ops, (const float *)coef,
                       (const float2 *)mats);
     }
-    allow_smem(k_gate_pass<double>, sm);
     return launch(k_gate_pass<double>, grid, threads, sm, st, (double2 *)psi, a, ops, (const double *)coef,
                   (const double2 *)mats);
 }
@@ -5288,7 +5289,6 @@ cudaError_t gate_reg_dispatch(cudaStream_t st, int grid, void *psi, const GatePa
     const int nt = 1 << (a.k - kRegBits);
     if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
     auto go = [&](auto kernel, int threads, auto... more) {
-        allow_smem(kernel, sm);
         return launch(kernel, grid, threads, sm, st, (Cx<R> *)psi, a, (const unsigned char *)image, more..., early ? 1 : 0);
     };
     const int kind = steps_kind(a);
@@ -5310,7 +5310,6 @@ cudaError_t adj_reg_dispatch(cudaStream_t st, int grid, void *psi, void *lam, co
     const int nt = 1 << (a.k - kRegBits);
     if (a.k < kRegMinTile || nt > (sizeof(R) == 4 ? 512 : 256)) return cudaErrorInvalidValue;
     auto go = [&](auto kernel) {
-        allow_smem(kernel, sm);
         return launch(kernel, grid, nt, sm, st, (Cx<R> *)psi, (Cx<R> *)lam, a, (const unsigned char *)image,
                       (const Cx<R> *)pmats, part, part_stride, early ? 1 : 0);
     };
@@ -5361,11 +5360,9 @@ cudaError_t launch_adj_pass(sv_dtype dt, cudaStream_t st, int grid, int threads,
                             double *part, int part_stride) {
     size_t sm = adj_smem(dt, a.k, a.nlow, a.op_end - a.op_begin, threads);
     if (dt == SV_C64) {
-        allow_smem(k_adj_pass<float>, sm);
         return launch(k_adj_pass<float>, grid, threads, sm, st, (float2 *)psi, (float2 *)lam, a, ops,
                       (const float *)coef, (const float2 *)mats, part, part_stride);
     }
-    allow_smem(k_adj_pass<double>, sm);
     return launch(k_adj_pass<double>, grid, threads, sm, st, (double2 *)psi, (double2 *)lam, a, ops,
                   (const double *)coef, (const double2 *)mats, part, part_stride);
 }
@@ -5447,7 +5444,6 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
         const size_t smr = 3 * (size_t)E * sizeof(Cx<R>) + ((size_t)1 << a.m) * 8;
 #define SV_EVCR_CASE(N)                                                                                      \
     case N:                                                                                                  \
-        allow_smem(k_evc_ring<R, N, 9>, smr);                                                                \
         return launch(k_evc_ring<R, N, 9>, grid, 512, smr, st, (const Cx<R> *)psi, a, groups, strs, part,    \
                       part_stride);
         switch (ept) {
@@ -5465,7 +5461,6 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
                            (size_t)kEvcFew * threads * (sizeof(R) + 4);
 #define SV_EVCF_CASE(N)                                                                                      \
     case N:                                                                                                  \
-        allow_smem(k_evc_few<R, N, 9>, smf);                                                                 \
         return launch(k_evc_few<R, N, 9>, grid, threads, smf, st, (const Cx<R> *)psi, a, groups, strs, part, \
                       part_stride);
         switch (ept) {
@@ -5489,7 +5484,6 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
     }
 #define SV_EVC_CASE(N)                                                                                       \
     case N:                                                                                                  \
-        allow_smem(k_evc_pass<R, N>, sm);                                                                    \
         return launch(k_evc_pass<R, N>, grid, threads, sm, st, (const Cx<R> *)psi, a, groups, strs, part,    \
                       part_stride, xform);
     switch (ept) {
@@ -5518,7 +5512,6 @@ bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, const CosetPass &cp) {
 cudaError_t launch_evc_unit(cudaStream_t st, int grid, const void *psi, const CosetArgs &a, const CosetPass &cp,
                             const EvcUnitItem *uitems, double *part, int part_stride) {
     const size_t sm = 3 * 8192 * sizeof(float2) + ((size_t)8 << kEvcUnitSpan) + kEvcUnitMax * 512 * sizeof(float);
-    allow_smem(k_evc_unit, sm);
     return launch(k_evc_unit, grid, 512, sm, st, (const float2 *)psi, a, uitems + cp.u_begin, cp.u_mid - cp.u_begin,
                   cp.u_end - cp.u_begin, part, part_stride);
 }
@@ -5532,11 +5525,9 @@ cudaError_t launch_evc_reg(sv_dtype dt, cudaStream_t st, int grid, const void *p
     const size_t sm = 2 * (es << (a.kl + a.m)) + evc_reg_layout(a.m, nslots, nph, nit, (int)es / 2).total;
     phases += cp.rp_begin;
     if (dt == SV_C64) {
-        allow_smem(k_evc_reg<float>, sm);
         return launch(k_evc_reg<float>, grid, 512, sm, st, (const float2 *)psi, a, phases, nph, cp.rp_first,
                       ritems, cp.ri_begin, nit, nslots, part, part_stride);
     }
-    allow_smem(k_evc_reg<double>, sm);
     return launch(k_evc_reg<double>, grid, 512, sm, st, (const double2 *)psi, a, phases, nph, cp.rp_first,
                   ritems, cp.ri_begin, nit, nslots, part, part_stride);
 }
@@ -5567,7 +5558,6 @@ cudaError_t hpsi_dispatch(cudaStream_t st, int grid, const void *psi, void *lam,
             // their split for the whole chain (the loads in flight then have 28 KB
             // of L1; n = 25, 317 strings: 140 -> 190 us a pass).
             auto go = [&](auto kernel) {
-                allow_smem(kernel, smv);
                 if (first)
                     return launch_drained(kernel, grid, 512, smv, st, (const float2 *)psi, (float2 *)lam, a, strs,
                                           first, last, epart);
@@ -5580,7 +5570,6 @@ cudaError_t hpsi_dispatch(cudaStream_t st, int grid, const void *psi, void *lam,
     }
 #define SV_HPSI_CASE(N)                                                                                      \
     case N:                                                                                                  \
-        allow_smem(k_hpsi_pass<R, N>, sm);                                                                   \
         return launch(k_hpsi_pass<R, N>, grid, threads, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, groups, \
                       strs, first, last, epart, status, limit);
     switch (ept) {
@@ -5621,10 +5610,8 @@ cudaError_t launch_evc_slice(sv_dtype dt, cudaStream_t st, const void *psi, cons
     const int S = std::max(1, std::min(want, most));
     const size_t es = dt == SV_C64 ? 8 : 16, sm = (size_t)E * es + ((size_t)8 << a.m);
     if (dt == SV_C64) {
-        allow_smem(k_evc_slice<float>, sm);
         return launch(k_evc_slice<float>, ncos * S, 512, sm, st, (const float2 *)psi, a, strs, part, part_stride, S);
     }
-    allow_smem(k_evc_slice<double>, sm);
     return launch(k_evc_slice<double>, ncos * S, 512, sm, st, (const double2 *)psi, a, strs, part, part_stride, S);
 }
 
@@ -5642,11 +5629,9 @@ cudaError_t hpsi_slice_dispatch(cudaStream_t st, const void *psi, void *lam, con
 #define SV_HS_CASE(N)                                                                                        \
     case N:                                                                                                  \
         if (grouped) {                                                                                       \
-            allow_smem(k_hpsi_slice<R, N, true>, sm);                                                        \
             return launch(k_hpsi_slice<R, N, true>, ncos * S, 512, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, \
                           a, strs, first, last, epart, S);                                                   \
         }                                                                                                    \
-        allow_smem(k_hpsi_slice<R, N, false>, sm);                                                           \
         return launch(k_hpsi_slice<R, N, false>, ncos * S, 512, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, \
                       strs, first, last, epart, S);
     switch (ept) {

@@ -7,6 +7,7 @@
 #include <numeric>
 #include <unordered_map>
 
+#include "kernels.h"
 #include "sv_internal.h"
 
 namespace sv {
@@ -449,6 +450,12 @@ void plan_gate_passes(QsuPlan &P, const std::vector<Op> &ops, int k, int low, in
 // non-diagonal gates (padded with the lowest free tile bits), then the phase
 // takes gates in order while they fit, a gate that does not fit blocking its
 // targets (C1 is kept).  The pass's ops are reordered phase by phase.
+//
+// The tables of a pass (a kilobyte a phase at 2^13 amplitudes, beside 128 KB of
+// tiles) stand in shared memory with its tiles; a pass with more phases than
+// fit is cut at a phase boundary into passes over the same staged bits.  94
+// random 4-qubit matrices on 13 qubits or about 180 Givens rotations (a phase
+// every few gates) reach that line.
 bool diag_kind(int kind) { return kind == SV_RZ || kind == SV_CZ; }
 int op_qubits(int kind) {
     return kind == SV_DEXC || kind == SV_MAT4 ? 4 : (kind == SV_CZ || kind == SV_GIVENS || kind == SV_MAT2) ? 2 : 1;
@@ -492,28 +499,75 @@ uint32_t phase_lanes(uint32_t rmask, int k) {
     return lanes;
 }
 
-void plan_phases(QsuPlan &P, bool pairs, int threads) {
+// what the operations of a register-blocked pass (or of a part of one) are
+void set_pass_kinds(const QsuPlan &P, GatePass &gp) {
+    gp.pairs = gp.others = gp.mat1 = gp.dense = 0;
+    for (int o = gp.op_begin; o < gp.op_end; ++o) {
+        const int kd = P.ops[o].kind;
+        if (kd == SV_MAT2 || kd == SV_MAT4) gp.dense = 1;
+        if (kd == SV_MAT1) gp.mat1 = 1;
+        if (kd == SV_GIVENS || kd == SV_DEXC) gp.pairs = 1;
+        else gp.others = 1;
+    }
+}
+
+// Shared memory of a register-blocked pass without diagonal blocks (they take
+// what is left), counting a step per operation; the reverse pass, which has
+// the gradient slots besides, unless dense matrices keep it out of registers.
+size_t reg_pass_bytes(const GatePass &gp, int amp) {
+    GatePassArgs a;
+    memset(&a, 0, sizeof(a));
+    a.k = gp.k;
+    a.nlow = gp.nlow;
+    a.op_end = a.st_end = gp.op_end - gp.op_begin;
+    a.ph_end = gp.ph_end - gp.ph_begin;
+    a.pairs = gp.pairs;
+    const sv_dtype dt = amp == 8 ? SV_C64 : SV_C128;
+    return gp.dense ? gate_reg_smem(dt, a) : adj_reg_smem(dt, a);
+}
+
+// The pass cut into passes whose tables fit (a single phase always does: at
+// most 256 operations and one set of thread places).
+void cut_pass(const QsuPlan &P, const GatePass &gp, int amp, std::vector<GatePass> &out) {
+    GatePass cur = gp;
+    cur.ph_end = gp.ph_begin;
+    for (int ph = gp.ph_begin; ph < gp.ph_end; ++ph) {
+        GatePass longer = cur;
+        longer.ph_end = ph + 1;
+        longer.op_end = P.phases[ph].op_end;
+        set_pass_kinds(P, longer);
+        if (cur.ph_end > cur.ph_begin && reg_pass_bytes(longer, amp) > (size_t)kRegSmemLimit) {
+            out.push_back(cur);
+            longer.ph_begin = ph;
+            longer.op_begin = P.phases[ph].op_begin;
+            set_pass_kinds(P, longer);
+        }
+        cur = longer;
+    }
+    out.push_back(cur);
+}
+
+void plan_phases(QsuPlan &P, bool pairs, int threads, int amp) {
+    std::vector<GatePass> passes;
     for (auto &gp : P.passes) {
         int r = kRegBits;
         if (threads) {
             r = gp.k;
             for (int t = threads; t > 1; t >>= 1) --r;
         }
-        if (r < 2 || (!threads && gp.k < kRegMinTile)) continue;
-        bool ok = true, dense = false;
+        bool ok = r >= 2 && (threads || gp.k >= kRegMinTile);
         for (int o = gp.op_begin; o < gp.op_end; ++o) {
             const int kd = P.ops[o].kind;
             // Givens rotations, double excitations and dense 2- and 4-qubit
             // matrices need their targets among four register bits
             const bool pair = kd == SV_GIVENS || kd == SV_DEXC || kd == SV_MAT2 || kd == SV_MAT4;
             if (kd != SV_RY && kd != SV_RZ && kd != SV_CZ && kd != SV_MAT1 && !(pairs && pair)) ok = false;
-            if (kd == SV_MAT2 || kd == SV_MAT4) dense = true;
-            if (kd == SV_MAT1) gp.mat1 = 1;
-            if (kd == SV_GIVENS || kd == SV_DEXC) gp.pairs = 1;
-            else gp.others = 1;
         }
-        if (!ok) continue;
-        gp.dense = dense;
+        set_pass_kinds(P, gp);
+        if (!ok) {
+            passes.push_back(gp);
+            continue;
+        }
         const uint32_t all = (gp.k >= 32) ? 0xFFFFFFFFu : ((1u << gp.k) - 1u);
         auto tmask = [&](const DevOp &d) {
             uint32_t m = 0;
@@ -574,7 +628,10 @@ void plan_phases(QsuPlan &P, bool pairs, int threads) {
         }
         gp.ph_end = (int32_t)P.phases.size();
         std::copy(out.begin(), out.end(), P.ops.begin() + gp.op_begin);
+        if (threads) passes.push_back(gp);   // the batched kernel gate by gate: no tables
+        else cut_pass(P, gp, amp, passes);
     }
+    P.passes.swap(passes);
 }
 
 // Steps of the register phases.  Inside a phase two operations on disjoint
@@ -1460,7 +1517,7 @@ std::string plan_qsu(int n, int g, const sv_gate *gates, size_t m, bool lazy, co
     if (P.tiles.empty()) P.final_l2p = l2p_init;
     int k = std::max(o.tile_bits, std::min(o.low_bits, P.nL) + 4);
     plan_gate_passes(P, ops, k, o.low_bits, o.fuse_max, o.diag_exempt);
-    plan_phases(P, o.reg_pairs, o.reg_threads);
+    plan_phases(P, o.reg_pairs, o.reg_threads, o.amp_bytes);
     plan_steps(P, std::min(o.max_diag, kMaxPassDiag), o.amp_bytes, o.image_limit);
     return "";
 }
