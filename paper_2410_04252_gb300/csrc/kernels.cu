@@ -1082,7 +1082,8 @@ enum : uint32_t {
     RO_MAT4 = 28,
     RO_RZ = 29,        // t0: tile bit, or kOutTarget + physical bit outside the tile
     RO_CZ = 30,        // t0, t1 likewise
-    RO_NOP = 31
+    RO_NOP = 31,
+    RO_SCALE = 32      // op_begin: the factor's bits (complex64)
 };
 #define SV_RO_GIVENS(CALL)                                                                       \
     case 0: CALL(1, 2); break;  case 1: CALL(1, 4); break;  case 2: CALL(1, 8); break;           \
@@ -1171,6 +1172,42 @@ __device__ __forceinline__ uint32_t diag_bit_mask(uint32_t t, uint32_t rmask, ui
     if (t >= (uint32_t)kOutTarget) return ((gbase >> (t - kOutTarget)) & 1ull) ? 0xFFFFu : 0u;
     return reg_or_thread_mask(t, rmask, base);
 }
+
+// every register amplitude times the factor of a SCALE step (complex64)
+template <typename R> __device__ __forceinline__ void reg_scale(RA<R> *x, int32_t bits) {
+    if constexpr (sizeof(R) == 4) {
+        const float g = __int_as_float(bits);
+        if (g == 1.f) return;
+        const unsigned long long gg = f2_pack(g, g);
+#pragma unroll
+        for (int v = 0; v < (1 << kRegBits); ++v) asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(x[v]) : "l"(gg));
+    }
+}
+
+// The product of RY factors, in two FP32 numbers for complex64: its error is
+// common to every amplitude, where a rotation's own roundings average out.
+template <typename R> struct RunProduct {
+    R f = 1, low = 0;
+    __device__ __forceinline__ void mul(R c, R clow) {
+        const R p = f * c;
+        if constexpr (sizeof(R) == 4) low = fmaf(low, c, fmaf(f, clow, fmaf(f, c, -p)));
+        f = p;
+    }
+    // the factor of a factored RY (t, f): the f that makes f (1, t) a unit vector
+    // for the rounded t, f + f r / 2 with r = 1 - f^2 (1 + t^2) to first order
+    __device__ __forceinline__ void mul_ry(Cx<R> k) {
+        R clow = 0;
+        if constexpr (sizeof(R) == 4) {
+            // (rounded products: contracted ones would not cancel)
+            const R t2 = __fmul_rn(k.x, k.x), w = 1 + t2, wl = (t2 - (w - 1)) + fmaf(k.x, k.x, -t2);   // 1 + t^2 = w + wl
+            const R c2 = __fmul_rn(k.y, k.y), q = __fmul_rn(c2, w);
+            const R r = (1 - q) - (fmaf(c2, w, -q) + fmaf(fmaf(k.y, k.y, -c2), w, c2 * wl));
+            clow = R(0.5) * k.y * r;
+        }
+        mul(k.y, clow);
+    }
+    __device__ __forceinline__ R value() const { return f + low; }
+};
 
 // A diagonal gate outside the blocks on the register amplitudes, m the
 // amplitudes whose bits are 1: CZ negates them, RZ turns them the other way.
@@ -1312,13 +1349,15 @@ struct PhaseS {
 // every CTA of every pass repeated them.  Block (pass, slice, direction): the
 // slices share a pass's phases and blocks, slice 0 writes the rest.
 constexpr int kImageSlices = 8;
-// `out` in shared or global memory; cs and st: shared room for the pass's
-// operations and steps; slice 0 of nslices writes what the slices don't share.
+constexpr float kScaleBelow = 1.f / 16;
+constexpr int kMaxPassSteps = kMaxPassOps + kMaxScaleSteps;
+// `out` in shared or global memory; cs, st and prod: shared room for the pass's
+// operations, steps and the steps' RY factors; slice 0 of nslices writes what the slices don't share.
 template <typename R>
 __device__ __forceinline__ void reg_tables(unsigned char *out, const RegLayout &L, const GatePassArgs &a,
                                            const DevOp *ops, const Phase *phases, const RegStep *steps, const R *coef,
                                            const DiagBlock *dblocks, const DiagMember *dmem, bool adj, Cx<R> *cs,
-                                           RegStep *st, int slice, int nslices) {
+                                           RegStep *st, Cx<R> *prod, int slice, int nslices) {
     constexpr int RB = kRegBits, V = 1 << RB;
     constexpr uint32_t P = 16 / sizeof(Cx<R>);
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -1360,6 +1399,8 @@ __device__ __forceinline__ void reg_tables(unsigned char *out, const RegLayout &
             S.op_begin = S.a - a.op_begin;
             S.a = (int32_t)(code | (t0 << 8) | (t1 << 16));
             S.op_end = op.pm;
+        } else if (S.type == SV_STEP_SCALE) {
+            S.a = (int32_t)RO_SCALE;
         }
         st[s] = S;
     }
@@ -1369,15 +1410,18 @@ __device__ __forceinline__ void reg_tables(unsigned char *out, const RegLayout &
     for (int s = tid; s < nst; s += nthr) {
         if (st[s].type != SV_STEP_ROT) continue;
         int o = st[s].op_begin - a.op_begin, forms = st[s].a;
+        RunProduct<R> f;
         for (int b = 0; b < RB; ++b) {
             if (!((st[s].a >> b) & 1)) continue;
             const Cx<R> k = cs[o];
             int fb;
             cs[o] = ry_factored<R>(k.x, k.y, fb);
+            f.mul_ry(cs[o]);
             if (fb) forms |= 1 << (8 + b);
             ++o;
         }
         st[s].a = forms;
+        prod[s] = mk<R>(f.f, f.low);
     }
     __syncthreads();
     if (first) {
@@ -1405,7 +1449,8 @@ __device__ __forceinline__ void reg_tables(unsigned char *out, const RegLayout &
             if (st[s].type == SV_STEP_OP)
                 *reinterpret_cast<uint64_t *>(reinterpret_cast<Cx<R> *>(out + L.rk) + 4 * st[s].op_begin + 3) =
                     (uint64_t)((uint32_t)st[s].a & 255u);
-        for (int s = tid; s < nst; s += nthr) reinterpret_cast<RegStep *>(out + L.steps)[s] = st[s];
+        for (int s = tid; s < nst; s += nthr)
+            if (st[s].type != SV_STEP_SCALE) reinterpret_cast<RegStep *>(out + L.steps)[s] = st[s];
         for (int b = a.db_begin + tid; b < a.db_end; b += nthr)
             reinterpret_cast<DiagBlock *>(out + L.blocks)[b - a.db_begin] = dblocks[b];
         for (int m = a.mem_begin + tid; m < a.mem_end; m += nthr)
@@ -1418,16 +1463,23 @@ __device__ __forceinline__ void reg_tables(unsigned char *out, const RegLayout &
                 reinterpret_cast<uint32_t *>(out + L.prb)[q * 4 + i] = swz_tile(rm & (0u - rm)) * (uint32_t)sizeof(Cx<R>);
         }
         // prefix products of the factors in execution order (forward: ascending
-        // steps; adjoint: descending), entry nst = the pass's total factor
+        // steps; adjoint: descending) since the SCALE step that last applied
+        // them, entry nst = what is left for the store
         R *sc = reinterpret_cast<R *>(out + L.sc);
         for (int i = tid; i <= nst; i += nthr) {
-            R f = 1;
+            RunProduct<R> f;
             for (int q = 0; q < i; ++q) {
-                const RegStep S = st[adj ? nst - 1 - q : q];
-                if (S.type != SV_STEP_ROT) continue;
-                for (int o = S.op_begin - a.op_begin; o < S.op_end - a.op_begin; ++o) f *= cs[o].y;
+                const int e = adj ? nst - 1 - q : q;
+                if (st[e].type == SV_STEP_ROT) f.mul(prod[e].x, prod[e].y);
+                else if (st[e].type == SV_STEP_SCALE && fabs(f.f) < kScaleBelow) f = RunProduct<R>();
             }
-            sc[i == nst ? nst : (adj ? nst - 1 - i : i)] = f;
+            const int s = i == nst ? nst : (adj ? nst - 1 - i : i);
+            sc[s] = f.value();
+            if (i < nst && st[s].type == SV_STEP_SCALE) {
+                RegStep S = st[s];
+                S.op_begin = __float_as_int(fabs(f.f) < kScaleBelow ? (float)f.value() : 1.f);
+                reinterpret_cast<RegStep *>(out + L.steps)[s] = S;
+            }
         }
     }
     // this slice's phases: the tile bits of every thread
@@ -1499,7 +1551,8 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
                                                    uint64_t dir_stride, int dir0) {
     __shared__ GatePassArgs a;
     __shared__ Cx<R> cs[kMaxPassOps];
-    __shared__ RegStep st[kMaxPassOps];
+    __shared__ RegStep st[kMaxPassSteps];
+    __shared__ Cx<R> prod[kMaxPassSteps];
     const bool adj = (int)blockIdx.z + dir0 != 0;
     for (int i = threadIdx.x; i < (int)(sizeof(GatePassArgs) / 4); i += blockDim.x)
         reinterpret_cast<uint32_t *>(&a)[i] = reinterpret_cast<const uint32_t *>(pargs + blockIdx.x)[i];
@@ -1508,7 +1561,7 @@ __global__ void __launch_bounds__(256) k_reg_image(const GatePassArgs *__restric
     pdl_wait();
     pdl_next();
     reg_tables<R>(out0 + (adj ? dir_stride : 0) + offs[blockIdx.x], L, a, ops, phases, steps, coef, dblocks, dmem, adj,
-                  cs, st, (int)blockIdx.y, kImageSlices);
+                  cs, st, prod, (int)blockIdx.y, kImageSlices);
 }
 
 // A pass's tables from global into shared memory (16 bytes at a time)
@@ -1689,8 +1742,11 @@ __device__ __forceinline__ void fwd_steps(RA<R> *x, const PhaseS &F, const GateP
                     case RO_MAT2 + 4: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 3>(x, M); } break;
                     case RO_MAT2 + 5: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 3>(x, M); } break;
                     case RO_MAT4: if constexpr (KIND == kStepsAll) { reg_mat4<R>(x, M); } break;
+                    case RO_SCALE: reg_scale<R>(x, S.op_begin); break;
                     default: break;
                     }
+                } else {
+                    reg_scale<R>(x, S.op_begin);
                 }
             }
         }
@@ -1842,12 +1898,19 @@ __device__ __forceinline__ void adj_steps(RA<R> *xp, RA<R> *xl, const PhaseS &F,
                     case RO_MAT1 + 1: if constexpr (KIND == kStepsAll) { reg_mat<R, 1, 1>(xp, M); reg_mat<R, 1, 1>(xl, M); } break;
                     case RO_MAT1 + 2: if constexpr (KIND == kStepsAll) { reg_mat<R, 2, 2>(xp, M); reg_mat<R, 2, 2>(xl, M); } break;
                     case RO_MAT1 + 3: if constexpr (KIND == kStepsAll) { reg_mat<R, 3, 3>(xp, M); reg_mat<R, 3, 3>(xl, M); } break;
+                    case RO_SCALE:
+                        reg_scale<R>(xp, S.op_begin);
+                        reg_scale<R>(xl, S.op_begin);
+                        break;
                     default: break;
                     }
                     if (code < RO_MAT1) {
                         g = warp_sum<R>(g) * fs2;
                         if (lane == 0) acc[S.op_begin * AS + warp] += g;
                     }
+                } else {
+                    reg_scale<R>(xp, S.op_begin);
+                    reg_scale<R>(xl, S.op_begin);
                 }
             }
         }
@@ -4615,6 +4678,9 @@ __device__ __noinline__ void batch_adj(unsigned char *smem, const BatchPass &B, 
 // Shared memory of the batched kernel with step loops, behind the two tiles:
 // span table, gradient slots of a pass, gradient per operation, coefficients,
 // then the tables of a pass (or of an H|psi> pass's strings).
+constexpr int kBatchProds = (kMaxPassSteps + 1) & ~1;   // (the steps behind them stay 16-byte aligned)
+static_assert(8 * (kMaxPassOps + kBatchProds) + 16 * kMaxPassSteps <= 4 * kAdjSlotStride * kMaxPassOps,
+              "the tables' scratch fits the gradient slots");
 constexpr uint32_t kBsSpan = 131072, kBsAcc = kBsSpan + 2048, kBsTot = kBsAcc + 4 * kAdjSlotStride * kMaxPassOps,
                    kBsCoef = kBsTot + 8 * 512, kBsTab = kBsCoef + 8 * 1024;
 
@@ -4655,11 +4721,11 @@ __global__ void __launch_bounds__(512, 1) k_batch(const BatchArgs a) {
             __syncthreads();
             const RegLayout L = reg_layout(sP, (int)sizeof(Cx<R>), adj);
             if (threadIdx.x == 0) sL = L;
-            Cx<R> *cs = reinterpret_cast<Cx<R> *>(opacc);
+            Cx<R> *cs = reinterpret_cast<Cx<R> *>(opacc), *prod = cs + kMaxPassOps;
             const BatchStepOff off = a.step[plan];
             reg_tables<R>(smem + kBsTab, L, sP, a.ops + a.plan_op_off[plan], a.phases + off.ph, a.steps + off.st, coef,
-                          a.dblocks + off.db, a.dmembers + off.dm, adj, cs, reinterpret_cast<RegStep *>(cs + kMaxPassOps),
-                          0, 1);
+                          a.dblocks + off.db, a.dmembers + off.dm, adj, cs,
+                          reinterpret_cast<RegStep *>(prod + kBatchProds), prod, 0, 1);
             __syncthreads();
             if (adj) {
                 for (int j = threadIdx.x; j < (sP.op_end - sP.op_begin) * kAdjSlotStride; j += NT) opacc[j] = 0;

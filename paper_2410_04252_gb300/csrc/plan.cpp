@@ -519,7 +519,8 @@ size_t reg_pass_bytes(const GatePass &gp, int amp) {
     memset(&a, 0, sizeof(a));
     a.k = gp.k;
     a.nlow = gp.nlow;
-    a.op_end = a.st_end = gp.op_end - gp.op_begin;
+    a.op_end = gp.op_end - gp.op_begin;
+    a.st_end = a.op_end + kMaxScaleSteps;
     a.ph_end = gp.ph_end - gp.ph_begin;
     a.pairs = gp.pairs;
     const sv_dtype dt = amp == 8 ? SV_C64 : SV_C128;
@@ -674,8 +675,12 @@ void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
         gp.db_begin = gp.db_end = (int32_t)P.dblocks.size();
         if (gp.ph_begin < 0) continue;
         const int nops = gp.op_end - gp.op_begin;
+        int rys = 0;    // RYs of the pass, then those since its last SCALE step
+        for (int o = gp.op_begin; o < gp.op_end; ++o) rys += amp == 8 && P.ops[o].kind == SV_RY;
+        const int nsteps = nops + rys / (kScaleRYs - 3);
+        rys = 0;
         const int limit = image_limit ? 2 * (1 << gp.k) * amp + nops * kAdjSlotStride * 8 + image_limit : kRegSmemLimit;
-        int budget = limit - reg_pass_fixed_bytes(gp.k, gp.nlow, nops, nops, gp.ph_end - gp.ph_begin, amp, gp.pairs != 0);
+        int budget = limit - reg_pass_fixed_bytes(gp.k, gp.nlow, nops, nsteps, gp.ph_end - gp.ph_begin, amp, gp.pairs != 0);
         int area = 0;   // bytes of the pass's block area handed out so far
         auto take_block = [&](int kind) {
             const int need = diag_block_bytes(kind, gp.k, amp);
@@ -781,26 +786,34 @@ void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
             };
             int left = N;
             while (left > 0) {
-                std::vector<int> rys, others, diags;
+                std::vector<int> ready, others, diags;
                 for (int i = 0; i < N; ++i) {
                     if (done[i] || npred[i]) continue;
-                    if (ry[i]) rys.push_back(i);
+                    if (ry[i]) ready.push_back(i);
                     else if (dg[i]) diags.push_back(i);
                     else others.push_back(i);
                 }
-                if (!rys.empty()) {
-                    std::sort(rys.begin(), rys.end(), [&](int a, int b) { return in[a].t[0] < in[b].t[0]; });
+                if (!ready.empty()) {
+                    std::sort(ready.begin(), ready.end(), [&](int a, int b) { return in[a].t[0] < in[b].t[0]; });
                     RegStep st;
+                    rys += amp == 8 ? (int)ready.size() : 0;
+                    if (rys > kScaleRYs) {
+                        st.type = SV_STEP_SCALE;
+                        st.a = 0;
+                        st.op_begin = st.op_end = F.op_begin + (int32_t)out.size();
+                        P.steps.push_back(st);
+                        rys = (int)ready.size();
+                    }
                     st.type = SV_STEP_ROT;
                     st.op_begin = F.op_begin + (int32_t)out.size();
                     st.a = 0;
-                    for (int i : rys) {
+                    for (int i : ready) {
                         st.a |= 1 << regidx(in[i].t[0]);
                         emit(i);
                     }
                     st.op_end = F.op_begin + (int32_t)out.size();
                     P.steps.push_back(st);
-                    left -= (int)rys.size();
+                    left -= (int)ready.size();
                     continue;
                 }
                 if (!others.empty()) {

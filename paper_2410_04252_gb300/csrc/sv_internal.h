@@ -122,7 +122,16 @@ struct Phase {
 // [op_begin, op_end) ordered by register bit, a = the register-bit mask.
 // DIAG: a diagonal block (a = its index in QsuPlan::dblocks), ops = its
 // members.  OP: one operation (a = op_begin), applied by the generic code.
-enum { SV_STEP_ROT = 0, SV_STEP_DIAG = 1, SV_STEP_OP = 2 };
+// SCALE: no operation; the register kernels apply the RYs without their larger
+// coefficient (each at least 2^-1/2) and the product of these factors at the
+// store, so that amplitudes grow by up to 2^(1/2) an RY meanwhile: 2^128 over a
+// full pass, past FP32.  A complex64 pass has a SCALE step after at most
+// kScaleRYs RYs, which applies the product there unless it is above 2^-4 (then
+// the next one does): what the registers hold stays within 2^52 of the
+// amplitudes, the gradient sums, products of two, within 2^104.
+enum { SV_STEP_ROT = 0, SV_STEP_DIAG = 1, SV_STEP_OP = 2, SV_STEP_SCALE = 3 };
+constexpr int kScaleRYs = 96;
+constexpr int kMaxScaleSteps = kMaxPassOps / (kScaleRYs - 3);   // (a ROT step holds up to four RYs)
 // The shared-memory slot of tile index i in the register-blocked passes: a
 // linear (XOR) swizzle, so that slot(a | b) = slot(a) ^ slot(b) for disjoint
 // a, b.  It keeps bit 0 (an even index and its successor stay one 16-byte
