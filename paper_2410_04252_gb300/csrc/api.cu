@@ -560,11 +560,7 @@ sv_status get_evc(sv_handle *h, const sv_pauli *p, const double *c, size_t nterm
                           ? plan_hpsi(h->n, p, c, nterms, po, h->l2p, ent->plan)
                           : plan_evc(h->n, h->g, p, c, nterms, sched != SV_SCHED_EAGER, po, h->l2p, ent->plan);
     if (!err.empty()) return fail(SV_EINVAL, std::string(hpsi ? "H|psi> plan: " : "EVC plan: ") + err);
-    if (!hpsi) {
-        const int r = h->dt == SV_C64 ? 5 : 4;
-        plan_evc_phases(ent->plan, r + 8, r);
-        if (h->dt == SV_C64) plan_evc_units(ent->plan);
-    }
+    if (!hpsi) plan_evc_kernels(ent->plan, h->dt);
     ent->plan_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     ent->key = key;
     ent->nterms = (int)nterms;

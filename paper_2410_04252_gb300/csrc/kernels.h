@@ -144,11 +144,11 @@ cudaError_t launch_evc_pass(sv_dtype dt, cudaStream_t st, int grid, const void *
 cudaError_t launch_hpsi_pass(sv_dtype dt, cudaStream_t st, int grid, const void *psi, void *lam,
                              const CosetArgs &a, const DevGroup *groups, const DevString *strs,
                              int first, int last, double *epart, int *status, long long limit);
-// Register phases of an expectation pass (plan_evc_phases).
+// Register phases of an expectation pass (plan_evc_kernels).
 bool evc_reg_fits(sv_dtype dt, const CosetArgs &a, const CosetPass &cp);
 cudaError_t launch_evc_reg(sv_dtype dt, cudaStream_t st, int grid, const void *psi, const CosetArgs &a,
                            const CosetPass &cp, const EvcRegPhase *phases, const EvcRegItem *ritems, double *part, int part_stride);
-// Few strings with their masks as the span basis (plan_evc_units; complex64).
+// Few strings with their masks as the span basis (plan_evc_kernels; complex64).
 cudaError_t launch_evc_unit(cudaStream_t st, int grid, const void *psi, const CosetArgs &a, const CosetPass &cp,
                             const EvcUnitItem *uitems, double *part, int part_stride);
 // Few cosets (coset_slices_pay): several CTAs share a coset.  Expectation:

@@ -162,9 +162,7 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
         slices = slices && sv::coset_slices_pay(dt, a) && a.nfree == args[0].nfree &&
                  ((size_t)nslots * sizeof(double) << a.nfree) <= kNoAllocScratchBytes / 4 * 3;
     if (!slices) {
-        const int rb = dt == SV_C64 ? 5 : 4;
-        sv::plan_evc_phases(P, rb + 8, rb);
-        if (dt == SV_C64) sv::plan_evc_units(P);
+        sv::plan_evc_kernels(P, dt);
         for (size_t i = 0; i < args.size(); ++i) {
             sv::CosetPass &cp = P.passes[i];
             if (cp.rp_end > cp.rp_begin && !sv::evc_reg_fits(dt, args[i], cp)) {

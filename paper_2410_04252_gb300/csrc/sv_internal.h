@@ -256,11 +256,11 @@ struct CosetPass {
     int32_t pivot[kMaxSpan] = {};
     int32_t g_begin = 0, g_end = 0;   // groups
     int32_t s_begin = 0, s_end = 0;   // strings (slots), contiguous
-    // register phases (plan_evc_phases): they take the groups before g_reg
+    // register phases (k_evc_reg): they take the groups before g_reg
     // (half of the warps run phases [rp_begin, rp_begin + rp_first), the others the rest)
     int32_t rp_begin = 0, rp_end = 0, rp_first = 0, g_reg = 0, s_reg = 0;
     int32_t ri_begin = 0, ri_end = 0;
-    // plan_evc_units: strings of the first and of the second half of the warps
+    // k_evc_unit: strings of the first and of the second half of the warps
     int32_t u_begin = 0, u_mid = 0, u_end = 0;
 };
 
@@ -316,11 +316,9 @@ std::string plan_evc(int n, int g, const sv_pauli *p, const double *coeffs, size
 // H|psi> grouping: one tile, no QR, cosets over all n bits.
 std::string plan_hpsi(int n, const sv_pauli *p, const double *coeffs, size_t nterms,
                       const PlanOptions &o, const std::vector<int32_t> &l2p, EvcPlan &out);
-// Register phases of the passes that stage 2^stage amplitudes and hold enough
-// groups of one or two staged bits (fewer than kXformMinStrings strings each).
-void plan_evc_phases(EvcPlan &P, int stage, int r);
-// The passes that k_evc_unit takes (complex64: 2^13 staged, runs of 2^5).
-void plan_evc_units(EvcPlan &P);
+// The kernels of the expectation passes that differ from the general ones:
+// few strings by k_evc_unit, else masks of one or two staged bits by k_evc_reg.
+void plan_evc_kernels(EvcPlan &P, sv_dtype dt);
 constexpr int kXformMinStrings = 16;  // groups with at least this many strings take the transform path
 constexpr int kEvcRegMinGroups = 6;
 // Write a bit permutation from layout `from` to layout `to` as at most two
