@@ -1118,11 +1118,14 @@ __device__ __forceinline__ MatRow<R, DIM> mat_row(const Cx<R> *M, int u) {
 }
 template <typename R, int DIM>
 __device__ __forceinline__ Cx<R> row_dot(const MatRow<R, DIM> &m, const Cx<R> *x) {
-    R re = 0, im = 0;
+    // four fused multiply-adds a term (complex128: FP64 operations bound it)
+    R re = m.m[0].x * x[0].x, im = m.m[0].x * x[0].y;
+    re = fma(-m.m[0].y, x[0].y, re);
+    im = fma(m.m[0].y, x[0].x, im);
 #pragma unroll
-    for (int w = 0; w < DIM; ++w) {
-        re += m.m[w].x * x[w].x - m.m[w].y * x[w].y;
-        im += m.m[w].x * x[w].y + m.m[w].y * x[w].x;
+    for (int w = 1; w < DIM; ++w) {
+        re = fma(-m.m[w].y, x[w].y, fma(m.m[w].x, x[w].x, re));
+        im = fma(m.m[w].y, x[w].x, fma(m.m[w].x, x[w].y, im));
     }
     return mk<R>(re, im);
 }
