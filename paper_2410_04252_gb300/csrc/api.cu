@@ -2,11 +2,15 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "kernels.h"
@@ -872,6 +876,41 @@ sv_status check_handle(const sv_handle *h) {
     return SV_OK;
 }
 
+// Plans of a batch's distinct circuits (state first[i] has the i-th), on several
+// host threads: the step loops' plans take about 30 us each (n = 13, 120 gates;
+// half of it gate by gate), and there may be hundreds (256 circuits: one thread
+// 11.9 ms a call, this way 4.7, of which the kernel runs for 0.6).
+// Returns the first failing plan's message with its state, in their order.
+std::string plan_batch(int n, const sv_gate *gates, const int32_t *gate_off, const std::vector<int32_t> &first,
+                       const PlanOptions &po, const std::vector<int32_t> &l2p, std::vector<QsuPlan> &plans) {
+    plans.assign(first.size(), QsuPlan());
+    std::vector<std::string> err(first.size());
+    std::atomic<size_t> next{0};
+    auto work = [&]() {
+        for (size_t i; (i = next.fetch_add(1)) < first.size();) {
+            const int b = first[i];
+            try {
+                err[i] = plan_qsu(n, 0, gates + gate_off[b], (size_t)(gate_off[b + 1] - gate_off[b]), true, po, l2p, plans[i]);
+            } catch (const std::exception &x) {
+                err[i] = x.what();
+            }
+        }
+    };
+    // a thread costs about as much as one plan: eight plans each, at most 16
+    const size_t want = std::min<size_t>({first.size() / 8, (size_t)std::thread::hardware_concurrency(), 16});
+    std::vector<std::thread> helpers;
+    helpers.reserve(want);
+    try {
+        while (helpers.size() + 1 < want) helpers.emplace_back(work);
+    } catch (const std::system_error &) {   // no more threads: this one does the rest
+    }
+    work();
+    for (auto &t : helpers) t.join();
+    for (size_t i = 0; i < err.size(); ++i)
+        if (!err[i].empty()) return "state " + std::to_string(first[i]) + ": " + err[i];
+    return "";
+}
+
 }  // namespace
 
 namespace sv {
@@ -1342,13 +1381,37 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
     std::vector<GatePassArgs> passes;
     std::vector<Phase> phases;
     std::vector<DevOp> ops;
-    std::vector<uint64_t> plan_keys;
-    std::vector<int32_t> gsize(batch);
+    std::vector<int32_t> gsize(batch), first;   // first state of each plan
+    std::vector<QsuPlan> plans;
     std::vector<BatchStepOff> step_off;
     std::vector<RegStep> steps;
     std::vector<DiagBlock> dblocks;
     std::vector<DiagMember> dmembers;
     auto t0 = std::chrono::steady_clock::now();
+    std::vector<uint64_t> plan_keys;
+    for (int b = 0; b < batch; ++b) {
+        const int gb = gate_off[b], ge = gate_off[b + 1];
+        const int pb = param_off[b], pe = param_off[b + 1];
+        if (ge < gb || pe < pb) return fail(SV_EINVAL, "offsets must be non-decreasing");
+        const size_t m = (size_t)(ge - gb), np = (size_t)(pe - pb);
+        if ((int)m > batch_max_gates()) return fail(SV_EINVAL, "sv_batch_run: more than 1024 gates in a state");
+        std::string err = validate_gates(n, gates + gb, m, np, 0);
+        if (!err.empty()) return fail(SV_EINVAL, "state " + std::to_string(b) + ": " + err);
+        for (size_t i = 0; i < np; ++i)
+            if (!std::isfinite(params[pb + i])) return fail(SV_EINVAL, "non-finite parameter");
+        for (size_t i = 0; i < m; ++i) {
+            const int k = gates[gb + i].kind;
+            gparam.push_back((k == SV_RY || k == SV_RZ || k == SV_GIVENS || k == SV_DEXC) ? gates[gb + i].param : -1);
+        }
+        gsize[b] = (int)m;
+        const uint64_t key = hash_bytes(gates + gb, m * sizeof(sv_gate));
+        const size_t pi = std::find(plan_keys.begin(), plan_keys.end(), key) - plan_keys.begin();
+        if (pi == plan_keys.size()) {
+            plan_keys.push_back(key);
+            first.push_back(b);
+        }
+        state_plan[b] = (int32_t)pi;
+    }
     // step loops where the kernel has them and the tables fit, else gate by gate
     bool stepped = dt == SV_C64 && kmax == 13 && o.threads == 512 && n >= 13;
     size_t step_smem = 0;
@@ -1357,67 +1420,43 @@ sv_status sv_batch_run(int n, sv_dtype dt, int batch, const sv_gate *gates, cons
         po.reg_pairs = stepped;                // gate by gate, phases hold RY / RZ / CZ only
         po.max_diag = stepped ? kMaxPassDiag : 0;
         po.image_limit = stepped ? batch_table_room() : 0;
+        const std::string err = plan_batch(n, gates, gate_off, first, po, l2p, plans);
+        if (!err.empty()) return fail(SV_EINVAL, err);
         plan_pass_off = {0};
         plan_op_off = {0};
-        gparam.clear(); passes.clear(); phases.clear(); ops.clear(); plan_keys.clear();
+        passes.clear(); phases.clear(); ops.clear();
         step_off.clear(); steps.clear(); dblocks.clear(); dmembers.clear();
-        for (int b = 0; b < batch; ++b) {
-            const int gb = gate_off[b], ge = gate_off[b + 1];
-            const int pb = param_off[b], pe = param_off[b + 1];
-            if (ge < gb || pe < pb) return fail(SV_EINVAL, "offsets must be non-decreasing");
-            const size_t m = (size_t)(ge - gb), np = (size_t)(pe - pb);
-            if ((int)m > batch_max_gates()) return fail(SV_EINVAL, "sv_batch_run: more than 1024 gates in a state");
-            std::string err = validate_gates(n, gates + gb, m, np, 0);
-            if (!err.empty()) return fail(SV_EINVAL, "state " + std::to_string(b) + ": " + err);
-            for (size_t i = 0; i < np; ++i)
-                if (!std::isfinite(params[pb + i])) return fail(SV_EINVAL, "non-finite parameter");
-            for (size_t i = 0; i < m; ++i) {
-                const int k = gates[gb + i].kind;
-                gparam.push_back((k == SV_RY || k == SV_RZ || k == SV_GIVENS || k == SV_DEXC) ? gates[gb + i].param : -1);
-            }
-            gsize[b] = (int)m;
-            const uint64_t key = hash_bytes(gates + gb, m * sizeof(sv_gate));
-            int pi = -1;
-            for (size_t k = 0; k < plan_keys.size(); ++k)
-                if (plan_keys[k] == key) pi = (int)k;
-            if (pi < 0) {
-                QsuPlan P;
-                err = plan_qsu(n, 0, gates + gb, m, true, po, l2p, P);
-                if (!err.empty()) return fail(SV_EINVAL, "state " + std::to_string(b) + ": " + err);
-                if ((int)P.ops.size() > batch_max_ops()) return fail(SV_EINVAL, "sv_batch_run: more than 512 gates in a state");
-                const int obase = (int)ops.size();
-                const int pbase = (int)phases.size();
-                step_off.push_back({pbase, (int32_t)steps.size(), (int32_t)dblocks.size(), (int32_t)dmembers.size()});
-                for (auto &gp : P.passes) {
-                    GatePassArgs a = gate_args(n, gp);
-                    if (!stepped) {
-                        a.op_begin += obase;
-                        a.op_end += obase;
-                        if (a.ph_begin >= 0) {
-                            a.ph_begin += pbase;
-                            a.ph_end += pbase;
-                        }
-                        a.db_begin = a.db_end = 0;
+        for (const QsuPlan &P : plans) {
+            if ((int)P.ops.size() > batch_max_ops()) return fail(SV_EINVAL, "sv_batch_run: more than 512 gates in a state");
+            const int obase = (int)ops.size();
+            const int pbase = (int)phases.size();
+            step_off.push_back({pbase, (int32_t)steps.size(), (int32_t)dblocks.size(), (int32_t)dmembers.size()});
+            for (auto &gp : P.passes) {
+                GatePassArgs a = gate_args(n, gp);
+                if (!stepped) {
+                    a.op_begin += obase;
+                    a.op_end += obase;
+                    if (a.ph_begin >= 0) {
+                        a.ph_begin += pbase;
+                        a.ph_end += pbase;
                     }
-                    passes.push_back(a);
+                    a.db_begin = a.db_end = 0;
                 }
-                for (Phase f : P.phases) {
-                    if (!stepped) {
-                        f.op_begin += obase;
-                        f.op_end += obase;
-                    }
-                    phases.push_back(f);
-                }
-                steps.insert(steps.end(), P.steps.begin(), P.steps.end());
-                dblocks.insert(dblocks.end(), P.dblocks.begin(), P.dblocks.end());
-                dmembers.insert(dmembers.end(), P.dmembers.begin(), P.dmembers.end());
-                ops.insert(ops.end(), P.ops.begin(), P.ops.end());
-                plan_pass_off.push_back((int32_t)passes.size());
-                plan_op_off.push_back((int32_t)ops.size());
-                pi = (int)plan_keys.size();
-                plan_keys.push_back(key);
+                passes.push_back(a);
             }
-            state_plan[b] = pi;
+            for (Phase f : P.phases) {
+                if (!stepped) {
+                    f.op_begin += obase;
+                    f.op_end += obase;
+                }
+                phases.push_back(f);
+            }
+            steps.insert(steps.end(), P.steps.begin(), P.steps.end());
+            dblocks.insert(dblocks.end(), P.dblocks.begin(), P.dblocks.end());
+            dmembers.insert(dmembers.end(), P.dmembers.begin(), P.dmembers.end());
+            ops.insert(ops.end(), P.ops.begin(), P.ops.end());
+            plan_pass_off.push_back((int32_t)passes.size());
+            plan_op_off.push_back((int32_t)ops.size());
         }
         if (!stepped) break;
         step_smem = batch_step_bytes(dt, n, kmax, o.threads, passes);

@@ -499,10 +499,9 @@ uint32_t phase_lanes(uint32_t rmask, int k) {
     return lanes;
 }
 
-// what the operations of a register-blocked pass (or of a part of one) are
-void set_pass_kinds(const QsuPlan &P, GatePass &gp) {
-    gp.pairs = gp.others = gp.mat1 = gp.dense = 0;
-    for (int o = gp.op_begin; o < gp.op_end; ++o) {
+// notes what operations [begin, end) are in the pass's kinds
+void add_kinds(const QsuPlan &P, GatePass &gp, int begin, int end) {
+    for (int o = begin; o < end; ++o) {
         const int kd = P.ops[o].kind;
         if (kd == SV_MAT2 || kd == SV_MAT4) gp.dense = 1;
         if (kd == SV_MAT1) gp.mat1 = 1;
@@ -511,10 +510,10 @@ void set_pass_kinds(const QsuPlan &P, GatePass &gp) {
     }
 }
 
-// Shared memory of a register-blocked pass without diagonal blocks (they take
-// what is left), counting a step per operation; the reverse pass, which has
-// the gradient slots besides, unless dense matrices keep it out of registers.
-size_t reg_pass_bytes(const GatePass &gp, int amp) {
+// Whether a register-blocked pass fits without diagonal blocks (they take what
+// is left), counting a step per operation; for the reverse pass, which has the
+// gradient slots besides, unless dense matrices keep it out of registers.
+bool reg_pass_fits(const GatePass &gp, int amp, int image_limit) {
     GatePassArgs a;
     memset(&a, 0, sizeof(a));
     a.k = gp.k;
@@ -524,32 +523,40 @@ size_t reg_pass_bytes(const GatePass &gp, int amp) {
     a.ph_end = gp.ph_end - gp.ph_begin;
     a.pairs = gp.pairs;
     const sv_dtype dt = amp == 8 ? SV_C64 : SV_C128;
-    return gp.dense ? gate_reg_smem(dt, a) : adj_reg_smem(dt, a);
+    if (image_limit) return reg_image_bytes(dt, a) <= (size_t)image_limit;
+    return (gp.dense ? gate_reg_smem(dt, a) : adj_reg_smem(dt, a)) <= (size_t)kRegSmemLimit;
 }
 
 // The pass cut into passes whose tables fit (a single phase always does: at
-// most 256 operations and one set of thread places).
-void cut_pass(const QsuPlan &P, const GatePass &gp, int amp, std::vector<GatePass> &out) {
+// most 256 operations and one set of thread places): with the tiles into
+// shared memory or, for the batched kernel, into image_limit bytes.
+void cut_pass(const QsuPlan &P, const GatePass &gp, int amp, int image_limit, std::vector<GatePass> &out) {
     GatePass cur = gp;
     cur.ph_end = gp.ph_begin;
+    cur.pairs = cur.others = cur.mat1 = cur.dense = 0;
     for (int ph = gp.ph_begin; ph < gp.ph_end; ++ph) {
+        const Phase &F = P.phases[ph];
         GatePass longer = cur;
         longer.ph_end = ph + 1;
-        longer.op_end = P.phases[ph].op_end;
-        set_pass_kinds(P, longer);
-        if (cur.ph_end > cur.ph_begin && reg_pass_bytes(longer, amp) > (size_t)kRegSmemLimit) {
+        longer.op_end = F.op_end;
+        add_kinds(P, longer, F.op_begin, F.op_end);
+        if (cur.ph_end > cur.ph_begin && !reg_pass_fits(longer, amp, image_limit)) {
             out.push_back(cur);
             longer.ph_begin = ph;
-            longer.op_begin = P.phases[ph].op_begin;
-            set_pass_kinds(P, longer);
+            longer.op_begin = F.op_begin;
+            longer.pairs = longer.others = longer.mat1 = longer.dense = 0;
+            add_kinds(P, longer, F.op_begin, F.op_end);
         }
         cur = longer;
     }
     out.push_back(cur);
 }
 
-void plan_phases(QsuPlan &P, bool pairs, int threads, int amp) {
+void plan_phases(QsuPlan &P, bool pairs, int threads, int amp, int image_limit) {
     std::vector<GatePass> passes;
+    std::vector<uint32_t> tm;            // in-tile targets of the pass's operations
+    std::vector<int32_t> remain, next;   // operations left, relative to the pass
+    std::vector<DevOp> out;
     for (auto &gp : P.passes) {
         int r = kRegBits;
         if (threads) {
@@ -564,26 +571,31 @@ void plan_phases(QsuPlan &P, bool pairs, int threads, int amp) {
             const bool pair = kd == SV_GIVENS || kd == SV_DEXC || kd == SV_MAT2 || kd == SV_MAT4;
             if (kd != SV_RY && kd != SV_RZ && kd != SV_CZ && kd != SV_MAT1 && !(pairs && pair)) ok = false;
         }
-        set_pass_kinds(P, gp);
         if (!ok) {
+            add_kinds(P, gp, gp.op_begin, gp.op_end);
             passes.push_back(gp);
             continue;
         }
         const uint32_t all = (gp.k >= 32) ? 0xFFFFFFFFu : ((1u << gp.k) - 1u);
-        auto tmask = [&](const DevOp &d) {
-            uint32_t m = 0;
-            const int nq = op_qubits(d.kind);
+        const DevOp *ops = P.ops.data() + gp.op_begin;
+        const int nops = gp.op_end - gp.op_begin;
+        tm.assign(nops, 0);
+        remain.resize(nops);
+        bool outside = false;            // operations without an in-tile target (nothing blocks them)
+        for (int o = 0; o < nops; ++o) {
+            const int nq = op_qubits(ops[o].kind);
             for (int i = 0; i < nq; ++i)
-                if (d.t[i] < kOutTarget) m |= 1u << d.t[i];
-            return m;
-        };
-        std::vector<DevOp> remain(P.ops.begin() + gp.op_begin, P.ops.begin() + gp.op_end), next, out;
+                if (ops[o].t[i] < kOutTarget) tm[o] |= 1u << ops[o].t[i];
+            outside |= !tm[o];
+            remain[o] = o;
+        }
+        out.clear();
         gp.ph_begin = (int32_t)P.phases.size();
         while (!remain.empty()) {
             uint32_t Rm = 0, avail = all;
-            for (auto &d : remain) {
-                const uint32_t t = tmask(d);
-                if (diag_kind(d.kind)) {
+            for (int32_t o : remain) {
+                const uint32_t t = tm[o];
+                if (diag_kind(ops[o].kind)) {
                     if (t & ~avail) avail &= ~t;
                     continue;
                 }
@@ -599,38 +611,45 @@ void plan_phases(QsuPlan &P, bool pairs, int threads, int amp) {
             ph.op_begin = gp.op_begin + (int32_t)out.size();
             uint32_t av = all;
             next.clear();
-            for (auto &d : remain) {
-                const uint32_t t = tmask(d);
-                const bool fits = (t & ~av) == 0 && (diag_kind(d.kind) || (t & ~Rm) == 0);
-                if (fits) out.push_back(d);
-                else {
-                    av &= ~t;
-                    next.push_back(d);
+            for (size_t i = 0; i < remain.size(); ++i) {
+                if (!av && !outside) {   // all bits are blocked
+                    next.insert(next.end(), remain.begin() + i, remain.end());
+                    break;
                 }
+                const int32_t o = remain[i];
+                const uint32_t t = tm[o];
+                if ((t & ~av) != 0 || (!diag_kind(ops[o].kind) && (t & ~Rm) != 0)) {
+                    av &= ~t;
+                    next.push_back(o);
+                    continue;
+                }
+                DevOp d = ops[o];
+                if (!threads && (d.kind == SV_MAT1 || d.kind == SV_MAT2 || d.kind == SV_MAT4)) {
+                    // the targets' places among the gate's register bits, ascending
+                    PrepMat pm;
+                    pm.nq = op_qubits(d.kind);
+                    pm.src = d.mat;
+                    pm.dst = P.prep_elems;
+                    for (int q = 0; q < 4; ++q)
+                        pm.perm[q] = (int8_t)(q < pm.nq ? __builtin_popcount(t & ((1u << d.t[q]) - 1u)) : 0);
+                    d.pm = pm.dst;
+                    P.prep_elems += 2 << (2 * pm.nq);
+                    P.prep.push_back(pm);
+                }
+                out.push_back(d);
             }
             ph.op_end = gp.op_begin + (int32_t)out.size();
-            for (int o = ph.op_begin - gp.op_begin; o < (int)out.size(); ++o) {
-                DevOp &d = out[o];
-                if (threads || (d.kind != SV_MAT1 && d.kind != SV_MAT2 && d.kind != SV_MAT4)) continue;
-                // the targets' places among the gate's register bits, ascending
-                PrepMat pm;
-                pm.nq = op_qubits(d.kind);
-                pm.src = d.mat;
-                pm.dst = P.prep_elems;
-                const uint32_t tm = tmask(d);
-                for (int t = 0; t < 4; ++t)
-                    pm.perm[t] = (int8_t)(t < pm.nq ? __builtin_popcount(tm & ((1u << d.t[t]) - 1u)) : 0);
-                d.pm = pm.dst;
-                P.prep_elems += 2 << (2 * pm.nq);
-                P.prep.push_back(pm);
-            }
             P.phases.push_back(ph);
             remain.swap(next);
         }
         gp.ph_end = (int32_t)P.phases.size();
         std::copy(out.begin(), out.end(), P.ops.begin() + gp.op_begin);
-        if (threads) passes.push_back(gp);   // the batched kernel gate by gate: no tables
-        else cut_pass(P, gp, amp, passes);
+        if (threads) {                   // the batched kernel gate by gate: no tables
+            add_kinds(P, gp, gp.op_begin, gp.op_end);
+            passes.push_back(gp);
+        } else {
+            cut_pass(P, gp, amp, image_limit, passes);
+        }
     }
     P.passes.swap(passes);
 }
@@ -671,6 +690,10 @@ void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
             if (d.t[i] >= 0 && d.t[i] < kOutTarget) m |= 1u << d.t[i];
         return m;
     };
+    std::vector<DevOp> in, thr, out, rops;
+    std::vector<uint32_t> m;
+    std::vector<char> dg, ry, done;
+    std::vector<int> ready, others, diags, run;
     for (auto &gp : P.passes) {
         gp.db_begin = gp.db_end = (int32_t)P.dblocks.size();
         if (gp.ph_begin < 0) continue;
@@ -693,10 +716,11 @@ void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
         for (int ph = gp.ph_begin; ph < gp.ph_end; ++ph) {
             Phase &F = P.phases[ph];
             F.st_begin = (int32_t)P.steps.size();
-            const std::vector<DevOp> all(P.ops.begin() + F.op_begin, P.ops.begin() + F.op_end);
             // thread-only diagonal operations: one thread block if room
-            std::vector<DevOp> in, thr;
-            for (auto &d : all) {
+            in.clear();
+            thr.clear();
+            for (int o = F.op_begin; o < F.op_end; ++o) {
+                const DevOp &d = P.ops[o];
                 if (in_tile_diag(d) && !(tm(d) & F.rmask)) thr.push_back(d);
                 else in.push_back(d);
             }
@@ -704,32 +728,25 @@ void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
             if (!thr.empty()) {
                 thr_off = take_block(1);
                 if (thr_off < 0) {
-                    in = all;
+                    in.assign(P.ops.begin() + F.op_begin, P.ops.begin() + F.op_end);
                     thr.clear();
                 }
             }
             const int N = (int)in.size();
-            std::vector<uint32_t> m(N);
-            std::vector<char> dg(N), ry(N), done(N, 0);
+            m.resize(N);
+            dg.resize(N);
+            ry.resize(N);
+            done.assign(N, 0);
             for (int i = 0; i < N; ++i) {
                 m[i] = tm(in[i]);
                 dg[i] = diag_kind(in[i].kind);
                 ry[i] = in[i].kind == SV_RY && in[i].t[0] < kOutTarget && (F.rmask >> in[i].t[0] & 1u);
             }
-            std::vector<int> npred(N, 0);
-            std::vector<std::vector<int>> succ(N);
-            for (int j = 0; j < N; ++j)
-                for (int i = 0; i < j; ++i)
-                    if ((m[i] & m[j]) && !(dg[i] && dg[j])) {
-                        ++npred[j];
-                        succ[i].push_back(j);
-                    }
-            std::vector<DevOp> out;
+            out.clear();
             auto regidx = [&](int t) { return __builtin_popcount(F.rmask & ((1u << t) - 1u)); };
             auto emit_op = [&](const DevOp &d) { out.push_back(d); };
             auto emit = [&](int i) {
                 done[i] = 1;
-                for (int j : succ[i]) --npred[j];
                 emit_op(in[i]);
             };
             auto push_op = [&](int i) {
@@ -786,9 +803,17 @@ void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
             };
             int left = N;
             while (left > 0) {
-                std::vector<int> ready, others, diags;
+                // ready: no earlier operation left that does not commute (bits of
+                // the non-diagonal and of the diagonal ones left before it)
+                ready.clear();
+                others.clear();
+                diags.clear();
+                uint32_t nd_left = 0, d_left = 0;
                 for (int i = 0; i < N; ++i) {
-                    if (done[i] || npred[i]) continue;
+                    if (done[i]) continue;
+                    const bool wait = (m[i] & nd_left) || (!dg[i] && (m[i] & d_left));
+                    (dg[i] ? d_left : nd_left) |= m[i];
+                    if (wait) continue;
                     if (ry[i]) ready.push_back(i);
                     else if (dg[i]) diags.push_back(i);
                     else others.push_back(i);
@@ -822,7 +847,7 @@ void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
                     continue;
                 }
                 // diagonal operations only: blockable ones as one run, the rest one by one
-                std::vector<int> run;
+                run.clear();
                 for (int i : diags) {
                     const DevOp &d = in[i];
                     // a thread-only member cannot go into a register block
@@ -831,7 +856,7 @@ void plan_steps(QsuPlan &P, int max_diag, int amp, int image_limit) {
                 }
                 left -= (int)diags.size();
                 if (run.empty()) continue;
-                std::vector<DevOp> rops;
+                rops.clear();
                 for (int i : run) rops.push_back(in[i]);
                 const int off = diag_run_pays(rops) ? take_block(0) : -1;
                 if (off < 0) {
@@ -1549,7 +1574,7 @@ std::string plan_qsu(int n, int g, const sv_gate *gates, size_t m, bool lazy, co
     if (P.tiles.empty()) P.final_l2p = l2p_init;
     int k = std::max(o.tile_bits, std::min(o.low_bits, P.nL) + 4);
     plan_gate_passes(P, ops, k, o.low_bits, o.fuse_max, o.diag_exempt);
-    plan_phases(P, o.reg_pairs, o.reg_threads, o.amp_bytes);
+    plan_phases(P, o.reg_pairs, o.reg_threads, o.amp_bytes, o.image_limit);
     plan_steps(P, std::min(o.max_diag, kMaxPassDiag), o.amp_bytes, o.image_limit);
     return "";
 }
