@@ -4301,9 +4301,9 @@ __global__ void __launch_bounds__(512) k_hpsi_slice(const Cx<R> *__restrict__ ps
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t E = 1u << (a.kl + a.m), O = E / (uint32_t)slices;
     Cx<R> *t = reinterpret_cast<Cx<R> *>(smem);
-    uint64_t *spanv = reinterpret_cast<uint64_t *>(t + E);
+    Cx<R> *red = t + E;                                              // [512] when strings are shared
+    uint64_t *spanv = reinterpret_cast<uint64_t *>(red + 512);       // (behind the 16-byte elements: 8 bytes when m = 0)
     HSliceStr<R> *tab = reinterpret_cast<HSliceStr<R> *>(spanv + (1u << a.m));
-    Cx<R> *red = reinterpret_cast<Cx<R> *>(tab + kHSliceTab);        // [512] when strings are shared
     __shared__ double wsum[16];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t c = blockIdx.x / (uint32_t)slices, sl = blockIdx.x % (uint32_t)slices;
