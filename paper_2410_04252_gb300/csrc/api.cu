@@ -657,7 +657,7 @@ sv_status run_forward(sv_handle *h, QsuEntry *q, sv_stats *st) {
         }
         for (; pi < P.passes.size() && P.passes[pi].tile == (int)t; ++pi, ++launched) {
             const GatePassArgs &a = q->args[pi];
-            if (a.ph_begin >= 0) {
+            if (a.ph_begin >= 0 && gate_reg_pays(h->dt, a)) {
                 Rec r(h, st, SV_K_GATE, 2.0 * (double)h->state_bytes());
                 const int rg = reg_pass_grid(h->dt, a, false, h->opt.blocks_per_sm);
                 SV_CK(launch_gate_reg(h->dt, h->stream, rg, h->psi, a, h->images.as<char>() + q->image[pi], h->pmats.p,
@@ -716,8 +716,7 @@ sv_status run_evc(sv_handle *h, EvcEntry *e, sv_stats *st) {
     int E = 1;
     for (auto &cp : P.passes) E = std::max(E, 1 << (cp.kl + cp.m));
     // a small state's cosets are shared by several CTAs; every pass then writes a row per coset
-    bool slices = !e->args.empty();
-    for (auto &a : e->args) slices = slices && coset_slices_pay(h->dt, a) && a.nfree == e->args[0].nfree;
+    const bool slices = evc_slices_pay(h->dt, P, e->args);
     const int grid = slices ? 1 << e->args[0].nfree : coset_grid(h->dt, E, h->opt.blocks_per_sm, false);
     SV_CK(h->part.ensure((size_t)grid * std::max(nslots, 1) * sizeof(double)));
     SV_CK(h->slotval.ensure(std::max(nslots, 1) * sizeof(double)));
@@ -787,7 +786,7 @@ sv_status run_hpsi(sv_handle *h, EvcEntry *e, sv_stats *st) {
     }
     for (int pi = 0; pi < np; ++pi) {
         Rec r(h, st, SV_K_HPSI, (pi == 0 ? 2.0 : 3.0) * (double)h->state_bytes());
-        if (coset_slices_pay(h->dt, e->args[pi])) {
+        if (hpsi_slices_pay(h->dt, e->args[pi])) {
             SV_CK(launch_hpsi_slice(h->dt, h->stream, h->psi, h->lam, e->args[pi], e->strings.as<DevString>(), pi == 0,
                                     pi == np - 1, h->part.as<double>(), &rows));
             continue;

@@ -2685,6 +2685,20 @@ __global__ void __launch_bounds__(512, 1) k_evc_pass(const Cx<R> *__restrict__ p
     const ThreadCoset tc = thread_coset(a.kl);
     // the transform path needs complex64, 16 per thread, 512 threads, 8192 staged, the scratch
     const bool use_d = sizeof(R) == 8 && EPT == 8 && blockDim.x == 512 && E == 4096u;
+    int zb = a.s_end, ze = a.s_end;          // complex128: the strings of the mask 0
+    if constexpr (sizeof(R) == 8 && EPT == 8) {
+        __shared__ int zrange[2];
+        if (threadIdx.x == 0) zrange[0] = zrange[1] = a.s_end;
+        __syncthreads();
+        for (int gi = a.g_begin + (int)threadIdx.x; gi < a.g_end; gi += (int)blockDim.x)
+            if (!groups[gi].X) {
+                zrange[0] = groups[gi].s_begin;
+                zrange[1] = groups[gi].s_end;
+            }
+        __syncthreads();
+        zb = zrange[0];
+        ze = zrange[1];
+    }
     bool use_x = false;
     float lsg[5] = {1.f, 1.f, 1.f, 1.f, 1.f};
     if constexpr (sizeof(R) == 4 && EPT == 16) {
@@ -2745,22 +2759,47 @@ __global__ void __launch_bounds__(512, 1) k_evc_pass(const Cx<R> *__restrict__ p
             // part it uses, one signed fold and its quarter of a four-value
             // reduction (12.5 FP64 operations a thread instead of 26); the pairs'
             // factor is applied at the end
-            for (int q0 = a.s_begin; use_d && q0 < a.s_end; q0 += 4) {
-                R c[4] = {0, 0, 0, 0};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (q0 + k >= a.s_end) continue;
-                    const DevString S = strs[q0 + k];
-                    const PairSel ps = S.X ? pair_split(tc, S.X, a.kl, EPT) : PairSel{-1, 0, 1};
-                    const uint32_t code = (uint32_t)(ps.h + 1) | ((uint32_t)ps.s << 3) | ((uint32_t)(S.nY & 1) << 4);
-                    const R v = evc_fast<R, EPT, 9>(t, own, S.X, code, S.bz >> tc.ash);
-                    const int neg = (__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz) ^
-                                     (S.X ? ((S.nY == 1) | (S.nY == 2)) : 0)) & 1;
-                    c[k] = neg ? -v : v;
-                }
+            auto add4 = [&](const R *c, int q0, int end) {
                 const R red = warp_sum4<R>(c[0], c[1], c[2], c[3]);
                 const int q = q0 + (lane >> 3);
-                if ((lane & 7) == 0 && q < a.s_end) acc[(q - a.s_begin) * nwarps + warp] += red;
+                if ((lane & 7) == 0 && q < end) acc[(q - a.s_begin) * nwarps + warp] += red;
+            };
+            for (int side = 0; use_d && side < 2; ++side) {
+                const int end = side ? a.s_end : zb;
+                for (int q0 = side ? ze : a.s_begin; q0 < end; q0 += 4) {
+                    R c[4] = {0, 0, 0, 0};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (q0 + k >= end) continue;
+                        const DevString S = strs[q0 + k];
+                        const PairSel ps = pair_split(tc, S.X, a.kl, EPT);
+                        const uint32_t code = (uint32_t)(ps.h + 1) | ((uint32_t)ps.s << 3) | ((uint32_t)(S.nY & 1) << 4);
+                        const R v = evc_fast<R, EPT, 9>(t, own, S.X, code, S.bz >> tc.ash);
+                        const int neg = (__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz) ^
+                                         ((S.nY == 1) | (S.nY == 2))) & 1;
+                        c[k] = neg ? -v : v;
+                    }
+                    add4(c, q0, end);
+                }
+            }
+            // mask 0: |psi|^2 once, a signed sum per string
+            if (use_d && zb < ze) {
+                R w[EPT];
+#pragma unroll
+                for (int j = 0; j < EPT; ++j) w[j] = fma(own[j].x, own[j].x, own[j].y * own[j].y);
+                for (int q0 = zb; q0 < ze; q0 += 4) {
+                    R c[4] = {0, 0, 0, 0};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (q0 + k >= ze) continue;
+                        const DevString S = strs[q0 + k];
+                        uint32_t m = walsh_mask(S.bz >> tc.ash);
+                        if ((__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz)) & 1) m = ~m;
+#pragma unroll
+                        for (int j = 0; j < EPT; ++j) c[k] += flip_by(w[j], m, j);
+                    }
+                    add4(c, q0, ze);
+                }
             }
         }
         for (int gi = use_d ? a.g_end : a.g_begin; gi < a.g_end; ++gi) {
@@ -5339,6 +5378,17 @@ static bool gate_two_pays(sv_dtype dt, const GatePassArgs &a) {
     return dt == SV_C64 && (steps_kind(a) == kStepsDiag || steps_kind(a) == kStepsPair) && a.ph_end - a.ph_begin >= kTwoPhases;
 }
 
+// With few gates to a pass (a double excitation fills a phase) the gate-by-gate
+// kernel's several CTAs an SM move a complex128 state better than one
+// register-blocked CTA.  Brick ansatz, forward, register phases against gate by
+// gate: n = 18 236 : 260 us, n = 20 495 : 456, n = 22 1823 : 1602, n = 23 3616 :
+// 3410; double excitations alone, n = 23, 2980 : 3250.  The reverse pass, which
+// holds two states, gains from its registers throughout.
+bool gate_reg_pays(sv_dtype dt, const GatePassArgs &a) {
+    return dt == SV_C64 || a.others || !(a.pairs & 2) || (a.pairs == 2 && a.n > kL2QubitsC128) ||
+           (1ull << a.nout) <= (uint64_t)device_sms();
+}
+
 int reg_pass_grid(sv_dtype dt, const GatePassArgs &a, bool adj, int blocks_per_sm) {
     const size_t sm = (adj ? adj_reg_smem(dt, a) : gate_reg_smem(dt, a)) + 1024;
     const bool two = !adj && gate_two_pays(dt, a);
@@ -5662,14 +5712,61 @@ cudaError_t launch_hpsi_pass(sv_dtype dt, cudaStream_t st, int grid, const void 
 }
 
 // Slices of a coset for the kernels above: about two CTAs for each SM in all,
-// as far as the strings (a warp each) or the outputs (at least 32) go.  The
-// line between whole cosets and slices is two cosets per SM: with fewer, the
-// double-buffered kernels have nothing to overlap.  complex64, n = 14, 256
-// random strings (2 cosets): an H|psi> pass 210 -> 12 us.  complex128 is bound
-// by its FP64 arithmetic, which one coset per SM already spreads; from there on
-// slices only repeat the loads (4 % slower at n = 20).
-bool coset_slices_pay(sv_dtype dt, const CosetArgs &a) {
-    return a.kl + a.m >= 6 && a.nfree < 16 && (1 << a.nfree) < (dt == SV_C64 ? 2 : 1) * device_sms();
+// as far as the strings (a warp each) or the outputs (at least 32) go.  With
+// fewer cosets than SMs, the double-buffered kernels leave SMs idle and have
+// nothing to overlap; but slices repeat the loads, and read every string's
+// partners from shared memory again.  The lines, from the times of all passes in
+// us, slices : whole cosets (of 2^13 complex64, 2^12 complex128; below that the
+// kernels for whole cosets have no fast paths, and complex64 takes slices):
+//   H|psi>, complex64, 200 random strings: 64 cosets 167 : 193, 128 245 : 229,
+//     256 372 : 316; with five strings a mask and more, whose coefficients are
+//     added up first, 301 : 313 at 128 and 529 : 614 at 256 (about nine a mask);
+//   complex128, 200 random strings: 64 cosets 575 : 627, 128 976 : 648; 64
+//     strings a mask 490 : 576 at 128.
+//   Expectation, complex64: by strings times cosets a pass, those on the mask 0
+//     twice (every element, not one of a pair).  700 Jordan-Wigner strings in 5
+//     passes, 500 of them on the mask 0: 16 cosets 81 : 102, 32 132 : 118, 128
+//     354 : 148; 200 strings in 4 passes: 32 cosets 48 : 69, 64 87 : 86, 128
+//     123 : 90; 1000 random strings in 56 passes, 256 cosets 1127 : 2277.  Nothing
+//     but strings on the mask 0 is one transform a coset: 300 of them 8 cosets
+//     17 : 16, 32 61 : 16.
+//   complex128: a pass is a chain of FP64 for one warp, 20 us at 2^12 (12 more on
+//     the mask 0), 12 and 7 at 2^11 and 2^10, where whole cosets take about 6 us
+//     and 3 a string: one string 20 : 13, an identity 32 : 13, 8 strings 44 : 36,
+//     200 of them 64 cosets 782 : 777.
+static bool sliceable(const CosetArgs &a) { return a.kl + a.m >= 6 && a.nfree < 16; }
+
+bool hpsi_slices_pay(sv_dtype dt, const CosetArgs &a) {
+    const int ncos = 1 << a.nfree, sms = device_sms();
+    if (!sliceable(a) || ncos >= (dt == SV_C64 ? 2 : 1) * sms) return false;
+    if (2 * ncos <= sms || (dt == SV_C64 && a.kl + a.m < 13)) return true;
+    return a.s_end - a.s_begin >= (dt == SV_C64 ? 5 : 16) * (a.g_end - a.g_begin);
+}
+
+bool evc_slices_pay(sv_dtype dt, const EvcPlan &plan, const std::vector<CosetArgs> &passes) {
+    if (passes.empty()) return false;
+    const int64_t ncos = (int64_t)1 << passes[0].nfree, sms = device_sms(), np = (int64_t)passes.size();
+    if (ncos >= 2 * sms) return false;
+    int64_t strings = 0, zero = 0, zgroups = 0;    // all strings; those on the mask 0, and their passes
+    bool full = true;                              // complex64 runs of cosets of 2^13
+    for (auto &a : passes) {
+        if (a.nfree != passes[0].nfree || !sliceable(a)) return false;
+        strings += a.s_end - a.s_begin;
+        full = full && a.kl + a.m == 13;
+    }
+    for (auto &g : plan.groups)
+        if (!g.X) {
+            zero += g.s_end - g.s_begin;
+            ++zgroups;
+        }
+    if (dt == SV_C128) {
+        const int bits = passes[0].kl + passes[0].m;
+        const int64_t chain = bits >= 12 ? 20 : bits == 11 ? 12 : bits == 10 ? 7 : 5, on_zero = chain * 3 / 5;
+        return 2 * ncos <= sms && 1000 * (chain * np + on_zero * zgroups) + 15 * (strings + 2 * zero) * ncos <
+                                      1000 * (6 * np + 3 * strings);
+    }
+    if (!full) return true;
+    return zero < strings && (ncos == 1 || (strings + zero) * ncos <= 6000 * np);
 }
 
 cudaError_t launch_evc_slice(sv_dtype dt, cudaStream_t st, const void *psi, const CosetArgs &a, const DevString *strs,

@@ -22,7 +22,7 @@ struct GatePassArgs {
     int st_begin, st_end;    // steps of the pass's register phases
     int area;                // bytes of the diagonal-block data
     int mem_begin, mem_end;  // diagonal-block members of the pass
-    int pairs;               // the phases hold pair rotations (Givens, double excitations)
+    int pairs;               // the phases hold pair rotations (1: Givens, 2: double excitations)
     int others;              // and gates besides pair rotations
     int mat1;                // the phases hold 1-qubit matrices
     int dense;               // the phases hold 2- or 4-qubit matrices (the reverse pass runs in k_adj_pass)
@@ -112,6 +112,8 @@ cudaError_t launch_adj_pass(sv_dtype dt, cudaStream_t st, int grid, int threads,
 // phases' steps (RegStep) are executed in order (forward) or in reverse
 // (adjoint); part receives the FP64 gradient partials of every operation.
 // pmats: the prepared matrices of launch_prep_mats.
+// whether the forward pass runs in its register phases (it may run gate by gate)
+bool gate_reg_pays(sv_dtype dt, const GatePassArgs &a);
 int reg_pass_grid(sv_dtype dt, const GatePassArgs &a, bool adj, int blocks_per_sm);
 cudaError_t launch_prep_mats(sv_dtype dt, cudaStream_t st, const PrepMat *prep, int count, const void *mats, void *out);
 // The tables of the register-blocked passes, made on the device once per call
@@ -151,9 +153,10 @@ cudaError_t launch_evc_reg(sv_dtype dt, cudaStream_t st, int grid, const void *p
 // Few strings with their masks as the span basis (plan_evc_kernels; complex64).
 cudaError_t launch_evc_unit(cudaStream_t st, int grid, const void *psi, const CosetArgs &a, const CosetPass &cp,
                             const EvcUnitItem *uitems, double *part, int part_stride);
-// Few cosets (coset_slices_pay): several CTAs share a coset.  Expectation:
-// part rows are the 2^nfree cosets; H|psi>: *rows energy partials.
-bool coset_slices_pay(sv_dtype dt, const CosetArgs &a);
+// Few cosets: several CTAs share a coset.  Expectation (all passes of a call or
+// none): part rows are the 2^nfree cosets; H|psi>: *rows energy partials.
+bool evc_slices_pay(sv_dtype dt, const EvcPlan &plan, const std::vector<CosetArgs> &passes);
+bool hpsi_slices_pay(sv_dtype dt, const CosetArgs &a);
 cudaError_t launch_evc_slice(sv_dtype dt, cudaStream_t st, const void *psi, const CosetArgs &a, const DevString *strs,
                              double *part, int part_stride);
 cudaError_t launch_hpsi_slice(sv_dtype dt, cudaStream_t st, const void *psi, void *lam, const CosetArgs &a,

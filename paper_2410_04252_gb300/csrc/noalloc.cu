@@ -157,10 +157,8 @@ extern "C" sv_status sv_expect_noalloc(const void *state, int n, sv_dtype dt, co
     // coset (three quarters of the scratch: the tables take far less than the
     // rest); else few strings go to the unit kernel and Jordan-Wigner masks to
     // register phases, as in sv_expect (n = 26, 177 strings: 5.0 -> 2.5 ms a call)
-    bool slices = true;
-    for (auto &a : args)
-        slices = slices && sv::coset_slices_pay(dt, a) && a.nfree == args[0].nfree &&
-                 ((size_t)nslots * sizeof(double) << a.nfree) <= kNoAllocScratchBytes / 4 * 3;
+    const bool slices = sv::evc_slices_pay(dt, P, args) &&
+                        ((size_t)nslots * sizeof(double) << args[0].nfree) <= kNoAllocScratchBytes / 4 * 3;
     if (!slices) {
         sv::plan_evc_kernels(P, dt);
         for (size_t i = 0; i < args.size(); ++i) {

@@ -505,7 +505,7 @@ void add_kinds(const QsuPlan &P, GatePass &gp, int begin, int end) {
         const int kd = P.ops[o].kind;
         if (kd == SV_MAT2 || kd == SV_MAT4) gp.dense = 1;
         if (kd == SV_MAT1) gp.mat1 = 1;
-        if (kd == SV_GIVENS || kd == SV_DEXC) gp.pairs = 1;
+        if (kd == SV_GIVENS || kd == SV_DEXC) gp.pairs |= kd == SV_DEXC ? 2 : 1;
         else gp.others = 1;
     }
 }
@@ -552,6 +552,20 @@ void cut_pass(const QsuPlan &P, const GatePass &gp, int amp, int image_limit, st
     out.push_back(cur);
 }
 
+// complex128 passes that gate by gate are no slower.  A double excitation moves
+// an eighth of the amplitudes but takes a phase of its own, which moves them all:
+// 80 of them, n = 21, 738 us gate by gate, 941 in register phases (n = 23, out of
+// L2, 3250 and 2980).  Tiles of 2^9 and 2^10 are one or two warps, which do not
+// keep FP64 busy but for the longest gates and the passes that take tables only:
+// n = 10, 80 gates: Givens 77 and 108, 2-qubit matrices 612 and 706, 4-qubit 4350
+// and 2870, RZ and CZ 88 and 12, RY 118 and 94 (2^9, with CZ: 111 and 123).
+bool reg_pays_c128(const GatePass &gp, const int *count, int n) {
+    const int all = gp.op_end - gp.op_begin;
+    if (2 * count[SV_DEXC] > all && n <= kL2QubitsC128) return false;
+    if (gp.k >= kRegMinTile + 2 || count[SV_MAT4]) return true;
+    return count[SV_RZ] + count[SV_CZ] + (gp.k > kRegMinTile ? count[SV_RY] : 0) == all;
+}
+
 void plan_phases(QsuPlan &P, bool pairs, int threads, int amp, int image_limit) {
     std::vector<GatePass> passes;
     std::vector<uint32_t> tm;            // in-tile targets of the pass's operations
@@ -564,13 +578,12 @@ void plan_phases(QsuPlan &P, bool pairs, int threads, int amp, int image_limit) 
             for (int t = threads; t > 1; t >>= 1) --r;
         }
         bool ok = r >= 2 && (threads || gp.k >= kRegMinTile);
-        for (int o = gp.op_begin; o < gp.op_end; ++o) {
-            const int kd = P.ops[o].kind;
-            // Givens rotations, double excitations and dense 2- and 4-qubit
-            // matrices need their targets among four register bits
-            const bool pair = kd == SV_GIVENS || kd == SV_DEXC || kd == SV_MAT2 || kd == SV_MAT4;
-            if (kd != SV_RY && kd != SV_RZ && kd != SV_CZ && kd != SV_MAT1 && !(pairs && pair)) ok = false;
-        }
+        int count[8] = {};
+        for (int o = gp.op_begin; o < gp.op_end; ++o) ++count[P.ops[o].kind];
+        // Givens rotations, double excitations and dense 2- and 4-qubit
+        // matrices need their targets among four register bits
+        if (!pairs && count[SV_GIVENS] + count[SV_DEXC] + count[SV_MAT2] + count[SV_MAT4]) ok = false;
+        if (amp == 16 && !threads && !reg_pays_c128(gp, count, P.n)) ok = false;
         if (!ok) {
             add_kinds(P, gp, gp.op_begin, gp.op_end);
             passes.push_back(gp);

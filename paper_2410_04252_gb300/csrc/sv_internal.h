@@ -65,7 +65,7 @@ struct GatePass {
     uint64_t bits = 0;                // physical staged bits
     int32_t op_begin = 0, op_end = 0; // into QsuPlan::ops
     int32_t ph_begin = -1, ph_end = -1;  // register phases (register-blocked passes), else -1
-    int32_t pairs = 0;                   // 1: the phases hold pair rotations
+    int32_t pairs = 0;                   // the phases hold pair rotations (1: Givens, 2: double excitations)
     int32_t others = 0;                  // 1: the phases hold gates besides pair rotations
     int32_t mat1 = 0;                    // 1: the phases hold 1-qubit matrices
     int32_t dense = 0;                   // 1: the phases hold 2- or 4-qubit matrices (forward only)
@@ -105,6 +105,7 @@ constexpr int kMaxPassDiag = 24;       // diagonal blocks per register-blocked p
 // so a tile of 2^k amplitudes takes 2^(k - kRegBits) threads, at least a warp.
 constexpr int kRegBits = 4;
 constexpr int kRegMinTile = kRegBits + 5;
+constexpr int kL2QubitsC128 = 22;    // complex128 states of 64 MB (half of L2)
 
 // A register phase of a register-blocked pass: each thread holds the
 // amplitudes spanned by the tile bits in rmask; ops [op_begin, op_end) are
