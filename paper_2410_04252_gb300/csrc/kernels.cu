@@ -1,17 +1,24 @@
 // Device kernels of the hot path (sm_103a).
 //
-//   k_gate_pass   K-GATE: stage 2^k amplitudes of a tile in shared memory,
-//                 apply a whole pass of narrow gates (Eq. apply_parallel:
+//   k_gate_pass   K-GATE gate by gate: stage 2^k amplitudes of a tile in shared
+//                 memory, apply a whole pass of narrow gates (Eq. apply_parallel:
 //                 every virtual chunk applies the same local operator), store.
+//   k_gate_reg    K-GATE in register phases (most passes); k_gate_two with two
+//                 tiles in work; their tables by k_reg_image, matrices by
+//                 k_prep_mats, once per call.
 //   k_adj_pass    K-ADJ: the same tiles of psi and lambda; per gate, in reverse,
-//                 the partial of Im<lambda|G|psi> and then U^dagger on both.
+//   k_adj_reg     the partial of Im<lambda|G|psi> and then U^dagger on both.
 //   k_bitswap     K-QR: in-place exchange of physical index bit pairs (the
 //                 qubit reordering of Sec. III-B-4: two elements whose indices
 //                 differ only at the paired bits are swapped).
 //   k_evc_pass    K-EVC: <psi|P|psi> for all strings whose X/Y mask pairs
 //                 amplitudes inside one staged coset (Eqs. evc, parallel_evc,
-//                 par_exp).
-//   k_hpsi_pass   K-HPSI: lambda += sum_t a_t P_t psi over the same cosets.
+//                 par_exp).  k_evc_few and k_evc_ring: few single strings;
+//                 k_evc_unit: those whose masks are the span's basis; k_evc_reg:
+//                 masks of one or two staged bits; k_evc_slice: few cosets.
+//   k_hpsi_pass   K-HPSI: lambda += sum_t a_t P_t psi over the same cosets;
+//                 k_hpsi_vec by element pairs, k_hpsi_slice for few cosets.
+//   k_batch       K-BATCH: whole states, one CTA each.
 //   k_reduce_rows K-RED: fixed-order FP64 reduction of per-CTA partials.
 //
 // All kernels are persistent grid-stride loops over independent work units
@@ -580,12 +587,14 @@ template <int OFF> __device__ __forceinline__ float2 lds_f2_off(uint32_t addr) {
 }
 
 // ------------------------------------------------- register-blocked passes --
-// A pass of RY / RZ / CZ / 1-qubit matrices runs in phases (host planned):
-// in a phase each of the 512 threads holds the 2^RB amplitudes spanned by
-// the phase's register bits (rmask) of the staged tile, gathered from shared
-// memory; non-diagonal gates act on register bits, diagonal gates on any bit
-// (a thread bit just selects the phase or sign for all of its registers).
-// One shared-memory transpose per phase instead of one barrier per gate.
+// A pass runs in phases (host planned): in a phase each of its 2^(k - RB)
+// threads holds the 2^RB amplitudes spanned by the phase's register bits
+// (rmask) of the staged tile, gathered from shared memory; non-diagonal gates
+// act on register bits, diagonal gates on any bit (a thread bit just selects
+// the phase or sign for all of its registers).  One shared-memory transpose per
+// phase instead of one barrier per gate.  The functions up to phase_base are
+// those of the batched kernel gate by gate (RY, RZ and CZ, 512 threads); the
+// others run decoded steps (k_gate_reg).
 __device__ __forceinline__ uint32_t swz_tile(uint32_t i) {
     return swz_slot(i);   // bijection; spreads strided lanes over the banks
 }
@@ -602,20 +611,6 @@ __device__ __forceinline__ void reg_rot(Cx<R> *x, R c, R s) {
         for (int v = 0; v < V; ++v)
             if (!(v & (1 << B))) rot<R>(x[v], x[v | (1 << B)], c, s);
     }
-}
-template <typename R, int V, int B>
-__device__ __forceinline__ void reg_mat1(Cx<R> *x, const Cx<R> *M, bool adj) {
-    const Cx<R> m00 = mel<R>(M, 2, 0, 0, adj), m01 = mel<R>(M, 2, 0, 1, adj);
-    const Cx<R> m10 = mel<R>(M, 2, 1, 0, adj), m11 = mel<R>(M, 2, 1, 1, adj);
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-        if (!(v & (1 << B))) {
-            const Cx<R> a = x[v], b = x[v | (1 << B)];
-            x[v] = mk<R>(m00.x * a.x - m00.y * a.y + m01.x * b.x - m01.y * b.y,
-                         m00.x * a.y + m00.y * a.x + m01.x * b.y + m01.y * b.x);
-            x[v | (1 << B)] = mk<R>(m10.x * a.x - m10.y * a.y + m11.x * b.x - m11.y * b.y,
-                                    m10.x * a.y + m10.y * a.x + m11.x * b.y + m11.y * b.x);
-        }
 }
 // multiply by (c, s) where bit B of v is 1 and by (c, -s) where it is 0
 template <typename R, int V, int B>
@@ -653,7 +648,7 @@ __device__ __forceinline__ void reg_neg_bit(Cx<R> *x) {
 // the thread's tile index bits outside rmask.
 template <typename R, int RB>
 __device__ __forceinline__ void reg_apply(Cx<R> *x, const DevOp &op, uint32_t rmask, uint32_t base, const R *coef,
-                                          const Cx<R> *mats, bool adj) {
+                                          bool adj) {
     constexpr int V = 1 << RB;
     const int t0 = op.t[0];
     const int b0 = __popc(rmask & ((1u << t0) - 1u));
@@ -661,13 +656,6 @@ __device__ __forceinline__ void reg_apply(Cx<R> *x, const DevOp &op, uint32_t rm
     case SV_RY: {
         const R c = coef[2 * op.gate], s = adj ? -coef[2 * op.gate + 1] : coef[2 * op.gate + 1];
 #define SV_C(B) reg_rot<R, V, B>(x, c, s)
-        SV_REG_SWITCH(b0, SV_C)
-#undef SV_C
-        break;
-    }
-    case SV_MAT1: {
-        const Cx<R> *M = mats + op.mat;
-#define SV_C(B) reg_mat1<R, V, B>(x, M, adj)
         SV_REG_SWITCH(b0, SV_C)
 #undef SV_C
         break;
@@ -711,29 +699,6 @@ __device__ __forceinline__ void reg_apply(Cx<R> *x, const DevOp &op, uint32_t rm
 #pragma unroll
             for (int v = 0; v < V; ++v) x[v] = mk<R>(-x[v].x, -x[v].y);
         }
-        break;
-    }
-    case SV_OP_PHASE: {
-        const R c = coef[2 * op.gate], s = adj ? -coef[2 * op.gate + 1] : coef[2 * op.gate + 1];
-        const R ss = op.t[0] ? s : -s;
-#pragma unroll
-        for (int v = 0; v < V; ++v) x[v] = mk<R>(c * x[v].x - ss * x[v].y, c * x[v].y + ss * x[v].x);
-        break;
-    }
-    case SV_OP_ZSIGN: {
-        if ((rmask >> t0) & 1u) {
-#define SV_C(B) reg_neg_bit<R, V, B>(x)
-            SV_REG_SWITCH(b0, SV_C)
-#undef SV_C
-        } else if ((base >> t0) & 1u) {
-#pragma unroll
-            for (int v = 0; v < V; ++v) x[v] = mk<R>(-x[v].x, -x[v].y);
-        }
-        break;
-    }
-    case SV_OP_NEG: {
-#pragma unroll
-        for (int v = 0; v < V; ++v) x[v] = mk<R>(-x[v].x, -x[v].y);
         break;
     }
     default:
@@ -785,7 +750,7 @@ __device__ __forceinline__ R reg_rz_adj(Cx<R> *p, Cx<R> *l, R c, R s) {
 
 template <typename R, int RB>
 __device__ __forceinline__ R reg_adjoint(Cx<R> *p, Cx<R> *l, const DevOp &op, uint32_t rmask, uint32_t base,
-                                         const R *coef, const Cx<R> *mats) {
+                                         const R *coef) {
     constexpr int V = 1 << RB;
     const int t0 = op.t[0];
     const int b0 = __popc(rmask & ((1u << t0) - 1u));
@@ -795,15 +760,14 @@ __device__ __forceinline__ R reg_adjoint(Cx<R> *p, Cx<R> *l, const DevOp &op, ui
 #define SV_C(B) g = reg_ry_adj<R, V, B>(p, l, c, s)
         SV_REG_SWITCH(b0, SV_C)
 #undef SV_C
-    } else if (op.kind == SV_RZ || op.kind == SV_OP_PHASE) {
+    } else if (op.kind == SV_RZ) {
         const R c = coef[2 * op.gate], s = -coef[2 * op.gate + 1];
-        if (op.kind == SV_RZ && ((rmask >> t0) & 1u)) {
+        if ((rmask >> t0) & 1u) {
 #define SV_C(B) g = reg_rz_adj<R, V, B>(p, l, c, s)
             SV_REG_SWITCH(b0, SV_C)
 #undef SV_C
         } else {
-            // the bit is the same for all registers: a thread bit, or a qubit outside the tile
-            const bool one = op.kind == SV_OP_PHASE ? op.t[0] != 0 : ((base >> t0) & 1u) != 0;
+            const bool one = (base >> t0) & 1u;     // a thread bit: the same for all registers
             const R ss = one ? s : -s;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -814,8 +778,8 @@ __device__ __forceinline__ R reg_adjoint(Cx<R> *p, Cx<R> *l, const DevOp &op, ui
             }
         }
     } else {
-        reg_apply<R, RB>(p, op, rmask, base, coef, mats, true);
-        reg_apply<R, RB>(l, op, rmask, base, coef, mats, true);
+        reg_apply<R, RB>(p, op, rmask, base, coef, true);
+        reg_apply<R, RB>(l, op, rmask, base, coef, true);
     }
     return g;
 }
@@ -3729,7 +3693,7 @@ __device__ __forceinline__ void eu_products(float *P, const float2 *x) {
 }
 struct __align__(16) EvcUnitS {
     float lev[4];
-    uint32_t code, sX;       // sX: swizzled slot of X
+    uint32_t code, sX;       // sX: the partner offset X
     float last;              // code 16, 17: the fifth sign
     float fac;               // 2 when each pair is taken once
 };
@@ -4547,7 +4511,7 @@ __device__ __noinline__ void batch_reg_forward(Cx<R> *tile, const GatePassArgs &
         base = phase_base(F.rmask, F.lanes, P.k, threadIdx.x);   // the phase's lane bits (conflict-free half-warps)
         Cx<R> x[V];
         batch_gather<R, V>(x, tile, base, sp, F.rmask & 1u);
-        for (int o = F.op_begin; o < F.op_end; ++o) reg_apply<R, RB>(x, ops[o], F.rmask, base, coef, nullptr, false);
+        for (int o = F.op_begin; o < F.op_end; ++o) reg_apply<R, RB>(x, ops[o], F.rmask, base, coef, false);
         batch_scatter<R, V>(x, tile, base, sp, F.rmask & 1u);
         __syncthreads();
     }
@@ -4590,7 +4554,7 @@ __device__ __noinline__ void batch_reg_adjoint(Cx<R> *tp, Cx<R> *tl, const GateP
         batch_gather<R, V>(xl, tl, base, sp, F.rmask & 1u);
         for (int o = F.op_end - 1; o >= F.op_begin; --o) {
             const DevOp op = ops[o];
-            R g = reg_adjoint<R, RB>(xp, xl, op, F.rmask, base, coef, nullptr);
+            R g = reg_adjoint<R, RB>(xp, xl, op, F.rmask, base, coef);
             if (has_param(op.kind)) {
                 g = warp_sum<R>(g);
                 if (lane == 0) opacc[(o - o0) * nwarps + warp] += g;
