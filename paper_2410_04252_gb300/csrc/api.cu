@@ -777,7 +777,7 @@ sv_status run_hpsi(sv_handle *h, EvcEntry *e, sv_stats *st) {
     for (auto &cp : P.passes) E = std::max(E, 1 << (cp.kl + cp.m));
     const int grid = coset_grid(h->dt, E, h->opt.blocks_per_sm, true);
     SV_CK(h->part.ensure((size_t)std::max(grid, 2 * device_sms()) * sizeof(double) + 64));
-    int rows = grid;         // energy partials of the last pass
+    int rows = grid;         // energy partials of the last pass (slices and whole cosets may take turns)
     const int np = (int)P.passes.size();
     if (np == 0) {
         SV_CK(cudaMemsetAsync(h->lam, 0, h->state_bytes(), h->stream));
@@ -791,6 +791,7 @@ sv_status run_hpsi(sv_handle *h, EvcEntry *e, sv_stats *st) {
                                     pi == np - 1, h->part.as<double>(), &rows));
             continue;
         }
+        rows = grid;
         SV_CK(launch_hpsi_pass(h->dt, h->stream, grid, h->psi, h->lam, e->args[pi], e->groups.as<DevGroup>(),
                                e->strings.as<DevString>(), pi == 0, pi == np - 1, h->part.as<double>(),
                                res_status(h), (long long)h->opt.wait_limit));

@@ -2649,19 +2649,19 @@ __global__ void __launch_bounds__(512, 1) k_evc_pass(const Cx<R> *__restrict__ p
     const ThreadCoset tc = thread_coset(a.kl);
     // the transform path needs complex64, 16 per thread, 512 threads, 8192 staged, the scratch
     const bool use_d = sizeof(R) == 8 && EPT == 8 && blockDim.x == 512 && E == 4096u;
-    int zb = a.s_end, ze = a.s_end;          // complex128: the strings of the mask 0
+    // complex128: the pass's groups of the mask 0 (a full group of 256 strings and
+    // the rest of them at most: a pass holds kMaxPassStrings)
+    constexpr int ZG = kMaxPassStrings / kMaxGroupStrings + 1;
+    __shared__ int zgroup[ZG], zcount;
     if constexpr (sizeof(R) == 8 && EPT == 8) {
-        __shared__ int zrange[2];
-        if (threadIdx.x == 0) zrange[0] = zrange[1] = a.s_end;
+        if (threadIdx.x == 0) zcount = 0;
         __syncthreads();
         for (int gi = a.g_begin + (int)threadIdx.x; gi < a.g_end; gi += (int)blockDim.x)
             if (!groups[gi].X) {
-                zrange[0] = groups[gi].s_begin;
-                zrange[1] = groups[gi].s_end;
+                const int at = atomicAdd(&zcount, 1);
+                if (at < ZG) zgroup[at] = gi;
             }
         __syncthreads();
-        zb = zrange[0];
-        ze = zrange[1];
     }
     bool use_x = false;
     float lsg[5] = {1.f, 1.f, 1.f, 1.f, 1.f};
@@ -2723,46 +2723,51 @@ __global__ void __launch_bounds__(512, 1) k_evc_pass(const Cx<R> *__restrict__ p
             // part it uses, one signed fold and its quarter of a four-value
             // reduction (12.5 FP64 operations a thread instead of 26); the pairs'
             // factor is applied at the end
-            auto add4 = [&](const R *c, int q0, int end) {
+            auto add4 = [&](const R *c, int q0, uint32_t take) {
                 const R red = warp_sum4<R>(c[0], c[1], c[2], c[3]);
-                const int q = q0 + (lane >> 3);
-                if ((lane & 7) == 0 && q < end) acc[(q - a.s_begin) * nwarps + warp] += red;
+                if ((lane & 7) == 0 && (take >> (lane >> 3)) & 1u) acc[(q0 + (lane >> 3) - a.s_begin) * nwarps + warp] += red;
             };
-            for (int side = 0; use_d && side < 2; ++side) {
-                const int end = side ? a.s_end : zb;
-                for (int q0 = side ? ze : a.s_begin; q0 < end; q0 += 4) {
-                    R c[4] = {0, 0, 0, 0};
+            const bool shared0 = zcount <= ZG;       // (more could not be listed: one by one)
+            for (int q0 = a.s_begin; use_d && q0 < a.s_end; q0 += 4) {
+                R c[4] = {0, 0, 0, 0};
+                uint32_t take = 0;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if (q0 + k >= end) continue;
-                        const DevString S = strs[q0 + k];
-                        const PairSel ps = pair_split(tc, S.X, a.kl, EPT);
-                        const uint32_t code = (uint32_t)(ps.h + 1) | ((uint32_t)ps.s << 3) | ((uint32_t)(S.nY & 1) << 4);
-                        const R v = evc_fast<R, EPT, 9>(t, own, S.X, code, S.bz >> tc.ash);
-                        const int neg = (__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz) ^
-                                         ((S.nY == 1) | (S.nY == 2))) & 1;
-                        c[k] = neg ? -v : v;
-                    }
-                    add4(c, q0, end);
+                for (int k = 0; k < 4; ++k) {
+                    if (q0 + k >= a.s_end) continue;
+                    const DevString S = strs[q0 + k];
+                    if (!S.X && shared0) continue;
+                    take |= 1u << k;
+                    const PairSel ps = S.X ? pair_split(tc, S.X, a.kl, EPT) : PairSel{-1, 0, 1};
+                    const uint32_t code = (uint32_t)(ps.h + 1) | ((uint32_t)ps.s << 3) | ((uint32_t)(S.nY & 1) << 4);
+                    const R v = evc_fast<R, EPT, 9>(t, own, S.X, code, S.bz >> tc.ash);
+                    const int neg = (__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz) ^
+                                     (S.X ? ((S.nY == 1) | (S.nY == 2)) : 0)) & 1;
+                    c[k] = neg ? -v : v;
                 }
+                if (take) add4(c, q0, take);
             }
             // mask 0: |psi|^2 once, a signed sum per string
-            if (use_d && zb < ze) {
+            if (use_d && zcount && shared0) {
                 R w[EPT];
 #pragma unroll
                 for (int j = 0; j < EPT; ++j) w[j] = fma(own[j].x, own[j].x, own[j].y * own[j].y);
-                for (int q0 = zb; q0 < ze; q0 += 4) {
-                    R c[4] = {0, 0, 0, 0};
+                for (int zi = 0; zi < zcount; ++zi) {
+                    const DevGroup G = groups[zgroup[zi]];
+                    for (int q0 = G.s_begin; q0 < G.s_end; q0 += 4) {
+                        R c[4] = {0, 0, 0, 0};
+                        uint32_t take = 0;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if (q0 + k >= ze) continue;
-                        const DevString S = strs[q0 + k];
-                        uint32_t m = walsh_mask(S.bz >> tc.ash);
-                        if ((__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz)) & 1) m = ~m;
+                        for (int k = 0; k < 4; ++k) {
+                            if (q0 + k >= G.s_end) continue;
+                            take |= 1u << k;
+                            const DevString S = strs[q0 + k];
+                            uint32_t m = walsh_mask(S.bz >> tc.ash);
+                            if ((__popcll((rep | tc.l) & S.z) ^ __popc(tc.a0 & S.bz)) & 1) m = ~m;
 #pragma unroll
-                        for (int j = 0; j < EPT; ++j) c[k] += flip_by(w[j], m, j);
+                            for (int j = 0; j < EPT; ++j) c[k] += flip_by(w[j], m, j);
+                        }
+                        add4(c, q0, take);
                     }
-                    add4(c, q0, ze);
                 }
             }
         }
@@ -5248,6 +5253,17 @@ cudaError_t launch_drained(void (*kernel)(A...), dim3 grid, int threads, size_t 
     return cudaLaunchKernelEx(&cfg, kernel, A(v)...);
 }
 
+// A coset kernel of one CTA an SM.  Overlapped, the blocks of the next pass are
+// placed beside running ones where two fit an SM, and not evenly: complex128,
+// passes of 2^8 amplitudes, 250 strings 3.4 -> 5.5 ms a call.  (The default
+// passes take more than half of an SM's shared memory.)
+template <typename... A, typename... V>
+cudaError_t launch_even(void (*kernel)(A...), int nfree, int grid, int threads, size_t smem, cudaStream_t st, V... v) {
+    if (2 * (smem + 1024) <= (size_t)228 * 1024 && (nfree >= 31 || (1 << nfree) >= device_sms()))
+        return launch_drained(kernel, grid, threads, smem, st, v...);
+    return launch(kernel, grid, threads, smem, st, v...);
+}
+
 size_t gate_smem(sv_dtype dt, int k, int nlow) {
     const size_t es = dt == SV_C64 ? 8 : 16;
     return ((size_t)1 << k) * es + ((size_t)1 << (k - nlow)) * 8 + 64;
@@ -5527,7 +5543,7 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
         const size_t smr = 3 * (size_t)E * sizeof(Cx<R>) + ((size_t)1 << a.m) * 8;
 #define SV_EVCR_CASE(N)                                                                                      \
     case N:                                                                                                  \
-        return launch(k_evc_ring<R, N, 9>, grid, 512, smr, st, (const Cx<R> *)psi, a, groups, strs, part,    \
+        return launch_even(k_evc_ring<R, N, 9>, a.nfree, grid, 512, smr, st, (const Cx<R> *)psi, a, groups, strs, part,    \
                       part_stride);
         switch (ept) {
             SV_EVCR_CASE(2)
@@ -5544,7 +5560,7 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
                            (size_t)kEvcFew * threads * (sizeof(R) + 4);
 #define SV_EVCF_CASE(N)                                                                                      \
     case N:                                                                                                  \
-        return launch(k_evc_few<R, N, 9>, grid, threads, smf, st, (const Cx<R> *)psi, a, groups, strs, part, \
+        return launch_even(k_evc_few<R, N, 9>, a.nfree, grid, threads, smf, st, (const Cx<R> *)psi, a, groups, strs, part, \
                       part_stride);
         switch (ept) {
             SV_EVCF_CASE(1)
@@ -5567,7 +5583,7 @@ cudaError_t evc_dispatch(cudaStream_t st, int grid, const void *psi, const Coset
     }
 #define SV_EVC_CASE(N)                                                                                       \
     case N:                                                                                                  \
-        return launch(k_evc_pass<R, N>, grid, threads, sm, st, (const Cx<R> *)psi, a, groups, strs, part,    \
+        return launch_even(k_evc_pass<R, N>, a.nfree, grid, threads, sm, st, (const Cx<R> *)psi, a, groups, strs, part,    \
                       part_stride, xform);
     switch (ept) {
         SV_EVC_CASE(1)
@@ -5653,7 +5669,7 @@ cudaError_t hpsi_dispatch(cudaStream_t st, int grid, const void *psi, void *lam,
     }
 #define SV_HPSI_CASE(N)                                                                                      \
     case N:                                                                                                  \
-        return launch(k_hpsi_pass<R, N>, grid, threads, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, groups, \
+        return launch_even(k_hpsi_pass<R, N>, a.nfree, grid, threads, sm, st, (const Cx<R> *)psi, (Cx<R> *)lam, a, groups, \
                       strs, first, last, epart, status, limit);
     switch (ept) {
         SV_HPSI_CASE(1)

@@ -1,6 +1,6 @@
 """Strings without X and Y (the mask 0: |psi|^2 with signs), alone and among
-others, in the numbers at which complex128 groups of four and the choice between
-slices and whole cosets change.  Bounds as for the other expectation tests:
+others, in the numbers at which complex128 groups of four, the groups a mask is split into
+(256 strings) and the choice between slices and whole cosets change.  Bounds as for the other expectation tests:
 1e-5 and 1e-12."""
 import numpy as np
 import pytest
@@ -19,7 +19,7 @@ sv = pytest.importorskip("paper_2410_04252_gb300.sv")
 # fewer staged bits than the state's, one coset, both sides of the lines of both types
 @pytest.mark.parametrize("dtype,n", [(sv.C64, 8), (sv.C64, 13), (sv.C64, 17), (sv.C64, 20), (sv.C64, 22),
                                      (sv.C128, 8), (sv.C128, 12), (sv.C128, 18), (sv.C128, 19), (sv.C128, 20)])
-@pytest.mark.parametrize("zeros,others", [(1, 0), (3, 0), (4, 30), (5, 9), (47, 0), (200, 60)])
+@pytest.mark.parametrize("zeros,others", [(1, 0), (3, 0), (4, 30), (5, 9), (47, 0), (200, 60), (300, 0), (300, 40)])
 def test_mask_zero(dtype, n, zeros, others):
     rng = np.random.default_rng(100 * n + zeros)
     z = np.unique((rng.random((zeros, n)) < 0.4) * W.PZ, axis=0).astype(np.uint8)

@@ -49,3 +49,26 @@ def test_states_of_one_run(dtype, n, g, run, ham):
     which = list(range(0, c.nparams, max(1, c.nparams // 6)))
     fd = ograd.finite_difference(c, params, h, 3, which=which)
     assert np.max(np.abs(got[which] - fd[which])) < (1e-7 if dtype == sv.C128 else 2e-5 * l1)
+
+
+@pytest.mark.parametrize("dtype,n", [(sv.C64, 20), (sv.C64, 21), (sv.C128, 18), (sv.C128, 19)])
+def test_hamiltonian_passes_of_both_kinds(dtype, n):
+    # one mask with many strings and eleven with one: passes in slices and of whole cosets in one call
+    rng = np.random.default_rng(n)
+    x = [rng.random(n) < 0.4 for _ in range(12)]
+    rows = [np.where(x[0], rng.choice([W.PX, W.PY], n), rng.choice([0, W.PZ], n)) for _ in range(60)]
+    rows += [np.where(m, rng.choice([W.PX, W.PY], n), rng.choice([0, W.PZ], n)) for m in x[1:]]
+    h = W.Hamiltonian(n, np.array(rows, np.uint8), np.linspace(-1.0, 1.0, len(rows)))
+    psi = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    psi = (psi / np.linalg.norm(psi)).astype(np.complex64 if dtype == sv.C64 else np.complex128)
+    wide = psi.astype(np.complex128)
+    l1 = float(np.abs(h.coeffs).sum())
+    for order in (slice(None), slice(None, None, -1)):
+        part = W.Hamiltonian(n, h.letters[order], h.coeffs[order])
+        s = sv.StateVector(n, 0, dtype)
+        s.set_state(psi)
+        e, lam = s.apply_hamiltonian(part)
+        vtol = 2 * len(rows) * l1 * (2.0 ** -24 if dtype == sv.C64 else 2.0 ** -53) * float(np.max(np.abs(psi)))
+        assert np.max(np.abs(lam.cpu().numpy().astype(np.complex128) - oracle.apply_hamiltonian(wide, part))) < vtol
+        ref = float(np.dot(part.coeffs, oracle.expect_terms(wide, part).real))
+        assert abs(e - ref) < (1e-5 if dtype == sv.C64 else 1e-12) * l1
