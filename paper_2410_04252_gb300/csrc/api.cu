@@ -809,7 +809,9 @@ sv_status run_reverse(sv_handle *h, QsuEntry *q, sv_stats *st) {
     const int threads = adj_threads(h);
     const int nops = (int)P.ops.size();
     int grid = 1;
-    // one grid for all passes, so that every pass writes the same partial rows
+    // one grid for all passes, so that every pass writes the same partial rows;
+    // passes with 2- and 4-qubit matrices go gate by gate: adj_steps has no form
+    // for them (two sets of 16 amplitudes and a matrix row exceed the registers)
     for (auto &a : q->args) {
         int ga;
         if (a.ph_begin >= 0 && !a.dense) {

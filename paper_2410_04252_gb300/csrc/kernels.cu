@@ -5869,7 +5869,9 @@ int batch_occupancy(sv_dtype dt, int kmax, int hio, int threads) {
 
 // Step loops in the batched kernel: complex64 tiles of 2^13 with 512 threads
 // whose passes' tables fit beside them (the largest of `passes`; 0: they do
-// not).  Smaller states and the other tile and CTA sizes go gate by gate.
+// not).  batch_fwd and batch_adj are written for that tile (two of them and the
+// tables fill the SM); complex128, smaller states and other CTA sizes have no
+// such form and go gate by gate.
 int batch_table_room() { return smem_optin() - 2048 - (int)kBsTab; }
 size_t batch_step_bytes(sv_dtype dt, int n, int kmax, int threads, const std::vector<GatePassArgs> &passes) {
     if (dt != SV_C64 || kmax != 13 || threads != 512 || n < 13) return 0;
