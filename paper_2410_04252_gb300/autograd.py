@@ -21,7 +21,7 @@ class VQEEnergy(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, params, sim, circ, ham, schedule, init_index):
-        p = params.detach().cpu().to(torch.float64).resolve_neg().numpy()
+        p = params.detach().cpu().resolve_neg().to(torch.float64).numpy()
         sim.reset(init_index)
         if isinstance(ham, tuple):
             e, g = sim.grad(circ, p, paulis=ham[0], coeffs=ham[1], schedule=schedule)
