@@ -1082,16 +1082,25 @@ __device__ __forceinline__ MatRow<R, DIM> mat_row(const Cx<R> *M, int u) {
 }
 template <typename R, int DIM>
 __device__ __forceinline__ Cx<R> row_dot(const MatRow<R, DIM> &m, const Cx<R> *x) {
-    // four fused multiply-adds a term (complex128: FP64 operations bound it)
-    R re = m.m[0].x * x[0].x, im = m.m[0].x * x[0].y;
-    re = fma(-m.m[0].y, x[0].y, re);
-    im = fma(m.m[0].y, x[0].x, im);
+    // four fused multiply-adds a term (complex128: FP64 operations bound it), a
+    // long row in two chains a part: half as many roundings each
+    if constexpr (DIM == 2) {
+        R re = m.m[0].x * x[0].x, im = m.m[0].x * x[0].y;
+        re = fma(-m.m[0].y, x[0].y, re);
+        im = fma(m.m[0].y, x[0].x, im);
+        re = fma(-m.m[1].y, x[1].y, fma(m.m[1].x, x[1].x, re));
+        im = fma(m.m[1].y, x[1].x, fma(m.m[1].x, x[1].y, im));
+        return mk<R>(re, im);
+    }
+    R xx = m.m[0].x * x[0].x, yy = m.m[0].y * x[0].y, xy = m.m[0].x * x[0].y, yx = m.m[0].y * x[0].x;
 #pragma unroll
     for (int w = 1; w < DIM; ++w) {
-        re = fma(-m.m[w].y, x[w].y, fma(m.m[w].x, x[w].x, re));
-        im = fma(m.m[w].y, x[w].x, fma(m.m[w].x, x[w].y, im));
+        xx = fma(m.m[w].x, x[w].x, xx);
+        yy = fma(m.m[w].y, x[w].y, yy);
+        xy = fma(m.m[w].x, x[w].y, xy);
+        yx = fma(m.m[w].y, x[w].x, yx);
     }
-    return mk<R>(re, im);
+    return mk<R>(xx - yy, xy + yx);
 }
 // the dim x dim matrix on register bits B0 (and B1 > B0)
 template <typename R, int B0, int B1>
@@ -1377,7 +1386,7 @@ __device__ __forceinline__ void reg_tables(unsigned char *out, const RegLayout &
     for (int s = tid; s < nst; s += nthr) {
         if (st[s].type != SV_STEP_ROT) continue;
         int o = st[s].op_begin - a.op_begin, forms = st[s].a;
-        RunProduct<R> f;
+        RunProduct<R> f;                       // (complex64; complex128 multiplies the operations' factors below)
         for (int b = 0; b < RB; ++b) {
             if (!((st[s].a >> b) & 1)) continue;
             const Cx<R> k = cs[o];
@@ -1437,8 +1446,12 @@ __device__ __forceinline__ void reg_tables(unsigned char *out, const RegLayout &
             RunProduct<R> f;
             for (int q = 0; q < i; ++q) {
                 const int e = adj ? nst - 1 - q : q;
-                if (st[e].type == SV_STEP_ROT) f.mul(prod[e].x, prod[e].y);
-                else if (st[e].type == SV_STEP_SCALE && fabs(f.f) < kScaleBelow) f = RunProduct<R>();
+                if (st[e].type == SV_STEP_ROT) {
+                    if constexpr (sizeof(R) == 4)
+                        f.mul(prod[e].x, prod[e].y);
+                    else
+                        for (int o = st[e].op_begin - a.op_begin; o < st[e].op_end - a.op_begin; ++o) f.mul(cs[o].y, 0);
+                } else if (st[e].type == SV_STEP_SCALE && fabs(f.f) < kScaleBelow) f = RunProduct<R>();
             }
             const int s = i == nst ? nst : (adj ? nst - 1 - i : i);
             sc[s] = f.value();
